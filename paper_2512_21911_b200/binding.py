@@ -1,8 +1,9 @@
-"""ctypes binding of libsv.so: the same entry points as include/sv.h, taking torch CUDA tensors.
+"""Binding of libsv.so: the same entry points as include/sv.h, taking torch CUDA tensors.
 
 Argument marshalling only -- every step of the path runs in the library's CUDA kernels.  torch is
-used for device memory and streams.  There is no CPU fallback: importing this module fails if the
-compiled library is missing.
+used for device memory and streams.  The calls of a decoding loop are marshalled by the compiled module
+_native (csrc/py_native.cpp), the rest through ctypes.  There is no CPU fallback: importing this module fails if
+a compiled library is missing.
 """
 from __future__ import annotations
 
@@ -14,6 +15,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsv.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 SV_OK = 0
 SV_TAIL_BLOCK = -1   # sv_block_reps(block_begin=SV_TAIL_BLOCK): refresh only each sequence's last block
@@ -97,6 +99,9 @@ def _load() -> ctypes.CDLL:
 
 
 _lib = _load()
+if not os.path.exists(NATIVE_PATH):
+    raise ImportError(f"{NATIVE_PATH} is missing: build it with `python paper_2512_21911_b200/build.py`")
+from . import _native   # noqa: E402
 
 
 def _strerror(status: int) -> str:
@@ -152,66 +157,41 @@ def sv_verify_attn_splits(geom: sv_geom, max_sel: int) -> int:
 
 def sv_block_reps(geom: sv_geom, kv: sv_kv, reps: torch.Tensor, block_begin: int = 0, block_end: int = -1,
                   stream=None) -> None:
-    _check(_lib.sv_block_reps(ctypes.byref(geom), ctypes.byref(kv), block_begin, block_end,
-                              _ptr(reps, torch.float32, "reps"), _stream(stream)), "sv_block_reps")
+    _check(_native.block_reps(geom, kv, reps, block_begin, block_end, stream, False), "sv_block_reps")
 
 
 def sv_block_reps_bf16(geom: sv_geom, kv: sv_kv, reps_bf16: torch.Tensor, block_begin: int = 0, block_end: int = -1,
                        stream=None) -> None:
     """sv_block_reps with the representatives stored in bfloat16."""
-    _check(_lib.sv_block_reps_bf16(ctypes.byref(geom), ctypes.byref(kv), block_begin, block_end,
-                                   _ptr(reps_bf16, torch.bfloat16, "reps_bf16"), _stream(stream)), "sv_block_reps_bf16")
+    _check(_native.block_reps(geom, kv, reps_bf16, block_begin, block_end, stream, True), "sv_block_reps_bf16")
 
 
 def sv_select_blocks_bf16reps(geom: sv_geom, q, reps_bf16, seq_lens, budget_blocks, n_sink: int, n_local: int, out_idx,
                               out_cnt, reuse_prev: bool = False, prev_idx=None, prev_cnt=None, out_scores=None,
                               stream=None) -> None:
     """sv_select_blocks reading bfloat16 representatives."""
-    _check(_lib.sv_select_blocks_bf16reps(ctypes.byref(geom), _ptr(q, torch.bfloat16, "q"),
-                                          _ptr(reps_bf16, torch.bfloat16, "reps_bf16"),
-                                          _ptr(seq_lens, torch.int32, "seq_lens"),
-                                          _ptr(budget_blocks, torch.int32, "budget_blocks"), n_sink, n_local,
-                                          1 if reuse_prev else 0, _ptr(prev_idx, torch.int32, "prev_idx"),
-                                          _ptr(prev_cnt, torch.int32, "prev_cnt"), _ptr(out_idx, torch.int32, "out_idx"),
-                                          _ptr(out_cnt, torch.int32, "out_cnt"), int(out_idx.shape[-1]),
-                                          _ptr(out_scores, torch.float32, "out_scores"), _stream(stream)),
-           "sv_select_blocks_bf16reps")
+    _check(_native.select_blocks(geom, q, reps_bf16, seq_lens, budget_blocks, n_sink, n_local, out_idx, out_cnt, reuse_prev,
+                                 prev_idx, prev_cnt, out_scores, stream, True), "sv_select_blocks_bf16reps")
 
 
 def sv_select_blocks(geom: sv_geom, q, reps, seq_lens, budget_blocks, n_sink: int, n_local: int, out_idx, out_cnt,
                      reuse_prev: bool = False, prev_idx=None, prev_cnt=None, out_scores=None, stream=None) -> None:
-    max_sel = int(out_idx.shape[-1])
-    _check(_lib.sv_select_blocks(ctypes.byref(geom), _ptr(q, torch.bfloat16, "q"), _ptr(reps, torch.float32, "reps"),
-                                 _ptr(seq_lens, torch.int32, "seq_lens"),
-                                 _ptr(budget_blocks, torch.int32, "budget_blocks"), n_sink, n_local,
-                                 1 if reuse_prev else 0, _ptr(prev_idx, torch.int32, "prev_idx"),
-                                 _ptr(prev_cnt, torch.int32, "prev_cnt"), _ptr(out_idx, torch.int32, "out_idx"),
-                                 _ptr(out_cnt, torch.int32, "out_cnt"), max_sel,
-                                 _ptr(out_scores, torch.float32, "out_scores"), _stream(stream)), "sv_select_blocks")
+    _check(_native.select_blocks(geom, q, reps, seq_lens, budget_blocks, n_sink, n_local, out_idx, out_cnt, reuse_prev,
+                                 prev_idx, prev_cnt, out_scores, stream, False), "sv_select_blocks")
 
 
 def sv_verify_attn(geom: sv_geom, q, kv: sv_kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse=None,
-                   workspace=None, softmax_scale: float = 0.0, status_word=None, stream=None, _fn=None, _name="sv_verify_attn") -> None:
-    max_sel = int(sel_idx.shape[-1]) if sel_idx is not None else int(geom.max_blocks)
-    ws_ptr = workspace.data_ptr() if workspace is not None else None
-    ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    if workspace is not None and not workspace.is_cuda:
-        raise TypeError("workspace must be a CUDA tensor")
-    _check((_fn or _lib.sv_verify_attn)(ctypes.byref(geom), _ptr(q, torch.bfloat16, "q"), ctypes.byref(kv),
-                               _ptr(draft_k, torch.bfloat16, "draft_k"), _ptr(draft_v, torch.bfloat16, "draft_v"),
-                               _ptr(parent, torch.int32, "parent"), _ptr(sel_idx, torch.int32, "sel_idx"),
-                               _ptr(sel_cnt, torch.int32, "sel_cnt"), max_sel, float(softmax_scale),
-                               _ptr(out, torch.bfloat16, "out"), _ptr(lse, torch.float32, "lse"), ws_ptr, ws_bytes,
-                               _ptr(status_word, torch.int32, "status_word"), _stream(stream)), _name)
+                   workspace=None, softmax_scale: float = 0.0, status_word=None, stream=None) -> None:
+    _check(_native.verify_attn(geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse, workspace, softmax_scale,
+                               status_word, stream, 0), "sv_verify_attn")
 
 
 def sv_verify_attn_reused(geom: sv_geom, q, kv: sv_kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse=None,
                           workspace=None, softmax_scale: float = 0.0, status_word=None, stream=None) -> None:
     """sv_verify_attn for a layer that reuses an earlier layer's block list: the caller vouches that the list, the tables,
     the lengths and the K/V pools are not written by the kernel just before, and the gather starts ahead of it."""
-    sv_verify_attn(geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse=lse, workspace=workspace,
-                   softmax_scale=softmax_scale, status_word=status_word, stream=stream, _fn=_lib.sv_verify_attn_reused,
-                   _name="sv_verify_attn_reused")
+    _check(_native.verify_attn(geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse, workspace, softmax_scale,
+                               status_word, stream, 1), "sv_verify_attn_reused")
 
 
 def sv_verify_attn_noalloc(geom: sv_geom, q, kv: sv_kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse=None,
@@ -223,27 +203,16 @@ def sv_verify_attn_noalloc(geom: sv_geom, q, kv: sv_kv, draft_k, draft_v, parent
     input and output tensors are passed through.  Problems whose partials do not fit raise
     SvError(SV_ERR_SCRATCH_LIMIT).  All calls on a device share that array, so calls that may overlap on
     the GPU must be serialised by the caller; make the first call on a device outside any stream capture."""
-    max_sel = int(sel_idx.shape[-1]) if sel_idx is not None else int(geom.max_blocks)
-    _check(_lib.sv_verify_attn_noalloc(ctypes.byref(geom), _ptr(q, torch.bfloat16, "q"), ctypes.byref(kv),
-                                       _ptr(draft_k, torch.bfloat16, "draft_k"),
-                                       _ptr(draft_v, torch.bfloat16, "draft_v"), _ptr(parent, torch.int32, "parent"),
-                                       _ptr(sel_idx, torch.int32, "sel_idx"), _ptr(sel_cnt, torch.int32, "sel_cnt"),
-                                       max_sel, float(softmax_scale), _ptr(out, torch.bfloat16, "out"),
-                                       _ptr(lse, torch.float32, "lse"), _ptr(status_word, torch.int32, "status_word"),
-                                       _stream(stream)), "sv_verify_attn_noalloc")
+    _check(_native.verify_attn(geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse, None, softmax_scale,
+                               status_word, stream, 2), "sv_verify_attn_noalloc")
 
 
 def sv_kv_append(geom: sv_geom, k_pool, v_pool, block_table, seq_lens, draft_k, draft_v, accept_idx, n_accept,
                  seq_lens_out, reps=None, stream=None) -> None:
     """Commit accepted draft tokens to the paged cache (pools modified in place), write the new lengths to
     seq_lens_out (a different tensor than seq_lens) and refresh the representatives of the grown blocks."""
-    _check(_lib.sv_kv_append(ctypes.byref(geom), _ptr(k_pool, torch.bfloat16, "k_pool"), _ptr(v_pool, torch.bfloat16, "v_pool"),
-                             int(k_pool.shape[0]), _ptr(block_table, torch.int32, "block_table"),
-                             _ptr(seq_lens, torch.int32, "seq_lens"), _ptr(draft_k, torch.bfloat16, "draft_k"),
-                             _ptr(draft_v, torch.bfloat16, "draft_v"), _ptr(accept_idx, torch.int32, "accept_idx"),
-                             _ptr(n_accept, torch.int32, "n_accept"), int(accept_idx.shape[-1]),
-                             _ptr(seq_lens_out, torch.int32, "seq_lens_out"), _ptr(reps, torch.float32, "reps"),
-                             _stream(stream)), "sv_kv_append")
+    _check(_native.kv_append(geom, k_pool, v_pool, block_table, seq_lens, draft_k, draft_v, accept_idx, n_accept, seq_lens_out,
+                             reps, stream), "sv_kv_append")
 
 
 def sv_anchor_jaccard(geom: sv_geom, sel_idx_all, sel_cnt_all, inter, uni, stream=None) -> None:
@@ -291,12 +260,8 @@ def sv_accept(p_target, p_draft, tokens, parent, u_accept, u_next, path, n_path,
     S, T, V = (int(x) for x in p_target.shape)
     if tuple(p_draft.shape) != (S, T, V) or tuple(tokens.shape) != (S, T) or tuple(path.shape) != (S, T):
         raise ValueError("sv_accept: shapes disagree")
-    _check(_lib.sv_accept(S, T, V, _ptr(p_target, torch.float32, "p_target"), _ptr(p_draft, torch.float32, "p_draft"),
-                          _ptr(tokens, torch.int32, "tokens"), _ptr(parent, torch.int32, "parent"),
-                          _ptr(u_accept, torch.float32, "u_accept"), _ptr(u_next, torch.float32, "u_next"),
-                          _ptr(path, torch.int32, "path"), _ptr(n_path, torch.int32, "n_path"),
-                          _ptr(next_token, torch.int32, "next_token"), _ptr(alpha, torch.float32, "alpha"),
-                          _stream(stream)), "sv_accept")
+    _check(_native.accept(p_target, p_draft, tokens, parent, u_accept, u_next, path, n_path, next_token, alpha, stream),
+           "sv_accept")
 
 
 def sv_pick_anchors(inter, uni, n_anchors: int):

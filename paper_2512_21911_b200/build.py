@@ -1,14 +1,19 @@
-"""Compile the CUDA sources under csrc/ into libsv.so (sm_100a only) next to this file."""
+"""Compile the CUDA sources under csrc/ into libsv.so (sm_100a only) and the Python module over it into _native.so, both next
+to this file."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsv.so")
+NATIVE = os.path.join(HERE, "_native.so")
+NATIVE_SOURCE = os.path.join(CSRC, "py_native.cpp")
 SOURCES = ["sv_api.cu", "block_reps.cu", "select_blocks.cu", "verify_attn.cu", "verify_attn_tc.cu", "kv_append.cu", "anchor_calib.cu",
            "select_variants.cu", "accept.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,11 +28,22 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def _native_command(out: str) -> list:
+    torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]   # without importing torch
+    inc = os.path.join(torch_dir, "include")
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", NATIVE_SOURCE, "-o", out,
+            "-I", os.path.join(ROOT, "include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
+            "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"],
+            "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+            "-L", HERE, "-l:libsv.so", "-Wl,-rpath,$ORIGIN"]
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(NATIVE)):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "sv.h"), __file__]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".o")] + [os.path.join(ROOT, "include", "sv.h"), __file__]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
@@ -53,6 +69,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".{os.getpid()}.tmp"
     subprocess.run([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"], check=True)
     os.replace(tmp, LIB)
+    tmp = NATIVE + f".{os.getpid()}.tmp"
+    subprocess.run(_native_command(tmp), check=True)
+    os.replace(tmp, NATIVE)
     return LIB
 
 

@@ -1,0 +1,265 @@
+// Python side of the C ABI: argument marshalling from torch tensors to the entry points of sv.h, as a CPython module.
+//
+// A layer of a verification step is two or three kernel launches (about 2.5 us of host time each), and a short one runs
+// for less than 10 us, so what the host spends between launches is what a small call costs: the same marshalling in
+// Python (type, device, dtype and layout checks per tensor, a ctypes call of 16 arguments) took 10-12 us per entry
+// point.  Here a tensor is unpacked and checked in a few tens of nanoseconds: back to back, an eager layer of a small model
+// (4K context) went from 30.5 to 12.3 us, an eager 32-layer step from 995 to 499 us.  The checks and the errors are those of
+// the Python binding: a tensor that is not a contiguous CUDA tensor of the expected type raises TypeError before
+// anything is launched, and the sv_status of the call is returned for the caller to map.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "sv.h"
+
+namespace {
+
+// A failed argument check: the Python exception is set, the call returns NULL.
+struct ArgError {};
+
+const at::Tensor &tensor(PyObject *o, at::ScalarType type, const char *name)
+{
+    if (THPVariable_Check(o)) {
+        const at::Tensor &t = THPVariable_Unpack(o);
+        if (t.is_cuda() && t.scalar_type() == type && t.is_contiguous()) return t;
+    }
+    PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor of torch.%s", name,
+                 type == at::kBFloat16 ? "bfloat16" : type == at::kFloat ? "float32" : "int32");
+    throw ArgError{};
+}
+
+// Device pointer of a tensor argument (None: NULL).
+void *ptr(PyObject *o, at::ScalarType type, const char *name)
+{
+    return o == Py_None ? nullptr : tensor(o, type, name).data_ptr();
+}
+void *bf16(PyObject *o, const char *name) { return ptr(o, at::kBFloat16, name); }
+float *f32(PyObject *o, const char *name) { return static_cast<float *>(ptr(o, at::kFloat, name)); }
+int32_t *i32(PyObject *o, const char *name) { return static_cast<int32_t *>(ptr(o, at::kInt, name)); }
+
+long long integer(PyObject *o)
+{
+    const long long v = PyLong_AsLongLong(o);
+    if (v == -1 && PyErr_Occurred()) throw ArgError{};
+    return v;
+}
+int32_t int32(PyObject *o)
+{
+    const long long v = integer(o);
+    if (v < INT32_MIN || v > INT32_MAX) {
+        PyErr_SetString(PyExc_OverflowError, "value does not fit in 32 bits");
+        throw ArgError{};
+    }
+    return (int32_t)v;
+}
+bool truth(PyObject *o)
+{
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) throw ArgError{};
+    return v != 0;
+}
+
+// A ctypes structure (sv_geom, sv_kv) by its bytes.
+template <class T>
+T structure(PyObject *o, const char *name)
+{
+    Py_buffer view;
+    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) {
+        PyErr_Format(PyExc_TypeError, "expected an %s", name);
+        throw ArgError{};
+    }
+    const bool fits = view.len == (Py_ssize_t)sizeof(T);
+    T v;
+    if (fits) memcpy(&v, view.buf, sizeof(T));
+    PyBuffer_Release(&view);
+    if (!fits) {
+        PyErr_Format(PyExc_TypeError, "expected an %s", name);
+        throw ArgError{};
+    }
+    return v;
+}
+sv_geom geometry(PyObject *o) { return structure<sv_geom>(o, "sv_geom"); }
+sv_kv cache(PyObject *o) { return structure<sv_kv>(o, "sv_kv"); }
+
+// The stream argument of the binding: a torch stream, or None for the current one.
+void *stream(PyObject *o)
+{
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    PyObject *h = PyObject_GetAttrString(o, "cuda_stream");
+    if (!h) throw ArgError{};
+    void *s = PyLong_AsVoidPtr(h);
+    Py_DECREF(h);
+    if (!s && PyErr_Occurred()) throw ArgError{};
+    return s;
+}
+
+// Last dimension of a list tensor: the row length max_sel.
+int32_t row_length(PyObject *o, const char *name) { return (int32_t)tensor(o, at::kInt, name).size(-1); }
+
+struct Scratch {
+    void *p;
+    size_t bytes;
+};
+Scratch scratch(PyObject *o)
+{
+    if (o == Py_None) return {nullptr, 0};
+    if (!THPVariable_Check(o) || !THPVariable_Unpack(o).is_cuda()) {
+        PyErr_SetString(PyExc_TypeError, "workspace must be a CUDA tensor");
+        throw ArgError{};
+    }
+    const at::Tensor &t = THPVariable_Unpack(o);
+    return {t.data_ptr(), (size_t)t.nbytes()};
+}
+
+// Every method: exactly N positional arguments, body returns a PyObject*.
+template <class F>
+PyObject *checked(Py_ssize_t n, Py_ssize_t want, F body)
+{
+    if (n != want) {
+        PyErr_Format(PyExc_TypeError, "expected %zd arguments, got %zd", want, n);
+        return nullptr;
+    }
+    try {
+        return body();
+    } catch (const ArgError &) {
+        return nullptr;
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+PyObject *status(sv_status st) { return PyLong_FromLong(st); }
+
+// geom, kv, reps, block_begin, block_end, stream, reps_bf16
+PyObject *block_reps(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 7, [&] {
+        const sv_geom g = geometry(a[0]);
+        const sv_kv kv = cache(a[1]);
+        if (truth(a[6])) return status(sv_block_reps_bf16(&g, &kv, int32(a[3]), int32(a[4]), bf16(a[2], "reps_bf16"), stream(a[5])));
+        return status(sv_block_reps(&g, &kv, int32(a[3]), int32(a[4]), f32(a[2], "reps"), stream(a[5])));
+    });
+}
+
+// geom, q, reps, seq_lens, budget_blocks, n_sink, n_local, out_idx, out_cnt, reuse_prev, prev_idx, prev_cnt, out_scores,
+// stream, reps_bf16
+PyObject *select_blocks(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 15, [&] {
+        const sv_geom g = geometry(a[0]);
+        const int32_t max_sel = row_length(a[7], "out_idx");
+        const void *q = bf16(a[1], "q");
+        const int32_t *lens = i32(a[3], "seq_lens"), *budget = i32(a[4], "budget_blocks");
+        const int32_t sink = int32(a[5]), local = int32(a[6]);
+        int32_t *idx = i32(a[7], "out_idx"), *cnt = i32(a[8], "out_cnt");
+        const int32_t reuse = truth(a[9]) ? 1 : 0;
+        const int32_t *pi = i32(a[10], "prev_idx"), *pc = i32(a[11], "prev_cnt");
+        float *scores = f32(a[12], "out_scores");
+        if (truth(a[14]))
+            return status(sv_select_blocks_bf16reps(&g, q, bf16(a[2], "reps_bf16"), lens, budget, sink, local, reuse, pi, pc, idx,
+                                                    cnt, max_sel, scores, stream(a[13])));
+        return status(sv_select_blocks(&g, q, f32(a[2], "reps"), lens, budget, sink, local, reuse, pi, pc, idx, cnt, max_sel,
+                                       scores, stream(a[13])));
+    });
+}
+
+// geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, out, lse, workspace, softmax_scale, status_word, stream, entry
+// (entry 0: sv_verify_attn, 1: sv_verify_attn_reused, 2: sv_verify_attn_noalloc)
+PyObject *verify_attn(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 15, [&] {
+        const sv_geom g = geometry(a[0]);
+        const sv_kv kv = cache(a[2]);
+        const int32_t max_sel = a[6] == Py_None ? g.max_blocks : row_length(a[6], "sel_idx");
+        const void *q = bf16(a[1], "q"), *dk = bf16(a[3], "draft_k"), *dv = bf16(a[4], "draft_v");
+        const int32_t *parent = i32(a[5], "parent"), *idx = i32(a[6], "sel_idx"), *cnt = i32(a[7], "sel_cnt");
+        void *out = bf16(a[8], "out");
+        float *lse = f32(a[9], "lse");
+        const Scratch ws = scratch(a[10]);
+        const double scale = PyFloat_AsDouble(a[11]);
+        if (scale == -1.0 && PyErr_Occurred()) throw ArgError{};
+        int32_t *word = i32(a[12], "status_word");
+        void *s = stream(a[13]);
+        switch (integer(a[14])) {
+            case 0: return status(sv_verify_attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s));
+            case 1: return status(sv_verify_attn_reused(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s));
+            default: return status(sv_verify_attn_noalloc(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, word, s));
+        }
+    });
+}
+
+// geom, k_pool, v_pool, block_table, seq_lens, draft_k, draft_v, accept_idx, n_accept, seq_lens_out, reps, stream
+PyObject *kv_append(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 12, [&] {
+        const sv_geom g = geometry(a[0]);
+        const int32_t pages = (int32_t)tensor(a[1], at::kBFloat16, "k_pool").size(0);
+        return status(sv_kv_append(&g, bf16(a[1], "k_pool"), bf16(a[2], "v_pool"), pages, i32(a[3], "block_table"),
+                                   i32(a[4], "seq_lens"), bf16(a[5], "draft_k"), bf16(a[6], "draft_v"), i32(a[7], "accept_idx"),
+                                   i32(a[8], "n_accept"), row_length(a[7], "accept_idx"), i32(a[9], "seq_lens_out"),
+                                   f32(a[10], "reps"), stream(a[11])));
+    });
+}
+
+// p_target, p_draft, tokens, parent, u_accept, u_next, path, n_path, next_token, alpha, stream
+PyObject *accept(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 11, [&] {
+        const at::Tensor &pt = tensor(a[0], at::kFloat, "p_target");
+        const int32_t S = (int32_t)pt.size(0), T = (int32_t)pt.size(1), V = (int32_t)pt.size(2);
+        return status(sv_accept(S, T, V, f32(a[0], "p_target"), f32(a[1], "p_draft"), i32(a[2], "tokens"), i32(a[3], "parent"),
+                                f32(a[4], "u_accept"), f32(a[5], "u_next"), i32(a[6], "path"), i32(a[7], "n_path"),
+                                i32(a[8], "next_token"), f32(a[9], "alpha"), stream(a[10])));
+    });
+}
+
+// One layer of a verification step: selection (an anchor layer) into sel_idx / sel_cnt or the reuse of what is there, then
+// attention, on the current stream.
+// geom, kv, q, reps [layers][...], layer, seq_lens, budget, n_sink, n_local, sel_idx, sel_cnt, draft_k, draft_v, parent, out,
+// lse, workspace, status_word, anchor, behind_own_layer -> (status, whether it is the selection's)
+PyObject *verify_layer(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 20, [&]() -> PyObject * {
+        const sv_geom g = geometry(a[0]);
+        const sv_kv kv = cache(a[1]);
+        const void *q = bf16(a[2], "q");
+        int32_t *idx = i32(a[9], "sel_idx"), *cnt = i32(a[10], "sel_cnt");
+        const int32_t max_sel = row_length(a[9], "sel_idx");
+        const void *dk = bf16(a[11], "draft_k"), *dv = bf16(a[12], "draft_v");
+        const int32_t *parent = i32(a[13], "parent");
+        void *out = bf16(a[14], "out");
+        float *lse = f32(a[15], "lse");
+        const Scratch ws = scratch(a[16]);
+        int32_t *word = i32(a[17], "status_word");
+        const bool anchor = truth(a[18]), behind = truth(a[19]);
+        void *s = stream(Py_None);
+        if (anchor) {
+            const at::Tensor &reps = tensor(a[3], at::kFloat, "reps");
+            long long layer = integer(a[4]);
+            if (layer < 0) layer += reps.size(0);
+            const float *r = reps.data_ptr<float>() + layer * reps.stride(0);
+            const sv_status st = sv_select_blocks(&g, q, r, i32(a[5], "seq_lens"), i32(a[6], "budget_blocks"), int32(a[7]), int32(a[8]),
+                                                  0, nullptr, nullptr, idx, cnt, max_sel, nullptr, s);
+            if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_True);
+        }
+        auto attn = behind && !anchor ? sv_verify_attn_reused : sv_verify_attn;
+        const sv_status st = attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, 0.f, out, lse, ws.p, ws.bytes, word, s);
+        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_False);
+        Py_RETURN_NONE;
+    });
+}
+
+#define METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {METHOD(block_reps), METHOD(select_blocks), METHOD(verify_attn), METHOD(kv_append), METHOD(accept),
+                         METHOD(verify_layer), {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the entry points of sv.h.", -1, methods,
+                      nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__native(void) { return PyModule_Create(&module); }

@@ -85,15 +85,12 @@ class SparseVerifier:
         behind_own_layer: the kernel just before this call in the stream is the preceding layer's attention / merge
         (as inside verify_step), which writes neither the block list nor the cache: a layer that reuses the list
         then starts its gather while that kernel drains (sv_verify_attn_reused)."""
-        if self.anchors[layer]:
-            sv.sv_select_blocks(self.geom, q, self.reps[layer], self.seq_lens, self.budget, self.n_sink,
-                                self.n_local, self.sel_idx, self.sel_cnt)
-        else:   # Eq. 9: same list as the preceding layer; in place, so nothing is launched
-            sv.sv_select_blocks(self.geom, None, None, None, None, self.n_sink, self.n_local, self.sel_idx,
-                                self.sel_cnt, reuse_prev=True, prev_idx=self.sel_idx, prev_cnt=self.sel_cnt)
-        attn = sv.sv_verify_attn_reused if (behind_own_layer and not self.anchors[layer]) else sv.sv_verify_attn
-        attn(self.geom, q, self.kv[layer], draft_k, draft_v, self.parent, self.sel_idx, self.sel_cnt, out, lse=lse,
-             workspace=self.workspace, status_word=self.status)
+        # a layer that reuses (Eq. 9) finds the preceding layer's list in place, so nothing is launched for it
+        failed = sv._native.verify_layer(self.geom, self.kv[layer], q, self.reps, layer, self.seq_lens, self.budget, self.n_sink,
+                                         self.n_local, self.sel_idx, self.sel_cnt, draft_k, draft_v, self.parent, out, lse,
+                                         self.workspace, self.status, self.anchors[layer], behind_own_layer)
+        if failed:
+            raise sv.SvError(failed[0], "sv_select_blocks" if failed[1] else "sv_verify_attn")
 
     def dense_layer(self, layer: int, q, draft_k, draft_v, out, lse=None) -> None:
         """Dense ("strict") verification attention over every cached block, for comparison."""
