@@ -7,7 +7,7 @@ Workload: the Llama-3.1-8B-shaped attention stack (32 layers, 32 query / 8 KV he
 bf16, batch 1, 32768 cached tokens in 64-token blocks, 64 kept blocks, 8 draft tokens as a chain),
 seeded synthetic tensors from sv_inputs.  One step = one pass of the whole hot path over all 32
 layers: refresh of the tail block's representative, block selection (every layer), sparse verification
-attention (split-KV + merge), the kernels chained by programmatic dependent launch.  The step is captured in a CUDA graph; K replays are timed with CUDA
+attention (split-KV + merge), layer after layer as a model reaches them, the kernels chained by programmatic dependent launch.  The step is captured in a CUDA graph; K replays are timed with CUDA
 events between barriers.  Every layer has its own 128 MiB KV pool and a step gathers 512 MiB from a
 4 GiB working set, so no iteration finds its K/V in the 126 MB L2.
 
@@ -333,7 +333,14 @@ def run_gpu(args):
         nvtx.range_pop()
         stream.synchronize()
     nvtx.range_push("capture")
-    g_step = capture(lambda: eng.verify_step(q, dk, dv, out, refresh_tail=True))
+
+    def by_layer(e, b=(q, dk, dv, out)):
+        """A step in the order in which a model reaches its layers: tail refresh of the stack, then layer after layer."""
+        e.refresh_tail_all()
+        for l in range(w.n_layers):
+            e.verify_layer(l, b[0][l], b[1][l], b[2][l], b[3][l], behind_own_layer=l > 0)
+
+    g_step = capture(lambda: by_layer(eng))
     nvtx.range_pop()
     if args.only_step:
         ms = time_replays(g_step, args.steps, args.warmup)
@@ -341,12 +348,13 @@ def run_gpu(args):
             print(json.dumps({"only_step": True, "layers": w.n_layers, "us_per_layer": ms * 1e3 / w.n_layers,
                               "kernels_per_step": eng.kernels_per_step(refresh_tail=True)}))
         return
-    g_reuse = capture(lambda: eng_reuse.verify_step(q, dk, dv, out, refresh_tail=True))
-    g_chain = capture(lambda: eng_chain.verify_step(q, dk, dv, out, refresh_tail=True))
+    g_reuse = capture(lambda: by_layer(eng_reuse))
+    g_chain = capture(lambda: by_layer(eng_chain))
     g_attn = capture(lambda: [sv.sv_verify_attn(eng.geom, q[l], eng.kv[l], dk[l], dv[l], None, eng.sel_idx, eng.sel_cnt,
                                                 out[l], workspace=eng.workspace, status_word=eng.status)
                               for l in range(w.n_layers)])
-    g_dense = capture(lambda: eng.dense_step(q, dk, dv, out))
+    g_dense = capture(lambda: [eng.dense_layer(l, q[l], dk[l], dv[l], out[l]) for l in range(w.n_layers)])
+    g_stack = capture(lambda: eng.verify_step(q, dk, dv, out, refresh_tail=True))   # the inputs of all layers at once
     # full rebuild of the block representatives of every layer (prefill-time cost; the step only refreshes tails)
     reps_scratch = torch.empty_like(eng.reps[0])
     g_reps = capture(lambda: [sv.sv_block_reps(eng.geom, eng.kv[l], reps_scratch) for l in range(w.n_layers)])
@@ -358,6 +366,7 @@ def run_gpu(args):
     side = max(10, min(args.steps, 200))
     ms_reuse = time_replays(g_reuse, side, 3)
     ms_chain = time_replays(g_chain, side, 3)
+    ms_stack = time_replays(g_stack, side, 3)
     ms_attn = time_replays(g_attn, side, 3)
     ms_dense = time_replays(g_dense, max(5, side // 4), 3)
     ms_reps = time_replays(g_reps, max(5, side // 4), 3)
@@ -366,7 +375,7 @@ def run_gpu(args):
     # outputs back.  Two sets of device buffers and three streams (copy-in, compute, copy-out) let the copies of
     # step i+1 / i-1 run under the kernels of step i; every step still pays its own copies inside the region.
     bufs = [(q, dk, dv, out), (torch.empty_like(q), torch.empty_like(dk), torch.empty_like(dv), torch.empty_like(out))]
-    graphs = [g_step, capture(lambda: eng.verify_step(bufs[1][0], bufs[1][1], bufs[1][2], bufs[1][3], refresh_tail=True))]
+    graphs = [g_step, capture(lambda: by_layer(eng, bufs[1]))]
     outs_h = [out_h, torch.empty_like(out_h).pin_memory()]
     s_in, s_out = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
 
@@ -446,6 +455,9 @@ def run_gpu(args):
     g_host = capture(lambda: eng.verify_step_from_host(q_h, dk_h, dv_h, q, dk, dv, out, out_h,
                                                        layers_per_chunk=e2e_chunks, refresh_tail=True))
     ms_e2e = time_e2e_serial(side, 4, g_host)
+    with torch.cuda.stream(stream):
+        g_stack.replay()
+        stream.synchronize()
     assert torch.equal(out_h, out.cpu()), "the host-fed step did not deliver the step's outputs"
     assert int(eng.status.item()) == 0 and int(eng_reuse.status.item()) == 0 and int(eng_chain.status.item()) == 0, \
         "a kernel gave up on a bounded wait"
@@ -460,6 +472,8 @@ def run_gpu(args):
     ms_step, ms_reuse, ms_chain, ms_attn, ms_dense, ms_e2e, ms_reps, ms_e2e_pipelined, ms_e2e_one_stream = (
         aggregate_over_ranks(x, world, allmax)[0]
         for x in (ms_step, ms_reuse, ms_chain, ms_attn, ms_dense, ms_e2e, ms_reps, ms_e2e_pipelined, ms_e2e_one_stream))
+
+    ms_stack = aggregate_over_ranks(ms_stack, world, allmax)[0]
 
     # algorithmic bytes of one sv_verify_attn launch (K+V of the kept tokens and draft tokens, Q in, O out)
     S, T, Hq, Hkv, D, B, N = w.n_seq, w.n_draft, w.n_q_heads, w.n_kv_heads, w.head_dim, w.block_size, w.budget_blocks
@@ -509,6 +523,9 @@ def run_gpu(args):
         "reuse_even_anchors": {"us_per_layer": ms_reuse * 1e3 / w.n_layers, "kernels_per_step": eng_reuse.kernels_per_step(True)},
         "reuse_previous_layer": {"us_per_layer": ms_chain * 1e3 / w.n_layers, "kernels_per_step": eng_chain.kernels_per_step(True),
                                  "note": "only layer 0 retrieves; every later layer attends over the previous layer's blocks"},
+        "all_layers_at_once": {"us_per_layer": ms_stack * 1e3 / w.n_layers,
+                               "note": "verify_step with the inputs of all layers in hand: one launch for all selections, one "
+                                       "for all attention (what the host-fed step runs per chunk); `value` goes layer by layer"},
         "dense_verify": {"us_per_layer": us_dense, "gbs": dense_bytes / (us_dense * 1e-6) / 1e9,
                          "frac": dense_bytes / (us_dense * 1e-6) / 1e9 / peak, "bytes_per_launch": dense_bytes},
         "block_reps_rebuild": {"us_per_layer": ms_reps * 1e3 / w.n_layers, "bytes_per_launch": reps_bytes,

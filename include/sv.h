@@ -373,6 +373,53 @@ SV_API sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, const 
                            const int32_t *tokens, const int32_t *parent, const float *u_accept, const float *u_next,
                            int32_t *path, int32_t *n_path, int32_t *next_token, float *alpha, void *stream);
 
+/*
+ * Several layers of a stack in one launch.  A caller that holds the queries of more than one layer (a step whose
+ * inputs for all layers are there at once) need not pay a layer's chain of latencies for each of them: the layers are
+ * independent problems but for the lists that non-anchor layers reuse (Eq. 9), and together they fill the GPU.
+ *
+ * sv_layer_table writes one row per layer (tensor maps over its pools, pool pointers, page count) to host memory;
+ * the caller copies the sv_layer_table_bytes(n_layers) bytes to device memory, 64-byte aligned, and keeps them as long
+ * as the pools.  All layers share the page table and the lengths (block_table / seq_lens of sv_layers; those of the
+ * sv_kv array are only checked).  n_layers <= SV_MAX_LAYERS, n_seq * n_layers <= 65535.
+ *
+ * In the calls below everything a layer owns is stacked over all n_layers layers -- q / out [L][S][T][Hq][D],
+ * draft_k / draft_v [L][S][T][Hkv][D], reps [L][S][Hkv][NBmax][D] -- and layers first <= l < end are processed.
+ * anchors (host, uint8 [L], anchors[0] != 0): the layers that select; lists are numbered by anchor,
+ * idx [A][S][Hkv][max_sel], cnt [A][S][Hkv], and a layer attends over the list of the last anchor up to it.
+ * Results are those of the single-layer calls; the splits of the attention are chosen for the whole stack, so that a
+ * layer's result does not depend on the layers it is launched with.
+ *   sv_block_reps_layers   layers l with which[l] != 0 (host, uint8 [L]; NULL: all)
+ *   sv_verify_attn_layers  sel_idx == NULL: dense verification (anchors may be NULL); workspace of
+ *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes
+ *   sv_kv_append_layers    advances seq_lens (which must be layers->seq_lens) in place; counters: dev uint32 [2 S], zeroed
+ *                          once by the caller and left to this call from then on
+ */
+#define SV_MAX_LAYERS 256
+typedef struct {
+    const void *table;          /* dev: rows written by sv_layer_table */
+    const int32_t *block_table; /* dev int32 [S][NBmax] */
+    const int32_t *seq_lens;    /* dev int32 [S] */
+    int32_t n_layers;           /* L: rows of the table */
+} sv_layers;
+SV_API size_t sv_layer_table_bytes(int32_t n_layers);
+SV_API sv_status sv_layer_table(const sv_geom *geom, const sv_kv *kv, int32_t n_layers, void *table_host);
+SV_API size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layers, int32_t max_sel);
+SV_API sv_status sv_block_reps_layers(const sv_geom *geom, const sv_layers *layers, const uint8_t *which, int32_t block_begin,
+                                      int32_t block_end, float *reps, void *stream);
+SV_API sv_status sv_select_blocks_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                         const uint8_t *anchors, const void *q, const float *reps,
+                                         const int32_t *budget_blocks, int32_t n_sink, int32_t n_local, int32_t *out_idx,
+                                         int32_t *out_cnt, int32_t max_sel, void *stream);
+SV_API sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                       const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
+                                       const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                       int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                                       size_t workspace_bytes, int32_t *status_word, void *stream);
+SV_API sv_status sv_kv_append_layers(const sv_geom *geom, const sv_layers *layers, const void *draft_k, const void *draft_v,
+                                     const int32_t *accept_idx, const int32_t *n_accept, int32_t max_accept,
+                                     int32_t *seq_lens, uint32_t *counters, float *reps, void *stream);
+
 /* Number of KV splits (CTAs per (sequence, KV head)) sv_verify_attn uses for this geometry. */
 SV_API int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel);
 

@@ -29,7 +29,9 @@ SV_NOALLOC_SCRATCH_BYTES = 4 * 1024 * 1024   # size of the library's built-in sc
 EXPORTS = ("sv_strerror", "sv_status_word_check", "sv_budget_blocks", "sv_workspace_bytes", "sv_block_reps", "sv_select_blocks",
            "sv_verify_attn", "sv_verify_attn_reused", "sv_verify_attn_splits", "sv_verify_attn_noalloc", "sv_kv_append", "sv_anchor_jaccard", "sv_pick_anchors",
            "sv_select_blocks_tokens", "sv_token_overlap", "sv_select_blocks_global", "sv_accept",
-           "sv_block_reps_bf16", "sv_select_blocks_bf16reps")
+           "sv_block_reps_bf16", "sv_select_blocks_bf16reps", "sv_layer_table_bytes", "sv_layer_table", "sv_workspace_bytes_layers",
+           "sv_block_reps_layers", "sv_select_blocks_layers", "sv_verify_attn_layers", "sv_kv_append_layers")
+SV_MAX_LAYERS = 256
 
 
 class SvError(RuntimeError):

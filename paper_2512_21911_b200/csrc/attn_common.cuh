@@ -13,6 +13,15 @@ namespace svk {
 constexpr int kStatusIndex = SV_STATUS_INDEX;   // a block index or page id outside its table was clamped
 constexpr int kStatusNoList = SV_STATUS_NO_LIST;  // a selection count was negative (block selection gave up on that list)
 
+// One layer of a layer table (sv_layer_table): what differs between the layers of a stack on the cache side.
+struct alignas(64) LayerRow {
+    CUtensorMap k_map, v_map;   // over the layer's pools, see pool_tensor_map
+    void *k_pool, *v_pool;
+    int32_t n_pages;
+    int32_t pad[11];
+};
+static_assert(sizeof(LayerRow) == 320, "rows stay 64-byte aligned, as tensor maps have to be");
+
 struct AttnParams {
     const __nv_bfloat16 *q;
     const __nv_bfloat16 *draft_k;
@@ -35,8 +44,17 @@ struct AttnParams {
     int early_gather;   // 1: nothing the gather reads comes from the kernel just before; it starts ahead of the dependency wait
 };
 
+// Several layers in one launch: grid.z = layers x sequences, layer-major.  What a layer owns (q, out, draft K/V, partials)
+// is numbered like the grid; tables, lengths and parents are those of the sequence, block lists of the layer's anchor.
+struct StackAttnParams : AttnParams {
+    const LayerRow *layers;           // device layer table, from the launch's first layer on
+    int S;                            // sequences of a layer
+    uint8_t list_of[SV_MAX_LAYERS];   // block list of a layer: the ordinal of the last anchor up to it
+};
+
 // tcgen05 / TMEM attention kernel (verify_attn_tc.cu): rows = G*T <= 128 packed as one M=128 tile.
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid,
                            cudaStream_t stream);
+cudaError_t launch_attn_tc_stack(const StackAttnParams &p, dim3 grid, cudaStream_t stream);
 
 }  // namespace svk

@@ -7,6 +7,9 @@
 // 512 bytes written per block.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
+#include "attn_common.cuh"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
 
@@ -15,15 +18,31 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kRowGroups = kThreads / 16;   // 16 threads cover one 256-byte key row
 
+// Several layers in one launch: grid.z = layers x sequences, the pool is the layer's.  A kernel of its own: with 30000
+// short CTAs even 270 bytes more of arguments and a branch cost a launch over one layer 10 %.
+struct OneLayer {};
+struct StackParams {
+    const svk::LayerRow *layers;
+    int S;
+    uint8_t layer_of[SV_MAX_LAYERS];
+};
+
 // OutT: float (the default representatives) or __nv_bfloat16 (storage variant: the fp32 mean rounded once).
-template <int B, typename OutT>
+template <int B, typename OutT, class Stack>
 __global__ void __launch_bounds__(kThreads) block_reps_kernel(const uint4 *__restrict__ k_pool,
                                                               const int32_t *__restrict__ block_table,
                                                               const int32_t *__restrict__ seq_lens,
                                                               OutT *__restrict__ reps, int Hkv, int NBmax,
-                                                              int block_begin, int block_end)
+                                                              int block_begin, int block_end, const Stack stack)
 {
-    const int s = blockIdx.z, h = blockIdx.y;
+    const int h = blockIdx.y, z = blockIdx.z;
+    int s = z, bz = z;   // sequence (table, length); batch index of the representatives
+    if constexpr (std::is_same_v<Stack, StackParams>) {
+        const int l = z / stack.S;
+        s = z - l * stack.S;
+        bz = stack.layer_of[l] * stack.S + s;
+        k_pool = static_cast<const uint4 *>(stack.layers[stack.layer_of[l]].k_pool);
+    }
     svk::grid_dependency_wait();      // the keys may come from the kernel just before (a cache append)
     svk::grid_launch_dependents();
     const int L = seq_lens[s];
@@ -62,26 +81,24 @@ __global__ void __launch_bounds__(kThreads) block_reps_kernel(const uint4 *__res
         float sum = 0.f;
 #pragma unroll
         for (int g = 0; g < kRowGroups; ++g) sum += part[g][threadIdx.x];
-        reps[(((size_t)s * Hkv + h) * NBmax + b) * 128 + threadIdx.x] = static_cast<OutT>(sum / (float)cnt);
+        reps[(((size_t)bz * Hkv + h) * NBmax + b) * 128 + threadIdx.x] = static_cast<OutT>(sum / (float)cnt);
     }
 }
 
 }  // namespace
 
-template <typename OutT>
-static sv_status launch_block_reps(const sv_geom *geom, const sv_kv *kv, int32_t block_begin, int32_t block_end,
-                                   OutT *reps, void *stream)
+// `n_batch`: sequences, or (layer, sequence) pairs of a stack.
+template <typename OutT, class Stack>
+static sv_status launch_block_reps(const sv_geom *geom, const void *k_pool, const int32_t *block_table, const int32_t *seq_lens,
+                                   const Stack &stack, int n_batch, int32_t block_begin, int32_t block_end, OutT *reps,
+                                   void *stream)
 {
-    sv_status st = svh::check_geom(geom);
-    if (st != SV_OK) return st;
-    st = svh::check_kv(geom, kv, false);
-    if (st != SV_OK) return st;
     if (!reps) return SV_ERR_NULL;
     if (!svh::aligned(reps, 16)) return SV_ERR_ALIGN;
     if (block_begin < 0 && block_begin != SV_TAIL_BLOCK) return SV_ERR_SHAPE;
     const int hi = (block_end < 0 || block_end > geom->max_blocks) ? geom->max_blocks : block_end;
     if (block_begin >= 0 && hi <= block_begin) return SV_OK;   // empty range: nothing to do
-    dim3 grid(block_begin < 0 ? 1 : hi - block_begin, geom->n_kv_heads, geom->n_seq);
+    dim3 grid(block_begin < 0 ? 1 : hi - block_begin, geom->n_kv_heads, n_batch);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kThreads);
@@ -90,24 +107,48 @@ static sv_status launch_block_reps(const sv_geom *geom, const sv_kv *kv, int32_t
     svh::pdl_attribute(attr);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const uint4 *pool = static_cast<const uint4 *>(kv->k_pool);
-    const cudaError_t e =
-        geom->block_size == 64
-            ? cudaLaunchKernelEx(&cfg, block_reps_kernel<64, OutT>, pool, kv->block_table, kv->seq_lens, reps,
-                                 (int)geom->n_kv_heads, (int)geom->max_blocks, (int)block_begin, (int)block_end)
-            : cudaLaunchKernelEx(&cfg, block_reps_kernel<128, OutT>, pool, kv->block_table, kv->seq_lens, reps,
-                                 (int)geom->n_kv_heads, (int)geom->max_blocks, (int)block_begin, (int)block_end);
+    const uint4 *pool = static_cast<const uint4 *>(k_pool);
+    const auto kernel = geom->block_size == 64 ? block_reps_kernel<64, OutT, Stack> : block_reps_kernel<128, OutT, Stack>;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, pool, block_table, seq_lens, reps, (int)geom->n_kv_heads,
+                                             (int)geom->max_blocks, (int)block_begin, (int)block_end, stack);
     return e == cudaSuccess ? svh::launch_status() : SV_ERR_CUDA;
+}
+
+template <typename OutT>
+static sv_status block_reps_impl(const sv_geom *geom, const sv_kv *kv, int32_t block_begin, int32_t block_end, OutT *reps,
+                                 void *stream)
+{
+    sv_status st = svh::check_geom(geom);
+    if (st != SV_OK) return st;
+    st = svh::check_kv(geom, kv, false);
+    if (st != SV_OK) return st;
+    return launch_block_reps(geom, kv->k_pool, kv->block_table, kv->seq_lens, OneLayer{}, geom->n_seq, block_begin, block_end, reps, stream);
 }
 
 extern "C" sv_status sv_block_reps(const sv_geom *geom, const sv_kv *kv, int32_t block_begin, int32_t block_end,
                                    float *reps, void *stream)
 {
-    return launch_block_reps<float>(geom, kv, block_begin, block_end, reps, stream);
+    return block_reps_impl<float>(geom, kv, block_begin, block_end, reps, stream);
 }
 
 extern "C" sv_status sv_block_reps_bf16(const sv_geom *geom, const sv_kv *kv, int32_t block_begin, int32_t block_end,
                                         void *reps_bf16, void *stream)
 {
-    return launch_block_reps<__nv_bfloat16>(geom, kv, block_begin, block_end, static_cast<__nv_bfloat16 *>(reps_bf16), stream);
+    return block_reps_impl<__nv_bfloat16>(geom, kv, block_begin, block_end, static_cast<__nv_bfloat16 *>(reps_bf16), stream);
+}
+
+extern "C" sv_status sv_block_reps_layers(const sv_geom *geom, const sv_layers *layers, const uint8_t *which, int32_t block_begin,
+                                          int32_t block_end, float *reps, void *stream)
+{
+    const sv_status st = svh::check_layers(geom, layers, 0, layers ? layers->n_layers : 1);
+    if (st != SV_OK) return st;
+    StackParams stack;
+    stack.layers = static_cast<const svk::LayerRow *>(layers->table);
+    stack.S = geom->n_seq;
+    int n = 0;
+    for (int l = 0; l < layers->n_layers; ++l)
+        if (!which || which[l]) stack.layer_of[n++] = (uint8_t)l;
+    if (n == 0) return SV_OK;
+    return launch_block_reps(geom, nullptr, layers->block_table, layers->seq_lens, stack, n * geom->n_seq, block_begin, block_end, reps,
+                             stream);
 }

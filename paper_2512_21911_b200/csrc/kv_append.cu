@@ -11,6 +11,7 @@
 // (sequence, KV head): latency-bound, not bandwidth-bound.
 #include <cuda_bf16.h>
 
+#include "attn_common.cuh"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
 
@@ -22,15 +23,23 @@ constexpr int kRowGroups = kThreads / 16;
 template <int B>
 __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__ k_pool, uint4 *__restrict__ v_pool,
                                                              const int32_t *__restrict__ block_table,
-                                                             const int32_t *__restrict__ seq_lens,
+                                                             const int32_t *seq_lens,
                                                              const uint4 *__restrict__ draft_k,
                                                              const uint4 *__restrict__ draft_v,
                                                              const int32_t *__restrict__ accept_idx,
                                                              const int32_t *__restrict__ n_accept, int max_accept,
-                                                             int32_t *__restrict__ seq_lens_out, float *__restrict__ reps,
-                                                             int T, int Hkv, int NBmax, int n_pages)
+                                                             int32_t *seq_lens_out, float *__restrict__ reps,
+                                                             int T, int Hkv, int NBmax, int n_pages,
+                                                             const svk::LayerRow *layers, uint32_t *readers)
 {
     const int h = blockIdx.x, s = blockIdx.y;
+    int bz = s;   // batch index of what the layer owns (draft K/V, representatives)
+    if (layers) {
+        const svk::LayerRow *row = layers + blockIdx.z;
+        bz += blockIdx.z * gridDim.y;
+        k_pool = static_cast<uint4 *>(row->k_pool), v_pool = static_cast<uint4 *>(row->v_pool);
+        n_pages = row->n_pages;
+    }
     svk::grid_dependency_wait();
     svk::grid_launch_dependents();
     const int L = seq_lens[s];
@@ -43,7 +52,23 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
         if (page < 0 || page >= n_pages) n = max(0, min(n, b * B - L));
     }
     const int Ln = L + n;
-    if (h == 0 && threadIdx.x == 0) seq_lens_out[s] = Ln;
+    if (readers) {
+        // The lengths are advanced in place, by the last CTA of the sequence to have read the old one; the counter wraps to
+        // zero behind it.  readers[S + s]: the new length on its way there (of the last layer, should the layers' pools
+        // hold different numbers of pages).
+        __syncthreads();   // every thread of this CTA holds the old length
+        if (threadIdx.x == 0) {
+            int *fresh = reinterpret_cast<int *>(readers) + gridDim.y + s;
+            if (h == 0 && blockIdx.z == gridDim.z - 1) atomicExch(fresh, Ln);
+            __threadfence();
+            if (atomicInc(readers + s, gridDim.x * gridDim.z - 1) == gridDim.x * gridDim.z - 1) {
+                __threadfence();
+                seq_lens_out[s] = atomicAdd(fresh, 0);
+            }
+        }
+    } else if (h == 0 && threadIdx.x == 0) {
+        seq_lens_out[s] = Ln;
+    }
     if (n <= 0) return;
 
     // copy the accepted rows: 16 threads per 256-byte row, K and V
@@ -53,7 +78,7 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
         const int t = L + a;
         const int page = block_table[(size_t)s * NBmax + t / B];
         const size_t dst = (((size_t)page * Hkv + h) * B + (t % B)) * 16 + c;
-        const size_t src = (((size_t)s * T + j) * Hkv + h) * 16 + c;
+        const size_t src = (((size_t)bz * T + j) * Hkv + h) * 16 + c;
         if (which)
             v_pool[dst] = __ldg(draft_v + src);
         else
@@ -93,7 +118,7 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
             float sum = 0.f;
 #pragma unroll
             for (int g = 0; g < kRowGroups; ++g) sum += part[g][threadIdx.x];
-            reps[(((size_t)s * Hkv + h) * NBmax + b) * 128 + threadIdx.x] = sum / (float)cnt;
+            reps[(((size_t)bz * Hkv + h) * NBmax + b) * 128 + threadIdx.x] = sum / (float)cnt;
         }
         __syncthreads();
     }
@@ -129,9 +154,36 @@ extern "C" sv_status sv_kv_append(const sv_geom *geom, void *k_pool, void *v_poo
         geom->block_size == 64
             ? cudaLaunchKernelEx(&cfg, kv_append_kernel<64>, kp, vp, block_table, seq_lens, dk, dv, accept_idx, n_accept,
                                  (int)max_accept, seq_lens_out, reps, (int)geom->n_draft, (int)geom->n_kv_heads,
-                                 (int)geom->max_blocks, (int)n_pages)
+                                 (int)geom->max_blocks, (int)n_pages, nullptr, nullptr)
             : cudaLaunchKernelEx(&cfg, kv_append_kernel<128>, kp, vp, block_table, seq_lens, dk, dv, accept_idx, n_accept,
                                  (int)max_accept, seq_lens_out, reps, (int)geom->n_draft, (int)geom->n_kv_heads,
-                                 (int)geom->max_blocks, (int)n_pages);
+                                 (int)geom->max_blocks, (int)n_pages, nullptr, nullptr);
+    return e == cudaSuccess ? svh::launch_status() : SV_ERR_CUDA;
+}
+
+extern "C" sv_status sv_kv_append_layers(const sv_geom *geom, const sv_layers *layers, const void *draft_k, const void *draft_v,
+                                         const int32_t *accept_idx, const int32_t *n_accept, int32_t max_accept,
+                                         int32_t *seq_lens, uint32_t *counters, float *reps, void *stream)
+{
+    const sv_status st = svh::check_layers(geom, layers, 0, layers ? layers->n_layers : 1);
+    if (st != SV_OK) return st;
+    if (!draft_k || !draft_v || !accept_idx || !n_accept || !seq_lens || !counters) return SV_ERR_NULL;
+    if (max_accept < 1 || max_accept > geom->n_draft) return SV_ERR_SHAPE;
+    if (seq_lens != layers->seq_lens) return SV_ERR_SHAPE;
+    if (!svh::aligned(draft_k, 16) || !svh::aligned(draft_v, 16) || !svh::aligned(counters, 4) || (reps && !svh::aligned(reps, 16)))
+        return SV_ERR_ALIGN;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(geom->n_kv_heads, geom->n_seq, layers->n_layers);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cudaLaunchAttribute attr[1];
+    svh::pdl_attribute(attr);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const auto kernel = geom->block_size == 64 ? kv_append_kernel<64> : kv_append_kernel<128>;
+    const cudaError_t e = cudaLaunchKernelEx(
+        &cfg, kernel, (uint4 *)nullptr, (uint4 *)nullptr, layers->block_table, (const int32_t *)seq_lens,
+        static_cast<const uint4 *>(draft_k), static_cast<const uint4 *>(draft_v), accept_idx, n_accept, (int)max_accept, seq_lens, reps,
+        (int)geom->n_draft, (int)geom->n_kv_heads, (int)geom->max_blocks, 0, static_cast<const svk::LayerRow *>(layers->table), counters);
     return e == cudaSuccess ? svh::launch_status() : SV_ERR_CUDA;
 }

@@ -10,7 +10,10 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
+#include <string.h>
+
 #include <ATen/core/Tensor.h>
+#include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -28,7 +31,7 @@ const at::Tensor &tensor(PyObject *o, at::ScalarType type, const char *name)
         if (t.is_cuda() && t.scalar_type() == type && t.is_contiguous()) return t;
     }
     PyErr_Format(PyExc_TypeError, "%s: expected a contiguous CUDA tensor of torch.%s", name,
-                 type == at::kBFloat16 ? "bfloat16" : type == at::kFloat ? "float32" : "int32");
+                 type == at::kBFloat16 ? "bfloat16" : type == at::kFloat ? "float32" : type == at::kByte ? "uint8" : "int32");
     throw ArgError{};
 }
 
@@ -253,9 +256,146 @@ PyObject *verify_layer(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// ---------------------------------------------------------------------- a stack of layers
+
+// Per-layer host flags as bytes.
+const uint8_t *flags(PyObject *o, int32_t n)
+{
+    if (o == Py_None) return nullptr;
+    if (!PyBytes_Check(o) || PyBytes_GET_SIZE(o) != n) {
+        PyErr_SetString(PyExc_TypeError, "expected one byte per layer");
+        throw ArgError{};
+    }
+    return reinterpret_cast<const uint8_t *>(PyBytes_AS_STRING(o));
+}
+
+// The layers of an engine: its table (uint8 tensor [n_layers][row bytes]) and the page table and lengths of a layer's sv_kv.
+sv_layers stack(PyObject *table, PyObject *kv)
+{
+    const at::Tensor &t = tensor(table, at::kByte, "layer table");
+    const sv_kv first = cache(kv);
+    return {t.data_ptr(), first.block_table, first.seq_lens, (int32_t)t.size(0)};
+}
+
+// Pointer of a tensor stacked over all layers, or null when the argument is something else (a list of per-layer tensors, a
+// strided view): the caller then goes layer by layer.
+void *stacked(PyObject *o, int64_t n_layers)
+{
+    if (!THPVariable_Check(o)) return nullptr;
+    const at::Tensor &t = THPVariable_Unpack(o);
+    if (!t.is_cuda() || t.scalar_type() != at::kBFloat16 || !t.is_contiguous() || t.dim() != 5 || t.size(0) != n_layers) return nullptr;
+    return t.data_ptr();
+}
+
+// geom, kv -> the layer's row of a layer table, as bytes
+PyObject *layer_row(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 2, [&]() -> PyObject * {
+        const sv_geom g = geometry(a[0]);
+        const sv_kv kv = cache(a[1]);
+        PyObject *row = PyBytes_FromStringAndSize(nullptr, (Py_ssize_t)sv_layer_table_bytes(1));
+        if (!row) return nullptr;
+        const sv_status st = sv_layer_table(&g, &kv, 1, PyBytes_AS_STRING(row));
+        if (st == SV_OK) return row;
+        Py_DECREF(row);
+        return status(st);
+    });
+}
+
+// geom, n_layers, max_sel -> bytes
+PyObject *workspace_bytes_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 3, [&] {
+        const sv_geom g = geometry(a[0]);
+        return PyLong_FromSize_t(sv_workspace_bytes_layers(&g, int32(a[1]), int32(a[2])));
+    });
+}
+
+// geom, table, kv, which (bytes or None), block_begin, block_end, reps
+PyObject *block_reps_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 7, [&] {
+        const sv_geom g = geometry(a[0]);
+        const sv_layers layers = stack(a[1], a[2]);
+        return status(sv_block_reps_layers(&g, &layers, flags(a[3], layers.n_layers), int32(a[4]), int32(a[5]), f32(a[6], "reps"),
+                                           stream(Py_None)));
+    });
+}
+
+// Layers first .. end - 1 of a step on the current stream: the selections of their anchors in one launch, their attention in
+// another (dense: attention only).  geom, table, kv, first, end, anchors, q, draft_k, draft_v, parent, out, reps, budget, n_sink,
+// n_local, idx, cnt (None: dense), workspace, status_word -> None, (status, whether it is the selection's), or False when the
+// inputs are not stacked tensors
+PyObject *verify_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 19, [&]() -> PyObject * {
+        const sv_geom g = geometry(a[0]);
+        const sv_layers layers = stack(a[1], a[2]);
+        const int32_t first = int32(a[3]), end = int32(a[4]);
+        const void *q = stacked(a[6], layers.n_layers), *dk = stacked(a[7], layers.n_layers), *dv = stacked(a[8], layers.n_layers);
+        void *out = stacked(a[10], layers.n_layers);
+        if (!q || !dk || !dv || !out) Py_RETURN_FALSE;
+        const uint8_t *anchors = flags(a[5], layers.n_layers);
+        const int32_t *parent = i32(a[9], "parent");
+        const bool dense = a[15] == Py_None;
+        int32_t *idx = i32(a[15], "idx"), *cnt = i32(a[16], "cnt");
+        const int32_t max_sel = dense ? g.max_blocks : row_length(a[15], "idx");
+        const Scratch ws = scratch(a[17]);
+        void *s = stream(Py_None);
+        if (!dense) {
+            const sv_status st = sv_select_blocks_layers(&g, &layers, first, end, anchors, q, f32(a[11], "reps"), i32(a[12], "budget_blocks"),
+                                                         int32(a[13]), int32(a[14]), idx, cnt, max_sel, s);
+            if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_True);
+        }
+        const sv_status st = sv_verify_attn_layers(&g, &layers, first, end, anchors, q, dk, dv, parent, idx, cnt, max_sel, 0.f, out, ws.p,
+                                                   ws.bytes, i32(a[18], "status_word"), s);
+        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_False);
+        Py_RETURN_NONE;
+    });
+}
+
+// geom, table, kv, draft_k, draft_v, path, n_path, seq_lens, counters, reps -> status, or False when the drafts are not stacked tensors
+PyObject *kv_append_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 10, [&]() -> PyObject * {
+        const sv_geom g = geometry(a[0]);
+        const sv_layers layers = stack(a[1], a[2]);
+        const void *dk = stacked(a[3], layers.n_layers), *dv = stacked(a[4], layers.n_layers);
+        int32_t *lens = i32(a[7], "seq_lens");
+        if (!dk || !dv || lens != layers.seq_lens) Py_RETURN_FALSE;
+        return status(sv_kv_append_layers(&g, &layers, dk, dv, i32(a[5], "accept_idx"), i32(a[6], "n_accept"),
+                                          row_length(a[5], "accept_idx"), lens, reinterpret_cast<uint32_t *>(i32(a[8], "counters")),
+                                          f32(a[9], "reps"), stream(Py_None)));
+    });
+}
+
+// accept with the outputs allocated here: p_target, p_draft, tokens, parent, u_accept, u_next, n_seq, n_draft
+// -> (path, n_path, next_token), or a status
+PyObject *accept_new(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 8, [&]() -> PyObject * {
+        const at::Tensor &pt = tensor(a[0], at::kFloat, "p_target"), &pd = tensor(a[1], at::kFloat, "p_draft");
+        const at::Tensor &tok = tensor(a[2], at::kInt, "tokens");
+        const int64_t S = integer(a[6]), T = integer(a[7]);
+        if (pt.dim() != 3 || pt.size(0) != S || pt.size(1) != T || !pd.sizes().equals(pt.sizes()) || !tok.sizes().equals({S, T})) {
+            PyErr_SetString(PyExc_ValueError, "sv_accept: shapes disagree");
+            throw ArgError{};
+        }
+        const auto opt = tok.options();
+        at::Tensor path = at::empty({S, T}, opt), n_path = at::empty({S}, opt), next = at::empty({S}, opt);
+        const sv_status st = sv_accept((int32_t)S, (int32_t)T, (int32_t)pt.size(2), pt.data_ptr<float>(), pd.data_ptr<float>(),
+                                       tok.data_ptr<int32_t>(), i32(a[3], "parent"), f32(a[4], "u_accept"), f32(a[5], "u_next"),
+                                       path.data_ptr<int32_t>(), n_path.data_ptr<int32_t>(), next.data_ptr<int32_t>(), nullptr,
+                                       stream(Py_None));
+        if (st != SV_OK) return status(st);
+        return Py_BuildValue("(NNN)", THPVariable_Wrap(path), THPVariable_Wrap(n_path), THPVariable_Wrap(next));
+    });
+}
+
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {METHOD(block_reps), METHOD(select_blocks), METHOD(verify_attn), METHOD(kv_append), METHOD(accept),
-                         METHOD(verify_layer), {nullptr, nullptr, 0, nullptr}};
+                         METHOD(verify_layer), METHOD(layer_row), METHOD(workspace_bytes_layers), METHOD(block_reps_layers),
+                         METHOD(verify_layers), METHOD(kv_append_layers), METHOD(accept_new), {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the entry points of sv.h.", -1, methods,
                       nullptr, nullptr, nullptr, nullptr};

@@ -16,6 +16,8 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "select_core.cuh"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
@@ -46,6 +48,13 @@ struct SelectParams {
     int T, Hq, Hkv, B, NBmax, n_sink, n_local, max_sel, chunk;
 };
 
+// Several layers in one launch: grid.z = selecting layers x sequences.  Query and representatives are those of layer
+// layer_of[z / S], lists are numbered by z; lengths and budgets by the sequence z % S.
+struct StackSelectParams : SelectParams {
+    int S;
+    uint8_t layer_of[SV_MAX_LAYERS];
+};
+
 // Cluster of CL CTAs per (sequence, KV head).  Every CTA scores a slice of the blocks and writes the
 // keys straight into CTA 0's shared memory (distributed shared memory) with stores that count their bytes
 // on an mbarrier there, and exits; CTA 0 waits for the expected number of bytes and selects.  The only cluster-wide barrier is split (arrive early, wait late) so that
@@ -53,15 +62,22 @@ struct SelectParams {
 // kBf16: the representatives are stored in bfloat16 (storage variant); scores are fp32 either way.
 // kDepth: passes whose rows a warp loads together (1, or 2 for slices of more than 64 blocks: eight rows in flight per
 // warp, half as many trips to DRAM; more would cost the second CTA per SM its registers).
-template <bool kBf16, int kDepth, int kThreads>
-__global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const SelectParams p)
+template <bool kBf16, int kDepth, int kThreads, bool kStack>
+__global__ void __launch_bounds__(kThreads, 1024 / kThreads)
+    select_kernel(const std::conditional_t<kStack, StackSelectParams, SelectParams> p)
 {
     constexpr int kWarps = kThreads / 32;
     constexpr int kStride = kWarps * kRowsPerIter;   // blocks the CTA covers per pass
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int CL = (int)cluster.num_blocks();
-    const int h = blockIdx.y, s = blockIdx.z;
+    const int h = blockIdx.y, z = blockIdx.z;
+    int s = z, bz = z;   // sequence; batch index of what the layer owns (query, representatives)
+    if constexpr (kStack) {
+        const int a = z / p.S;
+        s = z - a * p.S;
+        bz = p.layer_of[a] * p.S + s;
+    }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     extern __shared__ __align__(16) uint32_t keys_all[];         // [CL*chunk] keys of all blocks (used in CTA 0)
@@ -80,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // before any global request is in flight
     const int b0 = rank * p.chunk;
     constexpr int kRowBytes = kBf16 ? 256 : 512, kLaneBytes = kRowBytes / 32;
-    const char *rbase = static_cast<const char *>(p.reps) + ((size_t)s * p.Hkv + h) * p.NBmax * kRowBytes;
+    const char *rbase = static_cast<const char *>(p.reps) + ((size_t)bz * p.Hkv + h) * p.NBmax * kRowBytes;
     auto row_ptr = [&](int row) { return rbase + (size_t)row * kRowBytes + lane * kLaneBytes; };
     auto load_row = [&](int row) {
         if constexpr (kBf16) {
@@ -99,7 +115,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const
         for (int i = 0; i < kRowsPerIter; ++i)
             if (b + d * kStride + i < min(b0 + p.chunk, p.NBmax)) svk::prefetch_l2(row_ptr(b + d * kStride + i));
     const int G = p.Hq / p.Hkv;
-    const __nv_bfloat16 *q0 = p.q + ((size_t)s * p.T * p.Hq + (size_t)h * G) * 128;
+    const __nv_bfloat16 *q0 = p.q + ((size_t)bz * p.T * p.Hq + (size_t)h * G) * 128;
     if (tid < G * 2) svk::prefetch_l2(q0 + tid * 64);
     svk::grid_dependency_wait();
     svk::grid_launch_dependents();
@@ -159,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const
                     const int bb = bd + i;
                     const bool is_forced = bb < p.n_sink || bb >= nb - p.n_local;
                     kk[i] = is_forced ? kForcedKey : order_key(dot);
-                    if (p.out_scores && lane == 0 && bb < b1) p.out_scores[((size_t)s * p.Hkv + h) * p.NBmax + bb] = dot;
+                    if (p.out_scores && lane == 0 && bb < b1) p.out_scores[((size_t)z * p.Hkv + h) * p.NBmax + bb] = dot;
                 }
                 // rows bd .. bd+3 are 4 consecutive keys: one 16-byte store into CTA 0 (entries past nb are never read)
                 if (lane == 0 && !keep_all)
@@ -170,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const
     }
     if (rank != 0) return;
 
-    int32_t *out = p.out_idx + ((size_t)s * p.Hkv + h) * p.max_sel;
+    int32_t *out = p.out_idx + ((size_t)z * p.Hkv + h) * p.max_sel;
     int cnt_out;
     if (keep_all) {
         for (int bb = tid; bb < nb; bb += kThreads) out[bb] = bb;
@@ -184,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads) select_kernel(const
     }
     __syncthreads();   // every thread's entries of the list are written
     if (tid == 0) {
-        p.out_cnt[(size_t)s * p.Hkv + h] = cnt_out;
+        p.out_cnt[(size_t)z * p.Hkv + h] = cnt_out;
     }
 }
 
@@ -199,24 +215,25 @@ __global__ void copy_selection_kernel(const int32_t *__restrict__ prev_idx, cons
 
 }  // namespace
 
-template <int kThreads>
-static const void *select_fn(bool reps_bf16, bool deep)
+template <bool kBf16, bool kStack>
+static const void *select_fn(bool few, bool deep)
 {
-    return reps_bf16 ? (deep ? reinterpret_cast<const void *>(select_kernel<true, 2, kThreads>)
-                             : reinterpret_cast<const void *>(select_kernel<true, 1, kThreads>))
-                     : (deep ? reinterpret_cast<const void *>(select_kernel<false, 2, kThreads>)
-                             : reinterpret_cast<const void *>(select_kernel<false, 1, kThreads>));
+    return few ? (deep ? reinterpret_cast<const void *>(select_kernel<kBf16, 2, kThreadsFew, kStack>)
+                       : reinterpret_cast<const void *>(select_kernel<kBf16, 1, kThreadsFew, kStack>))
+               : (deep ? reinterpret_cast<const void *>(select_kernel<kBf16, 2, kThreadsMany, kStack>)
+                       : reinterpret_cast<const void *>(select_kernel<kBf16, 1, kThreadsMany, kStack>));
 }
 
 // Whether this device can hold clusters of 16 CTAs of the select kernel (asked once per device and instantiation).
-static bool clusters_of_16_fit(bool reps_bf16)
+template <bool kBf16, bool kStack>
+static bool clusters_of_16_fit()
 {
-    static std::atomic<int> state[2][svh::kMaxDevices];   // 0: not asked, 1: yes, 2: no
+    static std::atomic<int> state[svh::kMaxDevices];   // 0: not asked, 1: yes, 2: no
     const int dev = svh::current_device();
     if (dev < 0 || dev >= svh::kMaxDevices) return false;
-    int v = state[reps_bf16][dev].load(std::memory_order_acquire);
+    int v = state[dev].load(std::memory_order_acquire);
     if (v == 0) {
-        const void *fn = select_fn<kThreadsFew>(reps_bf16, true);   // (slices of 128 blocks)
+        const void *fn = select_fn<kBf16, kStack>(true, true);   // (slices of 128 blocks)
         v = 2;
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
             cudaLaunchConfig_t cfg = {};
@@ -234,10 +251,14 @@ static bool clusters_of_16_fit(bool reps_bf16)
             if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 8) v = 1;
         }
         (void)cudaGetLastError();   // a refusal is an answer, not an error of the call that asked
-        state[reps_bf16][dev].store(v, std::memory_order_release);
+        state[dev].store(v, std::memory_order_release);
     }
     return v == 1;
 }
+
+// The selection launch for `n_batch` (layer, sequence) pairs; p holds the pointers.
+template <bool kBf16, class Params>
+static sv_status launch_select(const sv_geom *geom, Params &p, int n_batch, cudaStream_t cs);
 
 static sv_status select_impl(const sv_geom *geom, const void *q, const void *reps, bool reps_bf16, const int32_t *seq_lens,
                              const int32_t *budget_blocks, int32_t n_sink, int32_t n_local, int32_t reuse_prev,
@@ -265,21 +286,6 @@ static sv_status select_impl(const sv_geom *geom, const void *q, const void *rep
     if (n_sink + n_local > max_sel) return SV_ERR_BUDGET;
     if (geom->max_blocks > svh::kMaxBlocksSelect) return SV_ERR_UNSUPPORTED;
 
-    // CTAs per (sequence, KV head): at least 32 blocks each, and no more CTAs than two per SM (a second wave costs more
-    // than the shorter slices save)
-    const int pairs = geom->n_seq * geom->n_kv_heads;
-    int CL = 1;
-    while (CL < 8 && geom->max_blocks / (CL * 2) >= 32 && pairs * CL * 2 <= 2 * svh::sm_count()) CL *= 2;
-    // Few pairs with very long block lists (one sequence of 128K tokens: 8 pairs x 2048 blocks) leave most SMs idle at
-    // 8 CTAs per pair, and reading the representatives (128 KB per CTA) is what the kernel then waits for: clusters of
-    // 16 (beyond the portable size, so the device is asked first whether it can hold them)
-    if (CL == 8 && geom->max_blocks >= 2048 && pairs * 16 <= svh::sm_count() && clusters_of_16_fit(reps_bf16)) CL = 16;
-    const int per = (geom->max_blocks + CL - 1) / CL;
-    const bool many = (long long)pairs * CL > 2 * svh::sm_count();   // more CTAs than fit at once: smaller CTAs, four per SM
-    const int threads = many ? kThreadsMany : kThreadsFew;
-    const int stride = threads / 32 * kRowsPerIter;              // blocks a CTA covers per pass
-    const int chunk = (per + stride - 1) / stride * stride;
-
     SelectParams p;
     p.q = static_cast<const __nv_bfloat16 *>(q);
     p.reps = reps;
@@ -288,16 +294,39 @@ static sv_status select_impl(const sv_geom *geom, const void *q, const void *rep
     p.out_idx = out_idx;
     p.out_cnt = out_cnt;
     p.out_scores = out_scores;
+    p.n_sink = n_sink, p.n_local = n_local, p.max_sel = max_sel;
+    return reps_bf16 ? launch_select<true>(geom, p, geom->n_seq, cs) : launch_select<false>(geom, p, geom->n_seq, cs);
+}
+
+template <bool kBf16, class Params>
+static sv_status launch_select(const sv_geom *geom, Params &p, int n_batch, cudaStream_t cs)
+{
+    constexpr bool kStack = std::is_same_v<Params, StackSelectParams>;
+    // CTAs per (sequence, KV head): at least 32 blocks each, and no more CTAs than two per SM (a second wave costs more
+    // than the shorter slices save)
+    const int pairs = n_batch * geom->n_kv_heads;
+    int CL = 1;
+    while (CL < 8 && geom->max_blocks / (CL * 2) >= 32 && pairs * CL * 2 <= 2 * svh::sm_count()) CL *= 2;
+    // Few pairs with very long block lists (one sequence of 128K tokens: 8 pairs x 2048 blocks) leave most SMs idle at
+    // 8 CTAs per pair, and reading the representatives (128 KB per CTA) is what the kernel then waits for: clusters of
+    // 16 (beyond the portable size, so the device is asked first whether it can hold them)
+    if (CL == 8 && geom->max_blocks >= 2048 && pairs * 16 <= svh::sm_count() && clusters_of_16_fit<kBf16, kStack>()) CL = 16;
+    const int per = (geom->max_blocks + CL - 1) / CL;
+    const bool many = (long long)pairs * CL > 2 * svh::sm_count();   // more CTAs than fit at once: smaller CTAs, four per SM
+    const int threads = many ? kThreadsMany : kThreadsFew;
+    const int stride = threads / 32 * kRowsPerIter;              // blocks a CTA covers per pass
+    const int chunk = (per + stride - 1) / stride * stride;
+
     p.T = geom->n_draft, p.Hq = geom->n_q_heads, p.Hkv = geom->n_kv_heads, p.B = geom->block_size;
-    p.NBmax = geom->max_blocks, p.n_sink = n_sink, p.n_local = n_local, p.max_sel = max_sel, p.chunk = chunk;
+    p.NBmax = geom->max_blocks, p.chunk = chunk;
 
     const size_t smem = (size_t)CL * chunk * sizeof(uint32_t);
     const bool deep = chunk > stride;   // more than one pass per warp: load two passes' rows together
-    const void *fn = many ? select_fn<kThreadsMany>(reps_bf16, deep) : select_fn<kThreadsFew>(reps_bf16, deep);
+    const void *fn = select_fn<kBf16, kStack>(!many, deep);
     if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return SV_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL, geom->n_kv_heads, geom->n_seq);
+    cfg.gridDim = dim3(CL, geom->n_kv_heads, n_batch);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = cs;
@@ -332,4 +361,39 @@ extern "C" sv_status sv_select_blocks_bf16reps(const sv_geom *geom, const void *
 {
     return select_impl(geom, q, reps_bf16, true, seq_lens, budget_blocks, n_sink, n_local, reuse_prev, prev_idx, prev_cnt,
                        out_idx, out_cnt, max_sel, out_scores, stream);
+}
+
+extern "C" sv_status sv_select_blocks_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                             const uint8_t *anchors, const void *q, const float *reps,
+                                             const int32_t *budget_blocks, int32_t n_sink, int32_t n_local, int32_t *out_idx,
+                                             int32_t *out_cnt, int32_t max_sel, void *stream)
+{
+    const sv_status st = svh::check_layers(geom, layers, first, end);
+    if (st != SV_OK) return st;
+    if (!anchors || !q || !reps || !budget_blocks || !out_idx || !out_cnt) return SV_ERR_NULL;
+    if (!svh::aligned(q, 16) || !svh::aligned(reps, 16)) return SV_ERR_ALIGN;
+    if (max_sel < 1 || n_sink < 0 || n_local < 0) return SV_ERR_SHAPE;
+    if (n_sink + n_local > max_sel) return SV_ERR_BUDGET;
+    if (geom->max_blocks > svh::kMaxBlocksSelect) return SV_ERR_UNSUPPORTED;
+    StackSelectParams p;
+    int before = 0, n = 0;   // anchors ahead of `first`, anchors of this call
+    for (int l = 0; l < end; ++l) {
+        if (!anchors[l]) continue;
+        if (l < first)
+            ++before;
+        else
+            p.layer_of[n++] = (uint8_t)l;
+    }
+    if (n == 0) return SV_OK;
+    const size_t lists = (size_t)before * geom->n_seq * geom->n_kv_heads;
+    p.q = static_cast<const __nv_bfloat16 *>(q);
+    p.reps = reps;
+    p.seq_lens = layers->seq_lens;
+    p.budget = budget_blocks;
+    p.out_idx = out_idx + lists * max_sel;
+    p.out_cnt = out_cnt + lists;
+    p.out_scores = nullptr;
+    p.n_sink = n_sink, p.n_local = n_local, p.max_sel = max_sel;
+    p.S = geom->n_seq;
+    return launch_select<false>(geom, p, n * geom->n_seq, static_cast<cudaStream_t>(stream));
 }

@@ -54,6 +54,19 @@ inline sv_status check_kv(const sv_geom *g, const sv_kv *kv, bool need_v)
     return SV_OK;
 }
 
+// Layers first .. end - 1 of a stack.
+inline sv_status check_layers(const sv_geom *g, const sv_layers *layers, int32_t first, int32_t end)
+{
+    const sv_status st = check_geom(g);
+    if (st != SV_OK) return st;
+    if (!layers || !layers->table || !layers->block_table || !layers->seq_lens) return SV_ERR_NULL;
+    if (layers->n_layers < 1 || layers->n_layers > SV_MAX_LAYERS || first < 0 || end > layers->n_layers || first >= end)
+        return SV_ERR_SHAPE;
+    if ((long long)g->n_seq * layers->n_layers > 65535) return SV_ERR_SHAPE;   // (layer, sequence) is a grid dimension
+    if (!aligned(layers->table, 64) || !aligned(layers->block_table, 4) || !aligned(layers->seq_lens, 4)) return SV_ERR_ALIGN;
+    return SV_OK;
+}
+
 // Launch attribute for programmatic dependent launch: the kernel may be scheduled while its
 // predecessor in the stream drains; every kernel of the library executes griddepcontrol.wait before it
 // reads anything the predecessor wrote.

@@ -16,6 +16,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <string.h>
+
 #include <mutex>
 
 #include "attn_common.cuh"
@@ -107,8 +109,22 @@ EncodeTiledFn encode_fn()
 
 // Tensor map over a pool viewed as a bf16 tensor [2 column halves][n_pages*Hkv*B rows][64 cols] (the halves 128 bytes
 // apart inside a 256-byte row); box = 2 halves x 64 rows x 64 cols (128 bytes wide, 128-byte swizzle), so that one copy
-// brings a 64-row unit as the two half tiles the tensor cores read.  Encoding costs microseconds of host time, so maps are kept in a
-// small fixed table keyed by (pool, rows) (no heap use; a full table is overwritten round-robin).
+// brings a 64-row unit as the two half tiles the tensor cores read.
+bool encode_pool_map(const void *pool, int64_t n_rows, CUtensorMap *out)
+{
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {64, (cuuint64_t)n_rows, 2};
+    const cuuint64_t strides[2] = {256, 128};
+    const cuuint32_t box[3] = {64, kUnit, 2};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(pool), dims, strides, box, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Encoding costs microseconds of host time, so the maps of single layers are kept in a small fixed table keyed by
+// (pool, rows) (no heap use; a full table is overwritten round-robin).
 bool pool_tensor_map(const void *pool, int64_t n_rows, CUtensorMap *out)
 {
     struct Entry {
@@ -126,17 +142,8 @@ bool pool_tensor_map(const void *pool, int64_t n_rows, CUtensorMap *out)
             *out = table[i].map;
             return true;
         }
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint64_t dims[3] = {64, (cuuint64_t)n_rows, 2};
-    const cuuint64_t strides[2] = {256, 128};
-    const cuuint32_t box[3] = {64, kUnit, 2};
-    const cuuint32_t estr[3] = {1, 1, 1};
     CUtensorMap tm;
-    if (fn(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(pool), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
+    if (!encode_pool_map(pool, n_rows, &tm)) return false;
     const int slot = used < kEntries ? used++ : (next++ % kEntries);
     table[slot].pool = pool;
     table[slot].rows = n_rows;
@@ -197,6 +204,78 @@ extern "C" size_t sv_workspace_bytes(const sv_geom *geom, int32_t max_sel)
     return workspace_bytes_for(geom, max_sel, true);
 }
 
+// What the entry points share once their arguments are checked: parameters and launches.  `rule`: the geometry that
+// the split and row-tile rules look at (all sequences of all layers of a stack, however many of its layers this launch
+// covers, so that a layer's result does not depend on the layers it is launched with).
+static void fill_params(AttnParams &p, const sv_geom *geom, const sv_geom *rule, int splits, const void *q, const void *draft_k,
+                        const void *draft_v, const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                        int32_t max_sel, float softmax_scale, void *out, float *lse, void *workspace, int32_t *status_word)
+{
+    const int G = geom->n_q_heads / geom->n_kv_heads;
+    p.q = static_cast<const __nv_bfloat16 *>(q);
+    p.draft_k = static_cast<const __nv_bfloat16 *>(draft_k);
+    p.draft_v = static_cast<const __nv_bfloat16 *>(draft_v);
+    p.parent = parent;
+    p.sel_idx = sel_idx;
+    p.sel_cnt = sel_cnt;
+    p.out = static_cast<__nv_bfloat16 *>(out);
+    p.lse = lse;
+    p.ws_o = static_cast<float *>(workspace);
+    p.status = status_word;
+    p.T = geom->n_draft, p.Hq = geom->n_q_heads, p.Hkv = geom->n_kv_heads, p.G = G, p.B = geom->block_size;
+    p.NBmax = geom->max_blocks, p.max_sel = max_sel, p.splits = splits;
+    p.Tt = svh::tokens_per_tile(geom), p.tiles = svh::row_tiles(geom);
+    p.pair = svh::pair_row_tiles(rule) ? 1 : 0;
+    p.early_gather = 0;
+    const float scale = softmax_scale > 0.f ? softmax_scale : 0.08838834764831845f;   // 1/sqrt(128)
+    p.scale_log2 = scale * 1.4426950408889634f;
+}
+
+// `attend`: launches the attention kernel on a grid.
+template <class Params, class Attend>
+static sv_status launch_attn(Params &p, const sv_geom *rule, int n_batch, cudaStream_t cs, Attend attend)
+{
+    const int rows = p.G * p.T;
+    p.ws_ml = p.ws_o ? p.ws_o + (size_t)n_batch * p.Hkv * p.splits * rows * 128 : nullptr;
+    const dim3 grid(p.splits * svh::row_groups(rule), p.Hkv, n_batch);   // one CTA per (row tile or pair of row tiles, split)
+    if (attend(grid) != cudaSuccess) return SV_ERR_CUDA;
+    if (p.splits > 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((rows * 32 + kMergeThreads - 1) / kMergeThreads, p.Hkv, n_batch);
+        cfg.blockDim = dim3(kMergeThreads);
+        cfg.stream = cs;
+        cudaLaunchAttribute attr[1];
+        svh::pdl_attribute(attr);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const AttnParams &mp = p;
+        const cudaError_t me = p.splits <= 4 ? cudaLaunchKernelEx(&cfg, merge_splits_kernel<4>, mp)
+                                             : cudaLaunchKernelEx(&cfg, merge_splits_kernel<20>, mp);
+        if (me != cudaSuccess) return SV_ERR_CUDA;
+    }
+    return SV_OK;
+}
+
+static sv_status check_attn_args(const void *q, const void *draft_k, const void *draft_v, const int32_t *sel_idx,
+                                 const int32_t *sel_cnt, int32_t max_sel, float softmax_scale, const void *out)
+{
+    if (!q || !draft_k || !draft_v || !out) return SV_ERR_NULL;
+    if (sel_idx && !sel_cnt) return SV_ERR_NULL;
+    if (!svh::aligned(q, 16) || !svh::aligned(draft_k, 16) || !svh::aligned(draft_v, 16) || !svh::aligned(out, 16))
+        return SV_ERR_ALIGN;
+    if (max_sel < 1) return SV_ERR_SHAPE;
+    if (!(softmax_scale >= 0.f)) return SV_ERR_SHAPE;
+    return SV_OK;
+}
+
+static sv_status check_workspace(int splits, const void *workspace, size_t bytes, size_t needed)
+{
+    if (splits <= 1) return SV_OK;
+    if (!workspace) return SV_ERR_NULL;
+    if (!svh::aligned(workspace, 16)) return SV_ERR_ALIGN;
+    return bytes < needed ? SV_ERR_WORKSPACE : SV_OK;
+}
+
 // `balance`: see choose_splits (the built-in-scratch entry point gives it up when the partials would not fit)
 static sv_status verify_attn_impl(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
                                   const void *draft_v, const int32_t *parent, const int32_t *sel_idx,
@@ -208,69 +287,26 @@ static sv_status verify_attn_impl(const sv_geom *geom, const void *q, const sv_k
     if (st != SV_OK) return st;
     st = svh::check_kv(geom, kv, true);
     if (st != SV_OK) return st;
-    if (!q || !draft_k || !draft_v || !out) return SV_ERR_NULL;
-    if (sel_idx && !sel_cnt) return SV_ERR_NULL;
-    if (!svh::aligned(q, 16) || !svh::aligned(draft_k, 16) || !svh::aligned(draft_v, 16) || !svh::aligned(out, 16))
-        return SV_ERR_ALIGN;
     if (!sel_idx) max_sel = geom->max_blocks;
-    if (max_sel < 1) return SV_ERR_SHAPE;
-    if (!(softmax_scale >= 0.f)) return SV_ERR_SHAPE;
-
-    const int G = geom->n_q_heads / geom->n_kv_heads;
-    const int rows = G * geom->n_draft;
+    st = check_attn_args(q, draft_k, draft_v, sel_idx, sel_cnt, max_sel, softmax_scale, out);
+    if (st != SV_OK) return st;
     const int splits = choose_splits(geom, max_sel, balance);
-    if (splits > 1) {
-        if (!workspace) return SV_ERR_NULL;
-        if (!svh::aligned(workspace, 16)) return SV_ERR_ALIGN;
-        if (workspace_bytes < workspace_bytes_for(geom, max_sel, balance)) return SV_ERR_WORKSPACE;
-    }
+    st = check_workspace(splits, workspace, workspace_bytes, workspace_bytes_for(geom, max_sel, balance));
+    if (st != SV_OK) return st;
 
     CUtensorMap tk, tv;
     const int64_t n_rows = (int64_t)kv->n_pages * geom->n_kv_heads * geom->block_size;
     if (!pool_tensor_map(kv->k_pool, n_rows, &tk) || !pool_tensor_map(kv->v_pool, n_rows, &tv)) return SV_ERR_CUDA;
 
     AttnParams p;
-    p.q = static_cast<const __nv_bfloat16 *>(q);
-    p.draft_k = static_cast<const __nv_bfloat16 *>(draft_k);
-    p.draft_v = static_cast<const __nv_bfloat16 *>(draft_v);
-    p.parent = parent;
+    fill_params(p, geom, geom, splits, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel, softmax_scale, out, lse, workspace,
+                status_word);
     p.block_table = kv->block_table;
     p.seq_lens = kv->seq_lens;
-    p.sel_idx = sel_idx;
-    p.sel_cnt = sel_cnt;
-    p.out = static_cast<__nv_bfloat16 *>(out);
-    p.lse = lse;
-    const size_t n_part_rows = (size_t)geom->n_seq * geom->n_kv_heads * splits * rows;
-    p.ws_o = static_cast<float *>(workspace);
-    p.ws_ml = workspace ? static_cast<float *>(workspace) + n_part_rows * 128 : nullptr;
-    p.status = status_word;
-    p.T = geom->n_draft, p.Hq = geom->n_q_heads, p.Hkv = geom->n_kv_heads, p.G = G, p.B = geom->block_size;
-    p.NBmax = geom->max_blocks, p.max_sel = max_sel, p.splits = splits;
-    p.Tt = svh::tokens_per_tile(geom), p.tiles = svh::row_tiles(geom);
-    p.pair = svh::pair_row_tiles(geom) ? 1 : 0;
     p.n_pages = kv->n_pages;
     p.early_gather = early_gather ? 1 : 0;
-    const float scale = softmax_scale > 0.f ? softmax_scale : 0.08838834764831845f;   // 1/sqrt(128)
-    p.scale_log2 = scale * 1.4426950408889634f;
-
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    dim3 grid(splits, geom->n_kv_heads, geom->n_seq);
-    grid.x = splits * svh::row_groups(geom);   // one CTA per (row tile or pair of row tiles, split)
-    if (launch_attn_tc(tk, tv, p, grid, cs) != cudaSuccess) return SV_ERR_CUDA;
-    if (splits > 1) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((rows * 32 + kMergeThreads - 1) / kMergeThreads, geom->n_kv_heads, geom->n_seq);
-        cfg.blockDim = dim3(kMergeThreads);
-        cfg.stream = cs;
-        cudaLaunchAttribute attr[1];
-        svh::pdl_attribute(attr);
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const cudaError_t me = splits <= 4 ? cudaLaunchKernelEx(&cfg, merge_splits_kernel<4>, p)
-                                           : cudaLaunchKernelEx(&cfg, merge_splits_kernel<20>, p);
-        if (me != cudaSuccess) return SV_ERR_CUDA;
-    }
-    return SV_OK;
+    return launch_attn(p, geom, geom->n_seq, cs, [&](dim3 grid) { return launch_attn_tc(tk, tv, p, grid, cs); });
 }
 
 extern "C" sv_status sv_verify_attn(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
@@ -291,6 +327,82 @@ extern "C" sv_status sv_verify_attn_reused(const sv_geom *geom, const void *q, c
 {
     return verify_attn_impl(geom, q, kv, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel, softmax_scale, out, lse,
                             workspace, workspace_bytes, status_word, stream, true, true);
+}
+
+// ---------------------------------------------------------------------- several layers at once
+
+extern "C" size_t sv_layer_table_bytes(int32_t n_layers)
+{
+    return n_layers < 1 || n_layers > SV_MAX_LAYERS ? 0 : (size_t)n_layers * sizeof(LayerRow);
+}
+
+extern "C" sv_status sv_layer_table(const sv_geom *geom, const sv_kv *kv, int32_t n_layers, void *table_host)
+{
+    sv_status st = svh::check_geom(geom);
+    if (st != SV_OK) return st;
+    if (!kv || !table_host) return SV_ERR_NULL;
+    if (n_layers < 1 || n_layers > SV_MAX_LAYERS) return SV_ERR_SHAPE;
+    for (int l = 0; l < n_layers; ++l) {
+        st = svh::check_kv(geom, kv + l, true);
+        if (st != SV_OK) return st;
+        LayerRow row = {};
+        const int64_t n_rows = (int64_t)kv[l].n_pages * geom->n_kv_heads * geom->block_size;
+        if (!encode_pool_map(kv[l].k_pool, n_rows, &row.k_map) || !encode_pool_map(kv[l].v_pool, n_rows, &row.v_map)) return SV_ERR_CUDA;
+        row.k_pool = const_cast<void *>(kv[l].k_pool), row.v_pool = const_cast<void *>(kv[l].v_pool);
+        row.n_pages = kv[l].n_pages;
+        memcpy(static_cast<char *>(table_host) + l * sizeof(LayerRow), &row, sizeof row);
+    }
+    return SV_OK;
+}
+
+// The geometry the split rules see for a stack: every (layer, sequence) is a sequence of one batch.
+static sv_geom stack_geom(const sv_geom *geom, int32_t n_layers)
+{
+    sv_geom g = *geom;
+    g.n_seq *= n_layers;
+    return g;
+}
+
+extern "C" size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layers, int32_t max_sel)
+{
+    if (svh::check_geom(geom) != SV_OK || n_layers < 1 || n_layers > SV_MAX_LAYERS || max_sel < 1) return 0;
+    const sv_geom g = stack_geom(geom, n_layers);
+    return svh::check_geom(&g) != SV_OK ? 0 : workspace_bytes_for(&g, max_sel, true);
+}
+
+extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                           const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
+                                           const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                           int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                                           size_t workspace_bytes, int32_t *status_word, void *stream)
+{
+    sv_status st = svh::check_layers(geom, layers, first, end);
+    if (st != SV_OK) return st;
+    if (!sel_idx) max_sel = geom->max_blocks;
+    st = check_attn_args(q, draft_k, draft_v, sel_idx, sel_cnt, max_sel, softmax_scale, out);
+    if (st != SV_OK) return st;
+    if (sel_idx && (!anchors || !anchors[0])) return SV_ERR_NULL;
+    const sv_geom rule = stack_geom(geom, layers->n_layers);
+    const int splits = choose_splits(&rule, max_sel);
+    st = check_workspace(splits, workspace, workspace_bytes, workspace_bytes_for(&rule, max_sel, true));
+    if (st != SV_OK) return st;
+    StackAttnParams p;
+    const size_t skip = (size_t)first * geom->n_seq * geom->n_draft * 128;   // rows of the layers ahead, per head
+    const auto from_first = [&](const void *x, int heads) { return static_cast<const __nv_bfloat16 *>(x) + skip * heads; };
+    fill_params(p, geom, &rule, splits, from_first(q, geom->n_q_heads), from_first(draft_k, geom->n_kv_heads),
+                from_first(draft_v, geom->n_kv_heads), parent, sel_idx, sel_cnt, max_sel, softmax_scale,
+                const_cast<__nv_bfloat16 *>(from_first(out, geom->n_q_heads)), nullptr, workspace, status_word);
+    p.block_table = layers->block_table;
+    p.seq_lens = layers->seq_lens;
+    p.n_pages = 0;   // (in the table)
+    p.layers = static_cast<const LayerRow *>(layers->table) + first;
+    p.S = geom->n_seq;
+    for (int l = 0, list = -1; l < end; ++l) {
+        if (sel_idx && anchors[l]) ++list;
+        if (l >= first) p.list_of[l - first] = (uint8_t)(list < 0 ? 0 : list);
+    }
+    cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    return launch_attn(p, &rule, geom->n_seq * (end - first), cs, [&](dim3 grid) { return launch_attn_tc_stack(p, grid, cs); });
 }
 
 // ---------------------------------------------------------------------- sv_verify_attn_noalloc

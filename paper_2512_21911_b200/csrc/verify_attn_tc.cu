@@ -30,6 +30,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "attn_common.cuh"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
@@ -78,10 +80,11 @@ enum Bar {
 // kPair (with kWide, NH = 4): the CTA serves two row tiles of its (sequence, KV head) from one gather: warpgroup w owns
 // row tile 2 * pair + w -- its own Q tile, S / P / O buffers -- and takes every unit instead of every other one.  The
 // host chooses it where it saves enough waves of CTAs (svh::pair_row_tiles).
-template <int NH, bool kWide, bool kPair, bool kUnitSlices>
+// kStack: several layers in one launch (StackAttnParams; the tensor maps are then those of the layer table).
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                          const AttnParams p)
+                          const std::conditional_t<kStack, StackAttnParams, AttnParams> p)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -113,7 +116,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     // those of the executing warpgroup (the query rows of draft tokens i0 .. i0 + Tq - 1).
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_groups = kPair ? (p.tiles + 1) / 2 : p.tiles;
-    const int split = kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, s = blockIdx.z;
+    const int split = kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, z = blockIdx.z;
+    // z numbers what the layer owns (q, out, draft, partials), s its sequence (tables, lengths, parents), lz its list
+    int s = z, lz = z;
+    const LayerRow *layer = nullptr;
+    if constexpr (kStack) {
+        const int l = z / p.S;
+        s = z - l * p.S;
+        lz = p.list_of[l] * p.S + s;
+        layer = p.layers + l;
+    }
     const int group = kWide ? blockIdx.x - split * n_groups : 0;
     const int tile = kPair ? 2 * group + ((warp >> 2) & 1) : group;
     const int i0 = kWide ? tile * p.Tt : 0, Tq = kWide ? max(0, min(p.Tt, p.T - i0)) : p.T;
@@ -182,9 +194,19 @@ __global__ void __launch_bounds__(kThreads, 1)
         reg_dealloc<40>();   // hand registers to the softmax warpgroups
         if (warp == 8) {
             // ---------------------------------------------------------- TMA producer
+            const CUtensorMap *mk = &tm_k, *mv = &tm_v;
+            int n_pages = p.n_pages;
+            if constexpr (kStack) {
+                mk = &layer->k_map, mv = &layer->v_map;
+                n_pages = layer->n_pages;
+                if (lane == 0) {   // (maps in global memory: the proxy that fetches them is told once)
+                    tensormap_acquire(mk);
+                    tensormap_acquire(mv);
+                }
+            }
             if (lane == 0) {
-                tma_prefetch_desc(&tm_k);
-                tma_prefetch_desc(&tm_v);
+                tma_prefetch_desc(mk);
+                tma_prefetch_desc(mv);
             }
             const uint64_t policy = policy_evict_first();
             // pull this sequence's block-table row towards L2 while the previous kernel drains
@@ -199,10 +221,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int j0_spec = kUnitSlices ? slice_begin(split, p.max_sel) >> 1 : slice_begin(split, p.max_sel);
             int blk_spec = 0;
             if (p.sel_idx && j0_spec + lane < p.max_sel)
-                blk_spec = p.sel_idx[((size_t)s * p.Hkv + h) * p.max_sel + j0_spec + lane];
+                blk_spec = p.sel_idx[((size_t)lz * p.Hkv + h) * p.max_sel + j0_spec + lane];
             const int L = p.seq_lens[s];
             const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-            const int cnt_in = p.sel_idx ? p.sel_cnt[(size_t)s * p.Hkv + h] : nb;
+            const int cnt_in = p.sel_idx ? p.sel_cnt[(size_t)lz * p.Hkv + h] : nb;
             // a negative count marks a list that block selection could not produce: attend over the draft tokens
             // only, and say so
             if (cnt_in < 0 && lane == 0 && p.status) atomicOr(p.status, kStatusNoList);
@@ -218,12 +240,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (j < j1) {
                     int blk = j;
                     if (p.sel_idx)
-                        blk = (base == j0 && j0 == j0_spec) ? blk_spec : p.sel_idx[((size_t)s * p.Hkv + h) * p.max_sel + j];
+                        blk = (base == j0 && j0 == j0_spec) ? blk_spec : p.sel_idx[((size_t)lz * p.Hkv + h) * p.max_sel + j];
                     // indices are clamped into their tables before any address is formed; a clamp that fires is reported
                     const int blk_in = blk;
                     blk = max(0, min(blk, p.NBmax - 1));
                     const int page_in = p.block_table[(size_t)s * p.NBmax + blk];
-                    const int page = max(0, min(page_in, p.n_pages - 1));
+                    const int page = max(0, min(page_in, n_pages - 1));
                     if ((blk != blk_in || page != page_in) && p.status) atomicOr(p.status, kStatusIndex);
                     row0 = (page * p.Hkv + h) * p.B;
                     tok0 = blk * p.B;
@@ -254,8 +276,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             mbar_arrive_expect_tx(fb, kStageBytes);
                             // one copy per operand: the box spans both 64-column halves (third coordinate), which
                             // land as two consecutive [64 rows][128 bytes] swizzled tiles
-                            tma_load_3d(dst, &tm_k, 0, y, 0, fb, policy);
-                            tma_load_3d(dst + 2 * kTile, &tm_v, 0, y, 0, fb, policy);
+                            tma_load_3d(dst, mk, 0, y, 0, fb, policy);
+                            tma_load_3d(dst + 2 * kTile, mv, 0, y, 0, fb, policy);
                         }
                     }
                 }
@@ -268,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 grid_dependency_wait();   // the lengths may come from the kernel just before (a cache commit)
                 const int L = p.seq_lens[s];
                 const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-                const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)s * p.Hkv + h], p.max_sel)) : nb;
+                const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
                 const int off = has_draft ? 1 : 0;
                 const int n_total = slice_units(split, n_sel) + off;
                 bool dead = !mbar_wait_bounded(bar(kStaged), 0);
@@ -390,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (idx < n_q) {
                 const int r = idx >> 4, c = idx & 15;
                 const int i = div_g(r), g = r - i * p.G;
-                v[x] = __ldg(reinterpret_cast<const uint4 *>(p.q + (((size_t)s * p.T + i0 + i) * p.Hq + h * p.G + g) * 128) + c);
+                v[x] = __ldg(reinterpret_cast<const uint4 *>(p.q + (((size_t)z * p.T + i0 + i) * p.Hq + h * p.G + g) * 128) + c);
             }
         }
         uint4 w[kDB];
@@ -399,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int idx = tid + x * 256;
             if (idx < n_d) {
                 const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;   // K rows, then V rows
-                const __nv_bfloat16 *src = (which ? p.draft_v : p.draft_k) + (((size_t)s * p.T + r) * p.Hkv + h) * 128;
+                const __nv_bfloat16 *src = (which ? p.draft_v : p.draft_k) + (((size_t)z * p.T + r) * p.Hkv + h) * 128;
                 w[x] = __ldg(reinterpret_cast<const uint4 *>(src) + c);
             }
         }
@@ -512,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int L = p.seq_lens[s];
     const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-    const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)s * p.Hkv + h], p.max_sel)) : nb;
+    const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
     const int off = has_draft ? 1 : 0;
     const int n_total = slice_units(split, n_sel) + off;
 
@@ -849,14 +871,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (row >= rows) continue;
             if (p.splits == 1) {
                 const int ii = div_g(row), g = row - ii * p.G;
-                const size_t orow = ((size_t)s * p.T + i0 + ii) * p.Hq + h * p.G + g;
+                const size_t orow = ((size_t)z * p.T + i0 + ii) * p.Hq + h * p.G + g;
                 const float inv = 1.f / lsum;
                 uint32_t *dst = reinterpret_cast<uint32_t *>(p.out + orow * 128) + ch * 32 + qd;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) dst[4 * j] = pack_bf16(o[i][2 * j] * inv, o[i][2 * j + 1] * inv);
                 if (p.lse && ch == 0 && qd == 0) p.lse[orow] = (M + log2f(lsum)) * 0.69314718055994531f;
             } else {
-                const size_t prow = (((size_t)s * p.Hkv + h) * p.splits + split) * (p.G * p.T) + i0 * p.G + row;
+                const size_t prow = (((size_t)z * p.Hkv + h) * p.splits + split) * (p.G * p.T) + i0 * p.G + row;
                 float2 *dst = reinterpret_cast<float2 *>(p.ws_o + prow * 128) + ch * 32 + qd;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) dst[4 * j] = make_float2(o[i][2 * j], o[i][2 * j + 1]);
@@ -868,15 +890,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-template <int NH, bool kWide, bool kPair, bool kUnitSlices = false>
-static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid,
-                             cudaStream_t stream)
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, class Params>
+static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
+    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>>;
     static svh::OncePerDevice once;   // function attributes belong to a device
-    const cudaError_t ce = once.run([] {
-        return cudaFuncSetAttribute(verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kSmemBytes);
-    });
+    const cudaError_t ce =
+        once.run([] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); });
     if (ce != cudaSuccess) return ce;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -887,29 +907,40 @@ static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, c
     svh::pdl_attribute(attr);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices>, tm_k, tm_v, p);
+    return cudaLaunchKernelEx(&cfg, kernel, tm_k, tm_v, p);
 }
 
 // grid.x = splits x groups, where a group is a row tile or (p.pair) a pair of row tiles
-cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid,
-                           cudaStream_t stream)
+template <class Params>
+static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
     const int rows = p.G * p.Tt;   // rows of a full row tile
     const bool units = p.B == 128;   // 128-row tiles over blocks of 128 tokens: slices cut at 64-key units
     if (p.pair) {   // (a full tile has more than 64 rows)
         return units ? launch_tc<4, true, true, true>(tm_k, tm_v, p, grid, stream)
-                     : launch_tc<4, true, true>(tm_k, tm_v, p, grid, stream);
+                     : launch_tc<4, true, true, false>(tm_k, tm_v, p, grid, stream);
     }
     if (p.tiles > 1 || p.T > 32) {
-        if (rows <= 32) return launch_tc<1, true, false>(tm_k, tm_v, p, grid, stream);
-        if (rows <= 64) return launch_tc<2, true, false>(tm_k, tm_v, p, grid, stream);
+        if (rows <= 32) return launch_tc<1, true, false, false>(tm_k, tm_v, p, grid, stream);
+        if (rows <= 64) return launch_tc<2, true, false, false>(tm_k, tm_v, p, grid, stream);
         return units ? launch_tc<4, true, false, true>(tm_k, tm_v, p, grid, stream)
-                     : launch_tc<4, true, false>(tm_k, tm_v, p, grid, stream);
+                     : launch_tc<4, true, false, false>(tm_k, tm_v, p, grid, stream);
     }
-    if (rows <= 32) return launch_tc<1, false, false>(tm_k, tm_v, p, grid, stream);
-    if (rows <= 64) return launch_tc<2, false, false>(tm_k, tm_v, p, grid, stream);
+    if (rows <= 32) return launch_tc<1, false, false, false>(tm_k, tm_v, p, grid, stream);
+    if (rows <= 64) return launch_tc<2, false, false, false>(tm_k, tm_v, p, grid, stream);
     return units ? launch_tc<4, false, false, true>(tm_k, tm_v, p, grid, stream)
-                 : launch_tc<4, false, false>(tm_k, tm_v, p, grid, stream);
+                 : launch_tc<4, false, false, false>(tm_k, tm_v, p, grid, stream);
+}
+
+cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid, cudaStream_t stream)
+{
+    return launch_any(tm_k, tm_v, p, grid, stream);
+}
+
+cudaError_t launch_attn_tc_stack(const StackAttnParams &p, dim3 grid, cudaStream_t stream)
+{
+    static const CUtensorMap none = {};
+    return launch_any(none, none, p, grid, stream);
 }
 
 }  // namespace svk

@@ -1,8 +1,10 @@
 """SparseVerifier: runs block selection and sparse verification attention for a stack of layers.
 
-A thin driver over the C-ABI calls: it owns the per-layer representatives, the shared block list,
-the split-KV workspace and the outputs, and enqueues, per layer, ``sv_select_blocks`` (anchor
-layers) or the reuse of the previous layer's list (Eq. 9), then ``sv_verify_attn``; after verification,
+A thin driver over the C-ABI calls: it owns the per-layer representatives, the block lists,
+the split-KV workspace and the outputs.  ``verify_layer`` enqueues one layer: ``sv_select_blocks`` (anchor
+layers) or the reuse of the previous layer's list (Eq. 9), then ``sv_verify_attn``.  ``verify_step`` is handed the inputs
+of all layers at once; but for the lists they reuse the layers are then independent problems, so it runs all
+selections in one launch and all attention in another.  After verification,
 ``accept`` (Eq. 2-3) and ``commit`` (append the kept rows to the cache) close the decoding step.  All compute
 is in the library's kernels; this class only holds buffers and calls them in order.
 """
@@ -29,51 +31,95 @@ class SparseVerifier:
         assert self.anchors[0], "layer 0 has no preceding layer to reuse"
         dev = torch.device(device)
         self.reps = torch.zeros((n_layers, n_seq, n_kv_heads, max_blocks, head_dim), dtype=torch.float32, device=dev)
-        self.sel_idx = torch.zeros((n_seq, n_kv_heads, max_sel), dtype=torch.int32, device=dev)
-        self.sel_cnt = torch.zeros((n_seq, n_kv_heads), dtype=torch.int32, device=dev)
+        self._make_lists(bytes(map(bool, self.anchors)), dev)
         self.workspace = torch.empty(max(16, sv.sv_workspace_bytes(self.geom, max_sel)), dtype=torch.uint8, device=dev)
         self.dense_workspace = None
         self.status = torch.zeros(1, dtype=torch.int32, device=dev)
         self.kv: List[Optional[sv.sv_kv]] = [None] * n_layers
         self._pools = [None] * n_layers   # keep the tensors alive
-        self._stack_kv = None
+        self._one_allocation = False
         self._copy_streams = None
+        self._stack_workspace = [None, None]   # sparse, dense
+        self._counters = torch.zeros(2 * n_seq, dtype=torch.int32, device=dev)   # see sv_kv_append_layers
+        # what the layers' kernels look up when several layers run in one launch (a row is valid once its layer has pools)
+        stackable = n_layers <= sv.SV_MAX_LAYERS and n_layers * n_seq <= 65535
+        row = sv._lib.sv_layer_table_bytes(1)
+        self._table = torch.zeros((n_layers, row), dtype=torch.uint8, device=dev) if stackable else None
+        self._rows_missing = n_layers
+
+    def _make_lists(self, flags: bytes, dev) -> None:
+        """One block list per anchor layer; sel_idx / sel_cnt is the last one, which is also what verify_layer keeps its
+        current list in."""
+        g, n = self.geom, max(1, sum(flags))
+        self._flags = flags
+        self._lists_idx = torch.zeros((n, g.n_seq, g.n_kv_heads, self.max_sel), dtype=torch.int32, device=dev)
+        self._lists_cnt = torch.zeros((n, g.n_seq, g.n_kv_heads), dtype=torch.int32, device=dev)
+        self.sel_idx, self.sel_cnt = self._lists_idx[-1], self._lists_cnt[-1]
 
     def set_layer_kv(self, layer: int, k_pool: torch.Tensor, v_pool: torch.Tensor) -> None:
+        new = self.kv[layer] is None
         self._pools[layer] = (k_pool, v_pool)
         self.kv[layer] = sv.make_kv(k_pool, v_pool, self.block_table, self.seq_lens)
+        if self._table is not None:
+            row = sv._native.layer_row(self.geom, self.kv[layer])
+            if isinstance(row, int):
+                self._table = None   # not a cache the kernels take: the call that uses it says so
+            else:
+                self._table[layer].copy_(torch.frombuffer(bytearray(row), dtype=torch.uint8))
+        self._rows_missing -= new
 
     def set_kv_stack(self, k_all: torch.Tensor, v_all: torch.Tensor) -> None:
-        """All layers' pools in one allocation, bf16 [layers][n_pages][Hkv][B][D].  Besides the per-layer
-        descriptors this builds a stacked view in which (layer, sequence) is the batch dimension, so that
-        the tail-block refresh of every layer is a single sv_block_reps launch."""
-        n_layers, n_pages = int(k_all.shape[0]), int(k_all.shape[1])
+        """All layers' pools in one allocation, bf16 [layers][n_pages][Hkv][B][D]."""
+        n_layers = int(k_all.shape[0])
         assert n_layers == self.n_layers and k_all.is_contiguous() and v_all.is_contiguous()
         for l in range(n_layers):
             self.set_layer_kv(l, k_all[l], v_all[l])
-        g = self.geom
-        self._stack_offs = (torch.arange(n_layers, device=k_all.device, dtype=torch.int32) * n_pages).view(n_layers, 1, 1)
-        self._stack_table = torch.empty((n_layers * g.n_seq, g.max_blocks), dtype=torch.int32, device=k_all.device)
-        self._stack_pages = n_pages
-        self.sync_block_table()
-        self._stack_lens = self.seq_lens.repeat(n_layers).contiguous()
-        self._stack_geom = sv.make_geom(g.n_seq * n_layers, g.n_q_heads, g.n_kv_heads, g.head_dim, g.block_size,
-                                        g.max_blocks, g.n_draft)
-        self._stack_pools = (k_all, v_all)
-        self._stack_kv = sv.make_kv(k_all.view(n_layers * n_pages, *k_all.shape[2:]),
-                                    v_all.view(n_layers * n_pages, *v_all.shape[2:]), self._stack_table,
-                                    self._stack_lens)
+        self._one_allocation = True
 
     def sync_block_table(self) -> None:
-        """Rebuild the stacked page table from block_table (call after assigning pages to a sequence; commit does it
-        itself).  Entries that are not pages of a layer's pool stay invalid in every layer."""
-        bt = self.block_table.unsqueeze(0)
-        ok = (bt >= 0) & (bt < self._stack_pages)
-        self._stack_table.copy_(torch.where(ok, bt + self._stack_offs, -1).reshape(self._stack_table.shape))
+        """Kept for callers that announce newly assigned pages: every launch reads block_table itself, so there is nothing
+        to rebuild."""
+
+    def _stacked(self) -> bool:
+        """Whether launches may cover several layers: every layer has its pools, over the same page table and lengths."""
+        return self._table is not None and self._rows_missing == 0
 
     def refresh_tail_all(self) -> None:
         """Recompute the representative of every sequence's last block in all layers (one launch)."""
-        sv.sv_block_reps(self._stack_geom, self._stack_kv, self.reps.view(-1, *self.reps.shape[2:]), sv.SV_TAIL_BLOCK)
+        self._refresh_tail(None)
+
+    def _refresh_tail(self, which: Optional[bytes]) -> None:
+        if self._stacked():
+            sv._check(sv._native.block_reps_layers(self.geom, self._table, self.kv[0], which, sv.SV_TAIL_BLOCK, -1, self.reps),
+                      "sv_block_reps_layers")
+            return
+        for l in range(self.n_layers):
+            if which is None or which[l]:
+                sv.sv_block_reps(self.geom, self.kv[l], self.reps[l], sv.SV_TAIL_BLOCK)
+
+    def _anchor_flags(self) -> bytes:
+        flags = bytes(map(bool, self.anchors))
+        if flags != self._flags:
+            self._make_lists(flags, self.workspace.device)
+        return flags
+
+    def _run_layers(self, first: int, end: int, q, draft_k, draft_v, out, dense: bool = False) -> bool:
+        """Layers first .. end - 1 in two launches (dense: one; three when the splits have to be merged).  False when the
+        inputs are not stacked tensors: the caller then goes layer by layer."""
+        if not self._stacked():
+            return False
+        flags = self._anchor_flags()
+        if self._stack_workspace[dense] is None:
+            n = sv._native.workspace_bytes_layers(self.geom, self.n_layers, self.geom.max_blocks if dense else self.max_sel)
+            self._stack_workspace[dense] = torch.empty(max(16, n), dtype=torch.uint8, device=self.workspace.device)
+        failed = sv._native.verify_layers(self.geom, self._table, self.kv[0], first, end, flags, q, draft_k, draft_v, self.parent, out,
+                                          self.reps, self.budget, self.n_sink, self.n_local, None if dense else self._lists_idx,
+                                          None if dense else self._lists_cnt, self._stack_workspace[dense], self.status)
+        if failed is False:
+            return False
+        if failed:
+            raise sv.SvError(failed[0], "sv_select_blocks_layers" if failed[1] else "sv_verify_attn_layers")
+        return True
 
     def build_reps(self, layer: int, block_begin: int = 0, block_end: int = -1) -> None:
         """(Re)compute block representatives of a layer; a decoding loop only refreshes the tail block."""
@@ -104,15 +150,16 @@ class SparseVerifier:
         """One verification step of the whole stack.  q/out: [layers][S][T][Hq][D]; draft_k/v: [layers][S][T][Hkv][D].
 
         refresh_tail: first recompute the representative of every sequence's last block (the block that
-        grew when the previous step's accepted tokens were appended) -- one launch for all layers when the
-        pools were given with set_kv_stack, else one per anchor layer."""
+        grew when the previous step's accepted tokens were appended), in one launch: of all layers when the pools were
+        given with set_kv_stack, else of the anchor layers.
+
+        All layers' selections are one launch and all their attention another (32 layers of a 32K context: about 115 us
+        instead of 470 layer by layer, where every layer pays the latency chain of its kernels).  A model whose layers
+        wait for one another calls verify_layer."""
         if refresh_tail:
-            if self._stack_kv is not None:
-                self.refresh_tail_all()
-            else:
-                for l in range(self.n_layers):
-                    if self.anchors[l]:
-                        sv.sv_block_reps(self.geom, self.kv[l], self.reps[l], sv.SV_TAIL_BLOCK)
+            self._refresh_tail(None if self._one_allocation else self._anchor_flags())
+        if self._run_layers(0, self.n_layers, q, draft_k, draft_v, out):
+            return
         for l in range(self.n_layers):
             self.verify_layer(l, q[l], draft_k[l], draft_v[l], out[l], behind_own_layer=l > 0)
 
@@ -157,17 +204,13 @@ class SparseVerifier:
                 ev.record(s_in)
                 arrived.append(ev)
         if refresh_tail:
-            if self._stack_kv is not None:
-                self.refresh_tail_all()
-            else:
-                for l in range(self.n_layers):
-                    if self.anchors[l]:
-                        sv.sv_block_reps(self.geom, self.kv[l], self.reps[l], sv.SV_TAIL_BLOCK)
+            self._refresh_tail(None if self._one_allocation else self._anchor_flags())
         for (c0, c1), ev in zip(chunks, arrived):
             main.wait_event(ev)
-            for l in range(c0, c1):
-                # the kernel before a chunk's first layer is not this stream's previous layer alone (the upload joins there)
-                self.verify_layer(l, q[l], draft_k[l], draft_v[l], out[l], behind_own_layer=l > c0)
+            if not self._run_layers(c0, c1, q, draft_k, draft_v, out):
+                for l in range(c0, c1):
+                    # the kernel before a chunk's first layer is not this stream's previous layer alone (the upload joins there)
+                    self.verify_layer(l, q[l], draft_k[l], draft_v[l], out[l], behind_own_layer=l > c0)
             done = torch.cuda.Event()
             done.record(main)
             s_out.wait_event(done)
@@ -179,31 +222,21 @@ class SparseVerifier:
     def accept(self, p_target, p_draft, tokens, u_accept, u_next):
         """Acceptance of the step's draft tokens (Eq. 2-3).  Returns (path [S][T], n_path [S], next_token [S]):
         the rows whose K/V enter the cache (root first) and the token drawn after the kept path."""
-        S, T = int(self.geom.n_seq), int(self.geom.n_draft)
-        dev = p_target.device
-        path = torch.empty((S, T), dtype=torch.int32, device=dev)
-        n_path = torch.empty((S,), dtype=torch.int32, device=dev)
-        next_token = torch.empty((S,), dtype=torch.int32, device=dev)
-        sv.sv_accept(p_target, p_draft, tokens, self.parent, u_accept, u_next, path, n_path, next_token)
-        return path, n_path, next_token
+        got = sv._native.accept_new(p_target, p_draft, tokens, self.parent, u_accept, u_next, self.geom.n_seq, self.geom.n_draft)
+        if isinstance(got, int):
+            raise sv.SvError(got, "sv_accept")
+        return got
 
     def commit(self, draft_k, draft_v, path, n_path) -> None:
         """Append the kept rows' K/V of every layer to the paged cache (sv_kv_append, which also refreshes the
-        representatives of the blocks that grew: one launch for all layers when the pools were given with
-        set_kv_stack, else one per layer) and advance the sequence lengths.  The block table
-        must already hold pages for the blocks the sequences grow into.  draft_k/v: [layers][S][T][Hkv][D]."""
-        if self._stack_kv is not None:   # one launch for all layers: (layer, sequence) is the batch dimension
-            self.sync_block_table()
-            L, g = self.n_layers, self.geom
-            k_all, v_all = self._stack_pools
-            new_len = torch.empty_like(self._stack_lens)
-            sv.sv_kv_append(self._stack_geom, k_all.view(-1, *k_all.shape[2:]), v_all.view(-1, *v_all.shape[2:]),
-                            self._stack_table, self._stack_lens, draft_k.reshape(L * g.n_seq, *draft_k.shape[2:]),
-                            draft_v.reshape(L * g.n_seq, *draft_v.shape[2:]), path.repeat(L, 1), n_path.repeat(L), new_len,
-                            self.reps.view(-1, *self.reps.shape[2:]))
-            self._stack_lens.copy_(new_len)
-            self.seq_lens.copy_(new_len[:g.n_seq])
-            return
+        representatives of the blocks that grew, in one launch for all layers) and advance the sequence lengths.  The
+        block table must already hold pages for the blocks the sequences grow into.  draft_k/v: [layers][S][T][Hkv][D]."""
+        if self._stacked():
+            st = sv._native.kv_append_layers(self.geom, self._table, self.kv[0], draft_k, draft_v, path, n_path, self.seq_lens,
+                                             self._counters, self.reps)
+            if st is not False:
+                sv._check(st, "sv_kv_append_layers")
+                return
         new_len = torch.empty_like(self.seq_lens)
         for l in range(self.n_layers):
             k_pool, v_pool = self._pools[l]
@@ -216,20 +249,23 @@ class SparseVerifier:
         on a bounded wait, clamped a block index or page id, or met a list that block selection marked invalid
         (count -1).  The outputs written since the word was last zero are then invalid."""
         st = sv.sv_status_word_check(int(self.status.item()))
-        if st == sv.SV_OK and int(self.sel_cnt.min().item()) < 0:
+        if st == sv.SV_OK and int(self._lists_cnt.min().item()) < 0:
             st = 9   # SV_ERR_INDEX: a list marked invalid that no attention call has consumed yet
         if st != sv.SV_OK:
             raise sv.SvError(st, "SparseVerifier.check_status")
 
     def dense_step(self, q, draft_k, draft_v, out) -> None:
+        if self._run_layers(0, self.n_layers, q, draft_k, draft_v, out, dense=True):
+            return
         for l in range(self.n_layers):
             self.dense_layer(l, q[l], draft_k[l], draft_v[l], out[l])
 
     def kernels_per_step(self, refresh_tail: bool = False, dense: bool = False) -> int:
-        """Kernel launches of one step: tail refresh and select per anchor layer; attention (+ merge) per layer."""
+        """Kernel launches of one step taken layer by layer (verify_layer, the order in which a model reaches its layers):
+        tail refresh, select per anchor layer, attention (+ merge) per layer."""
         splits = sv.sv_verify_attn_splits(self.geom, self.geom.max_blocks if dense else self.max_sel)
         attn = self.n_layers * (2 if splits > 1 else 1)
         if dense:
             return attn
-        refresh = 0 if not refresh_tail else (1 if self._stack_kv is not None else sum(self.anchors))
+        refresh = 0 if not refresh_tail else (1 if self._stacked() else sum(self.anchors))
         return refresh + sum(self.anchors) + attn
