@@ -391,7 +391,8 @@ SV_API sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, const 
  * layer's result does not depend on the layers it is launched with.
  *   sv_block_reps_layers   layers l with which[l] != 0 (host, uint8 [L]; NULL: all)
  *   sv_verify_attn_layers  sel_idx == NULL: dense verification (anchors may be NULL); workspace of
- *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes
+ *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes, the first 256 of them zeroed once by the
+ *                          caller and left to the call from then on (one workspace per stream)
  *   sv_kv_append_layers    advances seq_lens (which must be layers->seq_lens) in place; counters: dev uint32 [2 S], zeroed
  *                          once by the caller and left to this call from then on
  */

@@ -41,6 +41,8 @@ struct AttnParams {
     int Tt, tiles;   // draft tokens per row tile (G * Tt <= 128 query rows) and number of row tiles
     int pair;        // 1: a CTA serves two row tiles (grid.x = splits x ceil(tiles / 2)); 0: one (grid.x = splits x tiles)
     int n_pages;     // pages in each pool: page ids from the block table are clamped to it
+    int n_claims;       // > 0: that many lists are handed out to one CTA per SM (splits = 1)
+    uint32_t *claims;   // ... this many so far, less the first one of every CTA; zero before and after the launch
     int early_gather;   // 1: nothing the gather reads comes from the kernel just before; it starts ahead of the dependency wait
 };
 

@@ -18,6 +18,7 @@
 
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "attn_common.cuh"
@@ -227,6 +228,7 @@ static void fill_params(AttnParams &p, const sv_geom *geom, const sv_geom *rule,
     p.Tt = svh::tokens_per_tile(geom), p.tiles = svh::row_tiles(geom);
     p.pair = svh::pair_row_tiles(rule) ? 1 : 0;
     p.early_gather = 0;
+    p.n_claims = 0, p.claims = nullptr;
     const float scale = softmax_scale > 0.f ? softmax_scale : 0.08838834764831845f;   // 1/sqrt(128)
     p.scale_log2 = scale * 1.4426950408889634f;
 }
@@ -355,6 +357,16 @@ extern "C" sv_status sv_layer_table(const sv_geom *geom, const sv_kv *kv, int32_
     return SV_OK;
 }
 
+// Whether a stack's lists are handed out to resident CTAs (see verify_attn_tc.cu, kBal): more lists than SMs, so that CTAs
+// take several, and lists that are not cut to even out their lengths (choose_splits).  More than two row tiles are left to
+// CTAs of their own, which share their tiles through L2 by running side by side.  The rule looks at the whole stack: a
+// layer's result is the same whichever layers a launch covers.
+static bool hand_out(const sv_geom *rule, int max_sel)
+{
+    return svh::row_tiles(rule) <= 2 && (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
+}
+constexpr size_t kClaimsBytes = 256;
+
 // The geometry the split rules see for a stack: every (layer, sequence) is a sequence of one batch.
 static sv_geom stack_geom(const sv_geom *geom, int32_t n_layers)
 {
@@ -367,7 +379,8 @@ extern "C" size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layer
 {
     if (svh::check_geom(geom) != SV_OK || n_layers < 1 || n_layers > SV_MAX_LAYERS || max_sel < 1) return 0;
     const sv_geom g = stack_geom(geom, n_layers);
-    return svh::check_geom(&g) != SV_OK ? 0 : workspace_bytes_for(&g, max_sel, true);
+    if (svh::check_geom(&g) != SV_OK) return 0;
+    return hand_out(&g, max_sel) ? kClaimsBytes : workspace_bytes_for(&g, max_sel, true);
 }
 
 extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
@@ -384,7 +397,9 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
     if (sel_idx && (!anchors || !anchors[0])) return SV_ERR_NULL;
     const sv_geom rule = stack_geom(geom, layers->n_layers);
     const int splits = choose_splits(&rule, max_sel);
-    st = check_workspace(splits, workspace, workspace_bytes, workspace_bytes_for(&rule, max_sel, true));
+    const bool handed = hand_out(&rule, max_sel);
+    st = check_workspace(handed ? 2 : splits, workspace, workspace_bytes,
+                         handed ? kClaimsBytes : workspace_bytes_for(&rule, max_sel, true));
     if (st != SV_OK) return st;
     StackAttnParams p;
     const size_t skip = (size_t)first * geom->n_seq * geom->n_draft * 128;   // rows of the layers ahead, per head
@@ -402,6 +417,13 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
         if (l >= first) p.list_of[l - first] = (uint8_t)(list < 0 ? 0 : list);
     }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    if (handed) {
+        p.pair = p.tiles == 2;
+        p.n_claims = (end - first) * geom->n_seq * geom->n_kv_heads;
+        p.claims = static_cast<uint32_t *>(workspace);
+        p.ws_o = nullptr;
+        return launch_attn_tc_stack(p, dim3(std::min(sm_count(), p.n_claims)), cs) == cudaSuccess ? SV_OK : SV_ERR_CUDA;
+    }
     return launch_attn(p, &rule, geom->n_seq * (end - first), cs, [&](dim3 grid) { return launch_attn_tc_stack(p, grid, cs); });
 }
 

@@ -52,8 +52,9 @@ constexpr int kOffP = kStages * kStageBytes + kQBytes;   // (= 4 stages + 2 Q ti
 constexpr int kOffDraft = 0;                     // the draft unit is the first occupant of ring stage 0 (last split only)
 constexpr int kOffMisc = kOffP + 2 * kPBytes;
 constexpr int kSmemBytes = 1024 + kOffMisc + 1024;
-static_assert(kSmemBytes <= 232448, "shared memory budget");
-static_assert(2 * kMaxStages + 10 <= 32, "one lane of the producer warp per barrier");
+constexpr int kSmemBytesBal = kSmemBytes + 1024;   // (kBal) two sets of masks, segment descriptors
+static_assert(kSmemBytesBal <= 232448, "shared memory budget");
+static_assert(2 * kMaxStages + 17 <= 32, "one lane of the producer warp per barrier");
 static_assert((kStages - 1) * kStageBytes + 2 * kQBytes == kOffP, "both layouts put P at the same offset");
 constexpr int kTmemCols = 512;                   // S: 2 x 64 columns, O: 2 x 128 columns; 128-row tiles also P: 2 x 32 and
                                                  // Q: 64, or (two row tiles per CTA) Q: 2 x 64
@@ -70,8 +71,21 @@ enum Bar {
     kOReady = kPReady + 2,      // [2] the warpgroup's latest PV has been added to O in TMEM
     kStaged = kOReady + 2,      // Q (and the draft unit) are staged
     kTmemDone = kStaged + 1,    // all warps are done with TMEM
-    kNumBars = kTmemDone + 1
+    kLoaded = kTmemDone + 1,    // (kBal) the segment's descriptor, masks and Q tile are in shared memory
+    kTaken = kLoaded + 1,       // (kBal) ... and everybody has taken them from there: the next segment's may follow
+    kSlot = kTaken + 1,         // (kBal) the stage of the next draft unit is free
+    kClaim = kSlot + 1,         // (kBal) [2] the segment after next is known (segments take the two in turn)
+    kClaimTaken = kClaim + 2,   // (kBal) [2] ... and warp 11 has noted it
+    kNumBars = kClaimTaken + 2
 };
+
+// (kBal) One segment: the list of a (layer, sequence, KV head) and its draft tokens.
+struct alignas(16) Segment {
+    int n_total;   // units, the draft unit (the last one) included; -1: there is no further segment
+    int item;
+};
+constexpr uint32_t kLongWait = 1u << 22;   // polls of a wait that may last as long as a segment
+
 
 // NH = 8-row groups per TMEM lane quadrant that hold real query rows: 1 (rows <= 32), 2 (<= 64), 4 (<= 128).
 // kWide: more than one row tile per (sequence, KV head) or more than 32 draft tokens (64-bit ancestor masks).  The
@@ -81,7 +95,14 @@ enum Bar {
 // row tile 2 * pair + w -- its own Q tile, S / P / O buffers -- and takes every unit instead of every other one.  The
 // host chooses it where it saves enough waves of CTAs (svh::pair_row_tiles).
 // kStack: several layers in one launch (StackAttnParams; the tensor maps are then those of the layer table).
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack>
+// kBal: one resident CTA per SM that takes whole lists from a counter until there are none left (launches of more lists
+// than SMs).  Between two lists nothing drains: the TMA ring runs on into the next list, and warp 11 has that list's Q
+// tile, masks and draft K/V in shared memory by the time the warpgroups have written the last one's rows.  With one CTA
+// per list every list after an SM's first begins with an empty ring, 3 to 4 us of latencies for 45 us of HBM time (32 layers
+// of 8 lists of 65 units: 112.6 -> 108.8 us per step; 64 x 8 lists of 49 units: 155.7 -> 146.0).  Cutting lists so that all CTAs
+// end together costs more than it gains: the CTAs that are left have the HBM bandwidth to themselves, and partials have
+// to be written and merged (117 and 149 us).
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                           const std::conditional_t<kStack, StackAttnParams, AttnParams> p)
@@ -96,6 +117,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t *anc32 = reinterpret_cast<uint32_t *>(misc + 320);                     // [32] the same, up to 32 draft tokens
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 448);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + 456);
+    // (kBal) the masks of odd segments (64-bit: anc + 64), the segment descriptors, the claims on their way to warp 11
+    uint32_t *anc32_odd = reinterpret_cast<uint32_t *>(misc + 1536);
+    volatile Segment *segments = reinterpret_cast<volatile Segment *>(misc + 1664);
+    volatile int *claims = reinterpret_cast<volatile int *>(misc + 1696);
     auto bar = [&](int slot) { return bars + 8u * slot; };
 
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
@@ -109,6 +134,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int QR = NH == 4 ? 32 : 16;                    // tile rows per TMEM lane quadrant
     constexpr bool kPTmem = NH == 4 && !kPair;
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
+    // registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168); the roles of a balanced launch keep
+    // track of more
+    constexpr int kRegsMany = kBal ? (NH == 4 ? 216 : NH == 2 ? 208 : 200) : 232, kRegsFew = 504 - 2 * kRegsMany;
     constexpr int OFFQ = NS * kStageBytes;                   // the Q tile (kPair: of warpgroup 0; warpgroup 1's follows)
     // blockIdx.x = split * groups + group: the CTAs that gather the same slice of the blocks are neighbours in the grid
     // (they share those K/V tiles through L2; 1-2 % faster than group-major order).  A group is a row tile (kWide), or
@@ -116,21 +144,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     // those of the executing warpgroup (the query rows of draft tokens i0 .. i0 + Tq - 1).
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_groups = kPair ? (p.tiles + 1) / 2 : p.tiles;
-    const int split = kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, z = blockIdx.z;
+    const int split = kBal ? 0 : kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, z = blockIdx.z;   // (kBal: per segment)
     // z numbers what the layer owns (q, out, draft, partials), s its sequence (tables, lengths, parents), lz its list
     int s = z, lz = z;
     const LayerRow *layer = nullptr;
-    if constexpr (kStack) {
+    if constexpr (kStack && !kBal) {
         const int l = z / p.S;
         s = z - l * p.S;
         lz = p.list_of[l] * p.S + s;
         layer = p.layers + l;
     }
-    const int group = kWide ? blockIdx.x - split * n_groups : 0;
+    const int group = kWide && !kBal ? blockIdx.x - split * n_groups : 0;
     const int tile = kPair ? 2 * group + ((warp >> 2) & 1) : group;
     const int i0 = kWide ? tile * p.Tt : 0, Tq = kWide ? max(0, min(p.Tt, p.T - i0)) : p.T;
     const int upb = p.B / kUnit;
-    const bool has_draft = split == p.splits - 1;
+    const bool has_draft = kBal || split == p.splits - 1;
     const int rows = p.G * Tq;                               // query rows of this tile (0: the pair's second tile does not exist)
     constexpr int RPQ = 8 * NH;                              // query rows per TMEM lane quadrant
     const int n_active = min(4, (rows + RPQ - 1) / RPQ);     // warps of this softmax warpgroup that own real rows
@@ -174,28 +202,192 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t count = 1;
             if (lane == kSFree || lane == kPReady) count = na0;
             if (lane == kSFree + 1 || lane == kPReady + 1) count = max(1, na1);
-            if (lane == kStaged) count = 8;
+            if (lane == kStaged) count = kBal ? (kPair ? na0 + na1 : na0) : 8;
             if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0);
+            if (lane == kTaken) count = na0 + (n_wg == 2 ? na1 : 0) + 2;   // the softmax warps and both issuers
             mbar_init(bar(lane), count);
             mbar_fence_init();
         }
         if (lane == 0) *abort_flag = 0;
         __syncwarp();
-        named_bar_arrive(3, kThreads);
+        if constexpr (!kBal) named_bar_arrive(3, kThreads);
+    } else if constexpr (kBal) {
+        if (warp == 9) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+        tc_fence_before_sync();
     } else {
         if (warp == 9) tmem_alloc(smem_u32(tmem_slot), kTmemCols);
         tc_fence_before_sync();
         named_bar_sync(3, kThreads);
         tc_fence_after_sync();
     }
-    const uint32_t tmem_base = warp == 8 ? 0u : *tmem_slot;
+    // (kBal) what item i is made of: its list, the sequence it belongs to, its units without the draft unit
+    struct Item {
+        int z, h, s, lz, l;
+    };
+    auto item_at = [&](int i) {
+        Item it;
+        it.z = i / p.Hkv, it.h = i - it.z * p.Hkv;
+        it.s = it.z, it.lz = it.z, it.l = 0;
+        if constexpr (kStack) {
+            it.l = it.z / p.S;
+            it.s = it.z - it.l * p.S;
+            it.lz = p.list_of[it.l] * p.S + it.s;
+        }
+        return it;
+    };
+    // the number that says how many blocks (the list's count, or dense: the length), and the blocks it stands for
+    auto item_count = [&](const Item &it) { return p.sel_idx ? p.sel_cnt[(size_t)it.lz * p.Hkv + it.h] : p.seq_lens[it.s]; };
+    auto blocks_of = [&](int count) {
+        return p.sel_idx ? max(0, min(count, p.max_sel)) : max(0, min(p.B == 128 ? (count + 127) >> 7 : (count + 63) >> 6, p.NBmax));
+    };
+    auto item_blocks = [&](const Item &it) { return blocks_of(item_count(it)); };
+    // entry j of a list, and the page of a block
+    auto entry = [&](const Item &it, int j) {
+        if (!p.sel_idx) return j;
+        return j < p.max_sel ? p.sel_idx[((size_t)it.lz * p.Hkv + it.h) * p.max_sel + j] : 0;
+    };
+    auto page_of = [&](const Item &it, int blk) {
+        return p.block_table[(size_t)it.s * p.NBmax + max(0, min(blk, p.NBmax - 1))];
+    };
+    if constexpr (kBal) {
+        __syncthreads();   // the barriers are initialised, tensor memory is allocated
+        tc_fence_after_sync();
+    }
+    // after a wait that gave up: whatever this CTA still has in flight is through long before it frees its memory
+    auto let_copies_land = [] {
+        for (int i = 0; i < 100; ++i) __nanosleep(2000);
+    };
+    // query rows of a tile (draft tokens tok ..) to shared memory, 16 bytes per asynchronous copy, by n threads of which this is t
+    auto copy_q = [&](uint32_t tile_at, const Item &it, int tok, int n_rows, int t, int n) {
+        const int c = t & 15;
+        const __nv_bfloat16 *src = p.q + (((size_t)it.z * p.T + tok) * p.Hq + it.h * p.G) * 128 + c * 8;
+        const uint32_t dst = tile_at + (c >> 3) * (kQBytes / 2);
+#pragma unroll 4
+        for (int r = t >> 4; r < n_rows; r += n >> 4)
+            cp_async_16(dst + swz128((r / RPQ) * QR + (r % RPQ), c & 7), src + (r + div_g(r) * (p.Hq - p.G)) * 128);
+    };
+    const uint32_t tmem_base = warp == 8 && !kBal ? 0u : *tmem_slot;
 
     if (warp >= 8) {
-        reg_dealloc<40>();   // hand registers to the softmax warpgroups
+        reg_dealloc<kRegsFew>();   // hand registers to the softmax warpgroups
         if (warp == 8) {
             // ---------------------------------------------------------- TMA producer
             const CUtensorMap *mk = &tm_k, *mv = &tm_v;
             int n_pages = p.n_pages;
+            if constexpr (kBal) {
+                const uint64_t policy = policy_evict_first();
+                const int sh = upb - 1;   // units of a block: 1 << sh
+                bool dead = false;
+                if (!p.early_gather) grid_dependency_wait();   // the lists may come from the kernel just before
+                // A batch is 32 consecutive entries of one list, one per lane.  What the next segment needs -- its claim, count
+                // and first entries, their pages: three trips to L2, each needing the one before -- is fetched in steps
+                // between this segment's requests.
+                int ring = 0, draft_at = -1, layer_at = -1;
+                int claim = blockIdx.x;
+                Item cur = item_at(claim), nxt = cur;
+                int count = item_count(cur), L = p.seq_lens[cur.s];
+                int n_sel = blocks_of(count);
+                int blk_in = entry(cur, lane), page_in = page_of(cur, blk_in);
+                for (int seg = 0;; ++seg) {
+                    // a negative count marks a list that block selection could not produce: attend over the draft tokens
+                    // only, and say so
+                    if (p.sel_idx && count < 0 && lane == 0 && p.status) atomicOr(p.status, kStatusNoList);
+                    if constexpr (kStack) {
+                        if (cur.l != layer_at) {
+                            mk = &p.layers[cur.l].k_map, mv = &p.layers[cur.l].v_map;
+                            n_pages = p.layers[cur.l].n_pages;
+                            layer_at = cur.l;
+                            if (lane == 0) {
+                                tensormap_acquire(mk);
+                                tensormap_acquire(mv);
+                            }
+                        }
+                    }
+                    int count_next = 0, L_next = 0, blk_next = 0, page_next = 0, step = 0;
+                    if (lane == 0) claim = (int)atomicAdd(p.claims, 1u) + (int)gridDim.x;
+                    auto prepare_next = [&] {
+                        if (step == 0) {
+                            claim = __shfl_sync(0xffffffffu, claim, 0);
+                            // every CTA is refused once, so this many claims are made in all: the last one leaves zero behind
+                            if (lane == 0 && claim == p.n_claims + (int)gridDim.x - 1) atomicExch(p.claims, 0u);
+                            if (claim >= p.n_claims) claim = -1;
+                            // tell warp 11 (which has long noted the segment before this one)
+                            if (lane == 0 && !dead) {
+                                const int at = (seg + 1) & 1;
+                                if (seg >= 2 && (*abort_flag || !mbar_wait_bounded(bar(kClaimTaken + at), ((seg - 2) >> 1) & 1, kLongWait))) {
+                                    dead = true;
+                                    *abort_flag = 1;
+                                    if (p.status) atomicOr(p.status, 1);
+                                } else {
+                                    claims[at] = claim;
+                                    mbar_arrive(bar(kClaim + at));
+                                }
+                            }
+                            nxt = item_at(max(claim, 0));
+                            count_next = item_count(nxt), L_next = p.seq_lens[nxt.s];
+                            blk_next = entry(nxt, lane);
+                        } else if (step == 1) {
+                            page_next = page_of(nxt, blk_next);
+                        }
+                        ++step;
+                    };
+                    for (int base = 0; base < n_sel; base += 32) {
+                        // indices are clamped into their tables before any address is formed; a clamp that fires is reported
+                        const int blk = max(0, min(blk_in, p.NBmax - 1)), page = max(0, min(page_in, n_pages - 1));
+                        if ((blk != blk_in || page != page_in) && base + lane < n_sel && p.status) atomicOr(p.status, kStatusIndex);
+                        const int row0 = (page * p.Hkv + cur.h) * p.B, tok0 = blk * p.B;
+                        const bool more = base + 32 < n_sel;   // (more batches in this list)
+                        if (more) blk_in = entry(cur, base + 32 + lane);
+                        const int n_here = min(32, n_sel - base);
+                        for (int i = 0; i < n_here; ++i) {
+                            if (i & 1) prepare_next();
+                            if (i == n_here / 2 && more) page_in = page_of(cur, blk_in);
+                            const int r0 = __shfl_sync(0xffffffffu, row0, i);
+                            const int t0 = __shfl_sync(0xffffffffu, tok0, i);
+                            if (lane == 0 && !dead) {
+                                for (int uo = 0; uo < upb; ++uo) {
+                                    const int u = ring + ((base + i) << sh) + uo, stage = u % NS, it = u / NS;
+                                    if (it > 0 && (*abort_flag || !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
+                                        dead = true;
+                                        *abort_flag = 1;
+                                        if (p.status) atomicOr(p.status, 1);
+                                        break;
+                                    }
+                                    meta[stage] = max(0, min(kUnit, L - (t0 + uo * kUnit)));
+                                    const uint32_t fb = bar(kFull + stage), dst = smem0 + stage * kStageBytes;
+                                    mbar_arrive_expect_tx(fb, kStageBytes);
+                                    tma_load_3d(dst, mk, 0, r0 + uo * kUnit, 0, fb, policy);
+                                    tma_load_3d(dst + 2 * kTile, mv, 0, r0 + uo * kUnit, 0, fb, policy);
+                                }
+                            }
+                        }
+                    }
+                    ring += n_sel << sh;
+                    {
+                        // The draft unit's stage is filled by warp 11, which may be many rounds of the ring ahead; it is told
+                        // when the stage is free.  A barrier's parity only tells neighbouring rounds apart, so nobody is let
+                        // past a draft unit that is still on its way.
+                        if (lane == 0 && !dead) {
+                            const int stage = ring % NS, it = ring / NS;
+                            if (*abort_flag ||
+                                (draft_at >= 0 && ring - draft_at <= NS && !mbar_wait_bounded(bar(kFull + draft_at % NS), (draft_at / NS) & 1, kLongWait)) ||
+                                (it > 0 && !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
+                                dead = true;
+                                *abort_flag = 1;
+                                if (p.status) atomicOr(p.status, 1);
+                            } else {
+                                mbar_arrive(bar(kSlot));
+                            }
+                        }
+                        draft_at = ring++;
+                    }
+                    while (step < 2) prepare_next();
+                    if (claim < 0) break;
+                    cur = nxt, count = count_next, n_sel = blocks_of(count), L = L_next, blk_in = blk_next, page_in = page_next;
+                }
+                if (dead) let_copies_land();
+                return;
+            }
             if constexpr (kStack) {
                 mk = &layer->k_map, mv = &layer->v_map;
                 n_pages = layer->n_pages;
@@ -282,30 +474,157 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
             }
+        } else if (kBal && warp == 11) {
+            // ---------------------------------------------------------- (kBal) segments: descriptor, Q tile, masks, draft unit
+            int ring = 0, n_drafts = 0;
+            grid_dependency_wait();   // the queries may come from the kernel just before
+            for (int seg = 0;; ++seg) {
+                int claim = blockIdx.x;
+                bool ok = true;
+                if (seg > 0) {
+                    ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kClaim + (seg & 1)), ((seg - 1) >> 1) & 1, kLongWait));
+                    claim = claims[seg & 1];
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kClaimTaken + (seg & 1)));
+                    ok = ok && __all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kTaken), (seg - 1) & 1, kLongWait));
+                }
+                if (!ok) {
+                    *abort_flag = 1;
+                    if (p.status && lane == 0) atomicOr(p.status, 8);
+                    break;
+                }
+                volatile Segment *d = segments + (seg & 1);
+                if (claim < 0) {
+                    if (lane == 0) {
+                        d->n_total = -1;
+                        mbar_arrive(bar(kLoaded));
+                    }
+                    break;
+                }
+                const Item it = item_at(claim);
+                const int n_total = item_blocks(it) * upb + 1;
+                if (seg > 0) {   // (the first segment's is brought by the softmax warps)
+                    const uint32_t q_at = smem0 + OFFQ + (NH == 4 ? 0 : (seg & 1) * 8192);   // (an M = 64 tile fills half of either half)
+#pragma unroll
+                    for (int t = 0; t < (kPair ? 2 : 1); ++t)
+                        copy_q(q_at + t * kQBytes, it, t * p.Tt, t == 0 ? rows_w0 : rows_w1, lane, 32);
+                }
+                {   // lane i: tokens i and (kWide) 32 + i
+#pragma unroll
+                    for (int half = 0; half < (kWide ? 2 : 1); ++half) {
+                        const int tok = half * 32 + lane;
+                        unsigned long long mask = 0;
+                        if (!p.parent) {
+                            mask = tok >= p.T ? 0 : tok == 63 ? ~0ull : (1ull << (tok + 1)) - 1ull;
+                        } else {
+                            const int par0 = lane < p.T ? p.parent[(size_t)it.s * p.T + lane] : -1;
+                            const int par1 = kWide && 32 + lane < p.T ? p.parent[(size_t)it.s * p.T + 32 + lane] : -1;
+                            int at = tok < p.T ? tok : -1;
+                            for (int step = 0; step < p.T; ++step) {
+                                if (!__any_sync(0xffffffffu, at >= 0)) break;
+                                if (at >= 0) mask |= 1ull << at;
+                                const int n0 = __shfl_sync(0xffffffffu, par0, at & 31), n1 = __shfl_sync(0xffffffffu, par1, at & 31);
+                                const int up = at >= 32 ? n1 : n0;
+                                at = at >= 0 && up < at ? up : -1;   // parents must precede their children
+                            }
+                        }
+                        if constexpr (kWide)
+                            anc[(seg & 1) * 64 + tok] = mask;
+                        else
+                            (seg & 1 ? anc32_odd : anc32)[tok] = (uint32_t)mask;
+                    }
+                }
+                if (lane == 0) {
+                    d->n_total = n_total, d->item = claim;
+                }
+                cp_async_wait_all();
+                fence_proxy_async();
+                if (seg == 0) named_bar_sync(2, 288);   // the padding rows of the Q tiles are zero
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kLoaded));
+                {   // the last unit of the segment
+                    const int stage = (ring + n_total - 1) % NS;
+                    if (!__all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kSlot), n_drafts++ & 1, kLongWait))) {
+                        *abort_flag = 1;
+                        if (p.status && lane == 0) atomicOr(p.status, 1);
+                        break;
+                    }
+                    const uint32_t at = smem0 + stage * kStageBytes;
+                    for (int idx = lane; idx < 2 * p.T * 16; idx += 32) {   // K rows, then V rows
+                        const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;
+                        cp_async_16(at + which * (2 * kTile) + (c >> 3) * kTile + swz128(r, c & 7),
+                                    (which ? p.draft_v : p.draft_k) + (((size_t)it.z * p.T + r) * p.Hkv + it.h) * 128 + c * 8);
+                    }
+                    for (int idx = p.T * 16 + lane; idx < kUnit * 16; idx += 32) {   // (0 * junk must stay 0)
+                        const int r = idx >> 4, c = idx & 15;
+                        *reinterpret_cast<uint4 *>(smem + stage * kStageBytes + 2 * kTile + (c >> 3) * kTile + swz128(r, c & 7)) =
+                            make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    cp_async_wait_all();
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kFull + stage));
+                }
+                ring += n_total;
+            }
         } else if (warp == 9 || warp == 10) {
             // ---------------------------------------------------------- MMA issuers (one thread each)
             // warp 9 issues every S = Q K^T and owns the TMEM allocation; warp 10 issues every Ou = P V.
             // Descriptors are built once; per instruction only the 14-bit address field moves.
             if (lane == 0) {
-                grid_dependency_wait();   // the lengths may come from the kernel just before (a cache commit)
-                const int L = p.seq_lens[s];
-                const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-                const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
-                const int off = has_draft ? 1 : 0;
-                const int n_total = slice_units(split, n_sel) + off;
-                bool dead = !mbar_wait_bounded(bar(kStaged), 0);
+                int n_total = 0;
+                bool dead = false;
+                if constexpr (!kBal) {
+                    grid_dependency_wait();   // the lengths may come from the kernel just before (a cache commit)
+                    const int L = p.seq_lens[s];
+                    const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
+                    const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
+                    const int off = has_draft ? 1 : 0;
+                    n_total = slice_units(split, n_sel) + off;
+                    dead = !mbar_wait_bounded(bar(kStaged), 0);
+                }
+                // (kBal) per segment: its units, and what came before it: ring units, units of either warpgroup
+                int ring = 0, done0 = 0, done1 = 0;
+                bool end = false;
+                auto next_segment = [&](int seg, bool staged) {
+                    bool ok = !*abort_flag && mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait);
+                    if (ok) {
+                        n_total = segments[seg & 1].n_total;
+                        end = n_total < 0;
+                        if (end) return;
+                        // (before kTaken: a segment without units is over for the softmax warps once they have staged it)
+                        ok = !staged || mbar_wait_bounded(bar(kStaged), seg & 1);
+                    }
+                    if (ok) {
+                        mbar_arrive(bar(kTaken));
+                    } else {
+                        dead = true;
+                        *abort_flag = 1;
+                        if (p.status) atomicOr(p.status, 8);
+                    }
+                };
+                auto end_segment = [&] {
+                    ring += n_total;
+                    done0 += kPair ? n_total : (n_total + 1) >> 1;
+                    done1 += kPair ? n_total : n_total >> 1;
+                };
                 if (warp == 9) {
                     constexpr uint32_t idesc_s = umma_idesc_bf16(MT, kUnit, false);
                     const uint64_t dq = umma_desc_sw128(smem0 + OFFQ, 16, 1024);
                     const uint64_t dk = umma_desc_sw128(smem0, 16, 1024);
                     const uint32_t dq_lo = (uint32_t)dq, dk_lo = (uint32_t)dk;
                     const uint64_t d_hi = dq & 0xFFFFFFFF00000000ull;
+                    for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
+                    if constexpr (kBal) {
+                        next_segment(seg, kQTmem);
+                        if (end || dead) break;
+                    }
                     // one S per (unit, warpgroup that takes it): the warpgroups alternate units, or (kPair) each takes all
                     const int n_issue = kPair ? n_total * n_wg : n_total;
                     for (int x = 0; x < n_issue && !dead; ++x) {
                         const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
-                        const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = kPair ? u : (u >> 1);
-                        const int stage = u % NS, it = u / NS;
+                        const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = (kPair ? u : (u >> 1)) + (g ? done1 : done0);
+                        const int stage = (u + ring) % NS, it = (u + ring) / NS;
                         if (*abort_flag || !mbar_wait_bounded(bar(kFull + stage), it & 1) ||
                             (k > 0 && !mbar_wait_bounded(bar(kSFree + g), (k - 1) & 1))) {
                             dead = true;
@@ -318,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t d = tmem_base + g * kUnit;
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {
-                            const uint32_t qo = (uint32_t)(((kPair ? g * kQBytes : 0) + (ks >> 2) * (kQBytes / 2) + (ks & 3) * 32) >> 4);
+                            const uint32_t qo = (uint32_t)(((kPair ? g * kQBytes : 0) + (kBal ? (seg & 1) * 8192 : 0) + (ks >> 2) * (kQBytes / 2) + (ks & 3) * 32) >> 4);
                             const uint32_t ko = (uint32_t)(((ks >> 2) * kTile + (ks & 3) * 32) >> 4);
                             if constexpr (kQTmem)   // 16 dims = 8 packed columns of Q per instruction
                                 tc_mma_bf16_ta(d, tmem_base + (kPair ? kTmemP + g * 64 : kTmemQ) + ks * 8, d_hi | (k_lo + ko), idesc_s, ks > 0);
@@ -327,20 +646,28 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                         tc_commit(bar(kSReady + g));
                     }
+                    if constexpr (kBal) end_segment();
+                    }
+                    if (kBal && dead) let_copies_land();
                     // free TMEM only after every softmax warp has finished reading it
-                    if (!mbar_wait_bounded(bar(kTmemDone), 0) && p.status) atomicOr(p.status, 16);
+                    if (!mbar_wait_bounded(bar(kTmemDone), 0, kBal ? kLongWait : 1u << 19) && p.status) atomicOr(p.status, 16);
                 } else {
                     constexpr uint32_t idesc_pv = umma_idesc_bf16(MT, 128, true);
                     const uint64_t dp = umma_desc_sw128(smem0 + kOffP, 16, 1024);
                     const uint64_t dv = umma_desc_sw128(smem0 + 2 * kTile, kTile, 1024);
                     const uint32_t dp_lo = (uint32_t)dp, dv_lo = (uint32_t)dv;
                     const uint64_t dp_hi = dp & 0xFFFFFFFF00000000ull, dv_hi = dv & 0xFFFFFFFF00000000ull;
+                    for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
+                    if constexpr (kBal) {
+                        next_segment(seg, false);
+                        if (end || dead) break;
+                    }
                     const int n_issue = kPair ? n_total * n_wg : n_total;
                     for (int x = 0; x < n_issue && !dead; ++x) {
                         const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
                         const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = kPair ? u : (u >> 1);
-                        const int stage = u % NS;
-                        if (*abort_flag || !mbar_wait_bounded(bar(kPReady + g), k & 1)) {
+                        const int stage = (u + ring) % NS;
+                        if (*abort_flag || !mbar_wait_bounded(bar(kPReady + g), (k + (g ? done1 : done0)) & 1)) {
                             dead = true;
                             *abort_flag = 1;
                             if (p.status) atomicOr(p.status, 32);
@@ -362,6 +689,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         tc_commit(bar(kOReady + g));
                         if (!kPair || g == n_wg - 1) tc_commit(bar(kEmpty + stage));   // the last reader of the stage
                     }
+                    if constexpr (kBal) end_segment();
+                    }
                 }
             }
             if (warp == 9) {
@@ -374,23 +703,36 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 
     // ------------------------------------------------------------------ softmax warpgroups
-    reg_alloc<232>();
+    reg_alloc<kRegsMany>();
     // Stage Q and, in the last split, the draft tokens' K/V as one more unit; both in the swizzled layout
     // the tensor cores read.  Query row r = i*G + g (q[s][i][h*G + g][:]) goes to tile row
     // (r / RPQ)*32 + r % RPQ: RPQ rows per TMEM lane quadrant, so that all four warps of a warpgroup
     // share the softmax work even when only a few of the 128 tile rows are real.
     // The zero padding needs no input and is written while the previous kernel in the stream drains.
     // kPair: each warpgroup stages the Q tile of its own row tile (128 threads each); otherwise all 256 threads share one
+    if constexpr (kBal) grid_dependency_wait();   // the queries may come from the kernel just before
     constexpr int kQThreads = kPair ? 128 : 256;
     const int qtid = kPair ? (tid & 127) : tid;
     uint8_t *q_tile = smem + OFFQ + (kPair ? ((warp >> 2) & 1) * kQBytes : 0);
     for (int idx = qtid; idx < MT * 16; idx += kQThreads) {
         const int tr = idx >> 4, c = idx & 15;
         const int r = (tr / QR) * RPQ + (tr % QR);
-        if (!((tr % QR) < RPQ && r < rows))
+        if (!((tr % QR) < RPQ && r < rows)) {
             *reinterpret_cast<uint4 *>(q_tile + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = make_uint4(0u, 0u, 0u, 0u);
+            if (kBal && NH != 4)   // (two tiles, used in turn)
+                *reinterpret_cast<uint4 *>(q_tile + 8192 + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
-    if (has_draft) {
+    if (kBal) {
+        copy_q(smem0 + OFFQ + (kPair ? ((warp >> 2) & 1) * kQBytes : 0), item_at(blockIdx.x), i0, rows, qtid, kQThreads);   // (first segment)
+        // padding rows of Q in tensor memory that no active warp copies
+        if (kQTmem && (warp & 3) >= n_active && (kPair || warp < 4)) {
+            uint32_t zero[32] = {};
+            for (int half = 0; half < 2; ++half)
+                tmem_st_x32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (kPair ? kTmemP + (warp >> 2) * 64 : kTmemQ) + half * 32, zero);
+            tmem_st_wait();
+        }
+    } else if (has_draft) {
         for (int idx = tid; idx < 2 * kUnit * 16; idx += 256) {
             const int which = idx / (kUnit * 16);   // 0: K, 1: V
             const int r = (idx >> 4) % kUnit, c = idx & 15;
@@ -399,8 +741,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    grid_dependency_wait();
-    {
+    if constexpr (kBal) cp_async_wait_all();
+    if constexpr (!kBal) grid_dependency_wait();
+    if constexpr (!kBal) {
         // real rows: all loads of a thread are in flight together (16-byte chunks: Q up to 128 rows x 16, draft K and
         // V up to 64 tokens x 16 each)
         constexpr int kQB = (NH == 4 ? 8 : 4) * (kPair ? 2 : 1), kDB = kWide ? 8 : 4;
@@ -476,8 +819,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
     fence_proxy_async();   // the tensor cores read these tiles through the async proxy
-    named_bar_sync(2, 256);
-    if constexpr (kQTmem) {
+    if constexpr (kBal) {
+        tc_fence_before_sync();
+        named_bar_sync(2, 288);   // (with warp 11, which copies the real rows)
+        tc_fence_after_sync();
+    } else {
+        named_bar_sync(2, 256);
+    }
+    auto q_to_tmem = [&] {
         // Q goes on to tensor memory (thread = tile row = TMEM lane; the 64 32-bit words of the row are the 64 packed
         // columns): every S = Q K^T then reads only the K tile from shared memory, which is what bounds a
         // 128 x 64 x 16 MMA whose two operands both come from there.
@@ -496,9 +845,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             tmem_st_wait();
             tc_fence_before_sync();
         }
-    }
-    if (lane == 0) mbar_arrive(bar(kStaged));
-    if (has_draft && tid == 0) mbar_arrive(bar(kFull + 0));   // the draft unit fills stage 0 in place of a TMA load
+    };
+    if constexpr (kQTmem && !kBal) q_to_tmem();
+    if (!kBal && lane == 0) mbar_arrive(bar(kStaged));
+    if (!kBal && has_draft && tid == 0) mbar_arrive(bar(kFull + 0));   // the draft unit fills stage 0 in place of a TMA load
 
     const int wg = warp >> 2, quad = warp & 3;
     if (quad >= n_active) return;                                 // this warp's TMEM lanes hold padding only
@@ -507,13 +857,41 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t t_s = tmem_base + t_lane + wg * kUnit;
     const uint32_t t_o = tmem_base + t_lane + 128 + wg * 128;
     const int wg_threads = n_active * 32;
+    bool dead = false;
+    int ring = 0, k_before = 0;   // (kBal) ring units, and units of this warpgroup, of the segments before
+    for (int seg = 0;; ++seg) {   // (one pass unless kBal)
+    int seg_item = 0, seg_total = 0;
+    if constexpr (kBal) {
+        if (__any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait))) {
+            dead = true;
+            *abort_flag = 1;
+            if (p.status && lane == 0) atomicOr(p.status, 8);
+        } else {
+            const volatile Segment *d = segments + (seg & 1);
+            seg_total = d->n_total, seg_item = d->item;
+            if (seg_total < 0) {
+                grid_launch_dependents();
+                if (lane == 0) mbar_arrive(bar(kTmemDone));   // (behind this warp's last read of tensor memory)
+                return;
+            }
+            if constexpr (kQTmem) {
+                if (kPair || wg == 0) {
+                    q_to_tmem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kStaged));
+                }
+            }
+        }
+    }
+    const unsigned long long *anc_s = anc + (kBal ? (seg & 1) * 64 : 0);
+    const uint32_t *anc32_s = kBal && (seg & 1) ? anc32_odd : anc32;
     // per slot, the draft tokens the row may see: kWide: bit 2j + e <-> this thread's column 8j + 2qd + e; else bit = token
     uint32_t vis[NH];
     int trow[NH], lrow[NH];
     unsigned long long row_vis = ~0ull;   // NH == 4: the draft tokens row quad * 32 + lane may see
     if constexpr (NH == 4) {
         const int r = quad * 32 + lane;
-        if (has_draft && r < rows) row_vis = kWide ? anc[i0 + div_g(r)] : (unsigned long long)anc32[div_g(r)];
+        if (has_draft && r < rows) row_vis = kWide ? anc_s[i0 + div_g(r)] : (unsigned long long)anc32_s[div_g(r)];
     }
 #pragma unroll
     for (int i = 0; i < NH; ++i) {
@@ -521,22 +899,28 @@ __global__ void __launch_bounds__(kThreads, 1)
         trow[i] = quad * QR + 8 * i + lr;
         if constexpr (kWide) {
             const unsigned long long all_t = (p.T == 64) ? ~0ull : ((1ull << p.T) - 1ull);
-            const unsigned long long row_vis = (has_draft && lrow[i] < rows) ? anc[i0 + div_g(lrow[i])] : all_t;
+            const unsigned long long row_vis = (has_draft && lrow[i] < rows) ? anc_s[i0 + div_g(lrow[i])] : all_t;
             uint32_t mine = 0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) mine |= (uint32_t)((row_vis >> (8 * j + 2 * qd)) & 3ull) << (2 * j);
             vis[i] = mine;
         } else {
             const uint32_t all_t = (p.T == 32) ? 0xFFFFFFFFu : ((1u << p.T) - 1u);
-            vis[i] = (has_draft && lrow[i] < rows) ? anc32[div_g(lrow[i])] : all_t;
+            vis[i] = (has_draft && lrow[i] < rows) ? anc32_s[div_g(lrow[i])] : all_t;
         }
     }
 
-    const int L = p.seq_lens[s];
-    const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-    const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
+    int n_total = seg_total;
+    if constexpr (kBal) {
+        __syncwarp();
+        if (lane == 0 && !dead) mbar_arrive(bar(kTaken));
+    } else {
+        const int L = p.seq_lens[s];
+        const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
+        const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
+        n_total = slice_units(split, n_sel) + (has_draft ? 1 : 0);
+    }
     const int off = has_draft ? 1 : 0;
-    const int n_total = slice_units(split, n_sel) + off;
 
     // per slot (row): reference maximum of the exponentials (log2 units) and partial row sum
     float m[NH], l[NH];
@@ -545,12 +929,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         m[i] = -INFINITY;
         l[i] = 0.f;
     }
-    bool dead = false;
     constexpr float kLazy = 8.f;   // the reference maximum may trail the true one by up to 2^8
 
     // wait until the warpgroup's k-th PV has been added to O (warp-uniform outcome)
     auto wait_pv = [&](int k) {
-        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kOReady + wg), k & 1))) {
+        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kOReady + wg), (k_before + k) & 1))) {
             dead = true;
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 4);
@@ -560,15 +943,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     int k = 0;
     for (int u = kPair ? 0 : wg; u < n_total; u += kPair ? 1 : 2, ++k) {   // kPair: every unit, for this warpgroup's row tile
-        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kSReady + wg), k & 1))) {
+        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kSReady + wg), (k_before + k) & 1))) {
             dead = true;
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 2);
         }
         if (dead) break;
         tc_fence_after_sync();
-        const bool is_draft = u < off;
-        const int stage = u % NS;
+        const bool is_draft = kBal ? u == n_total - 1 : u < off;
+        const int stage = (u + ring) % NS;
         const int nvalid = is_draft ? p.T : min(meta[stage], kUnit);
         uint8_t *pbuf = smem + kOffP + wg * kPBytes;
         if constexpr (NH == 4) {
@@ -798,7 +1181,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Only now may the dependent kernel (the split merge) be scheduled: released at the start, its small CTAs would all
     // become resident on the few SMs this grid leaves idle and later do the whole merge from there; released here,
     // they spread over the SMs that the attention CTAs are about to vacate.
-    grid_launch_dependents();
+    if (!kBal) grid_launch_dependents();
     if (k > 0) wait_pv(k - 1);   // this warpgroup's accumulator is complete
     uint32_t ml_theirs[8] = {};   // (kPTmem) the other warpgroup's m, l of this thread's slots
     if constexpr (!kPair && kPTmem) {
@@ -827,6 +1210,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // a warpgroup without units never wrote its accumulator
     const bool have_mine = k > 0 && !dead, have_other = !kPair && n_total >= (wg == 0 ? 2 : 1);
     const uint32_t t_o_other = tmem_base + t_lane + 128 + (wg ^ 1) * 128;
+    bool stop = !kBal;
+    const int out_z = kBal ? seg_item / p.Hkv : z, out_h = kBal ? seg_item - out_z * p.Hkv : h;
     for (int ch = kPair ? 0 : wg; ch < (kPair ? 2 : wg + 1); ++ch) {   // column half: 64 output dims
         // this warp's rows of O, 16 output dims 64 ch + 8 j + 2 qd + e (index 2 j + e)
         float o[NH][16], row_m[NH], row_l[NH];
@@ -861,17 +1246,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (!kPair || ch == 1) {
             tc_fence_before_sync();
+            if constexpr (kBal && !kPair) {
+                // both accumulators have been read (and both exchanges): the next segment may overwrite them.  All warps
+                // leave together if one has given up.
+                stop = named_bar_or(1, n_sm, dead);
+            } else if constexpr (kBal) {
+                stop = dead;
+            }
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kTmemDone));   // this warp reads TMEM no more
+            if (lane == 0 && stop) mbar_arrive(bar(kTmemDone));   // this warp reads TMEM no more
         }
 #pragma unroll
         for (int i = 0; i < NH; ++i) {
             const float M = row_m[i], lsum = row_l[i];
             const int row = lrow[i];
-            if (row >= rows) continue;
-            if (p.splits == 1) {
+            if (row >= rows || (kBal && dead)) continue;
+            if (kBal || p.splits == 1) {
                 const int ii = div_g(row), g = row - ii * p.G;
-                const size_t orow = ((size_t)z * p.T + i0 + ii) * p.Hq + h * p.G + g;
+                const size_t orow = ((size_t)out_z * p.T + i0 + ii) * p.Hq + out_h * p.G + g;
                 const float inv = 1.f / lsum;
                 uint32_t *dst = reinterpret_cast<uint32_t *>(p.out + orow * 128) + ch * 32 + qd;
 #pragma unroll
@@ -886,22 +1278,25 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     }
+    if (stop) break;
+    ring += n_total, k_before += k;
+    }
 }
 
 }  // namespace
 
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, class Params>
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kBal = false, class Params>
 static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
-    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>>;
+    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>, kBal>;
+    constexpr int smem = kBal ? kSmemBytesBal : kSmemBytes;
     static svh::OncePerDevice once;   // function attributes belong to a device
-    const cudaError_t ce =
-        once.run([] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); });
+    const cudaError_t ce = once.run([] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (ce != cudaSuccess) return ce;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemBytes;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     svh::pdl_attribute(attr);
@@ -910,11 +1305,21 @@ static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, c
     return cudaLaunchKernelEx(&cfg, kernel, tm_k, tm_v, p);
 }
 
-// grid.x = splits x groups, where a group is a row tile or (p.pair) a pair of row tiles
+// grid.x = splits x groups, where a group is a row tile or (p.pair) a pair of row tiles; p.n_claims > 0: one CTA per SM
 template <class Params>
 static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
     const int rows = p.G * p.Tt;   // rows of a full row tile
+    if constexpr (std::is_same_v<Params, StackAttnParams>) if (p.n_claims > 0) {
+        if (p.pair) return launch_tc<4, true, true, false, true>(tm_k, tm_v, p, grid, stream);
+        if (p.T > 32) {
+            if (rows <= 64) return launch_tc<2, true, false, false, true>(tm_k, tm_v, p, grid, stream);
+            return launch_tc<4, true, false, false, true>(tm_k, tm_v, p, grid, stream);
+        }
+        if (rows <= 32) return launch_tc<1, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        if (rows <= 64) return launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        return launch_tc<4, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+    }
     const bool units = p.B == 128;   // 128-row tiles over blocks of 128 tokens: slices cut at 64-key units
     if (p.pair) {   // (a full tile has more than 64 rows)
         return units ? launch_tc<4, true, true, true>(tm_k, tm_v, p, grid, stream)

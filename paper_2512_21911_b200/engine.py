@@ -111,7 +111,7 @@ class SparseVerifier:
         flags = self._anchor_flags()
         if self._stack_workspace[dense] is None:
             n = sv._native.workspace_bytes_layers(self.geom, self.n_layers, self.geom.max_blocks if dense else self.max_sel)
-            self._stack_workspace[dense] = torch.empty(max(16, n), dtype=torch.uint8, device=self.workspace.device)
+            self._stack_workspace[dense] = torch.zeros(max(16, n), dtype=torch.uint8, device=self.workspace.device)
         failed = sv._native.verify_layers(self.geom, self._table, self.kv[0], first, end, flags, q, draft_k, draft_v, self.parent, out,
                                           self.reps, self.budget, self.n_sink, self.n_local, None if dense else self._lists_idx,
                                           None if dense else self._lists_cnt, self._stack_workspace[dense], self.status)
