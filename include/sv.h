@@ -421,6 +421,27 @@ SV_API sv_status sv_kv_append_layers(const sv_geom *geom, const sv_layers *layer
                                      const int32_t *accept_idx, const int32_t *n_accept, int32_t max_accept,
                                      int32_t *seq_lens, uint32_t *counters, float *reps, void *stream);
 
+/*
+ * A step of the whole stack with its inputs in pinned host memory and its outputs wanted there: sv_select_blocks_layers and
+ * sv_verify_attn_layers in chunks of layers (chunk_end: host, ascending, the last one n_layers), with the copies of other
+ * chunks in the background.  q / draft_k / draft_v / out: device, as above; the *_host ones their host counterparts.
+ * refresh_tail != 0: sv_block_reps_layers(refresh_which, SV_TAIL_BLOCK) first.  Everything is enqueued when the call
+ * returns, and `stream` ends behind the last copy.  stream_in / stream_out: two other streams, for the uploads and the
+ * downloads.  An sv_host_step holds the events of one caller; it belongs to the device that is current when it is created
+ * and serves one call at a time.
+ */
+#define SV_MAX_HOST_CHUNKS 256
+typedef struct sv_host_step sv_host_step;
+SV_API sv_host_step *sv_host_step_create(void);
+SV_API void sv_host_step_destroy(sv_host_step *step);
+SV_API sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors,
+                                          const int32_t *chunk_end, int32_t n_chunks, const void *q_host, const void *draft_k_host,
+                                          const void *draft_v_host, void *q, void *draft_k, void *draft_v,
+                                          const int32_t *parent, float *reps, const int32_t *budget_blocks, int32_t n_sink,
+                                          int32_t n_local, int32_t *idx, int32_t *cnt, int32_t max_sel, void *out, void *out_host,
+                                          void *workspace, size_t workspace_bytes, int32_t *status_word, int32_t refresh_tail,
+                                          const uint8_t *refresh_which, void *stream_in, void *stream_out, void *stream);
+
 /* Number of KV splits (CTAs per (sequence, KV head)) sv_verify_attn uses for this geometry. */
 SV_API int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel);
 

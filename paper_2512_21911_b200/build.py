@@ -15,7 +15,7 @@ LIB = os.path.join(HERE, "libsv.so")
 NATIVE = os.path.join(HERE, "_native.so")
 NATIVE_SOURCE = os.path.join(CSRC, "py_native.cpp")
 SOURCES = ["sv_api.cu", "block_reps.cu", "select_blocks.cu", "verify_attn.cu", "verify_attn_tc.cu", "kv_append.cu", "anchor_calib.cu",
-           "select_variants.cu", "accept.cu"]
+           "select_variants.cu", "accept.cu", "host_step.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
               "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -35,7 +35,7 @@ def _native_command(out: str) -> list:
     return ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", NATIVE_SOURCE, "-o", out,
             "-I", os.path.join(ROOT, "include"), "-I", inc, "-I", os.path.join(inc, "torch", "csrc", "api", "include"),
             "-I", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"],
-            "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
+            "-Wno-interference-size", "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10",
             "-L", HERE, "-l:libsv.so", "-Wl,-rpath,$ORIGIN"]
 
 

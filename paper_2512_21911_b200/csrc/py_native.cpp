@@ -12,6 +12,7 @@
 
 #include <string.h>
 
+#include <ATen/core/CachingHostAllocator.h>
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
@@ -354,6 +355,71 @@ PyObject *verify_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// Pointer of a stacked host tensor, or null: as stacked().
+void *stacked_host(PyObject *o, const at::Tensor &like)
+{
+    if (!THPVariable_Check(o)) return nullptr;
+    const at::Tensor &t = THPVariable_Unpack(o);
+    if (!t.is_cpu() || t.scalar_type() != at::kBFloat16 || !t.is_contiguous() || !t.sizes().equals(like.sizes())) return nullptr;
+    return t.data_ptr();
+}
+
+void destroy_host_step(PyObject *capsule) { sv_host_step_destroy(static_cast<sv_host_step *>(PyCapsule_GetPointer(capsule, "sv_host_step"))); }
+
+PyObject *host_step(PyObject *, PyObject *const *, Py_ssize_t n)
+{
+    return checked(n, 0, [&]() -> PyObject * {
+        sv_host_step *h = sv_host_step_create();
+        if (h) return PyCapsule_New(h, "sv_host_step", destroy_host_step);
+        return status(SV_ERR_CUDA);
+    });
+}
+
+// step, geom, table, kv, anchors, chunk_end (sequence of int), q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, parent, reps, budget,
+// n_sink, n_local, idx, cnt, out, out_host, workspace, status_word, refresh_tail, refresh_which (bytes or None),
+// stream_in, stream_out
+// -> status, or False when the tensors are not stacked ones
+PyObject *verify_step_from_host(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 27, [&]() -> PyObject * {
+        sv_host_step *h = static_cast<sv_host_step *>(PyCapsule_GetPointer(a[0], "sv_host_step"));
+        if (!h) throw ArgError{};
+        const sv_geom g = geometry(a[1]);
+        const sv_layers layers = stack(a[2], a[3]);
+        void *dev[4], *host[4];   // q, draft K, draft V, out
+        for (int i = 0; i < 4; ++i) {
+            PyObject *d = i < 3 ? a[9 + i] : a[19], *o = i < 3 ? a[6 + i] : a[20];
+            dev[i] = stacked(d, layers.n_layers);
+            if (!dev[i]) Py_RETURN_FALSE;
+            const at::Tensor &t = THPVariable_Unpack(d);
+            if (t.size(1) != g.n_seq || t.size(2) != g.n_draft || t.size(3) != (i == 1 || i == 2 ? g.n_kv_heads : g.n_q_heads) || t.size(4) != g.head_dim)
+                Py_RETURN_FALSE;
+            host[i] = stacked_host(o, t);
+            if (!host[i]) Py_RETURN_FALSE;
+        }
+        int32_t ends[SV_MAX_HOST_CHUNKS];
+        const Py_ssize_t chunks = PySequence_Fast_GET_SIZE(a[5]);
+        if (chunks > SV_MAX_HOST_CHUNKS) Py_RETURN_FALSE;
+        for (Py_ssize_t c = 0; c < chunks; ++c) ends[c] = int32(PySequence_Fast_GET_ITEM(a[5], c));
+        const Scratch ws = scratch(a[21]);
+        const sv_status st = sv_verify_step_from_host(
+            h, &g, &layers, flags(a[4], layers.n_layers), ends, (int32_t)chunks, host[0], host[1], host[2], dev[0], dev[1], dev[2],
+            i32(a[12], "parent"), f32(a[13], "reps"), i32(a[14], "budget_blocks"), int32(a[15]), int32(a[16]), i32(a[17], "idx"),
+            i32(a[18], "cnt"), row_length(a[17], "idx"), dev[3], host[3], ws.p, ws.bytes, i32(a[22], "status_word"), truth(a[23]),
+            flags(a[24], layers.n_layers), stream(a[25]), stream(a[26]), stream(Py_None));
+        // the allocator of pinned memory must not hand these out again before the copies are through
+        const auto device = c10::cuda::current_device();
+        for (int i = 0; i < 4; ++i) {
+            const at::Tensor &t = THPVariable_Unpack(i < 3 ? a[6 + i] : a[20]);
+            void *const context = t.storage().data_ptr().get_context();
+            at::getHostAllocator(at::kCUDA)->record_event(
+                host[i], context, c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream(a[i < 3 ? 25 : 26])), device).unwrap());
+            at::getHostAllocator(at::kCUDA)->record_event(host[i], context, c10::cuda::getCurrentCUDAStream().unwrap());
+        }
+        return status(st);
+    });
+}
+
 // geom, table, kv, draft_k, draft_v, path, n_path, seq_lens, counters, reps -> status, or False when the drafts are not stacked tensors
 PyObject *kv_append_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
@@ -395,7 +461,7 @@ PyObject *accept_new(PyObject *, PyObject *const *a, Py_ssize_t n)
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {METHOD(block_reps), METHOD(select_blocks), METHOD(verify_attn), METHOD(kv_append), METHOD(accept),
                          METHOD(verify_layer), METHOD(layer_row), METHOD(workspace_bytes_layers), METHOD(block_reps_layers),
-                         METHOD(verify_layers), METHOD(kv_append_layers), METHOD(accept_new), {nullptr, nullptr, 0, nullptr}};
+                         METHOD(verify_layers), METHOD(kv_append_layers), METHOD(accept_new), METHOD(host_step), METHOD(verify_step_from_host), {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the entry points of sv.h.", -1, methods,
                       nullptr, nullptr, nullptr, nullptr};

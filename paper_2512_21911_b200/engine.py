@@ -39,6 +39,7 @@ class SparseVerifier:
         self._pools = [None] * n_layers   # keep the tensors alive
         self._one_allocation = False
         self._copy_streams = None
+        self._host_step = None
         self._stack_workspace = [None, None]   # sparse, dense
         self._counters = torch.zeros(2 * n_seq, dtype=torch.int32, device=dev)   # see sv_kv_append_layers
         # what the layers' kernels look up when several layers run in one launch (a row is valid once its layer has pools)
@@ -103,18 +104,21 @@ class SparseVerifier:
             self._make_lists(flags, self.workspace.device)
         return flags
 
+    def _workspace_of_stack(self, dense: bool) -> torch.Tensor:
+        if self._stack_workspace[dense] is None:
+            n = sv._native.workspace_bytes_layers(self.geom, self.n_layers, self.geom.max_blocks if dense else self.max_sel)
+            self._stack_workspace[dense] = torch.zeros(max(16, n), dtype=torch.uint8, device=self.workspace.device)
+        return self._stack_workspace[dense]
+
     def _run_layers(self, first: int, end: int, q, draft_k, draft_v, out, dense: bool = False) -> bool:
         """Layers first .. end - 1 in two launches (dense: one; three when the splits have to be merged).  False when the
         inputs are not stacked tensors: the caller then goes layer by layer."""
         if not self._stacked():
             return False
         flags = self._anchor_flags()
-        if self._stack_workspace[dense] is None:
-            n = sv._native.workspace_bytes_layers(self.geom, self.n_layers, self.geom.max_blocks if dense else self.max_sel)
-            self._stack_workspace[dense] = torch.zeros(max(16, n), dtype=torch.uint8, device=self.workspace.device)
         failed = sv._native.verify_layers(self.geom, self._table, self.kv[0], first, end, flags, q, draft_k, draft_v, self.parent, out,
                                           self.reps, self.budget, self.n_sink, self.n_local, None if dense else self._lists_idx,
-                                          None if dense else self._lists_cnt, self._stack_workspace[dense], self.status)
+                                          None if dense else self._lists_cnt, self._workspace_of_stack(dense), self.status)
         if failed is False:
             return False
         if failed:
@@ -171,29 +175,15 @@ class SparseVerifier:
         q/draft_k/draft_v/out are the device staging tensors (shapes as for verify_step); the *_host tensors the pinned
         ones.  Returns with everything enqueued; the current stream ends behind the last download.  Capturable in a
         CUDA graph (the side streams fork from and join the current stream)."""
-        main = torch.cuda.current_stream()
+        chunks = self._chunks(layers_per_chunk)
         if self._copy_streams is None:
             self._copy_streams = (torch.cuda.Stream(device=q.device), torch.cuda.Stream(device=q.device))
+        if self._stacked() and self._from_host(chunks, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host, refresh_tail):
+            return
+        main = torch.cuda.current_stream()
         s_in, s_out = self._copy_streams
         s_in.wait_stream(main)
         s_out.wait_stream(main)
-        if layers_per_chunk is None:
-            # two layers first and last (their upload / download is what nothing hides), the rest in two halves (every
-            # chunk boundary costs the step a few microseconds): 32 layers measured 16.1 us/layer against 16.6 in chunks
-            # of four and 18.5 with the copies whole
-            mid = max(0, self.n_layers - 4)
-            layers_per_chunk = [2, (mid + 1) // 2, mid // 2, 2] if self.n_layers > 4 else [self.n_layers]
-        if isinstance(layers_per_chunk, int):
-            sizes = [layers_per_chunk] * -(-self.n_layers // layers_per_chunk)
-        else:   # a schedule: e.g. a small first and last chunk (their copies are the ones nothing hides), large ones between
-            sizes = list(layers_per_chunk)
-        chunks, c0 = [], 0
-        for n in sizes:
-            if c0 < self.n_layers and n > 0:
-                chunks.append((c0, min(c0 + n, self.n_layers)))
-                c0 += n
-        if c0 < self.n_layers:
-            chunks.append((c0, self.n_layers))
         arrived = []
         with torch.cuda.stream(s_in):
             for c0, c1 in chunks:
@@ -218,6 +208,43 @@ class SparseVerifier:
                 out_host[c0:c1].copy_(out[c0:c1], non_blocking=True)
         main.wait_stream(s_in)
         main.wait_stream(s_out)
+
+    def _chunks(self, layers_per_chunk):
+        if layers_per_chunk is None:
+            # Two chunks: every further one costs a launch that fills the GPU for a part of its time only.  The first is the
+            # smaller, its upload is not hidden (32 layers of a 32K context: 181 us in chunks of 14 / 18, 184 of 18 / 14,
+            # 201 of 8 / 10 / 14, 218 in one)
+            first = self.n_layers * 7 // 16
+            layers_per_chunk = [first, self.n_layers - first] if self.n_layers >= 4 else [self.n_layers]
+        if isinstance(layers_per_chunk, int):
+            sizes = [layers_per_chunk] * -(-self.n_layers // layers_per_chunk)
+        else:   # a schedule: e.g. a small first and last chunk (their copies are the ones nothing hides), large ones between
+            sizes = list(layers_per_chunk)
+        chunks, c0 = [], 0
+        for n in sizes:
+            if c0 < self.n_layers and n > 0:
+                chunks.append((c0, min(c0 + n, self.n_layers)))
+                c0 += n
+        if c0 < self.n_layers:
+            chunks.append((c0, self.n_layers))
+        return chunks
+
+    def _from_host(self, chunks, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host, refresh_tail) -> bool:
+        """verify_step_from_host in one call of the library.  False when the tensors are not stacked ones."""
+        flags = self._anchor_flags()
+        if self._host_step is None:
+            self._host_step = sv._native.host_step()
+            if isinstance(self._host_step, int):
+                raise sv.SvError(self._host_step, "sv_host_step_create")
+        st = sv._native.verify_step_from_host(
+            self._host_step, self.geom, self._table, self.kv[0], flags, [c1 for _, c1 in chunks], q_host, draft_k_host, draft_v_host, q,
+            draft_k, draft_v, self.parent, self.reps, self.budget, self.n_sink, self.n_local, self._lists_idx, self._lists_cnt, out,
+            out_host, self._workspace_of_stack(False), self.status, refresh_tail, None if self._one_allocation else flags,
+            *self._copy_streams)
+        if st is False:
+            return False
+        sv._check(st, "sv_verify_step_from_host")
+        return True
 
     def accept(self, p_target, p_draft, tokens, u_accept, u_next):
         """Acceptance of the step's draft tokens (Eq. 2-3).  Returns (path [S][T], n_path [S], next_token [S]):
