@@ -11,6 +11,13 @@
 // cumulative sum of the final p in vocabulary order: CTA totals -> the CTA that holds the target, block scan
 // of its thread sums -> the thread, a sequential walk of that thread's segment -> the token.
 // fp32 throughout; no spin-waits (cluster barriers only).
+//
+// A chain of latencies, not of bytes (a row of both distributions is 128 KB per CTA at a vocabulary of 128256): the
+// acceptance probabilities of all children are fetched together ahead of the walk, so the walk itself waits for nothing
+// until a rejection, and a row's range is copied once into shared memory (coalesced, asynchronous) for all of its passes --
+// every rejection, the sum and the draw -- laid out so that the threads' segments, of which each is read by one thread,
+// start in different banks.  Read from global memory in every pass, segment by segment, chains of 8 took
+// 18.1 us where they now take 13.9 us (one sequence, vocabulary 128256; 15.8 and 14.9 us at 151936).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -26,6 +33,7 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRows = 64;     // draft rows per step (the ancestor masks of the attention kernel are 64 bits)
 constexpr int kMaxCluster = 8;
+constexpr int kMaxStagedBytes = 2 * kThreads * 13 * 16;   // 13 words of either distribution per thread: 208 KB
 
 struct AcceptParams {
     const float *p_target;   // [S][T][V]
@@ -57,14 +65,21 @@ __device__ __forceinline__ float weight(float pt, float q, int r, const float *i
     return kResidual ? fmaxf(v - q, 0.f) : v;
 }
 
-// Sum of this thread's segment [y0, y1) in vocabulary order.
+// One thread's segment of a row of both distributions, four entries at a time: in global memory, or (kStaged) in the CTA's
+// copy, where a segment is `pad` 16-byte words after the one before.
+struct Segment {
+    const float4 *pt, *q;
+    int n;   // words
+};
+
+// Sum of a segment in vocabulary order.
 template <bool kResidual>
-__device__ __forceinline__ float segment_sum(const float *pt, const float *q, int y0, int y1, int r, const float *inv_z)
+__device__ __forceinline__ float segment_sum(const Segment &sg, int r, const float *inv_z)
 {
     float acc = 0.f;
-    for (int y = y0; y < y1; y += 4) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(pt + y));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(q + y));
+#pragma unroll 4
+    for (int i = 0; i < sg.n; ++i) {
+        const float4 a = sg.pt[i], b = sg.q[i];
         acc += weight<kResidual>(a.x, b.x, r, inv_z);
         acc += weight<kResidual>(a.y, b.y, r, inv_z);
         acc += weight<kResidual>(a.z, b.z, r, inv_z);
@@ -95,28 +110,37 @@ __device__ __forceinline__ float block_inclusive_scan(float v, float *warp_tot, 
     return before + inc;
 }
 
+// kStaged: a row's range fits in shared memory (vocabularies of up to 212992).
+template <bool kStaged>
 __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
     const int s = blockIdx.y, tid = threadIdx.x;
-    __shared__ int tok[kMaxRows], par[kMaxRows];
-    __shared__ float u[kMaxRows];
+    __shared__ int par[kMaxRows];
+    __shared__ float u[kMaxRows], px_of[kMaxRows], qx_of[kMaxRows];   // px, qx: a child's token in its parent's row
+    extern __shared__ float4 staged[];                                // [2][kThreads][pad]
     __shared__ float inv_z[kMaxRows];
     __shared__ float warp_tot[kWarps];
     __shared__ float cta_tot[2][kMaxCluster];   // totals of all CTAs, written by their owners; two buffers in turn
     __shared__ int s_first, s_last;
 
+    svk::cluster_arrive();
     svk::grid_dependency_wait();
     svk::grid_launch_dependents();
     if (tid < p.T) {
-        tok[tid] = p.tokens[(size_t)s * p.T + tid];
-        par[tid] = p.parent ? p.parent[(size_t)s * p.T + tid] : tid - 1;
+        const int x = min(max(p.tokens[(size_t)s * p.T + tid], 0), p.V - 1);
+        const int row = p.parent ? p.parent[(size_t)s * p.T + tid] : tid - 1;
+        par[tid] = row;
         u[tid] = p.u_accept[(size_t)s * p.T + tid];
+        if (row >= 0 && row < tid) {   // (a row that follows is never reached from it)
+            const size_t at = ((size_t)s * p.T + row) * p.V + x;
+            px_of[tid] = __ldg(p.p_target + at), qx_of[tid] = __ldg(p.p_draft + at);
+        }
     }
     const float u_next = p.u_next[s];
     __syncthreads();
-    cluster.sync();   // every CTA of the cluster is running: its shared memory may be written from here on
+    svk::cluster_wait();   // every CTA of the cluster is running: its shared memory may be written from here on
 
     const int lo = min(p.V, rank * p.chunk), hi = min(p.V, lo + p.chunk);
     const int y0 = min(hi, lo + tid * p.seg), y1 = min(hi, y0 + p.seg);
@@ -136,17 +160,35 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
 
     int cur = 0, n = 1, r = 0, buf = 0;
     if (writer) p.path[(size_t)s * p.T] = 0;
-    const float *pt = nullptr, *q = nullptr;
+    int at_hand = -1;   // the row in shared memory
+    auto segment_of = [&](int row) -> Segment {
+        const float4 *pt = reinterpret_cast<const float4 *>(p.p_target + ((size_t)s * p.T + row) * p.V + lo);
+        const float4 *q = reinterpret_cast<const float4 *>(p.p_draft + ((size_t)s * p.T + row) * p.V + lo);
+        if constexpr (kStaged) {
+            const int seg4 = p.seg >> 2, pad = seg4 | 1, words = (hi - lo) >> 2;
+            if (row != at_hand) {
+                __syncthreads();   // the row before has been read
+                for (int i = tid; i < words; i += kThreads) {
+                    const int t = i / seg4, at = t * pad + (i - t * seg4);
+                    svk::cp_async_16(svk::smem_u32(staged + at), pt + i);
+                    svk::cp_async_16(svk::smem_u32(staged + kThreads * pad + at), q + i);
+                }
+                svk::cp_async_wait_all();
+                __syncthreads();
+                at_hand = row;
+            }
+            return {staged + tid * pad, staged + (kThreads + tid) * pad, (y1 - y0) >> 2};
+        } else {
+            return {pt + ((y0 - lo) >> 2), q + ((y0 - lo) >> 2), (y1 - y0) >> 2};
+        }
+    };
     for (;;) {
-        pt = p.p_target + ((size_t)s * p.T + cur) * p.V;
-        q = p.p_draft + ((size_t)s * p.T + cur) * p.V;
         r = 0;
         bool moved = false;
         for (int c = cur + 1; c < p.T; ++c) {
             if (par[c] != cur) continue;
-            const int x = min(max(tok[c], 0), p.V - 1);
-            const float qx = __ldg(q + x);
-            const float px = adjusted(__ldg(pt + x), qx, r, inv_z);
+            const float qx = qx_of[c];
+            const float px = adjusted(px_of[c], qx, r, inv_z);
             const float a = (qx <= 0.f || px >= qx) ? 1.f : __fdiv_rn(px, qx);   // Eq. 2
             if (writer && p.alpha) p.alpha[(size_t)s * p.T + c] = a;
             if (u[c] < a) {
@@ -158,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
             }
             // rejected: Z = sum_y max(0, p - q) (Eq. 3); p itself is never stored
             float tot;
-            block_inclusive_scan(segment_sum<true>(pt, q, y0, y1, r, inv_z), warp_tot, tot);
+            block_inclusive_scan(segment_sum<true>(segment_of(cur), r, inv_z), warp_tot, tot);
             const float z = cluster_total(tot, buf);
             if (z > 0.f) {   // a residual without mass (p == q) leaves p as it is
                 if (tid == 0) inv_z[r] = __frcp_rn(z);
@@ -174,9 +216,10 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
     }
 
     // next token: the smallest x with  sum_{y <= x} p(y) >= u_next * sum_y p(y)  and p(x) > 0
+    const Segment mine = segment_of(cur);
     float tot;
-    const float mine = segment_sum<false>(pt, q, y0, y1, r, inv_z);
-    const float inc = block_inclusive_scan(mine, warp_tot, tot);
+    const float sum = segment_sum<false>(mine, r, inv_z);
+    const float inc = block_inclusive_scan(sum, warp_tot, tot);
     const float W = cluster_total(tot, buf);
     const float target = u_next * W;
     int owner = -1, last_pos = -1;
@@ -198,21 +241,26 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
     const float local = target - before;
     if (tid == 0) s_first = kThreads, s_last = -1;
     __syncthreads();
-    if (mine > 0.f) {
+    if (sum > 0.f) {
         if (inc >= local) atomicMin(&s_first, tid);
         atomicMax(&s_last, tid);
     }
     __syncthreads();
     const int chosen = s_first < kThreads ? s_first : s_last;
     if (tid != chosen) return;
-    float acc = inc - mine;
+    float acc = inc - sum;
     int pick = -1, last_y = -1;
-    for (int y = y0; y < y1 && pick < 0; ++y) {
-        const float w = weight<false>(__ldg(pt + y), __ldg(q + y), r, inv_z);
-        acc += w;
-        if (w > 0.f) {
-            last_y = y;
-            if (acc >= local) pick = y;
+    for (int i = 0; i < mine.n && pick < 0; ++i) {
+        const float4 a = mine.pt[i], b = mine.q[i];
+        const float w[4] = {weight<false>(a.x, b.x, r, inv_z), weight<false>(a.y, b.y, r, inv_z), weight<false>(a.z, b.z, r, inv_z),
+                            weight<false>(a.w, b.w, r, inv_z)};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            acc += w[e];
+            if (w[e] > 0.f && pick < 0) {
+                last_y = y0 + 4 * i + e;
+                if (acc >= local) pick = last_y;
+            }
         }
     }
     p.next_token[s] = pick >= 0 ? pick : last_y;
@@ -249,6 +297,17 @@ extern "C" sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, co
     svh::pdl_attribute(attr + 1);
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, accept_kernel, p) != cudaSuccess) return SV_ERR_CUDA;
+    const size_t bytes = (size_t)2 * kThreads * ((p.seg >> 2) | 1) * sizeof(float4);
+    // (one CTA per SM then: launches that would fill the GPU keep the form of which three fit an SM -- 16 sequences at a
+    // vocabulary of 151936: 24.6 against 26.9 us)
+    const bool staged = bytes <= kMaxStagedBytes && (2 * bytes <= kMaxStagedBytes || 3 * CL * n_seq <= 2 * svh::sm_count());
+    if (staged) {
+        static svh::OncePerDevice once;   // function attributes belong to a device
+        if (once.run([] { return cudaFuncSetAttribute(accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedBytes); }) !=
+            cudaSuccess)
+            return SV_ERR_CUDA;
+        cfg.dynamicSmemBytes = bytes;
+    }
+    if (cudaLaunchKernelEx(&cfg, staged ? accept_kernel<true> : accept_kernel<false>, p) != cudaSuccess) return SV_ERR_CUDA;
     return svh::launch_status();
 }
