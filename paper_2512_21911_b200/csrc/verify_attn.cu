@@ -358,12 +358,14 @@ extern "C" sv_status sv_layer_table(const sv_geom *geom, const sv_kv *kv, int32_
 }
 
 // Whether a stack's lists are handed out to resident CTAs (see verify_attn_tc.cu, kBal): more lists than SMs, so that CTAs
-// take several, and lists that are not cut to even out their lengths (choose_splits).  More than two row tiles are left to
-// CTAs of their own, which share their tiles through L2 by running side by side.  The rule looks at the whole stack: a
-// layer's result is the same whichever layers a launch covers.
+// take several, and lists that are not cut to even out their lengths (choose_splits).  Tiles of up to 64 rows only: 128-row
+// tiles are bound by their softmax, not by the gather, and the roles' bookkeeping takes registers from it (8 layers x 4
+// sequences of 96 rows: 95 us handed out, 84 with a CTA per list; 40 layers of 112 rows: 135 and 124).  The rule looks at
+// the whole stack: a layer's result is the same whichever layers a launch covers.
 static bool hand_out(const sv_geom *rule, int max_sel)
 {
-    return svh::row_tiles(rule) <= 2 && (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
+    return svh::row_tiles(rule) == 1 && rule->n_q_heads / rule->n_kv_heads * rule->n_draft <= 64 &&
+           (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
 }
 constexpr size_t kClaimsBytes = 256;
 
@@ -418,7 +420,6 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
     }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (handed) {
-        p.pair = p.tiles == 2;
         p.n_claims = (end - first) * geom->n_seq * geom->n_kv_heads;
         p.claims = static_cast<uint32_t *>(workspace);
         p.ws_o = nullptr;

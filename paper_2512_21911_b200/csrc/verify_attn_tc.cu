@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int *claims = reinterpret_cast<volatile int *>(misc + 1696);
     auto bar = [&](int slot) { return bars + 8u * slot; };
 
+    static_assert(!kBal || NH < 4, "lists are handed out for tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
     // 128-row tiles are bound by the tensor pipe when every MMA fetches both operands from shared memory (S = Q K^T: eight
     // 128 x 64 x 16 MMAs, each re-reading 4 KB of Q), so their Q lives in tensor memory (A operand from TMEM), and with a
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
     // registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168); the roles of a balanced launch keep
     // track of more
-    constexpr int kRegsMany = kBal ? (NH == 4 ? 216 : NH == 2 ? 208 : 200) : 232, kRegsFew = 504 - 2 * kRegsMany;
+    constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : 232, kRegsFew = 504 - 2 * kRegsMany;
     constexpr int OFFQ = NS * kStageBytes;                   // the Q tile (kPair: of warpgroup 0; warpgroup 1's follows)
     // blockIdx.x = split * groups + group: the CTAs that gather the same slice of the blocks are neighbours in the grid
     // (they share those K/V tiles through L2; 1-2 % faster than group-major order).  A group is a row tile (kWide), or
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t count = 1;
             if (lane == kSFree || lane == kPReady) count = na0;
             if (lane == kSFree + 1 || lane == kPReady + 1) count = max(1, na1);
-            if (lane == kStaged) count = kBal ? (kPair ? na0 + na1 : na0) : 8;
+            if (lane == kStaged) count = 8;
             if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0);
             if (lane == kTaken) count = na0 + (n_wg == 2 ? na1 : 0) + 2;   // the softmax warps and both issuers
             mbar_init(bar(lane), count);
@@ -257,13 +258,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto let_copies_land = [] {
         for (int i = 0; i < 100; ++i) __nanosleep(2000);
     };
-    // query rows of a tile (draft tokens tok ..) to shared memory, 16 bytes per asynchronous copy, by n threads of which this is t
-    auto copy_q = [&](uint32_t tile_at, const Item &it, int tok, int n_rows, int t, int n) {
+    // the query rows of a list to a Q tile, 16 bytes per asynchronous copy, by n threads of which this is t
+    auto copy_q = [&](uint32_t tile_at, const Item &it, int t, int n) {
         const int c = t & 15;
-        const __nv_bfloat16 *src = p.q + (((size_t)it.z * p.T + tok) * p.Hq + it.h * p.G) * 128 + c * 8;
+        const __nv_bfloat16 *src = p.q + ((size_t)it.z * p.T * p.Hq + it.h * p.G) * 128 + c * 8;
         const uint32_t dst = tile_at + (c >> 3) * (kQBytes / 2);
 #pragma unroll 4
-        for (int r = t >> 4; r < n_rows; r += n >> 4)
+        for (int r = t >> 4; r < rows; r += n >> 4)
             cp_async_16(dst + swz128((r / RPQ) * QR + (r % RPQ), c & 7), src + (r + div_g(r) * (p.Hq - p.G)) * 128);
     };
     const uint32_t tmem_base = warp == 8 && !kBal ? 0u : *tmem_slot;
@@ -504,10 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const Item it = item_at(claim);
                 const int n_total = item_blocks(it) * upb + 1;
                 if (seg > 0) {   // (the first segment's is brought by the softmax warps)
-                    const uint32_t q_at = smem0 + OFFQ + (NH == 4 ? 0 : (seg & 1) * 8192);   // (an M = 64 tile fills half of either half)
-#pragma unroll
-                    for (int t = 0; t < (kPair ? 2 : 1); ++t)
-                        copy_q(q_at + t * kQBytes, it, t * p.Tt, t == 0 ? rows_w0 : rows_w1, lane, 32);
+                    copy_q(smem0 + OFFQ + (seg & 1) * 8192, it, lane, 32);   // (an M = 64 tile fills half of either half)
                 }
                 {   // lane i: tokens i and (kWide) 32 + i
 #pragma unroll
@@ -586,17 +584,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 // (kBal) per segment: its units, and what came before it: ring units, units of either warpgroup
                 int ring = 0, done0 = 0, done1 = 0;
                 bool end = false;
-                auto next_segment = [&](int seg, bool staged) {
+                auto next_segment = [&](int seg) {
                     bool ok = !*abort_flag && mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait);
                     if (ok) {
                         n_total = segments[seg & 1].n_total;
                         end = n_total < 0;
-                        if (end) return;
-                        // (before kTaken: a segment without units is over for the softmax warps once they have staged it)
-                        ok = !staged || mbar_wait_bounded(bar(kStaged), seg & 1);
-                    }
-                    if (ok) {
-                        mbar_arrive(bar(kTaken));
+                        if (!end) mbar_arrive(bar(kTaken));
                     } else {
                         dead = true;
                         *abort_flag = 1;
@@ -605,8 +598,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 };
                 auto end_segment = [&] {
                     ring += n_total;
-                    done0 += kPair ? n_total : (n_total + 1) >> 1;
-                    done1 += kPair ? n_total : n_total >> 1;
+                    done0 += (n_total + 1) >> 1;
+                    done1 += n_total >> 1;
                 };
                 if (warp == 9) {
                     constexpr uint32_t idesc_s = umma_idesc_bf16(MT, kUnit, false);
@@ -616,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t d_hi = dq & 0xFFFFFFFF00000000ull;
                     for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
                     if constexpr (kBal) {
-                        next_segment(seg, kQTmem);
+                        next_segment(seg);
                         if (end || dead) break;
                     }
                     // one S per (unit, warpgroup that takes it): the warpgroups alternate units, or (kPair) each takes all
@@ -659,7 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint64_t dp_hi = dp & 0xFFFFFFFF00000000ull, dv_hi = dv & 0xFFFFFFFF00000000ull;
                     for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
                     if constexpr (kBal) {
-                        next_segment(seg, false);
+                        next_segment(seg);
                         if (end || dead) break;
                     }
                     const int n_issue = kPair ? n_total * n_wg : n_total;
@@ -719,19 +712,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = (tr / QR) * RPQ + (tr % QR);
         if (!((tr % QR) < RPQ && r < rows)) {
             *reinterpret_cast<uint4 *>(q_tile + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = make_uint4(0u, 0u, 0u, 0u);
-            if (kBal && NH != 4)   // (two tiles, used in turn)
+            if (kBal)   // (two tiles, used in turn)
                 *reinterpret_cast<uint4 *>(q_tile + 8192 + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = make_uint4(0u, 0u, 0u, 0u);
         }
     }
     if (kBal) {
-        copy_q(smem0 + OFFQ + (kPair ? ((warp >> 2) & 1) * kQBytes : 0), item_at(blockIdx.x), i0, rows, qtid, kQThreads);   // (first segment)
-        // padding rows of Q in tensor memory that no active warp copies
-        if (kQTmem && (warp & 3) >= n_active && (kPair || warp < 4)) {
-            uint32_t zero[32] = {};
-            for (int half = 0; half < 2; ++half)
-                tmem_st_x32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (kPair ? kTmemP + (warp >> 2) * 64 : kTmemQ) + half * 32, zero);
-            tmem_st_wait();
-        }
+        copy_q(smem0 + OFFQ, item_at(blockIdx.x), qtid, kQThreads);   // (first segment)
     } else if (has_draft) {
         for (int idx = tid; idx < 2 * kUnit * 16; idx += 256) {
             const int which = idx / (kUnit * 16);   // 0: K, 1: V
@@ -826,7 +812,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
         named_bar_sync(2, 256);
     }
-    auto q_to_tmem = [&] {
+    if constexpr (kQTmem) {
         // Q goes on to tensor memory (thread = tile row = TMEM lane; the 64 32-bit words of the row are the 64 packed
         // columns): every S = Q K^T then reads only the K tile from shared memory, which is what bounds a
         // 128 x 64 x 16 MMA whose two operands both come from there.
@@ -845,8 +831,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tmem_st_wait();
             tc_fence_before_sync();
         }
-    };
-    if constexpr (kQTmem && !kBal) q_to_tmem();
+    }
     if (!kBal && lane == 0) mbar_arrive(bar(kStaged));
     if (!kBal && has_draft && tid == 0) mbar_arrive(bar(kFull + 0));   // the draft unit fills stage 0 in place of a TMA load
 
@@ -857,13 +842,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t t_s = tmem_base + t_lane + wg * kUnit;
     const uint32_t t_o = tmem_base + t_lane + 128 + wg * 128;
     const int wg_threads = n_active * 32;
-    bool dead = false;
     int ring = 0, k_before = 0;   // (kBal) ring units, and units of this warpgroup, of the segments before
     for (int seg = 0;; ++seg) {   // (one pass unless kBal)
     int seg_item = 0, seg_total = 0;
+    bool lost = false;   // (the segment never came)
     if constexpr (kBal) {
         if (__any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait))) {
-            dead = true;
+            lost = true;
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 8);
         } else {
@@ -873,13 +858,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 grid_launch_dependents();
                 if (lane == 0) mbar_arrive(bar(kTmemDone));   // (behind this warp's last read of tensor memory)
                 return;
-            }
-            if constexpr (kQTmem) {
-                if (kPair || wg == 0) {
-                    q_to_tmem();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kStaged));
-                }
             }
         }
     }
@@ -910,17 +888,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
-    int n_total = seg_total;
     if constexpr (kBal) {
         __syncwarp();
-        if (lane == 0 && !dead) mbar_arrive(bar(kTaken));
-    } else {
-        const int L = p.seq_lens[s];
-        const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-        const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
-        n_total = slice_units(split, n_sel) + (has_draft ? 1 : 0);
+        if (lane == 0 && !lost) mbar_arrive(bar(kTaken));
     }
+    const int L = kBal ? 0 : p.seq_lens[s];
+    const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
+    const int n_sel = kBal ? 0 : p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
     const int off = has_draft ? 1 : 0;
+    const int n_total = kBal ? max(0, seg_total) : slice_units(split, n_sel) + off;
 
     // per slot (row): reference maximum of the exponentials (log2 units) and partial row sum
     float m[NH], l[NH];
@@ -929,6 +905,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         m[i] = -INFINITY;
         l[i] = 0.f;
     }
+    bool dead = kBal && lost;
     constexpr float kLazy = 8.f;   // the reference maximum may trail the true one by up to 2^8
 
     // wait until the warpgroup's k-th PV has been added to O (warp-uniform outcome)
@@ -1246,12 +1223,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (!kPair || ch == 1) {
             tc_fence_before_sync();
-            if constexpr (kBal && !kPair) {
+            if constexpr (kBal) {
                 // both accumulators have been read (and both exchanges): the next segment may overwrite them.  All warps
                 // leave together if one has given up.
                 stop = named_bar_or(1, n_sm, dead);
-            } else if constexpr (kBal) {
-                stop = dead;
             }
             __syncwarp();
             if (lane == 0 && stop) mbar_arrive(bar(kTmemDone));   // this warp reads TMEM no more
@@ -1311,14 +1286,9 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
 {
     const int rows = p.G * p.Tt;   // rows of a full row tile
     if constexpr (std::is_same_v<Params, StackAttnParams>) if (p.n_claims > 0) {
-        if (p.pair) return launch_tc<4, true, true, false, true>(tm_k, tm_v, p, grid, stream);
-        if (p.T > 32) {
-            if (rows <= 64) return launch_tc<2, true, false, false, true>(tm_k, tm_v, p, grid, stream);
-            return launch_tc<4, true, false, false, true>(tm_k, tm_v, p, grid, stream);
-        }
-        if (rows <= 32) return launch_tc<1, false, false, false, true>(tm_k, tm_v, p, grid, stream);
-        if (rows <= 64) return launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
-        return launch_tc<4, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        if (p.T > 32) return launch_tc<2, true, false, false, true>(tm_k, tm_v, p, grid, stream);
+        return rows <= 32 ? launch_tc<1, false, false, false, true>(tm_k, tm_v, p, grid, stream)
+                          : launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
     }
     const bool units = p.B == 128;   // 128-row tiles over blocks of 128 tokens: slices cut at 64-key units
     if (p.pair) {   // (a full tile has more than 64 rows)

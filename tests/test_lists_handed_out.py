@@ -57,7 +57,8 @@ def test_lists_handed_out_equal_layer_by_layer(shape):
         assert (b - a).norm() <= 5e-3 * a.norm() and (b - a).abs().max() <= 0.03 * a.abs().max()
         assert ((b - a).norm(dim=-1) <= 1e-2 * a.norm(dim=-1)).all()
 
-    assert L * S * Hkv > 148 and binding._native.workspace_bytes_layers(eng.geom, L, max_sel) == 256
+    handed = Hq // Hkv * T <= 64   # (128-row tiles are left to a CTA per list)
+    assert L * S * Hkv > 148 and (binding._native.workspace_bytes_layers(eng.geom, L, max_sel) == 256) == handed
     for _ in range(2):   # (the counter of the launch before must not matter)
         eng.verify_step(q, dk, dv, out)
     for l in range(L):
@@ -73,5 +74,5 @@ def test_lists_handed_out_equal_layer_by_layer(shape):
     for l in range(L):
         eng.dense_layer(l, q[l], dk[l], dv[l], want[l])
     check()
-    assert int(eng._stack_workspace[0].max()) == 0, "the launches left their counter behind"
+    assert not handed or int(eng._stack_workspace[0].max()) == 0, "the launches left their counter behind"
     eng.check_status()
