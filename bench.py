@@ -499,9 +499,9 @@ def run_gpu(args):
                 "note": "steps one after the other (a decoding loop cannot overlap neighbouring steps: the next queries "
                         "depend on this step's acceptance); every step is one call of SparseVerifier.verify_step_from_host: "
                         "Q and draft K/V of all layers from pinned host memory, the step, the outputs back to pinned host "
-                        "memory, the copies in chunks of a few layers on two side streams so that all but the first upload "
+                        "memory, the copies in two chunks of layers, in the background so that all but the first upload "
                         "and the last download run under the step's kernels; the KV cache is device-resident state",
-                "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "2 / half / half / 2",
+                "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "7/16, 9/16 of the layers",
                 "one_stream_value": ms_e2e_one_stream * 1e3 / (w.n_layers * world),
                 "one_stream_note": "the same bytes copied whole before and after the step on the step's own stream",
                 "pipelined_value": ms_e2e_pipelined * 1e3 / (w.n_layers * world),
@@ -923,7 +923,7 @@ def main():
     ap.add_argument("--configs", action="store_true",
                     help="timing lines for the batched (16 ragged sequences) and long-context (4 x 128K, tree) configurations")
     ap.add_argument("--e2e-chunk", default="", help="layers per copy chunk of the end-to-end step: a size, or sizes a,b,c,... "
-                                                     "(default: the engine's schedule, 2 / half / half / 2)")
+                                                     "(default: the engine's schedule, 7/16 and 9/16 of the layers)")
     ap.add_argument("--only", default="", help="with --configs: comma-separated configuration names (profiling aid: no dense pass)")
     ap.add_argument("--variants", action="store_true",
                     help="instead of the benchmark line: timings of the retrieval variants (shared budget, every token)")
