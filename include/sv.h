@@ -391,12 +391,15 @@ SV_API sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, const 
  * layer's result does not depend on the layers it is launched with.
  *   sv_block_reps_layers   layers l with which[l] != 0 (host, uint8 [L]; NULL: all)
  *   sv_verify_attn_layers  sel_idx == NULL: dense verification (anchors may be NULL); workspace of
- *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes, the first 256 of them zeroed once by the
- *                          caller and left to the call from then on (one workspace per stream)
+ *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes.  The first SV_STACK_STATE_BYTES of them
+ *                          are zeroed once by the caller and left to the call from then on (one workspace per stream); the
+ *                          zeros have to be there when the first call runs, so a captured call's own graph is no place for
+ *                          the fill: a call outside the graph may come before the first replay
  *   sv_kv_append_layers    advances seq_lens (which must be layers->seq_lens) in place; counters: dev uint32 [2 S], zeroed
  *                          once by the caller and left to this call from then on
  */
 #define SV_MAX_LAYERS 256
+#define SV_STACK_STATE_BYTES 256
 typedef struct {
     const void *table;          /* dev: rows written by sv_layer_table */
     const int32_t *block_table; /* dev int32 [S][NBmax] */

@@ -33,6 +33,7 @@ EXPORTS = ("sv_strerror", "sv_status_word_check", "sv_budget_blocks", "sv_worksp
            "sv_block_reps_layers", "sv_select_blocks_layers", "sv_verify_attn_layers", "sv_kv_append_layers", "sv_host_step_create",
            "sv_host_step_destroy", "sv_verify_step_from_host")
 SV_MAX_LAYERS = 256
+SV_STACK_STATE_BYTES = 256   # what a stack's launches keep at the start of their workspace
 
 
 class SvError(RuntimeError):

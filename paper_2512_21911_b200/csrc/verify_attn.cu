@@ -367,7 +367,6 @@ static bool hand_out(const sv_geom *rule, int max_sel)
     return svh::row_tiles(rule) == 1 && rule->n_q_heads / rule->n_kv_heads * rule->n_draft <= 64 &&
            (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
 }
-constexpr size_t kClaimsBytes = 256;
 
 // The geometry the split rules see for a stack: every (layer, sequence) is a sequence of one batch.
 static sv_geom stack_geom(const sv_geom *geom, int32_t n_layers)
@@ -382,7 +381,7 @@ extern "C" size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layer
     if (svh::check_geom(geom) != SV_OK || n_layers < 1 || n_layers > SV_MAX_LAYERS || max_sel < 1) return 0;
     const sv_geom g = stack_geom(geom, n_layers);
     if (svh::check_geom(&g) != SV_OK) return 0;
-    return hand_out(&g, max_sel) ? kClaimsBytes : workspace_bytes_for(&g, max_sel, true);
+    return hand_out(&g, max_sel) ? (size_t)SV_STACK_STATE_BYTES : workspace_bytes_for(&g, max_sel, true);
 }
 
 extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
@@ -401,7 +400,7 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
     const int splits = choose_splits(&rule, max_sel);
     const bool handed = hand_out(&rule, max_sel);
     st = check_workspace(handed ? 2 : splits, workspace, workspace_bytes,
-                         handed ? kClaimsBytes : workspace_bytes_for(&rule, max_sel, true));
+                         handed ? (size_t)SV_STACK_STATE_BYTES : workspace_bytes_for(&rule, max_sel, true));
     if (st != SV_OK) return st;
     StackAttnParams p;
     const size_t skip = (size_t)first * geom->n_seq * geom->n_draft * 128;   // rows of the layers ahead, per head

@@ -40,13 +40,19 @@ class SparseVerifier:
         self._one_allocation = False
         self._copy_streams = None
         self._host_step = None
-        self._stack_workspace = [None, None]   # sparse, dense
         self._counters = torch.zeros(2 * n_seq, dtype=torch.int32, device=dev)   # see sv_kv_append_layers
         # what the layers' kernels look up when several layers run in one launch (a row is valid once its layer has pools)
         stackable = n_layers <= sv.SV_MAX_LAYERS and n_layers * n_seq <= 65535
         row = sv._lib.sv_layer_table_bytes(1)
         self._table = torch.zeros((n_layers, row), dtype=torch.uint8, device=dev) if stackable else None
         self._rows_missing = n_layers
+        # Of a stack's workspaces (sparse, dense) those that hold only what the launches keep between calls are made and zeroed
+        # here: a fill in the first step would be a node of a graph, and not have run, when that step is captured.  The others
+        # are scratch of many megabytes, written before they are read: made when they are needed.
+        self._stack_bytes = [sv._native.workspace_bytes_layers(self.geom, n_layers, n) if stackable else 0
+                             for n in (max_sel, self.geom.max_blocks)]
+        self._stack_workspace = [torch.zeros(n, dtype=torch.uint8, device=dev) if n == sv.SV_STACK_STATE_BYTES else None
+                                 for n in self._stack_bytes]
 
     def _make_lists(self, flags: bytes, dev) -> None:
         """One block list per anchor layer; sel_idx / sel_cnt is the last one, which is also what verify_layer keeps its
@@ -106,8 +112,7 @@ class SparseVerifier:
 
     def _workspace_of_stack(self, dense: bool) -> torch.Tensor:
         if self._stack_workspace[dense] is None:
-            n = sv._native.workspace_bytes_layers(self.geom, self.n_layers, self.geom.max_blocks if dense else self.max_sel)
-            self._stack_workspace[dense] = torch.zeros(max(16, n), dtype=torch.uint8, device=self.workspace.device)
+            self._stack_workspace[dense] = torch.empty(max(16, self._stack_bytes[dense]), dtype=torch.uint8, device=self.workspace.device)
         return self._stack_workspace[dense]
 
     def _run_layers(self, first: int, end: int, q, draft_k, draft_v, out, dense: bool = False) -> bool:
