@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "attn_common.cuh"
+#include "list_claims.h"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
 
@@ -85,7 +86,12 @@ struct alignas(16) Segment {
     int item;
 };
 constexpr uint32_t kLongWait = 1u << 22;   // polls of a wait that may last as long as a segment
-
+// (kBal) the words of list_claims.h
+struct ClaimWords {
+    uint32_t *at;
+    __device__ uint32_t add(int i, uint32_t v) const { return atomicAdd(at + i, v); }
+    __device__ void set(int i, uint32_t v) const { atomicExch(at + i, v); }
+};
 
 // NH = 8-row groups per TMEM lane quadrant that hold real query rows: 1 (rows <= 32), 2 (<= 64), 4 (<= 128).
 // kWide: more than one row tile per (sequence, KV head) or more than 32 draft tokens (64-bit ancestor masks).  The
@@ -305,13 +311,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                     int count_next = 0, L_next = 0, blk_next = 0, page_next = 0, step = 0;
-                    if (lane == 0) claim = (int)atomicAdd(p.claims, 1u) + (int)gridDim.x;
+                    if (lane == 0) claim = (int)ClaimWords{p.claims}.add(0, 1u);
                     auto prepare_next = [&] {
                         if (step == 0) {
-                            claim = __shfl_sync(0xffffffffu, claim, 0);
-                            // every CTA is refused once, so this many claims are made in all: the last one leaves zero behind
-                            if (lane == 0 && claim == p.n_claims + (int)gridDim.x - 1) atomicExch(p.claims, 0u);
-                            if (claim >= p.n_claims) claim = -1;
+                            claim = claimed_list((uint32_t)__shfl_sync(0xffffffffu, claim, 0), p.n_claims, (int)gridDim.x);
                             // tell warp 11 (which has long noted the segment before this one)
                             if (lane == 0 && !dead) {
                                 const int at = (seg + 1) & 1;
@@ -383,8 +386,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                         draft_at = ring++;
                     }
                     while (step < 2) prepare_next();
-                    if (claim < 0) break;
+                    // a CTA that has given up claims nothing more: the lists that are left go to the others
+                    if (claim < 0 || __any_sync(0xffffffffu, dead || *abort_flag)) break;
                     cur = nxt, count = count_next, n_sel = blocks_of(count), L = L_next, blk_in = blk_next, page_in = page_next;
+                }
+                if (lane == 0) {
+                    __threadfence();   // (this CTA's claims are made before it leaves)
+                    leave_claims(ClaimWords{p.claims}, (int)gridDim.x);
                 }
                 if (dead) let_copies_land();
                 return;
