@@ -853,20 +853,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     int ring = 0, k_before = 0;   // (kBal) ring units, and units of this warpgroup, of the segments before
     for (int seg = 0;; ++seg) {   // (one pass unless kBal)
     int seg_item = 0, seg_total = 0;
-    bool lost = false;   // (the segment never came)
     if constexpr (kBal) {
-        if (__any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait))) {
-            lost = true;
+        // (lost: the segment never came)
+        const bool lost = __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait));
+        if (lost) {
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 8);
-        } else {
-            const volatile Segment *d = segments + (seg & 1);
-            seg_total = d->n_total, seg_item = d->item;
-            if (seg_total < 0) {
-                grid_launch_dependents();
-                if (lane == 0) mbar_arrive(bar(kTmemDone));   // (behind this warp's last read of tensor memory)
-                return;
-            }
+        }
+        // All warps leave together, here or behind a segment: what follows has barriers for all of them.
+        if (named_bar_or(1, 2 * wg_threads, lost)) {
+            if (lane == 0) mbar_arrive(bar(kTmemDone));
+            return;
+        }
+        const volatile Segment *d = segments + (seg & 1);
+        seg_total = d->n_total, seg_item = d->item;
+        if (seg_total < 0) {
+            grid_launch_dependents();
+            if (lane == 0) mbar_arrive(bar(kTmemDone));   // (behind this warp's last read of tensor memory)
+            return;
         }
     }
     const unsigned long long *anc_s = anc + (kBal ? (seg & 1) * 64 : 0);
@@ -898,13 +902,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if constexpr (kBal) {
         __syncwarp();
-        if (lane == 0 && !lost) mbar_arrive(bar(kTaken));
+        if (lane == 0) mbar_arrive(bar(kTaken));
     }
     const int L = kBal ? 0 : p.seq_lens[s];
     const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
     const int n_sel = kBal ? 0 : p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
     const int off = has_draft ? 1 : 0;
-    const int n_total = kBal ? max(0, seg_total) : slice_units(split, n_sel) + off;
+    const int n_total = kBal ? seg_total : slice_units(split, n_sel) + off;
 
     // per slot (row): reference maximum of the exponentials (log2 units) and partial row sum
     float m[NH], l[NH];
@@ -913,7 +917,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         m[i] = -INFINITY;
         l[i] = 0.f;
     }
-    bool dead = kBal && lost;
+    bool dead = false;
     constexpr float kLazy = 8.f;   // the reference maximum may trail the true one by up to 2^8
 
     // wait until the warpgroup's k-th PV has been added to O (warp-uniform outcome)
