@@ -26,7 +26,9 @@
 // third warpgroup gives its registers to the other two (setmaxnreg).  Everything is chained with mbarriers; tcgen05.commit signals MMA completion.
 // At the end warpgroup 0 reads both accumulators from TMEM (warp q of either warpgroup owns lane quadrant q),
 // merges them in registers and writes the rows (or the fp32 partial of its split) out.
-// All waits are bounded; a wait that gives up sets *status and the CTA drains and frees its TMEM.
+// All waits are bounded; a wait that gives up sets *status and the CTA drains: warp 9 leaves last, and before it
+// frees the TMEM and the CTA its shared memory it waits (again with a limit) for the MMAs that have been issued and, when somebody
+// has given up, for the copies that have been requested (else all of them have been read).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -34,6 +36,7 @@
 
 #include "attn_common.cuh"
 #include "list_claims.h"
+#include "ring_copies.h"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
 
@@ -71,7 +74,7 @@ enum Bar {
     kPReady = kSFree + 2,       // [2] P is in shared memory
     kOReady = kPReady + 2,      // [2] the warpgroup's latest PV has been added to O in TMEM
     kStaged = kOReady + 2,      // Q (and the draft unit) are staged
-    kTmemDone = kStaged + 1,    // all warps are done with TMEM
+    kTmemDone = kStaged + 1,    // all warps are done with TMEM, all MMAs are through, the producer has requested its last copy
     kLoaded = kTmemDone + 1,    // (kBal) the segment's descriptor, masks and Q tile are in shared memory
     kTaken = kLoaded + 1,       // (kBal) ... and everybody has taken them from there: the next segment's may follow
     kSlot = kTaken + 1,         // (kBal) the stage of the next draft unit is free
@@ -85,7 +88,9 @@ struct alignas(16) Segment {
     int n_total;   // units, the draft unit (the last one) included; -1: there is no further segment
     int item;
 };
-constexpr uint32_t kLongWait = 1u << 22;   // polls of a wait that may last as long as a segment
+// Polls of a wait that may last as long as a segment, and of the waits at the end of a CTA that has given up: more than the
+// other roles take to notice (each leaves the wait it is in, of 2^19 polls at most).
+constexpr uint32_t kLongWait = 1u << 22;
 // (kBal) the words of list_claims.h
 struct ClaimWords {
     uint32_t *at;
@@ -123,11 +128,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t *anc32 = reinterpret_cast<uint32_t *>(misc + 320);                     // [32] the same, up to 32 draft tokens
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 448);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + 456);
+    // the ring units the producer requests and the first of them; (kBal) a RingCopies
+    volatile uint32_t *requested = reinterpret_cast<volatile uint32_t *>(misc + 464);
     // (kBal) the masks of odd segments (64-bit: anc + 64), the segment descriptors, the claims on their way to warp 11
     uint32_t *anc32_odd = reinterpret_cast<uint32_t *>(misc + 1536);
     volatile Segment *segments = reinterpret_cast<volatile Segment *>(misc + 1664);
     volatile int *claims = reinterpret_cast<volatile int *>(misc + 1696);
     auto bar = [&](int slot) { return bars + 8u * slot; };
+    // (kBal) a wait that may last as long as a segment; it ends early when somebody has given up
+    auto long_wait = [&](int slot, uint32_t parity) {
+        for (uint32_t i = 0; i < kLongWait; ++i) {
+            if (mbar_try_wait(bar(slot), parity)) return true;
+            if ((i & 63) == 63 && *abort_flag) return false;
+        }
+        return false;
+    };
 
     static_assert(!kBal || NH < 4, "lists are handed out for tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
@@ -141,9 +156,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int QR = NH == 4 ? 32 : 16;                    // tile rows per TMEM lane quadrant
     constexpr bool kPTmem = NH == 4 && !kPair;
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
-    // registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168); the roles of a balanced launch keep
-    // track of more
-    constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : 232, kRegsFew = 504 - 2 * kRegsMany;
+    // Registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168).  At 232 / 40 the roles of the third spill
+    // inside their loops (16 sequences of 4-16K: 34.5 us a layer, 34.1 at 208 / 88; dense 32K 29.5 and 28.8; one 240-row tree 24.3
+    // and 23.9); the softmax needs no more than 208 in any form.  The roles of a balanced launch keep track of more.
+    constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : 208, kRegsFew = 504 - 2 * kRegsMany;
     constexpr int OFFQ = NS * kStageBytes;                   // the Q tile (kPair: of warpgroup 0; warpgroup 1's follows)
     // blockIdx.x = split * groups + group: the CTAs that gather the same slice of the blocks are neighbours in the grid
     // (they share those K/V tiles through L2; 1-2 % faster than group-major order).  A group is a row tile (kWide), or
@@ -210,12 +226,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == kSFree || lane == kPReady) count = na0;
             if (lane == kSFree + 1 || lane == kPReady + 1) count = max(1, na1);
             if (lane == kStaged) count = 8;
-            if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0);
+            if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0) + 3;   // the softmax warps, either issuer's MMAs, the producer
             if (lane == kTaken) count = na0 + (n_wg == 2 ? na1 : 0) + 2;   // the softmax warps and both issuers
             mbar_init(bar(lane), count);
             mbar_fence_init();
         }
-        if (lane == 0) *abort_flag = 0;
+        if (lane == 0) *abort_flag = 0, requested[0] = 0, requested[1] = 0;
         __syncwarp();
         if constexpr (!kBal) named_bar_arrive(3, kThreads);
     } else if constexpr (kBal) {
@@ -260,10 +276,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();   // the barriers are initialised, tensor memory is allocated
         tc_fence_after_sync();
     }
-    // after a wait that gave up: whatever this CTA still has in flight is through long before it frees its memory
-    auto let_copies_land = [] {
-        for (int i = 0; i < 100; ++i) __nanosleep(2000);
-    };
     // the query rows of a list to a Q tile, 16 bytes per asynchronous copy, by n threads of which this is t
     auto copy_q = [&](uint32_t tile_at, const Item &it, int t, int n) {
         const int c = t & 15;
@@ -285,6 +297,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint64_t policy = policy_evict_first();
                 const int sh = upb - 1;   // units of a block: 1 << sh
                 bool dead = false;
+                RingCopies copies;   // (lane 0's)
                 if (!p.early_gather) grid_dependency_wait();   // the lists may come from the kernel just before
                 // A batch is 32 consecutive entries of one list, one per lane.  What the next segment needs -- its claim, count
                 // and first entries, their pages: three trips to L2, each needing the one before -- is fetched in steps
@@ -318,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             // tell warp 11 (which has long noted the segment before this one)
                             if (lane == 0 && !dead) {
                                 const int at = (seg + 1) & 1;
-                                if (seg >= 2 && (*abort_flag || !mbar_wait_bounded(bar(kClaimTaken + at), ((seg - 2) >> 1) & 1, kLongWait))) {
+                                if (seg >= 2 && (*abort_flag || !long_wait(kClaimTaken + at, ((seg - 2) >> 1) & 1))) {
                                     dead = true;
                                     *abort_flag = 1;
                                     if (p.status) atomicOr(p.status, 1);
@@ -360,6 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                     meta[stage] = max(0, min(kUnit, L - (t0 + uo * kUnit)));
                                     const uint32_t fb = bar(kFull + stage), dst = smem0 + stage * kStageBytes;
                                     mbar_arrive_expect_tx(fb, kStageBytes);
+                                    copies.copied(stage, it);
                                     tma_load_3d(dst, mk, 0, r0 + uo * kUnit, 0, fb, policy);
                                     tma_load_3d(dst + 2 * kTile, mv, 0, r0 + uo * kUnit, 0, fb, policy);
                                 }
@@ -374,12 +388,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if (lane == 0 && !dead) {
                             const int stage = ring % NS, it = ring / NS;
                             if (*abort_flag ||
-                                (draft_at >= 0 && ring - draft_at <= NS && !mbar_wait_bounded(bar(kFull + draft_at % NS), (draft_at / NS) & 1, kLongWait)) ||
+                                (draft_at >= 0 && ring - draft_at <= NS && !long_wait(kFull + draft_at % NS, (draft_at / NS) & 1)) ||
                                 (it > 0 && !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
                                 dead = true;
                                 *abort_flag = 1;
                                 if (p.status) atomicOr(p.status, 1);
                             } else {
+                                copies.filled_otherwise(stage);
                                 mbar_arrive(bar(kSlot));
                             }
                         }
@@ -393,8 +408,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (lane == 0) {
                     __threadfence();   // (this CTA's claims are made before it leaves)
                     leave_claims(ClaimWords{p.claims}, (int)gridDim.x);
+                    requested[0] = copies.stages, requested[1] = copies.odd;
+                    mbar_arrive(bar(kTmemDone));
                 }
-                if (dead) let_copies_land();
                 return;
             }
             if constexpr (kStack) {
@@ -434,6 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int u0 = slice_begin(split, n_sel), u1 = slice_begin(split + 1, n_sel);
             const int j0 = kUnitSlices ? u0 >> 1 : u0, j1 = kUnitSlices ? (u1 + 1) >> 1 : u1;
             const int off = has_draft ? 1 : 0;
+            if (lane == 0) requested[0] = (kUnitSlices ? u1 - u0 : (j1 - j0) * upb) + off, requested[1] = off;
             bool dead = false;
             for (int base = j0; base < j1; base += 32) {
                 const int j = base + lane;
@@ -465,6 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 dead = true;
                                 *abort_flag = 1;
                                 if (p.status) atomicOr(p.status, 1);
+                                requested[0] = u + off;
                                 break;
                             }
                             const int nvalid = max(0, min(kUnit, L - (t0 + uo * kUnit)));
@@ -483,6 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
             }
+            if (lane == 0) mbar_arrive(bar(kTmemDone));
         } else if (kBal && warp == 11) {
             // ---------------------------------------------------------- (kBal) segments: descriptor, Q tile, masks, draft unit
             int ring = 0, n_drafts = 0;
@@ -491,11 +510,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 int claim = blockIdx.x;
                 bool ok = true;
                 if (seg > 0) {
-                    ok = __all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kClaim + (seg & 1)), ((seg - 1) >> 1) & 1, kLongWait));
+                    ok = __all_sync(0xffffffffu, !*abort_flag && long_wait(kClaim + (seg & 1), ((seg - 1) >> 1) & 1));
                     claim = claims[seg & 1];
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(kClaimTaken + (seg & 1)));
-                    ok = ok && __all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kTaken), (seg - 1) & 1, kLongWait));
+                    ok = ok && __all_sync(0xffffffffu, !*abort_flag && long_wait(kTaken, (seg - 1) & 1));
                 }
                 if (!ok) {
                     *abort_flag = 1;
@@ -550,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (lane == 0) mbar_arrive(bar(kLoaded));
                 {   // the last unit of the segment
                     const int stage = (ring + n_total - 1) % NS;
-                    if (!__all_sync(0xffffffffu, !*abort_flag && mbar_wait_bounded(bar(kSlot), n_drafts++ & 1, kLongWait))) {
+                    if (!__all_sync(0xffffffffu, !*abort_flag && long_wait(kSlot, n_drafts++ & 1))) {
                         *abort_flag = 1;
                         if (p.status && lane == 0) atomicOr(p.status, 1);
                         break;
@@ -593,7 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 int ring = 0, done0 = 0, done1 = 0;
                 bool end = false;
                 auto next_segment = [&](int seg) {
-                    bool ok = !*abort_flag && mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait);
+                    bool ok = !*abort_flag && long_wait(kLoaded, seg & 1);
                     if (ok) {
                         n_total = segments[seg & 1].n_total;
                         end = n_total < 0;
@@ -649,9 +668,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     if constexpr (kBal) end_segment();
                     }
-                    if (kBal && dead) let_copies_land();
-                    // free TMEM only after every softmax warp has finished reading it
-                    if (!mbar_wait_bounded(bar(kTmemDone), 0, kBal ? kLongWait : 1u << 19) && p.status) atomicOr(p.status, 16);
+                    tc_commit(bar(kTmemDone));
+                    // free TMEM only after every softmax warp has finished reading it and every MMA is through
+                    if (!mbar_wait_bounded(bar(kTmemDone), 0, kLongWait)) {
+                        *abort_flag = 1;
+                        if (p.status) atomicOr(p.status, 16);
+                    }
+                    if (*abort_flag) {
+                        const RingCopies copies = kBal ? RingCopies{requested[0], requested[1]}
+                                                       : copies_of_units((int)requested[1], (int)requested[0], NS);
+                        for (int stage = 0; stage < NS; ++stage)
+                            if (copies.waits_for(stage) && !mbar_wait_bounded(bar(kFull + stage), copies.parity(stage), kLongWait) && p.status)
+                                atomicOr(p.status, 1);
+                    }
                 } else {
                     constexpr uint32_t idesc_pv = umma_idesc_bf16(MT, 128, true);
                     const uint64_t dp = umma_desc_sw128(smem0 + kOffP, 16, 1024);
@@ -692,6 +721,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     if constexpr (kBal) end_segment();
                     }
+                    tc_commit(bar(kTmemDone));   // (arrives behind the last PV that was issued)
                 }
             }
             if (warp == 9) {
@@ -855,7 +885,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int seg_item = 0, seg_total = 0;
     if constexpr (kBal) {
         // (lost: the segment never came)
-        const bool lost = __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kLoaded), seg & 1, kLongWait));
+        const bool lost = __any_sync(0xffffffffu, *abort_flag || !long_wait(kLoaded, seg & 1));
         if (lost) {
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 8);
