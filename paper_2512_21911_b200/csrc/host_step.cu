@@ -105,6 +105,12 @@ extern "C" sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom 
     cudaStream_t main = static_cast<cudaStream_t>(stream), in = static_cast<cudaStream_t>(stream_in), back = static_cast<cudaStream_t>(stream_out);
     bool ok = true;
     auto cuda = [&](cudaError_t e) { ok = ok && e == cudaSuccess; };
+    // `to` goes on behind what is on `from` by now; whether it does
+    auto order = [&](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
+        const bool done = cudaEventRecord(e, from) == cudaSuccess && cudaStreamWaitEvent(to, e, 0) == cudaSuccess;
+        ok = ok && done;
+        return done;
+    };
     const size_t q_layer = (size_t)geom->n_seq * geom->n_draft * geom->n_q_heads * 256, kv_layer = (size_t)geom->n_seq * geom->n_draft * geom->n_kv_heads * 256;
     auto part = [&](void *to, const void *from, size_t layer, int c, cudaMemcpyKind kind, cudaStream_t s) {
         const size_t l0 = c ? chunk_end[c - 1] : 0, l1 = chunk_end[c];
@@ -140,9 +146,9 @@ extern "C" sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom 
                     {nq, nq + nk, nq + 2 * nk}});
     }
     // (the uploads of later chunks would only take bandwidth from the first one's)
-    cuda(cudaEventRecord(step->fork, main));
-    cuda(cudaStreamWaitEvent(in, step->fork, 0));
-    if (!direct_in) upload(0);
+    const bool in_forked = order(step->fork, main, in);
+    bool back_forked = false;
+    if (!direct_in && ok) upload(0);
     if (refresh_tail && ok) {
         st = sv_block_reps_layers(geom, layers, refresh_which, SV_TAIL_BLOCK, -1, reps, stream);
         ok = st == SV_OK;
@@ -166,19 +172,14 @@ extern "C" sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom 
                         {n, n, n}});
             continue;
         }
-        cuda(cudaEventRecord(step->done[c], main));
-        cuda(cudaStreamWaitEvent(back, step->done[c], 0));
+        if (!order(step->done[c], main, back)) break;
+        back_forked = true;
         part(out_host, out, q_layer, c, cudaMemcpyDeviceToHost, back);
     }
-    // the side streams join whatever happened (a captured stream may not be left forked)
-    const bool was_ok = ok;
-    ok = true;
-    cuda(cudaEventRecord(step->joined, in));
-    cuda(cudaStreamWaitEvent(main, step->joined, 0));
-    if (was_ok && st == SV_OK && (n_chunks > 1 || !direct_out)) {
-        cuda(cudaEventRecord(step->joined, back));
-        cuda(cudaStreamWaitEvent(main, step->joined, 0));
-    }
+    // The side streams that were forked join whatever happened: their copies still use the caller's memory, and a captured stream
+    // may not be left forked.
+    if (in_forked) order(step->joined, in, main);
+    if (back_forked) order(step->joined, back, main);
     if (st != SV_OK) return st;
-    return was_ok && ok ? SV_OK : SV_ERR_CUDA;
+    return ok ? SV_OK : SV_ERR_CUDA;
 }
