@@ -432,8 +432,12 @@ SV_API sv_status sv_kv_append_layers(const sv_geom *geom, const sv_layers *layer
  * returns, and `stream` ends behind the last copy.  stream_in / stream_out: two other streams, for the uploads and the
  * downloads.  An sv_host_step holds the events of one caller; it belongs to the device that is current when it is created
  * and serves one call at a time.
+ * workspace: as for sv_verify_attn_layers, of sv_workspace_bytes_layers bytes at least.  With sv_workspace_bytes_host_step bytes (a few
+ * megabytes more) a chunk of few lists is split over the SMs as if it were the whole stack, instead of one CTA a list; its
+ * outputs then equal those of sv_verify_attn_layers to bf16 rounding, and not bit for bit.
  */
 #define SV_MAX_HOST_CHUNKS 256
+SV_API size_t sv_workspace_bytes_host_step(const sv_geom *geom, int32_t n_layers, int32_t max_sel);
 typedef struct sv_host_step sv_host_step;
 SV_API sv_host_step *sv_host_step_create(void);
 SV_API void sv_host_step_destroy(sv_host_step *step);

@@ -161,8 +161,8 @@ extern "C" sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom 
         const int first = c ? chunk_end[c - 1] : 0, end = chunk_end[c];
         st = sv_select_blocks_layers(geom, layers, first, end, anchors, q, reps, budget_blocks, n_sink, n_local, idx, cnt, max_sel, stream);
         if (st == SV_OK)
-            st = sv_verify_attn_layers(geom, layers, first, end, anchors, q, draft_k, draft_v, parent, idx, cnt, max_sel, 0.f, out,
-                                       workspace, workspace_bytes, status_word, stream);
+            st = svh::verify_attn_layers(geom, layers, first, end, anchors, q, draft_k, draft_v, parent, idx, cnt, max_sel, 0.f, out,
+                                         workspace, workspace_bytes, status_word, stream, true);
         if (st != SV_OK) break;
         if (c == n_chunks - 1 && direct_out) {
             const size_t at = (c ? chunk_end[c - 1] : 0) * q_layer;

@@ -312,6 +312,15 @@ PyObject *workspace_bytes_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// geom, n_layers, max_sel -> bytes
+PyObject *workspace_bytes_host_step(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return checked(n, 3, [&] {
+        const sv_geom g = geometry(a[0]);
+        return PyLong_FromSize_t(sv_workspace_bytes_host_step(&g, int32(a[1]), int32(a[2])));
+    });
+}
+
 // geom, table, kv, which (bytes or None), block_begin, block_end, reps
 PyObject *block_reps_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
@@ -460,7 +469,7 @@ PyObject *accept_new(PyObject *, PyObject *const *a, Py_ssize_t n)
 
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {METHOD(block_reps), METHOD(select_blocks), METHOD(verify_attn), METHOD(kv_append), METHOD(accept),
-                         METHOD(verify_layer), METHOD(layer_row), METHOD(workspace_bytes_layers), METHOD(block_reps_layers),
+                         METHOD(verify_layer), METHOD(layer_row), METHOD(workspace_bytes_layers), METHOD(workspace_bytes_host_step), METHOD(block_reps_layers),
                          METHOD(verify_layers), METHOD(kv_append_layers), METHOD(accept_new), METHOD(host_step), METHOD(verify_step_from_host), {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Argument marshalling for the entry points of sv.h.", -1, methods,

@@ -144,6 +144,13 @@ inline int row_groups(const sv_geom *g)
     return pair_row_tiles(g) ? (t + 1) / 2 : t;
 }
 
+// sv_verify_attn_layers; own_splits: a launch of few lists may be split for itself instead of for the whole stack (the chunks of
+// a host-fed step; workspace of sv_workspace_bytes_host_step, without which the stack's rule holds).
+sv_status verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end, const uint8_t *anchors,
+                             const void *q, const void *draft_k, const void *draft_v, const int32_t *parent, const int32_t *sel_idx,
+                             const int32_t *sel_cnt, int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                             size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits);
+
 inline sv_status launch_status()
 {
     return cudaGetLastError() == cudaSuccess ? SV_OK : SV_ERR_CUDA;

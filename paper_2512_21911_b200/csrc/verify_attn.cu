@@ -376,6 +376,26 @@ static sv_geom stack_geom(const sv_geom *geom, int32_t n_layers)
     return g;
 }
 
+// Whether the launch of a chunk of a host-fed step is split for its own lists instead of the whole stack's.  The stack's rule leaves
+// the lists of a large stack whole, and a chunk of a few layers then runs on as many CTAs as it has lists, each with a
+// whole list in a row, while nothing fills the other SMs: the next chunk's launch waits for this one.  32 layers of a 32K context
+// (8 lists of 64 units a layer) in chunks of 1, 2, 4, 8 layers: 1519, 799, 413, 238 us by the stack's rule, 613, 375, 241, 188 split for
+// the launch; 16 layers x 4 sequences of 12K: 638, 349, 235 and 398, 277, 233; 16 layers of 128-row tiles: 542, 315, 236 and 383, 280,
+// 233.  Chunks that fill the SMs with whole lists come out the same by either rule.
+// The line: slices of at most eight units stay as the stack has them.  The shorter they are the less a split gains over the
+// partials and the merge it costs (20 layers in chunks of one: 16 units 428 -> 332 us, 10 units 377 -> 302; a launch of four units is
+// faster whole, see kUnsplitUnits), and what stays keeps the bits of the step on device tensors.  With several row tiles two halves
+// do not pay for their partials (24 layers x 2 sequences of 240 rows, 40 units, chunks of two layers: 1105 us whole, 1165 in
+// halves; chunks of one, four ways: 1600 and 1340).
+constexpr int kShortSliceUnits = 8;
+static bool split_for_launch(const sv_geom *rule, const sv_geom *launch, int max_sel)
+{
+    const int splits = choose_splits(rule, max_sel);
+    const int blocks = (max_sel + splits - 1) / splits;
+    const int at_least = svh::row_tiles(launch) > 1 ? 2 * splits + 1 : splits + 1;
+    return blocks * (rule->block_size / 64) > kShortSliceUnits && choose_splits(launch, max_sel) >= at_least;
+}
+
 extern "C" size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layers, int32_t max_sel)
 {
     if (svh::check_geom(geom) != SV_OK || n_layers < 1 || n_layers > SV_MAX_LAYERS || max_sel < 1) return 0;
@@ -384,11 +404,25 @@ extern "C" size_t sv_workspace_bytes_layers(const sv_geom *geom, int32_t n_layer
     return hand_out(&g, max_sel) ? (size_t)SV_STACK_STATE_BYTES : workspace_bytes_for(&g, max_sel, true);
 }
 
-extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
-                                           const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
-                                           const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
-                                           int32_t max_sel, float softmax_scale, void *out, void *workspace,
-                                           size_t workspace_bytes, int32_t *status_word, void *stream)
+extern "C" size_t sv_workspace_bytes_host_step(const sv_geom *geom, int32_t n_layers, int32_t max_sel)
+{
+    const size_t whole = sv_workspace_bytes_layers(geom, n_layers, max_sel);
+    if (svh::check_geom(geom) != SV_OK || n_layers < 1 || n_layers > SV_MAX_LAYERS || max_sel < 1) return 0;
+    const sv_geom rule = stack_geom(geom, n_layers);
+    if (svh::check_geom(&rule) != SV_OK) return 0;
+    size_t most = 0;
+    for (int32_t n = 1; n < n_layers; ++n) {
+        const sv_geom launch = stack_geom(geom, n);
+        if (split_for_launch(&rule, &launch, max_sel)) most = std::max(most, workspace_bytes_for(&launch, max_sel, true));
+    }
+    return most ? std::max(whole, (size_t)SV_STACK_STATE_BYTES + most) : whole;
+}
+
+sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                  const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
+                                  const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                  int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits)
 {
     sv_status st = svh::check_layers(geom, layers, first, end);
     if (st != SV_OK) return st;
@@ -396,9 +430,18 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
     st = check_attn_args(q, draft_k, draft_v, sel_idx, sel_cnt, max_sel, softmax_scale, out);
     if (st != SV_OK) return st;
     if (sel_idx && (!anchors || !anchors[0])) return SV_ERR_NULL;
-    const sv_geom rule = stack_geom(geom, layers->n_layers);
+    sv_geom rule = stack_geom(geom, layers->n_layers);
+    bool handed = hand_out(&rule, max_sel);
+    if (own_splits) {
+        const sv_geom launch = stack_geom(geom, end - first);
+        if (split_for_launch(&rule, &launch, max_sel) && workspace && svh::aligned(workspace, 16) &&
+            workspace_bytes >= (size_t)SV_STACK_STATE_BYTES + workspace_bytes_for(&launch, max_sel, true)) {
+            rule = launch, handed = false;
+            workspace = static_cast<char *>(workspace) + SV_STACK_STATE_BYTES;   // (what launches keep stays)
+            workspace_bytes -= SV_STACK_STATE_BYTES;
+        }
+    }
     const int splits = choose_splits(&rule, max_sel);
-    const bool handed = hand_out(&rule, max_sel);
     st = check_workspace(handed ? 2 : splits, workspace, workspace_bytes,
                          handed ? (size_t)SV_STACK_STATE_BYTES : workspace_bytes_for(&rule, max_sel, true));
     if (st != SV_OK) return st;
@@ -425,6 +468,16 @@ extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers 
         return launch_attn_tc_stack(p, dim3(std::min(sm_count(), p.n_claims)), cs) == cudaSuccess ? SV_OK : SV_ERR_CUDA;
     }
     return launch_attn(p, &rule, geom->n_seq * (end - first), cs, [&](dim3 grid) { return launch_attn_tc_stack(p, grid, cs); });
+}
+
+extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                           const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
+                                           const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                           int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                                           size_t workspace_bytes, int32_t *status_word, void *stream)
+{
+    return svh::verify_attn_layers(geom, layers, first, end, anchors, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel,
+                                   softmax_scale, out, workspace, workspace_bytes, status_word, stream, false);
 }
 
 // ---------------------------------------------------------------------- sv_verify_attn_noalloc

@@ -158,3 +158,27 @@ def test_pick_anchors_matches_oracle_on_host(svb):
         np.testing.assert_array_equal(a, oracle.pick_anchors(Jo, K))
     with pytest.raises(svb.SvError):
         svb.sv_pick_anchors(inter, uni, 13)
+
+
+def test_workspace_of_a_host_fed_step(svb):
+    """A chunk is split for itself only where the stack's slices are longer than eight units; every chunk's partials fit behind what
+    the launches keep."""
+    layers, step = svb._native.workspace_bytes_layers, svb._native.workspace_bytes_host_step
+    for heads, kv_heads, block, draft in ((32, 8, 64, 8), (64, 8, 128, 16), (32, 8, 64, 60), (8, 4, 64, 3)):
+        for n_layers in (1, 2, 3, 32, 64):
+            for seqs in (1, 3):
+                for keep in (1, 4, 8, 9, 40, 200):
+                    g = svb.make_geom(seqs, heads, kv_heads, 128, block, 256, draft)
+                    need, stack = step(g, n_layers, keep), layers(g, n_layers, keep)
+                    assert need >= stack
+                    if n_layers == 1 or keep * block // 64 <= 8:
+                        assert need == stack
+                    rows = heads // kv_heads * draft
+                    for n in range(1, n_layers):
+                        chunk = svb.make_geom(seqs * n, heads, kv_heads, 128, block, 256, draft)
+                        splits = svb.sv_verify_attn_splits(chunk, keep)
+                        whole = svb.sv_verify_attn_splits(svb.make_geom(seqs * n_layers, heads, kv_heads, 128, block, 256, draft), keep)
+                        if splits > (2 if rows > 128 else 1) * whole and -(-keep // whole) * (block // 64) > 8:
+                            assert need >= svb.SV_STACK_STATE_BYTES + seqs * n * kv_heads * splits * rows * 130 * 4
+    assert step(svb.make_geom(1, 32, 8, 128, 64, 512, 8), 32, 64) > 256
+    assert step(svb.make_geom(1, 32, 7, 128, 64, 512, 8), 32, 64) == 0 and step(svb.make_geom(1, 32, 8, 128, 64, 512, 8), 0, 64) == 0

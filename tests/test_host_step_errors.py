@@ -91,9 +91,11 @@ static sv_status work(void *s)
 sv_status sv_block_reps_layers(const sv_geom *, const sv_layers *, const uint8_t *, int32_t, int32_t, float *, void *s) { return work(s); }
 sv_status sv_select_blocks_layers(const sv_geom *, const sv_layers *, int32_t, int32_t, const uint8_t *, const void *, const float *,
                                   const int32_t *, int32_t, int32_t, int32_t *, int32_t *, int32_t, void *s) { return work(s); }
-sv_status sv_verify_attn_layers(const sv_geom *, const sv_layers *, int32_t, int32_t, const uint8_t *, const void *, const void *,
-                                const void *, const int32_t *, const int32_t *, const int32_t *, int32_t, float, void *, void *,
-                                size_t, int32_t *, void *s) { return work(s); }
+}
+namespace svh {
+sv_status verify_attn_layers(const sv_geom *, const sv_layers *, int32_t, int32_t, const uint8_t *, const void *, const void *,
+                             const void *, const int32_t *, const int32_t *, const int32_t *, int32_t, float, void *, void *,
+                             size_t, int32_t *, void *s, bool) { return work(s); }
 }
 
 int main()
