@@ -138,14 +138,31 @@ PyObject *checked(Py_ssize_t n, Py_ssize_t want, F body)
 }
 PyObject *status(sv_status st) { return PyLong_FromLong(st); }
 
+// The library call itself, without the interpreter lock: a launch waits when the queue of its device is full, and the threads that
+// drive other devices go on meanwhile.  All arguments are taken from Python before it (the caller holds the objects).  An eager layer
+// of a small model, back to back: 11.9 us with the lock held, 11.9-12.1 without.
+template <class F>
+sv_status unlocked(F call)
+{
+    struct Unlocked {
+        PyThreadState *const state = PyEval_SaveThread();
+        ~Unlocked() { PyEval_RestoreThread(state); }
+    } guard;
+    return call();
+}
+
 // geom, kv, reps, block_begin, block_end, stream, reps_bf16
 PyObject *block_reps(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return checked(n, 7, [&] {
         const sv_geom g = geometry(a[0]);
         const sv_kv kv = cache(a[1]);
-        if (truth(a[6])) return status(sv_block_reps_bf16(&g, &kv, int32(a[3]), int32(a[4]), bf16(a[2], "reps_bf16"), stream(a[5])));
-        return status(sv_block_reps(&g, &kv, int32(a[3]), int32(a[4]), f32(a[2], "reps"), stream(a[5])));
+        const int32_t begin = int32(a[3]), end = int32(a[4]);
+        const bool half = truth(a[6]);
+        void *const reps = half ? bf16(a[2], "reps_bf16") : f32(a[2], "reps"), *const s = stream(a[5]);
+        return status(unlocked([&] {
+            return half ? sv_block_reps_bf16(&g, &kv, begin, end, reps, s) : sv_block_reps(&g, &kv, begin, end, static_cast<float *>(reps), s);
+        }));
     });
 }
 
@@ -163,11 +180,15 @@ PyObject *select_blocks(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int32_t reuse = truth(a[9]) ? 1 : 0;
         const int32_t *pi = i32(a[10], "prev_idx"), *pc = i32(a[11], "prev_cnt");
         float *scores = f32(a[12], "out_scores");
-        if (truth(a[14]))
-            return status(sv_select_blocks_bf16reps(&g, q, bf16(a[2], "reps_bf16"), lens, budget, sink, local, reuse, pi, pc, idx,
-                                                    cnt, max_sel, scores, stream(a[13])));
-        return status(sv_select_blocks(&g, q, f32(a[2], "reps"), lens, budget, sink, local, reuse, pi, pc, idx, cnt, max_sel,
-                                       scores, stream(a[13])));
+        const bool half = truth(a[14]);
+        const void *const reps = half ? bf16(a[2], "reps_bf16") : f32(a[2], "reps");
+        void *const s = stream(a[13]);
+        return status(unlocked([&] {
+            if (half)
+                return sv_select_blocks_bf16reps(&g, q, reps, lens, budget, sink, local, reuse, pi, pc, idx, cnt, max_sel, scores, s);
+            return sv_select_blocks(&g, q, static_cast<const float *>(reps), lens, budget, sink, local, reuse, pi, pc, idx, cnt, max_sel,
+                                    scores, s);
+        }));
     });
 }
 
@@ -188,11 +209,14 @@ PyObject *verify_attn(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (scale == -1.0 && PyErr_Occurred()) throw ArgError{};
         int32_t *word = i32(a[12], "status_word");
         void *s = stream(a[13]);
-        switch (integer(a[14])) {
-            case 0: return status(sv_verify_attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s));
-            case 1: return status(sv_verify_attn_reused(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s));
-            default: return status(sv_verify_attn_noalloc(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, word, s));
-        }
+        const long long entry = integer(a[14]);
+        return status(unlocked([&] {
+            switch (entry) {
+                case 0: return sv_verify_attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s);
+                case 1: return sv_verify_attn_reused(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, ws.p, ws.bytes, word, s);
+                default: return sv_verify_attn_noalloc(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, (float)scale, out, lse, word, s);
+            }
+        }));
     });
 }
 
@@ -202,10 +226,15 @@ PyObject *kv_append(PyObject *, PyObject *const *a, Py_ssize_t n)
     return checked(n, 12, [&] {
         const sv_geom g = geometry(a[0]);
         const int32_t pages = (int32_t)tensor(a[1], at::kBFloat16, "k_pool").size(0);
-        return status(sv_kv_append(&g, bf16(a[1], "k_pool"), bf16(a[2], "v_pool"), pages, i32(a[3], "block_table"),
-                                   i32(a[4], "seq_lens"), bf16(a[5], "draft_k"), bf16(a[6], "draft_v"), i32(a[7], "accept_idx"),
-                                   i32(a[8], "n_accept"), row_length(a[7], "accept_idx"), i32(a[9], "seq_lens_out"),
-                                   f32(a[10], "reps"), stream(a[11])));
+        void *const k = bf16(a[1], "k_pool"), *const v = bf16(a[2], "v_pool");
+        const int32_t *const table = i32(a[3], "block_table"), *const lens = i32(a[4], "seq_lens");
+        const void *const dk = bf16(a[5], "draft_k"), *const dv = bf16(a[6], "draft_v");
+        const int32_t *const rows = i32(a[7], "accept_idx"), *const n_rows = i32(a[8], "n_accept");
+        const int32_t most = row_length(a[7], "accept_idx");
+        int32_t *const lens_out = i32(a[9], "seq_lens_out");
+        float *const reps = f32(a[10], "reps");
+        void *const s = stream(a[11]);
+        return status(unlocked([&] { return sv_kv_append(&g, k, v, pages, table, lens, dk, dv, rows, n_rows, most, lens_out, reps, s); }));
     });
 }
 
@@ -215,9 +244,15 @@ PyObject *accept(PyObject *, PyObject *const *a, Py_ssize_t n)
     return checked(n, 11, [&] {
         const at::Tensor &pt = tensor(a[0], at::kFloat, "p_target");
         const int32_t S = (int32_t)pt.size(0), T = (int32_t)pt.size(1), V = (int32_t)pt.size(2);
-        return status(sv_accept(S, T, V, f32(a[0], "p_target"), f32(a[1], "p_draft"), i32(a[2], "tokens"), i32(a[3], "parent"),
-                                f32(a[4], "u_accept"), f32(a[5], "u_next"), i32(a[6], "path"), i32(a[7], "n_path"),
-                                i32(a[8], "next_token"), f32(a[9], "alpha"), stream(a[10])));
+        const float *const target = f32(a[0], "p_target"), *const draft = f32(a[1], "p_draft");
+        const int32_t *const tokens = i32(a[2], "tokens"), *const parent = i32(a[3], "parent");
+        const float *const u_accept = f32(a[4], "u_accept"), *const u_next = f32(a[5], "u_next");
+        int32_t *const path = i32(a[6], "path"), *const n_path = i32(a[7], "n_path"), *const next = i32(a[8], "next_token");
+        float *const alpha = f32(a[9], "alpha");
+        void *const s = stream(a[10]);
+        return status(unlocked([&] {
+            return sv_accept(S, T, V, target, draft, tokens, parent, u_accept, u_next, path, n_path, next, alpha, s);
+        }));
     });
 }
 
@@ -241,18 +276,27 @@ PyObject *verify_layer(PyObject *, PyObject *const *a, Py_ssize_t n)
         int32_t *word = i32(a[17], "status_word");
         const bool anchor = truth(a[18]), behind = truth(a[19]);
         void *s = stream(Py_None);
+        const float *r = nullptr;
+        const int32_t *lens = nullptr, *budget = nullptr;
+        int32_t sink = 0, local = 0;
         if (anchor) {
             const at::Tensor &reps = tensor(a[3], at::kFloat, "reps");
             long long layer = integer(a[4]);
             if (layer < 0) layer += reps.size(0);
-            const float *r = reps.data_ptr<float>() + layer * reps.stride(0);
-            const sv_status st = sv_select_blocks(&g, q, r, i32(a[5], "seq_lens"), i32(a[6], "budget_blocks"), int32(a[7]), int32(a[8]),
-                                                  0, nullptr, nullptr, idx, cnt, max_sel, nullptr, s);
-            if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_True);
+            r = reps.data_ptr<float>() + layer * reps.stride(0);
+            lens = i32(a[5], "seq_lens"), budget = i32(a[6], "budget_blocks"), sink = int32(a[7]), local = int32(a[8]);
         }
         auto attn = behind && !anchor ? sv_verify_attn_reused : sv_verify_attn;
-        const sv_status st = attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, 0.f, out, lse, ws.p, ws.bytes, word, s);
-        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_False);
+        bool selecting = anchor;
+        const sv_status st = unlocked([&] {
+            if (anchor) {
+                const sv_status sel = sv_select_blocks(&g, q, r, lens, budget, sink, local, 0, nullptr, nullptr, idx, cnt, max_sel, nullptr, s);
+                if (sel != SV_OK) return sel;
+            }
+            selecting = false;
+            return attn(&g, q, &kv, dk, dv, parent, idx, cnt, max_sel, 0.f, out, lse, ws.p, ws.bytes, word, s);
+        });
+        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, selecting ? Py_True : Py_False);
         Py_RETURN_NONE;
     });
 }
@@ -327,8 +371,11 @@ PyObject *block_reps_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
     return checked(n, 7, [&] {
         const sv_geom g = geometry(a[0]);
         const sv_layers layers = stack(a[1], a[2]);
-        return status(sv_block_reps_layers(&g, &layers, flags(a[3], layers.n_layers), int32(a[4]), int32(a[5]), f32(a[6], "reps"),
-                                           stream(Py_None)));
+        const uint8_t *const which = flags(a[3], layers.n_layers);
+        const int32_t begin = int32(a[4]), end = int32(a[5]);
+        float *const reps = f32(a[6], "reps");
+        void *const s = stream(Py_None);
+        return status(unlocked([&] { return sv_block_reps_layers(&g, &layers, which, begin, end, reps, s); }));
     });
 }
 
@@ -352,14 +399,20 @@ PyObject *verify_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int32_t max_sel = dense ? g.max_blocks : row_length(a[15], "idx");
         const Scratch ws = scratch(a[17]);
         void *s = stream(Py_None);
-        if (!dense) {
-            const sv_status st = sv_select_blocks_layers(&g, &layers, first, end, anchors, q, f32(a[11], "reps"), i32(a[12], "budget_blocks"),
-                                                         int32(a[13]), int32(a[14]), idx, cnt, max_sel, s);
-            if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_True);
-        }
-        const sv_status st = sv_verify_attn_layers(&g, &layers, first, end, anchors, q, dk, dv, parent, idx, cnt, max_sel, 0.f, out, ws.p,
-                                                   ws.bytes, i32(a[18], "status_word"), s);
-        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, Py_False);
+        int32_t *const word = i32(a[18], "status_word");
+        const float *const reps = dense ? nullptr : f32(a[11], "reps");
+        const int32_t *const budget = dense ? nullptr : i32(a[12], "budget_blocks");
+        const int32_t sink = dense ? 0 : int32(a[13]), local = dense ? 0 : int32(a[14]);
+        bool selecting = !dense;
+        const sv_status st = unlocked([&] {
+            if (!dense) {
+                const sv_status sel = sv_select_blocks_layers(&g, &layers, first, end, anchors, q, reps, budget, sink, local, idx, cnt, max_sel, s);
+                if (sel != SV_OK) return sel;
+            }
+            selecting = false;
+            return sv_verify_attn_layers(&g, &layers, first, end, anchors, q, dk, dv, parent, idx, cnt, max_sel, 0.f, out, ws.p, ws.bytes, word, s);
+        });
+        if (st != SV_OK) return Py_BuildValue("(iO)", (int)st, selecting ? Py_True : Py_False);
         Py_RETURN_NONE;
     });
 }
@@ -411,18 +464,25 @@ PyObject *verify_step_from_host(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (chunks > SV_MAX_HOST_CHUNKS) Py_RETURN_FALSE;
         for (Py_ssize_t c = 0; c < chunks; ++c) ends[c] = int32(PySequence_Fast_GET_ITEM(a[5], c));
         const Scratch ws = scratch(a[21]);
-        const sv_status st = sv_verify_step_from_host(
-            h, &g, &layers, flags(a[4], layers.n_layers), ends, (int32_t)chunks, host[0], host[1], host[2], dev[0], dev[1], dev[2],
-            i32(a[12], "parent"), f32(a[13], "reps"), i32(a[14], "budget_blocks"), int32(a[15]), int32(a[16]), i32(a[17], "idx"),
-            i32(a[18], "cnt"), row_length(a[17], "idx"), dev[3], host[3], ws.p, ws.bytes, i32(a[22], "status_word"), truth(a[23]),
-            flags(a[24], layers.n_layers), stream(a[25]), stream(a[26]), stream(Py_None));
+        const uint8_t *const anchors = flags(a[4], layers.n_layers), *const which = flags(a[24], layers.n_layers);
+        const int32_t *const parent = i32(a[12], "parent"), *const budget = i32(a[14], "budget_blocks");
+        float *const reps = f32(a[13], "reps");
+        const int32_t sink = int32(a[15]), local = int32(a[16]), max_sel = row_length(a[17], "idx");
+        int32_t *const idx = i32(a[17], "idx"), *const cnt = i32(a[18], "cnt"), *const word = i32(a[22], "status_word");
+        const bool refresh = truth(a[23]);
+        void *const in = stream(a[25]), *const back = stream(a[26]), *const s = stream(Py_None);
+        const sv_status st = unlocked([&] {
+            return sv_verify_step_from_host(h, &g, &layers, anchors, ends, (int32_t)chunks, host[0], host[1], host[2], dev[0], dev[1], dev[2],
+                                            parent, reps, budget, sink, local, idx, cnt, max_sel, dev[3], host[3], ws.p, ws.bytes, word,
+                                            refresh, which, in, back, s);
+        });
         // the allocator of pinned memory must not hand these out again before the copies are through
         const auto device = c10::cuda::current_device();
         for (int i = 0; i < 4; ++i) {
             const at::Tensor &t = THPVariable_Unpack(i < 3 ? a[6 + i] : a[20]);
             void *const context = t.storage().data_ptr().get_context();
             at::getHostAllocator(at::kCUDA)->record_event(
-                host[i], context, c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream(a[i < 3 ? 25 : 26])), device).unwrap());
+                host[i], context, c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(i < 3 ? in : back), device).unwrap());
             at::getHostAllocator(at::kCUDA)->record_event(host[i], context, c10::cuda::getCurrentCUDAStream().unwrap());
         }
         return status(st);
@@ -438,9 +498,12 @@ PyObject *kv_append_layers(PyObject *, PyObject *const *a, Py_ssize_t n)
         const void *dk = stacked(a[3], layers.n_layers), *dv = stacked(a[4], layers.n_layers);
         int32_t *lens = i32(a[7], "seq_lens");
         if (!dk || !dv || lens != layers.seq_lens) Py_RETURN_FALSE;
-        return status(sv_kv_append_layers(&g, &layers, dk, dv, i32(a[5], "accept_idx"), i32(a[6], "n_accept"),
-                                          row_length(a[5], "accept_idx"), lens, reinterpret_cast<uint32_t *>(i32(a[8], "counters")),
-                                          f32(a[9], "reps"), stream(Py_None)));
+        const int32_t *const rows = i32(a[5], "accept_idx"), *const n_rows = i32(a[6], "n_accept");
+        const int32_t most = row_length(a[5], "accept_idx");
+        uint32_t *const counters = reinterpret_cast<uint32_t *>(i32(a[8], "counters"));
+        float *const reps = f32(a[9], "reps");
+        void *const s = stream(Py_None);
+        return status(unlocked([&] { return sv_kv_append_layers(&g, &layers, dk, dv, rows, n_rows, most, lens, counters, reps, s); }));
     });
 }
 
@@ -458,10 +521,14 @@ PyObject *accept_new(PyObject *, PyObject *const *a, Py_ssize_t n)
         }
         const auto opt = tok.options();
         at::Tensor path = at::empty({S, T}, opt), n_path = at::empty({S}, opt), next = at::empty({S}, opt);
-        const sv_status st = sv_accept((int32_t)S, (int32_t)T, (int32_t)pt.size(2), pt.data_ptr<float>(), pd.data_ptr<float>(),
-                                       tok.data_ptr<int32_t>(), i32(a[3], "parent"), f32(a[4], "u_accept"), f32(a[5], "u_next"),
-                                       path.data_ptr<int32_t>(), n_path.data_ptr<int32_t>(), next.data_ptr<int32_t>(), nullptr,
-                                       stream(Py_None));
+        const int32_t V = (int32_t)pt.size(2), *const tokens = tok.data_ptr<int32_t>(), *const parent = i32(a[3], "parent");
+        const float *const target = pt.data_ptr<float>(), *const draft = pd.data_ptr<float>();
+        const float *const u_accept = f32(a[4], "u_accept"), *const u_next = f32(a[5], "u_next");
+        void *const s = stream(Py_None);
+        const sv_status st = unlocked([&] {
+            return sv_accept((int32_t)S, (int32_t)T, V, target, draft, tokens, parent, u_accept, u_next, path.data_ptr<int32_t>(),
+                             n_path.data_ptr<int32_t>(), next.data_ptr<int32_t>(), nullptr, s);
+        });
         if (st != SV_OK) return status(st);
         return Py_BuildValue("(NNN)", THPVariable_Wrap(path), THPVariable_Wrap(n_path), THPVariable_Wrap(next));
     });
