@@ -458,7 +458,10 @@ def run_gpu(args):
     with torch.cuda.stream(stream):
         g_stack.replay()
         stream.synchronize()
-    assert torch.equal(out_h, out.cpu()), "the host-fed step did not deliver the step's outputs"
+    # (chunks of few layers are split over the SMs differently from the whole stack: the same to bf16 rounding, not bit for bit)
+    got, want = out_h.float(), out.cpu().float()
+    assert bool(torch.isfinite(got).all()) and float((got - want).norm()) <= 5e-3 * float(want.norm()), \
+        "the host-fed step did not deliver the step's outputs"
     assert int(eng.status.item()) == 0 and int(eng_reuse.status.item()) == 0 and int(eng_chain.status.item()) == 0, \
         "a kernel gave up on a bounded wait"
 
@@ -497,13 +500,17 @@ def run_gpu(args):
         "e2e": {"value": ms_e2e * 1e3 / (w.n_layers * world), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h,
                 "note": "steps one after the other (a decoding loop cannot overlap neighbouring steps: the next queries "
-                        "depend on this step's acceptance); every step is one call of SparseVerifier.verify_step_from_host: "
+                        "depend on this step's acceptance); within a step all layers' queries are there at once and the layers of "
+                        "a chunk run together, which a transformer's layers cannot (the queries of a layer depend on the output "
+                        "of the one before), so this is not `value`, which goes layer by layer, plus the copies: that is "
+                        "one_stream_value; every step is one call of SparseVerifier.verify_step_from_host: "
                         "Q and draft K/V of all layers from pinned host memory, the step, the outputs back to pinned host "
                         "memory, the copies in two chunks of layers, in the background so that all but the first upload "
                         "and the last download run under the step's kernels; the KV cache is device-resident state",
                 "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "7/16, 9/16 of the layers",
                 "one_stream_value": ms_e2e_one_stream * 1e3 / (w.n_layers * world),
-                "one_stream_note": "the same bytes copied whole before and after the step on the step's own stream",
+                "one_stream_note": "the step layer by layer, as in `value`, with the same bytes copied whole before and after it on "
+                                   "its own stream",
                 "pipelined_value": ms_e2e_pipelined * 1e3 / (w.n_layers * world),
                 "pipelined_note": "the same copies with two buffer sets and three streams, so that the copies of steps "
                                   "i+1 / i-1 run under the kernels of step i (an upper bound no real loop reaches)"},
