@@ -1390,10 +1390,10 @@ def test_accept_fuzz(sv):
 
 
 def test_benchmark_step_under_cuda_graph_replay(sv):
-    """The launch configuration the benchmark times: a stack of full-size cfg1 layers with their pools in one
-    allocation, one step (tail refresh of all layers in one launch, then select + attention + merge per layer, chained
-    with programmatic dependent launch) captured in a CUDA graph and replayed.  Every layer's output after the third
-    replay against the oracle on sampled rows; the last layer's block list exact."""
+    """verify_step of a stack of full-size cfg1 layers with their pools in one allocation (tail refresh, selection and
+    attention of all layers in a launch each, chained with programmatic dependent launch), captured in a CUDA graph and
+    replayed: the benchmark's all-at-once figure.  Its step layer by layer is in test_steps_against_oracle.  Every layer's output
+    after the third replay against the oracle on sampled rows; the last layer's block list exact."""
     n_layers = 3
     w = si.shrink(si.WORKLOADS["cfg1"], n_layers=n_layers)
     geom = si.make_geometry(w)
