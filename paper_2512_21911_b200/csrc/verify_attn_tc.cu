@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t *anc32 = reinterpret_cast<uint32_t *>(misc + 320);                     // [32] the same, up to 32 draft tokens
     volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 448);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + 456);
-    // the ring units the producer requests and the first of them; (kBal) a RingCopies
+    // where the producer stopped requesting, ~0: nowhere; (kBal) a RingCopies
     volatile uint32_t *requested = reinterpret_cast<volatile uint32_t *>(misc + 464);
     // (kBal) the masks of odd segments (64-bit: anc + 64), the segment descriptors, the claims on their way to warp 11
     uint32_t *anc32_odd = reinterpret_cast<uint32_t *>(misc + 1536);
@@ -158,8 +158,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
     // Registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168).  At 232 / 40 the roles of the third spill
     // inside their loops (16 sequences of 4-16K: 34.5 us a layer, 34.1 at 208 / 88; dense 32K 29.5 and 28.8; one 240-row tree 24.3
-    // and 23.9); the softmax needs no more than 208 in any form.  The roles of a balanced launch keep track of more.
-    constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : 208, kRegsFew = 504 - 2 * kRegsMany;
+    // and 23.9); the softmax needs no more than 208 in any form.  Up to 32 rows 56 do for the roles: a layer of a 32K context 14.59 us
+    // (selection, attention, merge) at 224 / 56, 14.63-14.69 at 208 / 88.  The roles of a balanced launch keep track of more.
+    constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : NH == 1 ? 224 : 208, kRegsFew = 504 - 2 * kRegsMany;
     constexpr int OFFQ = NS * kStageBytes;                   // the Q tile (kPair: of warpgroup 0; warpgroup 1's follows)
     // blockIdx.x = split * groups + group: the CTAs that gather the same slice of the blocks are neighbours in the grid
     // (they share those K/V tiles through L2; 1-2 % faster than group-major order).  A group is a row tile (kWide), or
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(bar(lane), count);
             mbar_fence_init();
         }
-        if (lane == 0) *abort_flag = 0, requested[0] = 0, requested[1] = 0;
+        if (lane == 0) *abort_flag = 0, requested[0] = kBal ? 0u : ~0u, requested[1] = 0;
         __syncwarp();
         if constexpr (!kBal) named_bar_arrive(3, kThreads);
     } else if constexpr (kBal) {
@@ -450,7 +451,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int u0 = slice_begin(split, n_sel), u1 = slice_begin(split + 1, n_sel);
             const int j0 = kUnitSlices ? u0 >> 1 : u0, j1 = kUnitSlices ? (u1 + 1) >> 1 : u1;
             const int off = has_draft ? 1 : 0;
-            if (lane == 0) requested[0] = (kUnitSlices ? u1 - u0 : (j1 - j0) * upb) + off, requested[1] = off;
             bool dead = false;
             for (int base = j0; base < j1; base += 32) {
                 const int j = base + lane;
@@ -675,8 +675,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if (p.status) atomicOr(p.status, 16);
                     }
                     if (*abort_flag) {
-                        const RingCopies copies = kBal ? RingCopies{requested[0], requested[1]}
-                                                       : copies_of_units((int)requested[1], (int)requested[0], NS);
+                        const uint32_t word = requested[0];
+                        const RingCopies copies = kBal ? RingCopies{word, requested[1]}
+                                                       : copies_of_units(has_draft ? 1 : 0, word == ~0u ? n_total : (int)word, NS);
                         for (int stage = 0; stage < NS; ++stage)
                             if (copies.waits_for(stage) && !mbar_wait_bounded(bar(kFull + stage), copies.parity(stage), kLongWait) && p.status)
                                 atomicOr(p.status, 1);
