@@ -110,7 +110,7 @@ struct ClaimWords {
 // than SMs).  Between two lists nothing drains: the TMA ring runs on into the next list, and warp 11 has that list's Q
 // tile, masks and draft K/V in shared memory by the time the warpgroups have written the last one's rows.  With one CTA
 // per list every list after an SM's first begins with an empty ring, 3 to 4 us of latencies for 45 us of HBM time (32 layers
-// of 8 lists of 65 units: 112.6 -> 108.8 us per step; 64 x 8 lists of 49 units: 155.7 -> 146.0).  Cutting lists so that all CTAs
+// of 8 lists of 65 units: 112.5 -> 106.9 us per step; 64 x 8 lists of 49 units: 155.7 -> 143.6).  Cutting lists so that all CTAs
 // end together costs more than it gains: the CTAs that are left have the HBM bandwidth to themselves, and partials have
 // to be written and merged (117 and 149 us).
 template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal>
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         return false;
     };
 
-    static_assert(!kBal || NH < 4, "lists are handed out for tiles of up to 64 rows");
+    static_assert(!kBal || (kStack && NH < 4), "lists are handed out for stacks, in tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
     // 128-row tiles are bound by the tensor pipe when every MMA fetches both operands from shared memory (S = Q K^T: eight
     // 128 x 64 x 16 MMAs, each re-reading 4 KB of Q), so their Q lives in tensor memory (A operand from TMEM), and with a
@@ -159,7 +159,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168).  At 232 / 40 the roles of the third spill
     // inside their loops (16 sequences of 4-16K: 34.5 us a layer, 34.1 at 208 / 88; dense 32K 29.5 and 28.8; one 240-row tree 24.3
     // and 23.9); the softmax needs no more than 208 in any form.  Up to 32 rows 56 do for the roles: a layer of a 32K context 14.59 us
-    // (selection, attention, merge) at 224 / 56, 14.63-14.69 at 208 / 88.  The roles of a balanced launch keep track of more.
+    // (selection, attention, merge) at 224 / 56, 14.63-14.69 at 208 / 88.  A balanced launch's roles keep
+    // track of more: 200 / 104 up to 32 rows (no spills; 192 and 208 the same within 0.3 %), else 208 / 88 (40 rows of 40 draft tokens, a
+    // stack of 12 layers x 2 sequences: 123 us, 129 at 200 and at 216, 131 at 192; 56 and 64 rows the same at 200 to 216).
     constexpr int kRegsMany = kBal ? (NH == 2 ? 208 : 200) : NH == 1 ? 224 : 208, kRegsFew = 504 - 2 * kRegsMany;
     constexpr int OFFQ = NS * kStageBytes;                   // the Q tile (kPair: of warpgroup 0; warpgroup 1's follows)
     // blockIdx.x = split * groups + group: the CTAs that gather the same slice of the blocks are neighbours in the grid
@@ -249,10 +251,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         int z, h, s, lz, l;
     };
     auto item_at = [&](int i) {
-        Item it;
-        it.z = i / p.Hkv, it.h = i - it.z * p.Hkv;
-        it.s = it.z, it.lz = it.z, it.l = 0;
-        if constexpr (kStack) {
+        Item it = {};
+        if constexpr (kStack) {   // (a single layer's parameters have neither S nor list_of)
+            it.z = i / p.Hkv, it.h = i - it.z * p.Hkv;
             it.l = it.z / p.S;
             it.s = it.z - it.l * p.S;
             it.lz = p.list_of[it.l] * p.S + it.s;
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int sh = upb - 1;   // units of a block: 1 << sh
                 bool dead = false;
                 RingCopies copies;   // (lane 0's)
-                if (!p.early_gather) grid_dependency_wait();   // the lists may come from the kernel just before
+                grid_dependency_wait();   // the lists may come from the kernel just before
                 // A batch is 32 consecutive entries of one list, one per lane.  What the next segment needs -- its claim, count
                 // and first entries, their pages: three trips to L2, each needing the one before -- is fetched in steps
                 // between this segment's requests.
@@ -313,15 +314,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // a negative count marks a list that block selection could not produce: attend over the draft tokens
                     // only, and say so
                     if (p.sel_idx && count < 0 && lane == 0 && p.status) atomicOr(p.status, kStatusNoList);
-                    if constexpr (kStack) {
-                        if (cur.l != layer_at) {
-                            mk = &p.layers[cur.l].k_map, mv = &p.layers[cur.l].v_map;
-                            n_pages = p.layers[cur.l].n_pages;
-                            layer_at = cur.l;
-                            if (lane == 0) {
-                                tensormap_acquire(mk);
-                                tensormap_acquire(mv);
-                            }
+                    if (cur.l != layer_at) {
+                        mk = &p.layers[cur.l].k_map, mv = &p.layers[cur.l].v_map;
+                        n_pages = p.layers[cur.l].n_pages;
+                        layer_at = cur.l;
+                        if (lane == 0) {
+                            tensormap_acquire(mk);
+                            tensormap_acquire(mv);
                         }
                     }
                     int count_next = 0, L_next = 0, blk_next = 0, page_next = 0, step = 0;
