@@ -387,8 +387,8 @@ SV_API sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, const 
  * draft_k / draft_v [L][S][T][Hkv][D], reps [L][S][Hkv][NBmax][D] -- and layers first <= l < end are processed.
  * anchors (host, uint8 [L], anchors[0] != 0): the layers that select; lists are numbered by anchor,
  * idx [A][S][Hkv][max_sel], cnt [A][S][Hkv], and a layer attends over the list of the last anchor up to it.
- * Results are those of the single-layer calls; the splits of the attention are chosen for the whole stack, so that a
- * layer's result does not depend on the layers it is launched with.
+ * Lists, representatives and cache rows are those of the single-layer calls; attention outputs are, to bf16 rounding.  The splits of the
+ * attention are chosen for the whole stack: a layer's result depends on n_layers, not on the layers it is launched with.
  *   sv_block_reps_layers   layers l with which[l] != 0 (host, uint8 [L]; NULL: all)
  *   sv_verify_attn_layers  sel_idx == NULL: dense verification (anchors may be NULL); workspace of
  *                          sv_workspace_bytes_layers(geom, n_layers, max_sel) bytes.  The first SV_STACK_STATE_BYTES of them
