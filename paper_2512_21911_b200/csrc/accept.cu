@@ -1,23 +1,26 @@
 // Acceptance of the draft tokens after verification (Section 2.1, Eq. 2-3), chains and trees.
 //
 // One thread-block cluster per sequence; the vocabulary is split into contiguous ranges, one per CTA, and
-// inside a CTA into contiguous segments, one per thread.  Every CTA runs the same walk from the root (row 0):
+// inside a CTA into contiguous ranges, one per warp, whose lanes read neighbouring 16-byte words.  Every CTA runs the same
+// walk from the root (row 0):
 // a child c of the current row with token x is accepted when u_accept[c] < min(1, p(x) / q(x)) (Eq. 2); a
 // rejected child replaces p by norm(max(0, p - q)) (Eq. 3), which is never materialised: after k rejections at
 // a row, p_k(y) follows from p_target(y), q(y) and the k normalisers Z_1..Z_k by k subtract-clamp-scale steps.
-// Each normaliser is one pass over the vocabulary: per-thread segment sums, a block reduction in fixed order,
-// CTA totals exchanged through distributed shared memory, one hardware cluster barrier.  All CTAs add the
+// Each normaliser is one pass over the vocabulary: sums per thread, per warp and per CTA in a fixed order, CTA totals
+// exchanged through distributed shared memory, one hardware cluster barrier.  All CTAs add the
 // totals in the same order, so every CTA takes the same decisions.  The next token is drawn by inverting the
-// cumulative sum of the final p in vocabulary order: CTA totals -> the CTA that holds the target, block scan
-// of its thread sums -> the thread, a sequential walk of that thread's segment -> the token.
+// cumulative sum of the final p in vocabulary order: CTA totals -> the CTA that holds the target, warp totals -> the warp,
+// a scan over that warp's words -> the token.  Behind the rejection of a row's last child the residual's own pass serves the
+// draw too: max(0, p - q) is drawn from as it is, against u_next * Z.
 // fp32 throughout; no spin-waits (cluster barriers only).
 //
-// A chain of latencies, not of bytes (a row of both distributions is 128 KB per CTA at a vocabulary of 128256): the
-// acceptance probabilities of all children are fetched together ahead of the walk, so the walk itself waits for nothing
-// until a rejection, and a row's range is copied once into shared memory (coalesced, asynchronous) for all of its passes --
-// every rejection, the sum and the draw -- laid out so that the threads' segments, of which each is read by one thread,
-// start in different banks.  Read from global memory in every pass, segment by segment, chains of 8 took
-// 18.1 us where they now take 13.9 us (one sequence, vocabulary 128256; 15.8 and 14.9 us at 151936).
+// A chain of latencies, not of bytes (64 KB of both distributions per CTA and row at a vocabulary of 128256): the
+// acceptance probabilities of all children are fetched together ahead of the walk, so the walk itself -- ballots over rows that lie
+// in the lanes -- waits for nothing until a rejection, and a row's range is loaded once, straight into registers, for all of its
+// passes.  The rest is the code itself, which every launch fetches anew: one place for the pass, and as little as possible
+// between its trips (a second copy of it and a walk of ballots cost 2 us).  One sequence of 8 rows, vocabulary 128256: 4.8 us on the
+// device (12 when a row's range went to shared memory and every pass was followed by another for the draw); four
+// sequences behind an attention launch, nothing in L2: 6.7 us (17).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -32,8 +35,8 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRows = 64;     // draft rows per step (the ancestor masks of the attention kernel are 64 bits)
-constexpr int kMaxCluster = 8;
-constexpr int kMaxStagedBytes = 2 * kThreads * 13 * 16;   // 13 words of either distribution per thread: 208 KB
+constexpr int kMaxCluster = 16;
+constexpr int kMaxHeld = 8;      // words of either distribution that a thread holds (64 registers)
 
 struct AcceptParams {
     const float *p_target;   // [S][T][V]
@@ -46,224 +49,284 @@ struct AcceptParams {
     int32_t *n_path;         // [S]
     int32_t *next_token;     // [S]
     float *alpha;            // [S][T] or nullptr
-    int T, V, chunk, seg;    // chunk: vocabulary entries per CTA, seg: per thread (multiples of 4)
+    int T, V;
+    int batches;             // batches of NW words per thread that make up a CTA's range
 };
 
-// p after `r` rejections at the current row, at one vocabulary entry
-__device__ __forceinline__ float adjusted(float pt, float q, int r, const float *inv_z)
-{
-    float v = pt;
-    for (int k = 0; k < r; ++k) v = fmaxf(v - q, 0.f) * inv_z[k];
-    return v;
-}
+// p(y) after another rejection: norm(max(0, p - q)), Z^-1 = inv_z
+__device__ __forceinline__ float rejected(float p, float q, float inv_z) { return fmaxf(p - q, 0.f) * inv_z; }
+__device__ __forceinline__ float alpha_of(float px, float qx) { return (qx <= 0.f || px >= qx) ? 1.f : __fdiv_rn(px, qx); }   // Eq. 2
 
-// Weight of entry y in the current pass: kResidual ? max(0, p_r - q) : p_r
-template <bool kResidual>
-__device__ __forceinline__ float weight(float pt, float q, int r, const float *inv_z)
+// The part of a running sum that the target falls into: lane l holds part l (0: not there).  Returns the lane, -1 when there is no mass;
+// `ahead` grows by the parts before it.  Rounding may leave the target just above the total: then the last part with mass.
+__device__ __forceinline__ int part_of(float t, float target, float &ahead)
 {
-    const float v = adjusted(pt, q, r, inv_z);
-    return kResidual ? fmaxf(v - q, 0.f) : v;
-}
-
-// One thread's segment of a row of both distributions, four entries at a time: in global memory, or (kStaged) in the CTA's
-// copy, where a segment is `pad` 16-byte words after the one before.
-struct Segment {
-    const float4 *pt, *q;
-    int n;   // words
-};
-
-// Sum of a segment in vocabulary order.
-template <bool kResidual>
-__device__ __forceinline__ float segment_sum(const Segment &sg, int r, const float *inv_z)
-{
-    float acc = 0.f;
-#pragma unroll 4
-    for (int i = 0; i < sg.n; ++i) {
-        const float4 a = sg.pt[i], b = sg.q[i];
-        acc += weight<kResidual>(a.x, b.x, r, inv_z);
-        acc += weight<kResidual>(a.y, b.y, r, inv_z);
-        acc += weight<kResidual>(a.z, b.z, r, inv_z);
-        acc += weight<kResidual>(a.w, b.w, r, inv_z);
-    }
-    return acc;
-}
-
-// Inclusive prefix of `v` over the CTA in thread order (fixed association); total returned through `total`.
-__device__ __forceinline__ float block_inclusive_scan(float v, float *warp_tot, float &total)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float inc = v;
+    const int lane = threadIdx.x & 31;
+    float inc = t;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
+    for (int o = 1; o < 16; o <<= 1) {
+        const float v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
     }
-    __syncthreads();   // warp_tot of the previous scan has been consumed
-    if (lane == 31) warp_tot[warp] = inc;
-    __syncthreads();
-    float before = 0.f, tot = 0.f;
-    for (int w = 0; w < kWarps; ++w) {
-        if (w == warp) before = tot;
-        tot += warp_tot[w];
-    }
-    total = tot;
-    return before + inc;
+    const unsigned hit = __ballot_sync(0xffffffffu, t > 0.f && ahead + inc >= target), any = __ballot_sync(0xffffffffu, t > 0.f);
+    if (!any) return -1;
+    const int at = hit ? __ffs(hit) - 1 : 31 - __clz(any);
+    ahead += __shfl_sync(0xffffffffu, inc - t, at);
+    return at;
 }
 
-// kStaged: a row's range fits in shared memory (vocabularies of up to 212992).
-template <bool kStaged>
+// NW: 16-byte words of either distribution that a thread holds.  kHeld: they are its whole share of a row (one batch);
+// otherwise a pass loads batch after batch.
+template <int NW, bool kHeld>
 __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank(), CL = (int)cluster.num_blocks();
-    const int s = blockIdx.y, tid = threadIdx.x;
-    __shared__ int par[kMaxRows];
-    __shared__ float u[kMaxRows], px_of[kMaxRows], qx_of[kMaxRows];   // px, qx: a child's token in its parent's row
-    extern __shared__ float4 staged[];                                // [2][kThreads][pad]
+    const int s = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ int par_of[kMaxRows];
+    __shared__ float u_of[kMaxRows], px_of[kMaxRows], qx_of[kMaxRows];   // px, qx: a child's token in its parent's row
+    __shared__ unsigned first_child[kMaxRows];   // 2 c: the row's first child is c and accepted; 2 c + 1: rejected
     __shared__ float inv_z[kMaxRows];
-    __shared__ float warp_tot[kWarps];
+    __shared__ float warp_tot[2][kWarps];
     __shared__ float cta_tot[2][kMaxCluster];   // totals of all CTAs, written by their owners; two buffers in turn
-    __shared__ int s_first, s_last;
 
+    if (tid < kMaxRows) first_child[tid] = ~0u;
+    if (tid < 2 * kMaxCluster) (&cta_tot[0][0])[tid] = 0.f;   // (clusters of fewer CTAs)
     svk::cluster_arrive();
+    __syncthreads();
     svk::grid_dependency_wait();
     svk::grid_launch_dependents();
-    if (tid < p.T) {
-        const int x = min(max(p.tokens[(size_t)s * p.T + tid], 0), p.V - 1);
-        const int row = p.parent ? p.parent[(size_t)s * p.T + tid] : tid - 1;
-        par[tid] = row;
-        u[tid] = p.u_accept[(size_t)s * p.T + tid];
-        if (row >= 0 && row < tid) {   // (a row that follows is never reached from it)
-            const size_t at = ((size_t)s * p.T + row) * p.V + x;
-            px_of[tid] = __ldg(p.p_target + at), qx_of[tid] = __ldg(p.p_draft + at);
+    if (tid < kMaxRows) {
+        int row = -1;
+        float u = 0.f, px = 0.f, qx = 0.f;
+        if (tid < p.T) {
+            const int x = min(max(p.tokens[(size_t)s * p.T + tid], 0), p.V - 1);
+            row = p.parent ? p.parent[(size_t)s * p.T + tid] : tid - 1;
+            u = p.u_accept[(size_t)s * p.T + tid];
+            if (row >= 0 && row < tid) {   // (a row that follows is never reached from it)
+                const size_t at = ((size_t)s * p.T + row) * p.V + x;
+                px = __ldg(p.p_target + at), qx = __ldg(p.p_draft + at);
+                atomicMin(&first_child[row], 2u * tid + (u < alpha_of(px, qx) ? 0u : 1u));
+            } else {
+                row = -1;
+            }
         }
+        par_of[tid] = row, u_of[tid] = u, px_of[tid] = px, qx_of[tid] = qx;
     }
     const float u_next = p.u_next[s];
     __syncthreads();
     svk::cluster_wait();   // every CTA of the cluster is running: its shared memory may be written from here on
 
-    const int lo = min(p.V, rank * p.chunk), hi = min(p.V, lo + p.chunk);
-    const int y0 = min(hi, lo + tid * p.seg), y1 = min(hi, y0 + p.seg);
     const bool writer = rank == 0 && tid == 0;
-    int n_red = 0;
-
-    // total over the cluster of the CTAs' sums; leaves the per-CTA sums in cta_tot[buf]
-    auto cluster_total = [&](float cta_sum, int &buf) {
-        buf = n_red & 1;
-        ++n_red;
-        if (tid < CL) *cluster.map_shared_rank(&cta_tot[buf][rank], tid) = cta_sum;
-        cluster.sync();
-        float t = 0.f;
-        for (int c = 0; c < CL; ++c) t += cta_tot[buf][c];
-        return t;
-    };
-
-    int cur = 0, n = 1, r = 0, buf = 0;
-    if (writer) p.path[(size_t)s * p.T] = 0;
-    int at_hand = -1;   // the row in shared memory
-    auto segment_of = [&](int row) -> Segment {
-        const float4 *pt = reinterpret_cast<const float4 *>(p.p_target + ((size_t)s * p.T + row) * p.V + lo);
-        const float4 *q = reinterpret_cast<const float4 *>(p.p_draft + ((size_t)s * p.T + row) * p.V + lo);
-        if constexpr (kStaged) {
-            const int seg4 = p.seg >> 2, pad = seg4 | 1, words = (hi - lo) >> 2;
-            if (row != at_hand) {
-                __syncthreads();   // the row before has been read
-                for (int i = tid; i < words; i += kThreads) {
-                    const int t = i / seg4, at = t * pad + (i - t * seg4);
-                    svk::cp_async_16(svk::smem_u32(staged + at), pt + i);
-                    svk::cp_async_16(svk::smem_u32(staged + kThreads * pad + at), q + i);
-                }
-                svk::cp_async_wait_all();
-                __syncthreads();
-                at_hand = row;
-            }
-            return {staged + tid * pad, staged + (kThreads + tid) * pad, (y1 - y0) >> 2};
-        } else {
-            return {pt + ((y0 - lo) >> 2), q + ((y0 - lo) >> 2), (y1 - y0) >> 2};
+    const int batches = kHeld ? 1 : p.batches;
+    const int words = p.V >> 2, word0 = (rank * kWarps + warp) * batches * NW * 32 + lane;   // this lane's first word
+    int cur = 0, n = 1;   // the current row, rows on the path
+    int r = 0;            // rejections at the current row
+    float4 pt[NW], q[NW];
+    auto load = [&](int batch) {
+        const float4 *a = reinterpret_cast<const float4 *>(p.p_target + ((size_t)s * p.T + cur) * p.V);
+        const float4 *b = reinterpret_cast<const float4 *>(p.p_draft + ((size_t)s * p.T + cur) * p.V);
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+            const int w = word0 + (batch * NW + i) * 32;
+            const bool in = w < words;
+            pt[i] = in ? __ldg(a + w) : make_float4(0.f, 0.f, 0.f, 0.f);
+            q[i] = in ? __ldg(b + w) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     };
+    int at_hand = -1, applied = 0;   // (kHeld) the row in registers, and how many of its rejections they have seen
+    // The words of a batch, as p after r rejections.
+    auto fetch = [&](int batch) {
+        if (!kHeld || at_hand != cur) {
+            load(batch);
+            at_hand = cur, applied = 0;
+        }
+        for (; applied < r; ++applied) {
+            const float iz = inv_z[applied];
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                pt[i].x = rejected(pt[i].x, q[i].x, iz), pt[i].y = rejected(pt[i].y, q[i].y, iz);
+                pt[i].z = rejected(pt[i].z, q[i].z, iz), pt[i].w = rejected(pt[i].w, q[i].w, iz);
+            }
+        }
+    };
+    bool residual = false;   // the weights of the last pass: max(0, p - q), else p
+    auto weights = [&](int i) {
+        const float4 a = pt[i], b = q[i];
+        return residual ? make_float4(fmaxf(a.x - b.x, 0.f), fmaxf(a.y - b.y, 0.f), fmaxf(a.z - b.z, 0.f), fmaxf(a.w - b.w, 0.f)) : a;
+    };
+
+    // The walk.  First along first children that are accepted (no other is tried, and nothing but the table is needed) ...
+    if (writer) p.path[(size_t)s * p.T] = 0;
+    if (!p.alpha) {
+        for (unsigned next; !((next = first_child[cur]) & 1);) {
+            cur = (int)(next >> 1);
+            if (writer) p.path[(size_t)s * p.T + n] = cur;
+            ++n;
+        }
+    }
+    // ... then child by child, in row order: lane l holds rows l and 32 + l.
+    const int par_lo = par_of[lane], par_hi = par_of[32 + lane];
+    auto children = [&] {
+        const unsigned a = __ballot_sync(0xffffffffu, par_lo == cur), b = __ballot_sync(0xffffffffu, par_hi == cur);
+        return (unsigned long long)b << 32 | a;
+    };
+    unsigned long long left = children();
+    int n_pass = 0;
+    float W;   // total of the last pass's weights
     for (;;) {
-        r = 0;
-        bool moved = false;
-        for (int c = cur + 1; c < p.T; ++c) {
-            if (par[c] != cur) continue;
+        residual = false;
+        while (left) {
+            const int c = __ffsll(left) - 1;
+            left &= left - 1;
             const float qx = qx_of[c];
-            const float px = adjusted(px_of[c], qx, r, inv_z);
-            const float a = (qx <= 0.f || px >= qx) ? 1.f : __fdiv_rn(px, qx);   // Eq. 2
+            float px = px_of[c];
+            for (int k = 0; k < r; ++k) px = rejected(px, qx, inv_z[k]);
+            const float a = alpha_of(px, qx);
             if (writer && p.alpha) p.alpha[(size_t)s * p.T + c] = a;
-            if (u[c] < a) {
-                if (writer) p.path[(size_t)s * p.T + n] = c;
-                ++n;
-                cur = c;
-                moved = true;
+            if (!(u_of[c] < a)) {
+                residual = true;   // rejected: Z = sum_y max(0, p - q) (Eq. 3); p itself is never stored
                 break;
             }
-            // rejected: Z = sum_y max(0, p - q) (Eq. 3); p itself is never stored
-            float tot;
-            block_inclusive_scan(segment_sum<true>(segment_of(cur), r, inv_z), warp_tot, tot);
-            const float z = cluster_total(tot, buf);
-            if (z > 0.f) {   // a residual without mass (p == q) leaves p as it is
-                if (tid == 0) inv_z[r] = __frcp_rn(z);
-                ++r;
-                __syncthreads();
+            if (writer) p.path[(size_t)s * p.T + n] = c;
+            ++n;
+            cur = c, r = 0;
+            left = children();
+        }
+        // one pass over the row: the total over the cluster; the CTAs' sums stay in cta_tot, this CTA's warps' in warp_tot
+        float sum = 0.f;
+        for (int batch = 0; batch < batches; ++batch) {
+            fetch(batch);
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const float4 w = weights(i);
+                sum += (w.x + w.y) + (w.z + w.w);
             }
         }
-        if (!moved) break;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        const int buf = n_pass++ & 1;
+        if (lane == 0) warp_tot[buf][warp] = sum;
+        __syncthreads();
+        if (warp == 0) {
+            float t = warp_tot[buf][lane & (kWarps - 1)];
+#pragma unroll
+            for (int o = kWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane < CL) *cluster.map_shared_rank(&cta_tot[buf][rank], lane) = t;
+        }
+        cluster.sync();
+        W = cta_tot[buf][lane & (kMaxCluster - 1)];
+#pragma unroll
+        for (int o = kMaxCluster / 2; o > 0; o >>= 1) W += __shfl_xor_sync(0xffffffffu, W, o);
+        if (!residual) break;
+        if (W > 0.f) {   // a residual without mass (p == q) leaves p as it is
+            if (!left) break;   // nothing else is tried: the draw is from this residual
+            if (tid == 0) inv_z[r] = __frcp_rn(W);
+            ++r;
+            __syncthreads();
+        }
     }
     if (writer) {
         p.n_path[s] = n;
         for (int i = n; i < p.T; ++i) p.path[(size_t)s * p.T + i] = -1;
     }
 
-    // next token: the smallest x with  sum_{y <= x} p(y) >= u_next * sum_y p(y)  and p(x) > 0
-    const Segment mine = segment_of(cur);
-    float tot;
-    const float sum = segment_sum<false>(mine, r, inv_z);
-    const float inc = block_inclusive_scan(sum, warp_tot, tot);
-    const float W = cluster_total(tot, buf);
+    // next token: the smallest x with  sum_{y <= x} w(y) >= u_next * sum_y w(y)  and w(x) > 0
+    const int buf = (n_pass - 1) & 1;
     const float target = u_next * W;
-    int owner = -1, last_pos = -1;
-    float before = 0.f, before_last = 0.f, run = 0.f;
-    for (int c = 0; c < CL; ++c) {
-        const float t = cta_tot[buf][c];
-        if (t > 0.f) {
-            if (owner < 0 && run + t >= target) owner = c, before = run;
-            last_pos = c, before_last = run;
-        }
-        run += t;
-    }
-    if (owner < 0) owner = last_pos, before = before_last;   // rounding left the target just above the total
-    if (owner < 0) {                                         // no mass anywhere
+    float before = 0.f;
+    const int owner = part_of(lane < kMaxCluster ? cta_tot[buf][lane] : 0.f, target, before);
+    if (owner < 0) {   // no mass anywhere
         if (writer) p.next_token[s] = p.V - 1;
         return;
     }
     if (rank != owner) return;
-    const float local = target - before;
-    if (tid == 0) s_first = kThreads, s_last = -1;
-    __syncthreads();
-    if (sum > 0.f) {
-        if (inc >= local) atomicMin(&s_first, tid);
-        atomicMax(&s_last, tid);
-    }
-    __syncthreads();
-    const int chosen = s_first < kThreads ? s_first : s_last;
-    if (tid != chosen) return;
-    float acc = inc - sum;
-    int pick = -1, last_y = -1;
-    for (int i = 0; i < mine.n && pick < 0; ++i) {
-        const float4 a = mine.pt[i], b = mine.q[i];
-        const float w[4] = {weight<false>(a.x, b.x, r, inv_z), weight<false>(a.y, b.y, r, inv_z), weight<false>(a.z, b.z, r, inv_z),
-                            weight<false>(a.w, b.w, r, inv_z)};
+    if (warp != part_of(lane < kWarps ? warp_tot[buf][lane] : 0.f, target, before)) return;
+    int last = -1;   // the last entry with mass that this lane has seen
+    for (int batch = 0; batch < batches; ++batch) {
+        if (!kHeld) fetch(batch);
+        float sum[NW], inc[NW];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            acc += w[e];
-            if (w[e] > 0.f && pick < 0) {
-                last_y = y0 + 4 * i + e;
-                if (acc >= local) pick = last_y;
+        for (int i = 0; i < NW; ++i) {
+            const float4 w = weights(i);
+            inc[i] = sum[i] = (w.x + w.y) + (w.z + w.w);
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const float t = __shfl_up_sync(0xffffffffu, inc[i], o);
+                if (lane >= o) inc[i] += t;
             }
+        // the first word whose scan reaches the target; its lane finds the entry
+        bool found = false;
+        float4 at_word = make_float4(0.f, 0.f, 0.f, 0.f);
+        float ahead = 0.f;
+        int y = 0;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+            const float4 w = weights(i);
+            const unsigned hit = __ballot_sync(0xffffffffu, sum[i] > 0.f && before + inc[i] >= target);
+            const int y_i = 4 * (word0 + (batch * NW + i) * 32);
+            if (!found && sum[i] > 0.f) last = w.w > 0.f ? y_i + 3 : w.z > 0.f ? y_i + 2 : w.y > 0.f ? y_i + 1 : y_i;
+            if (!found && hit) {
+                found = true;
+                if (lane == __ffs(hit) - 1) at_word = w, ahead = before + (inc[i] - sum[i]), y = y_i;
+                else last = -1;
+            }
+            before += __shfl_sync(0xffffffffu, inc[i], 31);
+        }
+        if (found) {
+            if (last >= 0) {
+                const float r0 = ahead + at_word.x, r1 = r0 + at_word.y, r2 = r1 + at_word.z;
+                p.next_token[s] = at_word.x > 0.f && r0 >= target ? y : at_word.y > 0.f && r1 >= target ? y + 1
+                                : at_word.z > 0.f && r2 >= target ? y + 2 : last;
+            }
+            return;
         }
     }
-    p.next_token[s] = pick >= 0 ? pick : last_y;
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (lane == 0) p.next_token[s] = last;
+}
+
+template <int NW = 1>
+const void *accept_fn(int held)   // kernel for `held` words per thread; more than kMaxHeld: several batches
+{
+    if constexpr (NW <= kMaxHeld) {
+        return held <= NW ? reinterpret_cast<const void *>(accept_kernel<NW, true>) : accept_fn<NW + 1>(held);
+    } else {
+        return reinterpret_cast<const void *>(accept_kernel<kMaxHeld, false>);
+    }
+}
+
+// How many clusters of 16 CTAs of the kernel this device holds at once (asked once per device; more than the portable size).
+int clusters_of_16(const void *fn, int held)
+{
+    static std::atomic<int> known[svh::kMaxDevices][kMaxHeld + 2];   // the number + 1; 0: not asked
+    const int dev = svh::current_device();
+    if (dev < 0 || dev >= svh::kMaxDevices) return 0;
+    std::atomic<int> &at = known[dev][held <= kMaxHeld ? held : kMaxHeld + 1];
+    int v = at.load(std::memory_order_acquire);
+    if (v == 0) {
+        int n = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(16, 1);
+            cfg.blockDim = dim3(kThreads);
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 16;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) n = 0;
+        }
+        (void)cudaGetLastError();   // a refusal is an answer, not an error of the call that asked
+        v = n + 1;
+        at.store(v, std::memory_order_release);
+    }
+    return v - 1;
 }
 
 }  // namespace
@@ -277,14 +340,20 @@ extern "C" sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, co
     if (n_draft < 1) return SV_ERR_SHAPE;
     if (n_draft > kMaxRows) return SV_ERR_UNSUPPORTED;
     if (vocab % 4 != 0 || !svh::aligned(p_target, 16) || !svh::aligned(p_draft, 16)) return SV_ERR_ALIGN;
+    // At least 4096 entries per CTA (2048: the same within 1 %).  Clusters of 16 while the device holds them all at once: with an
+    // L2 full of other data, one sequence of 128256 entries takes 10.3 us, 12.2 in a cluster of 8 (151936: 10.2 and 14.3); 8
+    // sequences, for which there is not room, 16.4 and 12.4.
     int CL = 1;
-    while (CL < kMaxCluster && vocab / (CL * 2) >= 4096) CL *= 2;   // at least 4096 entries per CTA
+    while (CL < 8 && vocab / (CL * 2) >= 4096) CL *= 2;
+    const auto held_by = [&](int ctas) { return (vocab / 4 + ctas * kThreads - 1) / (ctas * kThreads); };   // words per thread
+    if (CL == 8 && vocab / 16 >= 4096 && n_seq <= clusters_of_16(accept_fn(held_by(16)), held_by(16))) CL = 16;
+    const int held = held_by(CL);
+    const void *fn = accept_fn(held);
     AcceptParams p;
     p.p_target = p_target, p.p_draft = p_draft, p.tokens = tokens, p.parent = parent, p.u_accept = u_accept;
     p.u_next = u_next, p.path = path, p.n_path = n_path, p.next_token = next_token, p.alpha = alpha;
     p.T = n_draft, p.V = vocab;
-    p.chunk = ((vocab / 4 + CL - 1) / CL) * 4;
-    p.seg = ((p.chunk / 4 + kThreads - 1) / kThreads) * 4;
+    p.batches = (held + kMaxHeld - 1) / kMaxHeld;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CL, n_seq);
     cfg.blockDim = dim3(kThreads);
@@ -297,17 +366,7 @@ extern "C" sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, co
     svh::pdl_attribute(attr + 1);
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const size_t bytes = (size_t)2 * kThreads * ((p.seg >> 2) | 1) * sizeof(float4);
-    // (one CTA per SM then: launches that would fill the GPU keep the form of which three fit an SM -- 16 sequences at a
-    // vocabulary of 151936: 24.6 against 26.9 us)
-    const bool staged = bytes <= kMaxStagedBytes && (2 * bytes <= kMaxStagedBytes || 3 * CL * n_seq <= 2 * svh::sm_count());
-    if (staged) {
-        static svh::OncePerDevice once;   // function attributes belong to a device
-        if (once.run([] { return cudaFuncSetAttribute(accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxStagedBytes); }) !=
-            cudaSuccess)
-            return SV_ERR_CUDA;
-        cfg.dynamicSmemBytes = bytes;
-    }
-    if (cudaLaunchKernelEx(&cfg, staged ? accept_kernel<true> : accept_kernel<false>, p) != cudaSuccess) return SV_ERR_CUDA;
+    void *args[] = {&p};
+    if (cudaLaunchKernelExC(&cfg, fn, args) != cudaSuccess) return SV_ERR_CUDA;
     return svh::launch_status();
 }
