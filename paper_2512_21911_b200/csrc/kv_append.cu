@@ -5,10 +5,14 @@
 //
 // One CTA per (KV head, sequence).  At most 64 tokens are appended per sequence, so at most two blocks are
 // touched: the rows are copied with 128-bit loads/stores (K and V), then the one or two affected block
-// means are recomputed from the pool exactly as sv_block_reps does (fp32 sums in a fixed order), which keeps
+// means are recomputed exactly as sv_block_reps does (fp32 sums in a fixed order), which keeps
 // them bit-identical to a full rebuild.  Page ids are checked against the pool size before anything is
-// written: a table entry that is not a page of the pool ends the table (the rows are dropped).  Traffic: n*512 bytes copied + at most 2*B*256 bytes re-read per
-// (sequence, KV head): latency-bound, not bandwidth-bound.
+// written: a table entry that is not a page of the pool ends the table (the rows are dropped).  Traffic: n*512 bytes copied + at
+// most B*256 bytes read per (sequence, KV head): latency-bound, not bandwidth-bound.  Three trips to memory, each needing
+// the one before: length, count and kept rows' numbers; page ids and draft rows; the rows that the block held already.  The appended
+// rows are summed from shared memory, and the length is advanced by a warp of its own, whose fences and atomics would
+// otherwise hold up the copy (32 layers of one sequence: 3.9 us behind the acceptance, 5 before, when rows were written, read back
+// and waited for the atomics).
 #include <cuda_bf16.h>
 
 #include "attn_common.cuh"
@@ -17,11 +21,12 @@
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;       // that copy and sum; one more warp advances the length
 constexpr int kRowGroups = kThreads / 16;
+constexpr int kMaxAppended = 64;    // rows per sequence (svh::kMaxDraft)
 
 template <int B>
-__global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__ k_pool, uint4 *__restrict__ v_pool,
+__global__ void __launch_bounds__(kThreads + 32) kv_append_kernel(uint4 *__restrict__ k_pool, uint4 *__restrict__ v_pool,
                                                              const int32_t *__restrict__ block_table,
                                                              const int32_t *seq_lens,
                                                              const uint4 *__restrict__ draft_k,
@@ -32,7 +37,9 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
                                                              int T, int Hkv, int NBmax, int n_pages,
                                                              const svk::LayerRow *layers, uint32_t *readers)
 {
-    const int h = blockIdx.x, s = blockIdx.y;
+    __shared__ uint4 fresh[kMaxAppended * 16];   // the appended K rows
+    __shared__ float part[kRowGroups][128];
+    const int h = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
     int bz = s;   // batch index of what the layer owns (draft K/V, representatives)
     if (layers) {
         const svk::LayerRow *row = layers + blockIdx.z;
@@ -42,68 +49,86 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
     }
     svk::grid_dependency_wait();
     svk::grid_launch_dependents();
+    // first trip: length, number of rows, and (thread: 32 per row, K and V) the draft row that is kept
+    const int which = (tid >> 4) & 1, c = tid & 15;
+    const auto kept = [&](int a) { return a < max_accept ? accept_idx[(size_t)s * max_accept + a] : 0; };
+    const auto draft_row = [&](int j) {
+        const size_t src = (((size_t)bz * T + min(max(j, 0), T - 1)) * Hkv + h) * 16 + c;
+        return __ldg((which ? draft_v : draft_k) + src);
+    };
     const int L = seq_lens[s];
-    int n = min(max(n_accept[s], 0), max_accept);
+    int n = n_accept[s];
+    const int j_first = kept(tid >> 5);
+    // second trip: the page or pages, and the draft row
+    const int *pages = block_table + (size_t)s * NBmax;
+    const int b0 = L < 0 ? 0 : L / B;
+    const int page0 = b0 < NBmax ? pages[b0] : -1, page1 = b0 + 1 < NBmax ? pages[b0 + 1] : -1;
+    const uint4 first = draft_row(j_first);
+    n = min(max(n, 0), max_accept);
     n = L < 0 ? 0 : max(0, min(n, NBmax * B - L));   // never past the last page of the table (nothing if L is already there)
     // A block whose table entry is not a page of the pool (not assigned yet: -1, or stale) ends the table: no row
     // enters it.  n <= 64 <= B, so the rows touch at most the blocks L / B and L / B + 1.
-    for (int b = L / B; n > 0 && b <= (L + n - 1) / B; ++b) {
-        const int page = block_table[(size_t)s * NBmax + b];
-        if (page < 0 || page >= n_pages) n = max(0, min(n, b * B - L));
-    }
+    if (page0 < 0 || page0 >= n_pages) n = 0;
+    if (page1 < 0 || page1 >= n_pages) n = min(n, (b0 + 1) * B - L);
     const int Ln = L + n;
     if (readers) {
         // The lengths are advanced in place, by the last CTA of the sequence to have read the old one; the counter wraps to
         // zero behind it.  readers[S + s]: the new length on its way there (of the last layer, should the layers' pools
-        // hold different numbers of pages).
-        __syncthreads();   // every thread of this CTA holds the old length
-        if (threadIdx.x == 0) {
-            int *fresh = reinterpret_cast<int *>(readers) + gridDim.y + s;
-            if (h == 0 && blockIdx.z == gridDim.z - 1) atomicExch(fresh, Ln);
-            __threadfence();
-            if (atomicInc(readers + s, gridDim.x * gridDim.z - 1) == gridDim.x * gridDim.z - 1) {
+        // hold different numbers of pages).  Fences and atomics take as long as the rest of the kernel, so a warp of its own
+        // does this.
+        if (tid >= kThreads) {
+            svk::named_bar_sync(1, kThreads + 32);   // every thread of this CTA holds the old length
+            if (tid == kThreads) {
+                int *fresh_len = reinterpret_cast<int *>(readers) + gridDim.y + s;
+                if (h == 0 && blockIdx.z == gridDim.z - 1) atomicExch(fresh_len, Ln);
                 __threadfence();
-                seq_lens_out[s] = atomicAdd(fresh, 0);
+                if (atomicInc(readers + s, gridDim.x * gridDim.z - 1) == gridDim.x * gridDim.z - 1) {
+                    __threadfence();
+                    seq_lens_out[s] = atomicAdd(fresh_len, 0);
+                }
             }
+            return;
         }
-    } else if (h == 0 && threadIdx.x == 0) {
-        seq_lens_out[s] = Ln;
+        svk::named_bar_arrive(1, kThreads + 32);
+    } else {
+        if (tid >= kThreads) return;
+        if (h == 0 && tid == 0) seq_lens_out[s] = Ln;
     }
     if (n <= 0) return;
 
-    // copy the accepted rows: 16 threads per 256-byte row, K and V
-    for (int idx = threadIdx.x; idx < n * 32; idx += kThreads) {
-        const int a = idx >> 5, which = (idx >> 4) & 1, c = idx & 15;
-        const int j = min(max(accept_idx[(size_t)s * max_accept + a], 0), T - 1);
-        const int t = L + a;
-        const int page = block_table[(size_t)s * NBmax + t / B];
-        const size_t dst = (((size_t)page * Hkv + h) * B + (t % B)) * 16 + c;
-        const size_t src = (((size_t)bz * T + j) * Hkv + h) * 16 + c;
-        if (which)
-            v_pool[dst] = __ldg(draft_v + src);
-        else
-            k_pool[dst] = __ldg(draft_k + src);
-    }
-    if (!reps) return;
-    __syncthreads();   // the rows written above are read back below by other threads of this CTA
-
-    __shared__ float part[kRowGroups][128];
-    const int chunk = threadIdx.x & 15, rg = threadIdx.x >> 4;
-    for (int b = L / B; b <= (Ln - 1) / B; ++b) {
-        const int cnt = min(B, Ln - b * B);
-        const int page = block_table[(size_t)s * NBmax + b];
-        const uint4 *tile = k_pool + ((size_t)page * Hkv + h) * (B * 16);
-        constexpr int kIter = B / kRowGroups;
-        uint4 v[kIter];
+    // third trip: the rows that the first block held already
+    constexpr int kIter = B / kRowGroups;
+    const int chunk = tid & 15, rg = tid >> 4;
+    uint4 v[kIter];
+    if (reps) {
+        const uint4 *tile = k_pool + ((size_t)page0 * Hkv + h) * (B * 16);
 #pragma unroll
         for (int i = 0; i < kIter; ++i) {
             const int row = rg + i * kRowGroups;
-            v[i] = row < cnt ? tile[row * 16 + chunk] : make_uint4(0u, 0u, 0u, 0u);   // plain loads: some rows were just written
+            v[i] = b0 * B + row < L ? tile[row * 16 + chunk] : make_uint4(0u, 0u, 0u, 0u);
         }
+    }
+    // copy the accepted rows: 16 threads per 256-byte row, K and V
+    for (int a = tid >> 5; a < n; a += kThreads / 32) {
+        const uint4 row = a == tid >> 5 ? first : draft_row(kept(a));
+        const int t = L + a;
+        const size_t dst = (((size_t)(t / B == b0 ? page0 : page1) * Hkv + h) * B + (t % B)) * 16 + c;
+        (which ? v_pool : k_pool)[dst] = row;
+        if (!which) fresh[a * 16 + c] = row;
+    }
+    if (!reps) return;
+    svk::named_bar_sync(2, kThreads);
+
+    // the means of the one or two blocks that grew (a second one holds appended rows only)
+    for (int b = b0; b <= (Ln - 1) / B; ++b) {
+        const int cnt = min(B, Ln - b * B);
         float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < kIter; ++i) {
-            const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&v[i]);
+            const int row = rg + i * kRowGroups, t = b * B + row;
+            uint4 x = b == b0 ? v[i] : make_uint4(0u, 0u, 0u, 0u);
+            if (t >= L && row < cnt) x = fresh[(t - L) * 16 + chunk];
+            const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&x);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float2 f = __bfloat1622float2(p2[j]);
@@ -113,14 +138,14 @@ __global__ void __launch_bounds__(kThreads) kv_append_kernel(uint4 *__restrict__
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) part[rg][chunk * 8 + j] = acc[j];
-        __syncthreads();
-        if (threadIdx.x < 128) {
+        svk::named_bar_sync(2, kThreads);
+        if (tid < 128) {
             float sum = 0.f;
 #pragma unroll
-            for (int g = 0; g < kRowGroups; ++g) sum += part[g][threadIdx.x];
-            reps[(((size_t)bz * Hkv + h) * NBmax + b) * 128 + threadIdx.x] = sum / (float)cnt;
+            for (int g = 0; g < kRowGroups; ++g) sum += part[g][tid];
+            reps[(((size_t)bz * Hkv + h) * NBmax + b) * 128 + tid] = sum / (float)cnt;
         }
-        __syncthreads();
+        svk::named_bar_sync(2, kThreads);
     }
 }
 
@@ -142,7 +167,7 @@ extern "C" sv_status sv_kv_append(const sv_geom *geom, void *k_pool, void *v_poo
         return SV_ERR_ALIGN;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(geom->n_kv_heads, geom->n_seq);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kThreads + 32);
     cfg.stream = static_cast<cudaStream_t>(stream);
     cudaLaunchAttribute attr[1];
     svh::pdl_attribute(attr);
@@ -174,7 +199,7 @@ extern "C" sv_status sv_kv_append_layers(const sv_geom *geom, const sv_layers *l
         return SV_ERR_ALIGN;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(geom->n_kv_heads, geom->n_seq, layers->n_layers);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kThreads + 32);
     cfg.stream = static_cast<cudaStream_t>(stream);
     cudaLaunchAttribute attr[1];
     svh::pdl_attribute(attr);
