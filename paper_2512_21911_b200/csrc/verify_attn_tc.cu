@@ -22,7 +22,8 @@
 //
 // Warp roles (384 threads): warps 0-3 and 4-7 are two softmax warpgroups that take units alternately,
 // each with its own S / P / O buffers; warp 8 is the TMA producer, one thread of warp 9 issues every
-// S = Q K^T (and the warp owns the TMEM allocation), one thread of warp 10 issues every O += P V.  The
+// S = Q K^T (and the warp owns the TMEM allocation; 128-row tiles: those of the first warpgroup, and a thread of warp 11 those of the
+// second), one thread of warp 10 issues every O += P V.  The
 // third warpgroup gives its registers to the other two (setmaxnreg).  Everything is chained with mbarriers; tcgen05.commit signals MMA completion.
 // At the end warpgroup 0 reads both accumulators from TMEM (warp q of either warpgroup owns lane quadrant q),
 // merges them in registers and writes the rows (or the fp32 partial of its split) out.
@@ -135,6 +136,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile Segment *segments = reinterpret_cast<volatile Segment *>(misc + 1664);
     volatile int *claims = reinterpret_cast<volatile int *>(misc + 1696);
     auto bar = [&](int slot) { return bars + 8u * slot; };
+    // a wait that ends early when somebody has given up; the flag is only looked at while there is something to wait for
+    auto wait_for = [&](int slot, uint32_t parity) {
+        for (uint32_t i = 0; i < (1u << 19); ++i) {
+            if (mbar_try_wait(bar(slot), parity)) return true;
+            if ((i & 15) == 15 && *abort_flag) return false;
+        }
+        return false;
+    };
     // (kBal) a wait that may last as long as a segment; it ends early when somebody has given up
     auto long_wait = [&](int slot, uint32_t parity) {
         for (uint32_t i = 0; i < kLongWait; ++i) {
@@ -155,6 +164,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int MT = NH == 4 ? 128 : 64;                   // rows of the Q and P tiles and of the MMAs
     constexpr int QR = NH == 4 ? 32 : 16;                    // tile rows per TMEM lane quadrant
     constexpr bool kPTmem = NH == 4 && !kPair;
+    // 128-row tiles: two threads issue S, one for either warpgroup.  One thread took 1180 cycles from one S to the next -- 520 for
+    // the eight MMAs, 90 for the commit, 275 for either wait even when there was nothing to wait for, behind the
+    // exponentials of two softmax warps on the same scheduler -- and everybody else waited for it: the softmax of a pair of units
+    // takes 1800 cycles, the tensor pipe 1230.  12 trees of 240 rows, a layer: 108 -> 93 us together with the flag of the waits
+    // (wait_for), which alone is 5 of these; one such tree 24.3 -> 23.5, 4 x 128K with 128 rows 32.4 -> 31.9.
+    constexpr bool kTwoS = NH == 4;
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
     // Registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168).  At 232 / 40 the roles of the third spill
     // inside their loops (16 sequences of 4-16K: 34.5 us a layer, 34.1 at 208 / 88; dense 32K 29.5 and 28.8; one 240-row tree 24.3
@@ -229,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == kSFree || lane == kPReady) count = na0;
             if (lane == kSFree + 1 || lane == kPReady + 1) count = max(1, na1);
             if (lane == kStaged) count = 8;
-            if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0) + 3;   // the softmax warps, either issuer's MMAs, the producer
+            if (lane == kTmemDone) count = na0 + (n_wg == 2 ? na1 : 0) + (kTwoS ? 4 : 3);   // the softmax warps, the issuers' MMAs, the producer
             if (lane == kTaken) count = na0 + (n_wg == 2 ? na1 : 0) + 2;   // the softmax warps and both issuers
             mbar_init(bar(lane), count);
             mbar_fence_init();
@@ -591,9 +606,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 ring += n_total;
             }
-        } else if (warp == 9 || warp == 10) {
+        } else if (warp == 9 || warp == 10 || kTwoS) {
             // ---------------------------------------------------------- MMA issuers (one thread each)
-            // warp 9 issues every S = Q K^T and owns the TMEM allocation; warp 10 issues every Ou = P V.
+            // warp 9 issues every S = Q K^T (kTwoS: of warpgroup 0, warp 11 of warpgroup 1) and owns the TMEM allocation; warp
+            // 10 issues every Ou = P V.
             // Descriptors are built once; per instruction only the 14-bit address field moves.
             if (lane == 0) {
                 int n_total = 0;
@@ -627,7 +643,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     done0 += (n_total + 1) >> 1;
                     done1 += n_total >> 1;
                 };
-                if (warp == 9) {
+                if (warp == 9 || (kTwoS && warp == 11)) {
                     constexpr uint32_t idesc_s = umma_idesc_bf16(MT, kUnit, false);
                     const uint64_t dq = umma_desc_sw128(smem0 + OFFQ, 16, 1024);
                     const uint64_t dk = umma_desc_sw128(smem0, 16, 1024);
@@ -639,13 +655,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if (end || dead) break;
                     }
                     // one S per (unit, warpgroup that takes it): the warpgroups alternate units, or (kPair) each takes all
-                    const int n_issue = kPair ? n_total * n_wg : n_total;
-                    for (int x = 0; x < n_issue && !dead; ++x) {
-                        const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
-                        const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = (kPair ? u : (u >> 1)) + (g ? done1 : done0);
-                        const int stage = (u + ring) % NS, it = (u + ring) / NS;
-                        if (*abort_flag || !mbar_wait_bounded(bar(kFull + stage), it & 1) ||
-                            (k > 0 && !mbar_wait_bounded(bar(kSFree + g), (k - 1) & 1))) {
+                    const int g_mine = kTwoS && warp == 11 ? 1 : 0;
+                    const int step = kTwoS && !kPair ? 2 : 1;
+                    const int u_end = kPair && g_mine == 1 && n_wg == 1 ? 0 : n_total;
+                    for (int u = kPair ? 0 : g_mine, stage = (u + ring) % NS, turn = (u + ring) / NS; u < u_end && !dead; u += step) {
+                        const int g = kTwoS ? g_mine : u & 1, k = kPair ? u : (u >> 1) + (g ? done1 : done0);
+                        if (!wait_for(kFull + stage, turn & 1) || (k > 0 && !wait_for(kSFree + g, (k - 1) & 1))) {
                             dead = true;
                             *abort_flag = 1;
                             if (p.status) atomicOr(p.status, 8);
@@ -664,10 +679,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 tc_mma_bf16(d, d_hi | (dq_lo + qo), d_hi | (k_lo + ko), idesc_s, ks > 0);
                         }
                         tc_commit(bar(kSReady + g));
+                        stage += step;
+                        if (stage >= NS) stage -= NS, ++turn;
                     }
                     if constexpr (kBal) end_segment();
                     }
                     tc_commit(bar(kTmemDone));
+                    if (warp == 11) return;
                     // free TMEM only after every softmax warp has finished reading it and every MMA is through
                     if (!mbar_wait_bounded(bar(kTmemDone), 0, kLongWait)) {
                         *abort_flag = 1;
@@ -693,11 +711,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if (end || dead) break;
                     }
                     const int n_issue = kPair ? n_total * n_wg : n_total;
-                    for (int x = 0; x < n_issue && !dead; ++x) {
+                    for (int x = 0, stage = ring % NS; x < n_issue && !dead; ++x) {
                         const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
                         const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = kPair ? u : (u >> 1);
-                        const int stage = (u + ring) % NS;
-                        if (*abort_flag || !mbar_wait_bounded(bar(kPReady + g), (k + (g ? done1 : done0)) & 1)) {
+                        if (!wait_for(kPReady + g, (k + (g ? done1 : done0)) & 1)) {
                             dead = true;
                             *abort_flag = 1;
                             if (p.status) atomicOr(p.status, 32);
@@ -717,7 +734,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                                             idesc_pv, (k > 0 || kk > 0) ? 1u : 0u);
                         }
                         tc_commit(bar(kOReady + g));
-                        if (!kPair || g == n_wg - 1) tc_commit(bar(kEmpty + stage));   // the last reader of the stage
+                        if (!kPair || g == n_wg - 1) {   // the last reader of the stage
+                            tc_commit(bar(kEmpty + stage));
+                            if (++stage == NS) stage = 0;
+                        }
                     }
                     if constexpr (kBal) end_segment();
                     }
@@ -952,7 +972,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // wait until the warpgroup's k-th PV has been added to O (warp-uniform outcome)
     auto wait_pv = [&](int k) {
-        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kOReady + wg), (k_before + k) & 1))) {
+        if (!dead && !__all_sync(0xffffffffu, wait_for(kOReady + wg, (k_before + k) & 1))) {
             dead = true;
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 4);
@@ -962,7 +982,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     int k = 0;
     for (int u = kPair ? 0 : wg; u < n_total; u += kPair ? 1 : 2, ++k) {   // kPair: every unit, for this warpgroup's row tile
-        if (!dead && __any_sync(0xffffffffu, *abort_flag || !mbar_wait_bounded(bar(kSReady + wg), (k_before + k) & 1))) {
+        if (!dead && !__all_sync(0xffffffffu, wait_for(kSReady + wg, (k_before + k) & 1))) {
             dead = true;
             *abort_flag = 1;
             if (p.status && lane == 0) atomicOr(p.status, 2);
