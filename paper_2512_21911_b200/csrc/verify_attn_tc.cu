@@ -293,14 +293,23 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();   // the barriers are initialised, tensor memory is allocated
         tc_fence_after_sync();
     }
-    // the query rows of a list to a Q tile, 16 bytes per asynchronous copy, by n threads of which this is t
-    auto copy_q = [&](uint32_t tile_at, const Item &it, int t, int n) {
+    // the query rows of this tile to shared memory, 16 bytes per asynchronous copy, by n threads of which this is t; z_q, h_q: whose
+    auto copy_q = [&](uint32_t tile_at, int z_q, int h_q, int t, int n) {
         const int c = t & 15;
-        const __nv_bfloat16 *src = p.q + ((size_t)it.z * p.T * p.Hq + it.h * p.G) * 128 + c * 8;
+        const __nv_bfloat16 *src = p.q + (((size_t)z_q * p.T + i0) * p.Hq + h_q * p.G) * 128 + c * 8;
         const uint32_t dst = tile_at + (c >> 3) * (kQBytes / 2);
 #pragma unroll 4
         for (int r = t >> 4; r < rows; r += n >> 4)
             cp_async_16(dst + swz128((r / RPQ) * QR + (r % RPQ), c & 7), src + (r + div_g(r) * (p.Hq - p.G)) * 128);
+    };
+    // the draft tokens' K rows, then their V rows, to a unit's place in shared memory
+    auto copy_draft = [&](uint32_t unit_at, int z_d, int h_d, int t, int n) {
+#pragma unroll 4
+        for (int idx = t; idx < 2 * p.T * 16; idx += n) {
+            const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;
+            cp_async_16(unit_at + which * (2 * kTile) + (c >> 3) * kTile + swz128(r, c & 7),
+                        (which ? p.draft_v : p.draft_k) + (((size_t)z_d * p.T + r) * p.Hkv + h_d) * 128 + c * 8);
+        }
     };
     const uint32_t tmem_base = warp == 8 && !kBal ? 0u : *tmem_slot;
 
@@ -546,7 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const Item it = item_at(claim);
                 const int n_total = item_blocks(it) * upb + 1;
                 if (seg > 0) {   // (the first segment's is brought by the softmax warps)
-                    copy_q(smem0 + OFFQ + (seg & 1) * 8192, it, lane, 32);   // (an M = 64 tile fills half of either half)
+                    copy_q(smem0 + OFFQ + (seg & 1) * 8192, it.z, it.h, lane, 32);   // (an M = 64 tile fills half of either half)
                 }
                 {   // lane i: tokens i and (kWide) 32 + i
 #pragma unroll
@@ -589,11 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         break;
                     }
                     const uint32_t at = smem0 + stage * kStageBytes;
-                    for (int idx = lane; idx < 2 * p.T * 16; idx += 32) {   // K rows, then V rows
-                        const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;
-                        cp_async_16(at + which * (2 * kTile) + (c >> 3) * kTile + swz128(r, c & 7),
-                                    (which ? p.draft_v : p.draft_k) + (((size_t)it.z * p.T + r) * p.Hkv + it.h) * 128 + c * 8);
-                    }
+                    copy_draft(at, it.z, it.h, lane, 32);
                     for (int idx = p.T * 16 + lane; idx < kUnit * 16; idx += 32) {   // (0 * junk must stay 0)
                         const int r = idx >> 4, c = idx & 15;
                         *reinterpret_cast<uint4 *>(smem + stage * kStageBytes + 2 * kTile + (c >> 3) * kTile + swz128(r, c & 7)) =
@@ -774,8 +779,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 *reinterpret_cast<uint4 *>(q_tile + 8192 + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    if (kBal) {
-        copy_q(smem0 + OFFQ, item_at(blockIdx.x), qtid, kQThreads);   // (first segment)
+    if constexpr (kBal) {
+        const Item it = item_at(blockIdx.x);
+        copy_q(smem0 + OFFQ, it.z, it.h, qtid, kQThreads);   // (first segment)
     } else if (has_draft) {
         for (int idx = tid; idx < 2 * kUnit * 16; idx += 256) {
             const int which = idx / (kUnit * 16);   // 0: K, 1: V
@@ -785,33 +791,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     make_uint4(0u, 0u, 0u, 0u);
         }
     }
-    if constexpr (kBal) cp_async_wait_all();
-    if constexpr (!kBal) grid_dependency_wait();
     if constexpr (!kBal) {
-        // real rows: all loads of a thread are in flight together (16-byte chunks: Q up to 128 rows x 16, draft K and
-        // V up to 64 tokens x 16 each)
-        constexpr int kQB = (NH == 4 ? 8 : 4) * (kPair ? 2 : 1), kDB = kWide ? 8 : 4;
-        const int n_q = rows * 16, n_d = has_draft ? 2 * p.T * 16 : 0;
-        uint4 v[kQB];
-#pragma unroll
-        for (int x = 0; x < kQB; ++x) {
-            const int idx = qtid + x * kQThreads;
-            if (idx < n_q) {
-                const int r = idx >> 4, c = idx & 15;
-                const int i = div_g(r), g = r - i * p.G;
-                v[x] = __ldg(reinterpret_cast<const uint4 *>(p.q + (((size_t)z * p.T + i0 + i) * p.Hq + h * p.G + g) * 128) + c);
-            }
-        }
-        uint4 w[kDB];
-#pragma unroll
-        for (int x = 0; x < kDB; ++x) {
-            const int idx = tid + x * 256;
-            if (idx < n_d) {
-                const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;   // K rows, then V rows
-                const __nv_bfloat16 *src = (which ? p.draft_v : p.draft_k) + (((size_t)z * p.T + r) * p.Hkv + h) * 128;
-                w[x] = __ldg(reinterpret_cast<const uint4 *>(src) + c);
-            }
-        }
+        grid_dependency_wait();
+        // all copies are in flight together (through registers, sixteen loads of a thread of the pair form went one after
+        // the other: 4 us ahead of the first S)
+        copy_q(smem_u32(q_tile), z, h, qtid, kQThreads);
+        if (has_draft) copy_draft(smem0 + kOffDraft, z, h, tid, 256);
         if (!kWide && has_draft && tid < 32) {
             uint32_t mask = 0;
             if (tid < p.T) {
@@ -844,24 +829,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             anc[tid] = mask;
         }
-#pragma unroll
-        for (int x = 0; x < kQB; ++x) {
-            const int idx = qtid + x * kQThreads;
-            if (idx < n_q) {
-                const int r = idx >> 4, c = idx & 15;
-                const int tr = (r / RPQ) * QR + (r % RPQ);
-                *reinterpret_cast<uint4 *>(q_tile + (c >> 3) * (kQBytes / 2) + swz128(tr, c & 7)) = v[x];
-            }
-        }
-#pragma unroll
-        for (int x = 0; x < kDB; ++x) {
-            const int idx = tid + x * 256;
-            if (idx < n_d) {
-                const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;
-                *reinterpret_cast<uint4 *>(smem + kOffDraft + which * (2 * kTile) + (c >> 3) * kTile + swz128(r, c & 7)) = w[x];
-            }
-        }
     }
+    cp_async_wait_all();
     fence_proxy_async();   // the tensor cores read these tiles through the async proxy
     if constexpr (kBal) {
         tc_fence_before_sync();
