@@ -505,9 +505,9 @@ def run_gpu(args):
                         "of the one before), so this is not `value`, which goes layer by layer, plus the copies: that is "
                         "one_stream_value; every step is one call of SparseVerifier.verify_step_from_host: "
                         "Q and draft K/V of all layers from pinned host memory, the step, the outputs back to pinned host "
-                        "memory, the copies in two chunks of layers, in the background so that all but the first upload "
+                        "memory, the copies in chunks of layers, in the background so that all but the first upload "
                         "and the last download run under the step's kernels; the KV cache is device-resident state",
-                "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "7/16, 9/16 of the layers",
+                "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "the engine's schedule",
                 "one_stream_value": ms_e2e_one_stream * 1e3 / (w.n_layers * world),
                 "one_stream_note": "the step layer by layer, as in `value`, with the same bytes copied whole before and after it on "
                                    "its own stream",
@@ -930,7 +930,7 @@ def main():
     ap.add_argument("--configs", action="store_true",
                     help="timing lines for the batched (16 ragged sequences) and long-context (4 x 128K, tree) configurations")
     ap.add_argument("--e2e-chunk", default="", help="layers per copy chunk of the end-to-end step: a size, or sizes a,b,c,... "
-                                                     "(default: the engine's schedule, 7/16 and 9/16 of the layers)")
+                                                     "(default: the engine's schedule)")
     ap.add_argument("--only", default="", help="with --configs: comma-separated configuration names (profiling aid: no dense pass)")
     ap.add_argument("--variants", action="store_true",
                     help="instead of the benchmark line: timings of the retrieval variants (shared budget, every token)")

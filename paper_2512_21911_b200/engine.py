@@ -17,6 +17,9 @@ import torch
 from . import binding as sv
 
 
+ONE_CHUNK_BYTES = 7 << 18   # see SparseVerifier._chunks
+
+
 class SparseVerifier:
     def __init__(self, *, n_seq: int, n_q_heads: int, n_kv_heads: int, head_dim: int, block_size: int,
                  max_blocks: int, n_draft: int, n_layers: int, block_table: torch.Tensor, seq_lens: torch.Tensor,
@@ -182,7 +185,7 @@ class SparseVerifier:
         CUDA graph (the side streams fork from and join the current stream).
 
         A chunk of few lists is split over the SMs for itself, so the outputs are those of verify_step to bf16 rounding.  Large
-        chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 178 us in two
+        chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 177 us in two
         chunks, 188 in chunks of eight layers, 241 of four, 613 of one)."""
         chunks = self._chunks(layers_per_chunk)
         if self._copy_streams is None:
@@ -220,12 +223,22 @@ class SparseVerifier:
 
     def _chunks(self, layers_per_chunk):
         if layers_per_chunk is None:
-            # Two chunks: every further one costs a launch that fills the GPU for a part of its time only.  The first is the
-            # smaller, its upload is not hidden (32 layers of a 32K context: 181 us in chunks of 14 / 18, 184 of 18 / 14,
-            # 201 of 8 / 10 / 14, 218 in one).  Not the best for every stack: 32 layers of an 8K context 165-205 us, 145 in
-            # halves; 16 layers x 4 sequences of 12K 245, 233 in chunks of four.
-            first = self.n_layers * 7 // 16
-            layers_per_chunk = [first, self.n_layers - first] if self.n_layers >= 4 else [self.n_layers]
+            # Nothing hides the first upload and the last download, and every chunk is a launch more that fills the GPU for a part of its
+            # time only.  A step of few bytes goes in one chunk: its copies take no longer than another launch (us per step, one chunk and
+            # 7/16 + 9/16 of the layers: 12 layers x 4K, 0.2 MB 29 and 45; 32 x 2K, 0.8 MB 62 and 68; 8 x 32K, 1.2 MB 88 and 92;
+            # 16 x 20K, 1.6 MB 101 and 102; 8 x 2 sequences x 100K, 2.4 MB 180 and 182; 32 x 8K, 3.1 MB 171 and 153).
+            # Larger ones: a short last chunk where a quarter of the layers still has lists for the SMs (5/16, 7/16, 1/4
+            # against 7/16 + 9/16: 24 x 3 sequences x 6K 205 and 232, 20 x 8 x 4K 225 and 254, 24 x 2 with 240 rows 990 and
+            # 1146, 8 x 2 x 100K 165 and 182, but 16 x 4 x 12K 257 and 249), halves otherwise (32 x 1 x 8K 143 and 153, 32 x 1 x
+            # 32K 177 both, where the three chunks take 182).
+            g, n = self.geom, self.n_layers
+            upload = n * g.n_seq * g.n_draft * (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim * 2
+            if n < 4 or upload <= ONE_CHUNK_BYTES:
+                layers_per_chunk = [n]
+            elif g.n_seq * g.n_kv_heads < 16:
+                layers_per_chunk = [n // 2, n - n // 2]
+            else:
+                layers_per_chunk = [n * 5 // 16, n - n * 5 // 16 - n // 4, n // 4]
         if isinstance(layers_per_chunk, int):
             sizes = [layers_per_chunk] * -(-self.n_layers // layers_per_chunk)
         else:   # a schedule: e.g. a small first and last chunk (their copies are the ones nothing hides), large ones between
