@@ -162,25 +162,37 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     if (need_scores) {
         const float4 qv = reinterpret_cast<const float4 *>(qbar)[lane];
         for (; b < b1; b += kDepth * kStride) {
+            float dot[kDepth * kRowsPerIter];
 #pragma unroll
-            for (int d = 0; d < kDepth; ++d) {
-                const int bd = b + d * kStride;
-                if (bd >= b1) break;   // (warp-uniform)
-                uint32_t kk[kRowsPerIter];
+            for (int d = 0; d < kDepth; ++d)
 #pragma unroll
-                for (int i = 0; i < kRowsPerIter; ++i) {
-                    float dot = r[d][i].x * qv.x + r[d][i].y * qv.y + r[d][i].z * qv.z + r[d][i].w * qv.w;
+                for (int i = 0; i < kRowsPerIter; ++i)
+                    dot[d * kRowsPerIter + i] = r[d][i].x * qv.x + r[d][i].y * qv.y + r[d][i].z * qv.z + r[d][i].w * qv.w;
+            // The sums over the lanes, all rows at once: with every exchange a lane keeps one half of the rows and hands the other half
+            // over, until it holds one (the same additions as row by row, in the same order, so the same bits).  13 shuffles for eight
+            // rows instead of 40: with two CTAs per SM, 1300 of them ahead of the selection (a layer of 16 ragged sequences, selection
+            // and attention: 33.6 -> 32.6 us; 4 x 128K 31.9 -> 30.9; one tree of 60 at 32K 23.0 -> 22.6).
+            int o = 16;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                    const int bb = bd + i;
-                    const bool is_forced = bb < p.n_sink || bb >= nb - p.n_local;
-                    kk[i] = is_forced ? kForcedKey : order_key(dot);
-                    if (p.out_scores && lane == 0 && bb < b1) p.out_scores[((size_t)z * p.Hkv + h) * p.NBmax + bb] = dot;
+            for (int n = kDepth * kRowsPerIter / 2; n > 0; n /= 2, o /= 2)
+#pragma unroll
+                for (int i = 0; i < n; ++i) {
+                    const float keep = lane & o ? dot[n + i] : dot[i], give = lane & o ? dot[i] : dot[n + i];
+                    dot[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
                 }
-                // rows bd .. bd+3 are 4 consecutive keys: one 16-byte store into CTA 0 (entries past nb are never read)
-                if (lane == 0 && !keep_all)
-                    svk::st_async_cluster_v4(keys0 + 4u * (uint32_t)bd, make_uint4(kk[0], kk[1], kk[2], kk[3]), ready0);
-            }
+#pragma unroll
+            for (; o > 0; o /= 2) dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], o);
+            // lane group l / kGroup holds row (l / kGroup) of the kDepth x 4
+            constexpr int kGroup = 32 / (kDepth * kRowsPerIter);
+            const int bd = b + lane / (kGroup * kRowsPerIter) * kStride, bb = bd + lane / kGroup % kRowsPerIter;
+            if (p.out_scores && lane % kGroup == 0 && bb < b1) p.out_scores[((size_t)z * p.Hkv + h) * p.NBmax + bb] = dot[0];
+            const uint32_t key = bb < p.n_sink || bb >= nb - p.n_local ? kForcedKey : order_key(dot[0]);
+            uint32_t kk[kRowsPerIter];   // the keys of this half's four rows (kDepth = 1: of the four)
+#pragma unroll
+            for (int i = 0; i < kRowsPerIter; ++i) kk[i] = __shfl_sync(0xffffffffu, key, lane / (kGroup * kRowsPerIter) * (kGroup * kRowsPerIter) + i * kGroup);
+            // rows bd .. bd+3 are 4 consecutive keys: one 16-byte store into CTA 0 (entries past nb are never read)
+            if (lane % (kGroup * kRowsPerIter) == 0 && bd < b1 && !keep_all)
+                svk::st_async_cluster_v4(keys0 + 4u * (uint32_t)bd, make_uint4(kk[0], kk[1], kk[2], kk[3]), ready0);
             if (b + kDepth * kStride < b1) load_rows(b + kDepth * kStride, b1);
         }
     }

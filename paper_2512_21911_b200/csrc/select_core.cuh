@@ -185,10 +185,8 @@ __device__ __forceinline__ void select_top(const uint32_t *keys_all, int nb, int
                 }
                 if (lane == 31) sc.warp_sel[warp] = incl;
                 sync();
-                uint32_t pos = incl - n_mine;
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w)
-                    if (w < warp) pos += sc.warp_sel[w];
+                // (one load per lane: a loop over the warps ahead is up to 15 loads of every thread)
+                uint32_t pos = incl - n_mine + __reduce_add_sync(0xffffffffu, lane < warp ? sc.warp_sel[lane] : 0u);
 #pragma unroll
                 for (int c = 0; c < NC; ++c)
                     if ((sel_bits >> c) & 1u) emit((int)pos++, NC * tid + c);
