@@ -32,6 +32,7 @@ namespace {
 // 128 sequences 31 -> 24 us per call and 216 -> 208 us with the attention behind it; with one wave the smaller CTAs
 // finish a stand-alone call sooner too, but the attention behind them starts later -- 4 x 128K: 31.0 against 29.8 us).
 constexpr int kThreadsFew = 512, kThreadsMany = 256;
+constexpr int kFirstHeads = 8;    // query heads of a group whose rows are loaded together (the others follow one by one)
 constexpr int kRowsPerIter = 4;   // consecutive representative rows a warp scores per pass (one 16-byte store of keys)
 
 using svsel::kForcedKey;
@@ -131,10 +132,17 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
             for (int i = 0; i < kRowsPerIter; ++i)
                 r[d][i] = (bb + d * kStride + i < hi) ? load_row(bb + d * kStride + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
+    // The query ahead of the rows: what an SM has asked for arrives in that order, and two CTAs' rows take it a microsecond (16 ragged
+    // sequences, selection and attention: 32.65 -> 32.27 us; 4 x 128K 30.95 -> 30.75; four heads together: 32.38, 30.80).
+    float q_first[kFirstHeads];
+#pragma unroll
+    for (int g = 0; g < kFirstHeads; ++g) q_first[g] = tid < 128 && g < G ? __bfloat162float(q0[(size_t)g * 128 + tid]) : 0.f;
     load_rows(b, min(b0 + p.chunk, p.NBmax));
     float qsum = 0.f;
+#pragma unroll
+    for (int g = 0; g < kFirstHeads; ++g) qsum += q_first[g];
     if (tid < 128)
-        for (int g = 0; g < G; ++g) qsum += __bfloat162float(q0[(size_t)g * 128 + tid]);
+        for (int g = kFirstHeads; g < G; ++g) qsum += __bfloat162float(q0[(size_t)g * 128 + tid]);
     // CTA 0's barrier is initialised (every CTA arrived before its first global request); the wait costs a few hundred
     // cycles even then, so it sits here, behind the loads it can overlap with
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
