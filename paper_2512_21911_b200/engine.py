@@ -17,7 +17,39 @@ import torch
 from . import binding as sv
 
 
-ONE_CHUNK_BYTES = 7 << 18   # see SparseVerifier._chunks
+# What the schedule of a host-fed step reckons with: bytes per microsecond over PCIe and from HBM, microseconds per chunk (its
+# launches; the copies of a further one), and the lists of a launch from which on the GPU gathers at full speed.
+PCIE_RATE, HBM_RATE, LAUNCH_US, COPY_US, FULL_LISTS = 49e3, 6.6e6, 14.0, 16.0, 148 / 2.5
+
+
+def host_step_us(sizes: Sequence[int], upload: float, download: float, gathered: float, lists: int) -> float:
+    """What a host-fed step in chunks of these sizes takes, by bytes and lists per layer: uploads one after the other, a chunk's
+    kernels behind its upload and the chunk before, its download behind them."""
+    up = computed = down = 0.0
+    for i, n in enumerate(sizes):
+        up += n * upload / PCIE_RATE + (COPY_US if i else 0.0)
+        computed = max(up, computed) + LAUNCH_US + n * gathered / HBM_RATE / min(1.0, n * lists / FULL_LISTS)
+        down = max(computed, down) + n * download / PCIE_RATE
+    return down
+
+
+def host_step_schedule(n: int, upload: float, download: float, gathered: float, lists: int) -> List[int]:
+    """Layers per chunk of a host-fed step of n layers.  Nothing hides the first upload and the last download, and every chunk costs
+    launches: a step of few bytes is one chunk, one with much to move and to compute ends soonest with a short last chunk.  7/16 and
+    9/16 of the layers unless another split is reckoned to be 3 % faster.  Over 135 steps (4 to 32 layers, 1 to 7 sequences of 1K to
+    100K tokens, 1 to 16 draft tokens, 0.2 to 18 MB of inputs, 7 to 750 MB gathered) what this picks takes 0.884 of the time of
+    7/16 + 9/16 in the geometric mean and 1.033 at worst, 1.02 of the best of these four: 12 layers x 4K 45 -> 29 us, 24 layers x 3
+    sequences x 6K 232 -> 205, 24 x 2 with 240 rows 1146 -> 990."""
+    if n == 1:
+        return [1]
+    first = max(1, n * 7 // 16)
+    usual, others = [first, n - first], [[n], [n // 2, n - n // 2]]
+    if n >= 4:
+        third = max(1, n * 5 // 16)
+        others.append([third, n - third - n // 4, n // 4])
+    reckon = lambda sizes: host_step_us(sizes, upload, download, gathered, lists)
+    best = min(others, key=reckon)
+    return best if reckon(best) < 0.97 * reckon(usual) else usual
 
 
 class SparseVerifier:
@@ -43,6 +75,10 @@ class SparseVerifier:
         self._one_allocation = False
         self._copy_streams = None
         self._host_step = None
+        rows, pairs = n_seq * n_draft * head_dim * 2, n_seq * n_kv_heads
+        self._schedule = host_step_schedule(
+            n_layers, rows * (n_q_heads + 2 * n_kv_heads), rows * n_q_heads,
+            pairs * head_dim * 4 * (min(max_sel, max_blocks) * block_size + max_blocks * sum(map(bool, self.anchors)) / n_layers), pairs)
         self._counters = torch.zeros(2 * n_seq, dtype=torch.int32, device=dev)   # see sv_kv_append_layers
         # what the layers' kernels look up when several layers run in one launch (a row is valid once its layer has pools)
         stackable = n_layers <= sv.SV_MAX_LAYERS and n_layers * n_seq <= 65535
@@ -223,22 +259,7 @@ class SparseVerifier:
 
     def _chunks(self, layers_per_chunk):
         if layers_per_chunk is None:
-            # Nothing hides the first upload and the last download, and every chunk is a launch more that fills the GPU for a part of its
-            # time only.  A step of few bytes goes in one chunk: its copies take no longer than another launch (us per step, one chunk and
-            # 7/16 + 9/16 of the layers: 12 layers x 4K, 0.2 MB 29 and 45; 32 x 2K, 0.8 MB 62 and 68; 8 x 32K, 1.2 MB 88 and 92;
-            # 16 x 20K, 1.6 MB 101 and 102; 8 x 2 sequences x 100K, 2.4 MB 180 and 182; 32 x 8K, 3.1 MB 171 and 153).
-            # Larger ones: a short last chunk where a quarter of the layers still has lists for the SMs (5/16, 7/16, 1/4
-            # against 7/16 + 9/16: 24 x 3 sequences x 6K 205 and 232, 20 x 8 x 4K 225 and 254, 24 x 2 with 240 rows 990 and
-            # 1146, 8 x 2 x 100K 165 and 182, but 16 x 4 x 12K 257 and 249), halves otherwise (32 x 1 x 8K 143 and 153, 32 x 1 x
-            # 32K 177 both, where the three chunks take 182).
-            g, n = self.geom, self.n_layers
-            upload = n * g.n_seq * g.n_draft * (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim * 2
-            if n < 4 or upload <= ONE_CHUNK_BYTES:
-                layers_per_chunk = [n]
-            elif g.n_seq * g.n_kv_heads < 16:
-                layers_per_chunk = [n // 2, n - n // 2]
-            else:
-                layers_per_chunk = [n * 5 // 16, n - n * 5 // 16 - n // 4, n // 4]
+            layers_per_chunk = self._schedule
         if isinstance(layers_per_chunk, int):
             sizes = [layers_per_chunk] * -(-self.n_layers // layers_per_chunk)
         else:   # a schedule: e.g. a small first and last chunk (their copies are the ones nothing hides), large ones between
