@@ -126,10 +126,11 @@ inline int sm_count()
 // from one gather, each softmax warpgroup taking every unit for its own tile).  One per tile is the default: the CTAs
 // that share a slice of the blocks sit next to each other in the grid, request the same K/V tiles at about the same
 // time, and all but the first find them in L2 (240 rows, one sequence: 29.6 MB from DRAM for 29.8 MB algorithmic), and
-// the finer CTAs fill the SMs better.  A paired CTA takes 1.93 times as long as a single-tile one (batches of 240-row
-// trees: 99.5 against 51.6 us per wave of CTAs), so pairs are used where they save enough waves to pay for that -- in
-// practice when the row-tile CTAs just miss fitting the SMs once or twice (10 to 16 such sequences of 8 KV heads:
-// 99 against 103 us).
+// the finer CTAs fill the SMs better.  A paired CTA takes 1.75 to 1.93 times as long as a single-tile one (batches of 240-row
+// trees with lists of 74 blocks: 75 against 42 us per wave of CTAs, 38.8 and 22 with lists of 30; 99.5 and 51.6 when one thread issued all
+// of a CTA's S), so pairs are used where they save enough waves to pay for that -- in
+// practice when the row-tile CTAs just miss fitting the SMs once or twice (10 to 18 such sequences of 8 KV heads:
+// 75 against 84 us).  Within that range of the factor the rule gives the same answer up to nine waves.
 inline bool pair_row_tiles(const sv_geom *g)
 {
     const int t = row_tiles(g);
