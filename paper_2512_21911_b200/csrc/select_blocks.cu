@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "select_core.cuh"
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    extern __shared__ __align__(16) uint32_t keys_all[];         // [CL*chunk] keys of all blocks (used in CTA 0)
+    extern __shared__ __align__(16) uint32_t keys_all[];         // keys of all blocks (used in CTA 0)
     __shared__ float qbar[128];
     __shared__ svsel::Scratch scratch;
     __shared__ uint64_t keys_ready;                // mbarrier in CTA 0: the bytes of all keys (one arrival: CTA 0 itself)
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     }
     scratch.init(tid, kThreads);
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // before any global request is in flight
-    const int b0 = rank * p.chunk;
+    const int b0 = rank * p.chunk, b_end = rank == CL - 1 ? p.NBmax : min(b0 + p.chunk, p.NBmax);   // this CTA's slice
     constexpr int kRowBytes = kBf16 ? 256 : 512, kLaneBytes = kRowBytes / 32;
     const char *rbase = static_cast<const char *>(p.reps) + ((size_t)bz * p.Hkv + h) * p.NBmax * kRowBytes;
     auto row_ptr = [&](int row) { return rbase + (size_t)row * kRowBytes + lane * kLaneBytes; };
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     for (int d = 0; d < kDepth; ++d)
 #pragma unroll
         for (int i = 0; i < kRowsPerIter; ++i)
-            if (b + d * kStride + i < min(b0 + p.chunk, p.NBmax)) svk::prefetch_l2(row_ptr(b + d * kStride + i));
+            if (b + d * kStride + i < b_end) svk::prefetch_l2(row_ptr(b + d * kStride + i));
     const int G = p.Hq / p.Hkv;
     const __nv_bfloat16 *q0 = p.q + ((size_t)bz * p.T * p.Hq + (size_t)h * G) * 128;
     if (tid < G * 2) svk::prefetch_l2(q0 + tid * 64);
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     float q_first[kFirstHeads];
 #pragma unroll
     for (int g = 0; g < kFirstHeads; ++g) q_first[g] = tid < 128 && g < G ? __bfloat162float(q0[(size_t)g * 128 + tid]) : 0.f;
-    load_rows(b, min(b0 + p.chunk, p.NBmax));
+    load_rows(b, b_end);
     float qsum = 0.f;
 #pragma unroll
     for (int g = 0; g < kFirstHeads; ++g) qsum += q_first[g];
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     const bool keep_all = N >= nb;
     if (keep_all) N = nb;
     const bool need_scores = !keep_all || p.out_scores;
-    const int b1 = min(b0 + p.chunk, nb);
+    const int b1 = min(b_end, nb);
 
     // retrieval query: mean of the first draft token's query over the GQA group
     if (tid < 128) qbar[tid] = qsum / (float)G;
@@ -335,12 +336,18 @@ static sv_status launch_select(const sv_geom *geom, Params &p, int n_batch, cuda
     const bool many = (long long)pairs * CL > 2 * svh::sm_count();   // more CTAs than fit at once: smaller CTAs, four per SM
     const int threads = many ? kThreadsMany : kThreadsFew;
     const int stride = threads / 32 * kRowsPerIter;              // blocks a CTA covers per pass
-    const int chunk = (per + stride - 1) / stride * stride;
+    // Slices are multiples of four blocks (one store of keys); the last CTA's goes on to the end of the table.  A table has room for the
+    // draft, so it is often one block longer than a round number: slices rounded up to whole passes left CTAs idle (513
+    // blocks: four of eight) or cost another pass (257 over two CTAs: 192 and 65), so a slice is rounded down where rounding it up
+    // would cost a pass.  Selection and attention of 16 ragged sequences of up to 16K 32.4 -> 31.3 us, 4 x 128K 30.7 -> 29.6, one
+    // request of 32K with a tree of 60 rows 22.4 -> 22.2.
+    const int up = (per + 3) / 4 * 4, down = std::max(4, geom->max_blocks / CL / 4 * 4);
+    const int chunk = (up + stride - 1) / stride > (down + stride - 1) / stride ? down : up;
 
     p.T = geom->n_draft, p.Hq = geom->n_q_heads, p.Hkv = geom->n_kv_heads, p.B = geom->block_size;
     p.NBmax = geom->max_blocks, p.chunk = chunk;
 
-    const size_t smem = (size_t)CL * chunk * sizeof(uint32_t);
+    const size_t smem = (size_t)std::max(CL * chunk, (geom->max_blocks + 3) / 4 * 4) * sizeof(uint32_t);
     const bool deep = chunk > stride;   // more than one pass per warp: load two passes' rows together
     const void *fn = select_fn<kBf16, kStack>(!many, deep);
     if (smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
