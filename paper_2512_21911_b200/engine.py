@@ -17,39 +17,47 @@ import torch
 from . import binding as sv
 
 
-# What the schedule of a host-fed step reckons with: bytes per microsecond over PCIe and from HBM, microseconds per chunk (its
-# launches; the copies of a further one), and the lists of a launch from which on the GPU gathers at full speed.
-PCIE_RATE, HBM_RATE, LAUNCH_US, COPY_US, FULL_LISTS = 49e3, 6.6e6, 14.0, 16.0, 148 / 2.5
+# What the schedule of a host-fed step reckons with: bytes per microsecond up, down, from HBM and by one CTA alone, microseconds per
+# chunk (its launches; the copies of a further one).  Fitted to the differences between the schedules of 184 stacks on two
+# machines (the sums come out 15 % high): a B200 on a PCIe 5 link, of which only the proportions matter here.
+UP_RATE, DOWN_RATE, HBM_RATE, CTA_RATE, LAUNCH_US, COPY_US = 36e3, 57e3, 6.4e6, 76e3, 18.0, 18.0
 
 
-def host_step_us(sizes: Sequence[int], upload: float, download: float, gathered: float, lists: int) -> float:
+def host_step_us(sizes: Sequence[int], upload: float, download: float, gathered: float, lists: int, sms: int = 148) -> float:
     """What a host-fed step in chunks of these sizes takes, by bytes and lists per layer: uploads one after the other, a chunk's
-    kernels behind its upload and the chunk before, its download behind them."""
+    kernels behind its upload and the chunk before, its download behind them.  A chunk gathers at the rate of HBM however few its
+    lists are (they are split over the SMs); where there are more lists than SMs, the last of them run on a part of the SMs (32
+    layers of 8 lists in chunks of 14 + 18 layers: 178 us, of 12 + 20 layers, 160 lists: 213)."""
     up = computed = down = 0.0
     for i, n in enumerate(sizes):
-        up += n * upload / PCIE_RATE + (COPY_US if i else 0.0)
-        computed = max(up, computed) + LAUNCH_US + n * gathered / HBM_RATE / min(1.0, n * lists / FULL_LISTS)
-        down = max(computed, down) + n * download / PCIE_RATE
+        up += n * upload / UP_RATE + (COPY_US if i else 0.0)
+        computed = max(up, computed) + LAUNCH_US + n * gathered / HBM_RATE
+        if n * lists > sms:
+            computed += gathered / lists / CTA_RATE * (-n * lists % sms) / sms
+        down = max(computed, down) + n * download / DOWN_RATE
     return down
 
 
-def host_step_schedule(n: int, upload: float, download: float, gathered: float, lists: int) -> List[int]:
+def host_step_schedule(n: int, upload: float, download: float, gathered: float, lists: int, sms: int = 148) -> List[int]:
     """Layers per chunk of a host-fed step of n layers.  Nothing hides the first upload and the last download, and every chunk costs
-    launches: a step of few bytes is one chunk, one with much to move and to compute ends soonest with a short last chunk.  7/16 and
-    9/16 of the layers unless another split is reckoned to be 3 % faster.  Over 135 steps (4 to 32 layers, 1 to 7 sequences of 1K to
-    100K tokens, 1 to 16 draft tokens, 0.2 to 18 MB of inputs, 7 to 750 MB gathered) what this picks takes 0.884 of the time of
-    7/16 + 9/16 in the geometric mean and 1.033 at worst, 1.02 of the best of these four: 12 layers x 4K 45 -> 29 us, 24 layers x 3
-    sequences x 6K 232 -> 205, 24 x 2 with 240 rows 1146 -> 990."""
+    launches and copies: a step of few bytes is one chunk, one with much to move and to compute ends soonest with a short last
+    chunk.  7/16 and 9/16 of the layers (fewer than four: all at once) unless another split is reckoned to be 2 % faster.
+
+    Over 331 timings of stacks on three machines (2 to 32 layers, 1 to 8 sequences of 1K to 131K tokens, 1 to 60 draft tokens), the 147 of
+    one machine not part of the fit, what this picks takes 0.938 of the time of that usual split in the geometric mean, more than 1.01 of it for ten of them
+    and 1.05 at worst (7.7 MB up and 34 MB gathered, in three chunks), and 1.006 of the best of these four: 13 layers x 57K 53 -> 37
+    us, 31 layers x 5 sequences 501 -> 460, 3 x 8 sequences of 32K 327 -> 272; 32 layers of a 32K context 178 (183 in 10 + 14 + 8)."""
     if n == 1:
         return [1]
     first = max(1, n * 7 // 16)
-    usual, others = [first, n - first], [[n], [n // 2, n - n // 2]]
+    splits = [[first, n - first], [n], [n // 2, n - n // 2]]
     if n >= 4:
         third = max(1, n * 5 // 16)
-        others.append([third, n - third - n // 4, n // 4])
-    reckon = lambda sizes: host_step_us(sizes, upload, download, gathered, lists)
-    best = min(others, key=reckon)
-    return best if reckon(best) < 0.97 * reckon(usual) else usual
+        splits.append([third, n - third - n // 4, n // 4])
+    usual = splits[0] if n >= 4 else splits[1]
+    reckon = lambda sizes: host_step_us(sizes, upload, download, gathered, lists, sms)
+    best = min(splits, key=reckon)
+    return best if reckon(best) < 0.98 * reckon(usual) else usual
 
 
 class SparseVerifier:
@@ -78,7 +86,8 @@ class SparseVerifier:
         rows, pairs = n_seq * n_draft * head_dim * 2, n_seq * n_kv_heads
         self._schedule = host_step_schedule(
             n_layers, rows * (n_q_heads + 2 * n_kv_heads), rows * n_q_heads,
-            pairs * head_dim * 4 * (min(max_sel, max_blocks) * block_size + max_blocks * sum(map(bool, self.anchors)) / n_layers), pairs)
+            pairs * head_dim * 4 * (min(max_sel, max_blocks) * block_size + max_blocks * sum(map(bool, self.anchors)) / n_layers), pairs,
+            torch.cuda.get_device_properties(dev).multi_processor_count)
         self._counters = torch.zeros(2 * n_seq, dtype=torch.int32, device=dev)   # see sv_kv_append_layers
         # what the layers' kernels look up when several layers run in one launch (a row is valid once its layer has pools)
         stackable = n_layers <= sv.SV_MAX_LAYERS and n_layers * n_seq <= 65535
@@ -221,7 +230,7 @@ class SparseVerifier:
         CUDA graph (the side streams fork from and join the current stream).
 
         A chunk of few lists is split over the SMs for itself, so the outputs are those of verify_step to bf16 rounding.  Large
-        chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 177 us in two
+        chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 178 us in two
         chunks, 188 in chunks of eight layers, 241 of four, 613 of one)."""
         chunks = self._chunks(layers_per_chunk)
         if self._copy_streams is None:
