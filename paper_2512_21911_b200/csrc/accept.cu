@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "accept_share.h"
 #include "sv_host.h"
 #include "sv_ptx.cuh"
 
@@ -32,11 +33,11 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int kThreads = 512;
+constexpr int kThreads = svk::kAcceptThreads;
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxRows = 64;     // draft rows per step (the ancestor masks of the attention kernel are 64 bits)
 constexpr int kMaxCluster = 16;
-constexpr int kMaxHeld = 8;      // words of either distribution that a thread holds (64 registers)
+constexpr int kMaxHeld = svk::kAcceptHeld;
 
 struct AcceptParams {
     const float *p_target;   // [S][T][V]
@@ -289,23 +290,27 @@ __global__ void __launch_bounds__(kThreads) accept_kernel(const AcceptParams p)
     if (lane == 0) p.next_token[s] = last;
 }
 
+// The kernel for a share; several batches have more than half of kMaxHeld words each.
 template <int NW = 1>
-const void *accept_fn(int held)   // kernel for `held` words per thread; more than kMaxHeld: several batches
+const void *accept_fn(svk::AcceptShare share)
 {
-    if constexpr (NW <= kMaxHeld) {
-        return held <= NW ? reinterpret_cast<const void *>(accept_kernel<NW, true>) : accept_fn<NW + 1>(held);
-    } else {
-        return reinterpret_cast<const void *>(accept_kernel<kMaxHeld, false>);
+    if constexpr (NW < kMaxHeld) {
+        if (share.words > NW) return accept_fn<NW + 1>(share);
     }
+    if constexpr (2 * NW > kMaxHeld) {
+        if (share.batches > 1) return reinterpret_cast<const void *>(accept_kernel<NW, false>);
+    }
+    return reinterpret_cast<const void *>(accept_kernel<NW, true>);
 }
 
 // How many clusters of 16 CTAs of the kernel this device holds at once (asked once per device; more than the portable size).
-int clusters_of_16(const void *fn, int held)
+int clusters_of_16(svk::AcceptShare share)
 {
-    static std::atomic<int> known[svh::kMaxDevices][kMaxHeld + 2];   // the number + 1; 0: not asked
+    static std::atomic<int> known[svh::kMaxDevices][2 * kMaxHeld + 1];   // by kernel: the number + 1; 0: not asked
     const int dev = svh::current_device();
     if (dev < 0 || dev >= svh::kMaxDevices) return 0;
-    std::atomic<int> &at = known[dev][held <= kMaxHeld ? held : kMaxHeld + 1];
+    const void *fn = accept_fn(share);
+    std::atomic<int> &at = known[dev][share.words + (share.batches > 1 ? kMaxHeld : 0)];
     int v = at.load(std::memory_order_acquire);
     if (v == 0) {
         int n = 0;
@@ -345,15 +350,14 @@ extern "C" sv_status sv_accept(int32_t n_seq, int32_t n_draft, int32_t vocab, co
     // sequences, for which there is not room, 16.4 and 12.4.
     int CL = 1;
     while (CL < 8 && vocab / (CL * 2) >= 4096) CL *= 2;
-    const auto held_by = [&](int ctas) { return (vocab / 4 + ctas * kThreads - 1) / (ctas * kThreads); };   // words per thread
-    if (CL == 8 && vocab / 16 >= 4096 && n_seq <= clusters_of_16(accept_fn(held_by(16)), held_by(16))) CL = 16;
-    const int held = held_by(CL);
-    const void *fn = accept_fn(held);
+    if (CL == 8 && vocab / 16 >= 4096 && n_seq <= clusters_of_16(svk::accept_share(vocab, 16))) CL = 16;
+    const svk::AcceptShare share = svk::accept_share(vocab, CL);
+    const void *fn = accept_fn(share);
     AcceptParams p;
     p.p_target = p_target, p.p_draft = p_draft, p.tokens = tokens, p.parent = parent, p.u_accept = u_accept;
     p.u_next = u_next, p.path = path, p.n_path = n_path, p.next_token = next_token, p.alpha = alpha;
     p.T = n_draft, p.V = vocab;
-    p.batches = (held + kMaxHeld - 1) / kMaxHeld;
+    p.batches = share.batches;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CL, n_seq);
     cfg.blockDim = dim3(kThreads);
