@@ -34,4 +34,14 @@ SV_RING_FN RingCopies copies_of_units(int first, int end, int n_stages)
     return ring;
 }
 
+// Whether threads that take every step-th unit of a ring each may wait for the units' full barriers.  A wait names a parity and passes
+// while the barrier is in a phase of the other one, so it tells a unit only from the one before it on the same stage.  A thread that
+// has waited for that one itself cannot be early; where it was another thread's, it may not have landed yet, and the
+// wait for the unit a round later passes: the tile is read while it is being written, and the stage handed back with its copy in
+// flight, so that its barrier is armed twice in a phase.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr bool stages_keep_their_thread(int n_stages, int step) { return n_stages % step == 0; }
+
 }  // namespace svk

@@ -171,6 +171,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // (wait_for), which alone is 5 of these; one such tree 24.3 -> 23.5, 4 x 128K with 128 rows 32.4 -> 31.9.
     constexpr bool kTwoS = NH == 4;
     constexpr int NS = kPair ? kStages - 1 : kPTmem ? kStages + 1 : kStages;   // ring stages
+    // (of a pair either thread takes every unit; a single 128-row tile has six stages, tiles of up to 64 rows five: not for two threads)
+    static_assert(!kTwoS || stages_keep_their_thread(NS, kPair ? 1 : 2), "a thread that issues S waits for all units of its stages");
     // Registers of the softmax warpgroups and of the third (2 x many + few = 3 x 168).  At 232 / 40 the roles of the third spill
     // inside their loops (16 sequences of 4-16K: 34.5 us a layer, 34.1 at 208 / 88; dense 32K 29.5 and 28.8; one 240-row tree 24.3
     // and 23.9); the softmax needs no more than 208 in any form.  Up to 32 rows 56 do for the roles: a layer of a 32K context 14.59 us
