@@ -25,9 +25,9 @@ UP_RATE, DOWN_RATE, HBM_RATE, CTA_RATE, LAUNCH_US, COPY_US = 36e3, 57e3, 6.4e6, 
 
 def host_step_us(sizes: Sequence[int], upload: float, download: float, gathered: float, lists: int, sms: int = 148) -> float:
     """What a host-fed step in chunks of these sizes takes, by bytes and lists per layer: uploads one after the other, a chunk's
-    kernels behind its upload and the chunk before, its download behind them.  A chunk gathers at the rate of HBM however few its
-    lists are (they are split over the SMs); where there are more lists than SMs, the last of them run on a part of the SMs (32
-    layers of 8 lists in chunks of 14 + 18 layers: 178 us, of 12 + 20 layers, 160 lists: 213)."""
+    kernels behind its upload and the chunk before, its download behind them.  A chunk is taken to gather at the rate of HBM however
+    few its lists are (few are split over the SMs); where there are more lists than SMs, the last of them run on a part of the SMs
+    (32 layers of 8 lists in chunks of 14 + 18 layers: 178 us, of 12 + 20 layers, 160 lists: 213)."""
     up = computed = down = 0.0
     for i, n in enumerate(sizes):
         up += n * upload / UP_RATE + (COPY_US if i else 0.0)

@@ -1,5 +1,6 @@
-"""Acceptance with a row's range in shared memory: vocabularies at the edges of the threads' segments and of what fits there (212992
-entries for a cluster of eight), against the oracle and with every child of a row rejected in turn."""
+"""Acceptance at vocabularies around the threads' and CTAs' shares of a row (4 entries a word; 65536 on eight CTAs are four words a thread;
+151936 and 212992 also ones that a real model has, or that took another path when rows were staged in shared memory), against the
+oracle and with every child of a row rejected in turn."""
 import numpy as np
 import pytest
 
