@@ -19,7 +19,7 @@ from . import binding as sv
 
 # What the schedule of a host-fed step reckons with: bytes per microsecond up, down, from HBM and by one CTA alone, microseconds per
 # chunk (its launches; the copies of a further one).  Fitted to the differences between the schedules of 184 stacks on two
-# machines (the sums come out 15 % high): a B200 on a PCIe 5 link, of which only the proportions matter here.
+# machines (the sums come out 4 % high on average): a B200 on a PCIe 5 link, of which only the proportions matter here.
 UP_RATE, DOWN_RATE, HBM_RATE, CTA_RATE, LAUNCH_US, COPY_US = 36e3, 57e3, 6.4e6, 76e3, 18.0, 18.0
 
 
