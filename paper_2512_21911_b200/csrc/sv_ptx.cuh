@@ -56,6 +56,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     return false;
 }
 
+// One lane of a converged warp, always the same one.  Where a warp's loop is uniform and one lane issues -- tcgen05.mma, commits, TMA:
+// instructions whose operands are uniform registers -- this, unlike `lane == 0`, says that there is one.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(one));
+    return one != 0;
+}
+
 // ---------------------------------------------------------------- thread-block clusters / distributed shared memory
 // address of the same shared-memory location in CTA `rank` of this cluster
 __device__ __forceinline__ uint32_t cluster_map_shared(uint32_t addr, uint32_t rank)

@@ -144,6 +144,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         return false;
     };
+    // the same for a whole warp that goes on together
+    auto warp_wait = [&](int slot, uint32_t parity) { return __all_sync(0xffffffffu, wait_for(slot, parity)) != 0; };
     // (kBal) a wait that may last as long as a segment; it ends early when somebody has given up
     auto long_wait = [&](int slot, uint32_t parity) {
         for (uint32_t i = 0; i < kLongWait; ++i) {
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // (they share those K/V tiles through L2; 1-2 % faster than group-major order).  A group is a row tile (kWide), or
     // a pair of row tiles (kPair) of which softmax warpgroup w owns tile 2 * group + w; `tile`, `i0`, `Tq`, `rows` are
     // those of the executing warpgroup (the query rows of draft tokens i0 .. i0 + Tq - 1).
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform, for all that hangs on it)
     const int n_groups = kPair ? (p.tiles + 1) / 2 : p.tiles;
     const int split = kBal ? 0 : kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, z = blockIdx.z;   // (kBal: per segment)
     // z numbers what the layer owns (q, out, draft, partials), s its sequence (tables, lengths, parents), lz its list
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         (which ? p.draft_v : p.draft_k) + (((size_t)z_d * p.T + r) * p.Hkv + h_d) * 128 + c * 8);
         }
     };
-    const uint32_t tmem_base = warp == 8 && !kBal ? 0u : *tmem_slot;
+    const uint32_t tmem_base = warp == 8 && !kBal ? 0u : __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     if (warp >= 8) {
         reg_dealloc<kRegsFew>();   // hand registers to the softmax warpgroups
@@ -325,15 +327,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint64_t policy = policy_evict_first();
                 const int sh = upb - 1;   // units of a block: 1 << sh
                 bool dead = false;
-                RingCopies copies;   // (lane 0's)
+                RingCopies copies;
                 grid_dependency_wait();   // the lists may come from the kernel just before
                 // A batch is 32 consecutive entries of one list, one per lane.  What the next segment needs -- its claim, count
                 // and first entries, their pages: three trips to L2, each needing the one before -- is fetched in steps
                 // between this segment's requests.
                 int ring = 0, draft_at = -1, layer_at = -1;
+                int stage = 0, turn = 0;   // of the next unit: ring % NS, ring / NS
+                auto next_stage = [&] {
+                    if (++stage == NS) stage = 0, ++turn;
+                };
+                auto give_up = [&] {
+                    dead = true;
+                    if (lane == 0) {
+                        *abort_flag = 1;
+                        if (p.status) atomicOr(p.status, 1);
+                    }
+                };
                 int claim = blockIdx.x;
                 Item cur = item_at(claim), nxt = cur;
-                int count = item_count(cur), L = p.seq_lens[cur.s];
+                auto uniform = [](int x) { return __shfl_sync(0xffffffffu, x, 0); };
+                int count = uniform(item_count(cur)), L = uniform(p.seq_lens[cur.s]);
                 int n_sel = blocks_of(count);
                 int blk_in = entry(cur, lane), page_in = page_of(cur, blk_in);
                 for (int seg = 0;; ++seg) {
@@ -355,13 +369,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                         if (step == 0) {
                             claim = claimed_list((uint32_t)__shfl_sync(0xffffffffu, claim, 0), p.n_claims, (int)gridDim.x);
                             // tell warp 11 (which has long noted the segment before this one)
-                            if (lane == 0 && !dead) {
+                            if (!dead) {
                                 const int at = (seg + 1) & 1;
-                                if (seg >= 2 && (*abort_flag || !long_wait(kClaimTaken + at, ((seg - 2) >> 1) & 1))) {
-                                    dead = true;
-                                    *abort_flag = 1;
-                                    if (p.status) atomicOr(p.status, 1);
-                                } else {
+                                if (seg >= 2 && !__all_sync(0xffffffffu, !*abort_flag && long_wait(kClaimTaken + at, ((seg - 2) >> 1) & 1))) {
+                                    give_up();
+                                } else if (lane == 0) {
                                     claims[at] = claim;
                                     mbar_arrive(bar(kClaim + at));
                                 }
@@ -387,22 +399,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                             if (i == n_here / 2 && more) page_in = page_of(cur, blk_in);
                             const int r0 = __shfl_sync(0xffffffffu, row0, i);
                             const int t0 = __shfl_sync(0xffffffffu, tok0, i);
-                            if (lane == 0 && !dead) {
-                                for (int uo = 0; uo < upb; ++uo) {
-                                    const int u = ring + ((base + i) << sh) + uo, stage = u % NS, it = u / NS;
-                                    if (it > 0 && (*abort_flag || !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
-                                        dead = true;
-                                        *abort_flag = 1;
-                                        if (p.status) atomicOr(p.status, 1);
-                                        break;
-                                    }
+                            for (int uo = 0; uo < upb && !dead; ++uo) {
+                                if (turn > 0 && !warp_wait(kEmpty + stage, (turn - 1) & 1)) {
+                                    give_up();
+                                    break;
+                                }
+                                copies.copied(stage, turn);
+                                if (elect_one()) {
                                     meta[stage] = max(0, min(kUnit, L - (t0 + uo * kUnit)));
                                     const uint32_t fb = bar(kFull + stage), dst = smem0 + stage * kStageBytes;
                                     mbar_arrive_expect_tx(fb, kStageBytes);
-                                    copies.copied(stage, it);
                                     tma_load_3d(dst, mk, 0, r0 + uo * kUnit, 0, fb, policy);
                                     tma_load_3d(dst + 2 * kTile, mv, 0, r0 + uo * kUnit, 0, fb, policy);
                                 }
+                                __syncwarp();
+                                next_stage();
                             }
                         }
                     }
@@ -411,25 +422,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                         // The draft unit's stage is filled by warp 11, which may be many rounds of the ring ahead; it is told
                         // when the stage is free.  A barrier's parity only tells neighbouring rounds apart, so nobody is let
                         // past a draft unit that is still on its way.
-                        if (lane == 0 && !dead) {
-                            const int stage = ring % NS, it = ring / NS;
-                            if (*abort_flag ||
-                                (draft_at >= 0 && ring - draft_at <= NS && !long_wait(kFull + draft_at % NS, (draft_at / NS) & 1)) ||
-                                (it > 0 && !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
-                                dead = true;
-                                *abort_flag = 1;
-                                if (p.status) atomicOr(p.status, 1);
+                        if (!dead) {
+                            const bool ok = !*abort_flag &&
+                                            !(draft_at >= 0 && ring - draft_at <= NS && !long_wait(kFull + draft_at % NS, (draft_at / NS) & 1)) &&
+                                            !(turn > 0 && !wait_for(kEmpty + stage, (turn - 1) & 1));
+                            if (!__all_sync(0xffffffffu, ok)) {
+                                give_up();
                             } else {
                                 copies.filled_otherwise(stage);
-                                mbar_arrive(bar(kSlot));
+                                if (lane == 0) mbar_arrive(bar(kSlot));
                             }
                         }
                         draft_at = ring++;
+                        next_stage();
                     }
                     while (step < 2) prepare_next();
                     // a CTA that has given up claims nothing more: the lists that are left go to the others
                     if (claim < 0 || __any_sync(0xffffffffu, dead || *abort_flag)) break;
-                    cur = nxt, count = count_next, n_sel = blocks_of(count), L = L_next, blk_in = blk_next, page_in = page_next;
+                    cur = nxt, count = uniform(count_next), n_sel = blocks_of(count), L = uniform(L_next), blk_in = blk_next, page_in = page_next;
                 }
                 if (lane == 0) {
                     __threadfence();   // (this CTA's claims are made before it leaves)
@@ -465,9 +475,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             int blk_spec = 0;
             if (p.sel_idx && j0_spec + lane < p.max_sel)
                 blk_spec = p.sel_idx[((size_t)lz * p.Hkv + h) * p.max_sel + j0_spec + lane];
-            const int L = p.seq_lens[s];
+            const int L_in = p.seq_lens[s];
+            const int cnt_list = p.sel_idx ? p.sel_cnt[(size_t)lz * p.Hkv + h] : 0;
+            const int L = __shfl_sync(0xffffffffu, L_in, 0);
             const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-            const int cnt_in = p.sel_idx ? p.sel_cnt[(size_t)lz * p.Hkv + h] : nb;
+            const int cnt_in = p.sel_idx ? __shfl_sync(0xffffffffu, cnt_list, 0) : nb;
             // a negative count marks a list that block selection could not produce: attend over the draft tokens
             // only, and say so
             if (cnt_in < 0 && lane == 0 && p.status) atomicOr(p.status, kStatusNoList);
@@ -475,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // blocks j0 .. j1 - 1 of the list; kUnitSlices: units u0 .. u1 - 1 of the list, which those blocks hold
             const int u0 = slice_begin(split, n_sel), u1 = slice_begin(split + 1, n_sel);
             const int j0 = kUnitSlices ? u0 >> 1 : u0, j1 = kUnitSlices ? (u1 + 1) >> 1 : u1;
-            const int off = has_draft ? 1 : 0;
+            int stage = has_draft ? 1 : 0, turn = 0;   // of the next unit (the draft unit, if any, came first)
             bool dead = false;
             for (int base = j0; base < j1; base += 32) {
                 const int j = base + lane;
@@ -497,21 +509,20 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int i = 0; i < n_here; ++i) {
                     const int r0 = __shfl_sync(0xffffffffu, row0, i);
                     const int t0 = __shfl_sync(0xffffffffu, tok0, i);
-                    if (lane == 0 && !dead) {
-                        const int ub = 2 * (base + i);   // (kUnitSlices) first unit of the block
-                        for (int uo = kUnitSlices ? max(0, u0 - ub) : 0; uo < (kUnitSlices ? min(2, u1 - ub) : upb); ++uo) {
-                            // ring unit; the draft unit (if any) came first
-                            const int u = kUnitSlices ? ub + uo - u0 : (base - j0 + i) * upb + uo;
-                            const int stage = (u + off) % NS, it = (u + off) / NS;
-                            if (it > 0 && (*abort_flag || !mbar_wait_bounded(bar(kEmpty + stage), (it - 1) & 1))) {
-                                dead = true;
+                    const int ub = 2 * (base + i);   // (kUnitSlices) first unit of the block
+                    const int uo0 = kUnitSlices ? max(0, u0 - ub) : 0, uo1 = kUnitSlices ? min(2, u1 - ub) : upb;
+                    for (int uo = uo0; uo < uo1 && !dead; ++uo) {
+                        if (turn > 0 && !warp_wait(kEmpty + stage, (turn - 1) & 1)) {
+                            dead = true;
+                            if (lane == 0) {
                                 *abort_flag = 1;
                                 if (p.status) atomicOr(p.status, 1);
-                                requested[0] = u + off;
-                                break;
+                                requested[0] = turn * NS + stage;
                             }
-                            const int nvalid = max(0, min(kUnit, L - (t0 + uo * kUnit)));
-                            meta[stage] = nvalid;
+                            break;
+                        }
+                        if (elect_one()) {
+                            meta[stage] = max(0, min(kUnit, L - (t0 + uo * kUnit)));
                             const uint32_t fb = bar(kFull + stage);
                             const uint32_t dst = smem0 + stage * kStageBytes;
                             const int y = r0 + uo * kUnit;
@@ -523,6 +534,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                             tma_load_3d(dst, mk, 0, y, 0, fb, policy);
                             tma_load_3d(dst + 2 * kTile, mv, 0, y, 0, fb, policy);
                         }
+                        __syncwarp();
+                        if (++stage == NS) stage = 0, ++turn;
                     }
                 }
             }
@@ -614,68 +627,74 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ring += n_total;
             }
         } else if (warp == 9 || warp == 10 || kTwoS) {
-            // ---------------------------------------------------------- MMA issuers (one thread each)
+            // ---------------------------------------------------------- MMA issuers (one lane of each warp, whose loop is uniform)
+            // All lanes wait and count, one that elect.sync names issues (as in the producer).  With the whole loop behind `lane == 0`
+            // every MMA, commit and copy was compiled for any set of lanes, and a CTA took 1250-1360 cycles per unit even with all K/V in
+            // L2, whatever its rows: 32 layers of 8 lists of 65 units 115.6 -> 110.6 us, 16 layers x 4 sequences 165.7 -> 158.6, dense 32K
+            // 28.6 -> 27.7, dense 4 x 128K 459 -> 422, 16 ragged sequences 31.8 -> 30.8, 12 trees of 240 rows 96.9 -> 94.8.
             // warp 9 issues every S = Q K^T (kTwoS: of warpgroup 0, warp 11 of warpgroup 1) and owns the TMEM allocation; warp
             // 10 issues every Ou = P V.
             // Descriptors are built once; per instruction only the 14-bit address field moves.
-            if (lane == 0) {
-                int n_total = 0;
-                bool dead = false;
-                if constexpr (!kBal) {
-                    grid_dependency_wait();   // the lengths may come from the kernel just before (a cache commit)
-                    const int L = p.seq_lens[s];
-                    const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
-                    const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
-                    const int off = has_draft ? 1 : 0;
-                    n_total = slice_units(split, n_sel) + off;
-                    dead = !mbar_wait_bounded(bar(kStaged), 0);
+            int n_total = 0;
+            bool dead = false;
+            if constexpr (!kBal) {
+                grid_dependency_wait();   // the lengths may come from the kernel just before (a cache commit)
+                const int L = p.seq_lens[s];
+                const int nb = min(p.B == 128 ? (L + 127) >> 7 : (L + 63) >> 6, p.NBmax);
+                const int n_sel = p.sel_idx ? max(0, min(p.sel_cnt[(size_t)lz * p.Hkv + h], p.max_sel)) : nb;
+                const int off = has_draft ? 1 : 0;
+                n_total = __shfl_sync(0xffffffffu, slice_units(split, n_sel) + off, 0);
+                dead = !warp_wait(kStaged, 0);
+            }
+            // (kBal) per segment: its units, and what came before it: ring units, units of either warpgroup
+            int ring = 0, done0 = 0, done1 = 0;
+            bool end = false;
+            auto give_up = [&](int bit) {
+                dead = true;
+                if (lane == 0) {
+                    *abort_flag = 1;
+                    if (p.status) atomicOr(p.status, bit);
                 }
-                // (kBal) per segment: its units, and what came before it: ring units, units of either warpgroup
-                int ring = 0, done0 = 0, done1 = 0;
-                bool end = false;
-                auto next_segment = [&](int seg) {
-                    bool ok = !*abort_flag && long_wait(kLoaded, seg & 1);
-                    if (ok) {
-                        n_total = segments[seg & 1].n_total;
-                        end = n_total < 0;
-                        if (!end) mbar_arrive(bar(kTaken));
-                    } else {
-                        dead = true;
-                        *abort_flag = 1;
-                        if (p.status) atomicOr(p.status, 8);
+            };
+            auto next_segment = [&](int seg) {
+                if (__all_sync(0xffffffffu, !*abort_flag && long_wait(kLoaded, seg & 1))) {
+                    n_total = __shfl_sync(0xffffffffu, segments[seg & 1].n_total, 0);
+                    end = n_total < 0;
+                    if (!end && lane == 0) mbar_arrive(bar(kTaken));
+                } else {
+                    give_up(8);
+                }
+            };
+            auto end_segment = [&] {
+                ring += n_total;
+                done0 += (n_total + 1) >> 1;
+                done1 += n_total >> 1;
+            };
+            if (warp == 9 || (kTwoS && warp == 11)) {
+                constexpr uint32_t idesc_s = umma_idesc_bf16(MT, kUnit, false);
+                const uint64_t dq = umma_desc_sw128(smem0 + OFFQ, 16, 1024);
+                const uint64_t dk = umma_desc_sw128(smem0, 16, 1024);
+                const uint32_t dq_lo = (uint32_t)dq, dk_lo = (uint32_t)dk;
+                const uint64_t d_hi = dq & 0xFFFFFFFF00000000ull;
+                for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
+                if constexpr (kBal) {
+                    next_segment(seg);
+                    if (end || dead) break;
+                }
+                // one S per (unit, warpgroup that takes it): the warpgroups alternate units, or (kPair) each takes all
+                const int g_mine = kTwoS && warp == 11 ? 1 : 0;
+                const int step = kTwoS && !kPair ? 2 : 1;
+                const int u_end = kPair && g_mine == 1 && n_wg == 1 ? 0 : n_total;
+                for (int u = kPair ? 0 : g_mine, stage = (u + ring) % NS, turn = (u + ring) / NS; u < u_end && !dead; u += step) {
+                    const int g = kTwoS ? g_mine : u & 1, k = kPair ? u : (u >> 1) + (g ? done1 : done0);
+                    if (!warp_wait(kFull + stage, turn & 1) || (k > 0 && !warp_wait(kSFree + g, (k - 1) & 1))) {
+                        give_up(8);
+                        break;
                     }
-                };
-                auto end_segment = [&] {
-                    ring += n_total;
-                    done0 += (n_total + 1) >> 1;
-                    done1 += n_total >> 1;
-                };
-                if (warp == 9 || (kTwoS && warp == 11)) {
-                    constexpr uint32_t idesc_s = umma_idesc_bf16(MT, kUnit, false);
-                    const uint64_t dq = umma_desc_sw128(smem0 + OFFQ, 16, 1024);
-                    const uint64_t dk = umma_desc_sw128(smem0, 16, 1024);
-                    const uint32_t dq_lo = (uint32_t)dq, dk_lo = (uint32_t)dk;
-                    const uint64_t d_hi = dq & 0xFFFFFFFF00000000ull;
-                    for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
-                    if constexpr (kBal) {
-                        next_segment(seg);
-                        if (end || dead) break;
-                    }
-                    // one S per (unit, warpgroup that takes it): the warpgroups alternate units, or (kPair) each takes all
-                    const int g_mine = kTwoS && warp == 11 ? 1 : 0;
-                    const int step = kTwoS && !kPair ? 2 : 1;
-                    const int u_end = kPair && g_mine == 1 && n_wg == 1 ? 0 : n_total;
-                    for (int u = kPair ? 0 : g_mine, stage = (u + ring) % NS, turn = (u + ring) / NS; u < u_end && !dead; u += step) {
-                        const int g = kTwoS ? g_mine : u & 1, k = kPair ? u : (u >> 1) + (g ? done1 : done0);
-                        if (!wait_for(kFull + stage, turn & 1) || (k > 0 && !wait_for(kSFree + g, (k - 1) & 1))) {
-                            dead = true;
-                            *abort_flag = 1;
-                            if (p.status) atomicOr(p.status, 8);
-                            break;
-                        }
-                        tc_fence_after_sync();
-                        const uint32_t k_lo = dk_lo + (uint32_t)((stage * kStageBytes) >> 4);
-                        const uint32_t d = tmem_base + g * kUnit;
+                    tc_fence_after_sync();
+                    const uint32_t k_lo = dk_lo + (uint32_t)((stage * kStageBytes) >> 4);
+                    const uint32_t d = tmem_base + g * kUnit;
+                    if (elect_one()) {
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {
                             const uint32_t qo = (uint32_t)(((kPair ? g * kQBytes : 0) + (kBal ? (seg & 1) * 8192 : 0) + (ks >> 2) * (kQBytes / 2) + (ks & 3) * 32) >> 4);
@@ -686,51 +705,54 @@ __global__ void __launch_bounds__(kThreads, 1)
                                 tc_mma_bf16(d, d_hi | (dq_lo + qo), d_hi | (k_lo + ko), idesc_s, ks > 0);
                         }
                         tc_commit(bar(kSReady + g));
-                        stage += step;
-                        if (stage >= NS) stage -= NS, ++turn;
                     }
-                    if constexpr (kBal) end_segment();
+                    __syncwarp();
+                    stage += step;
+                    if (stage >= NS) stage -= NS, ++turn;
+                }
+                if constexpr (kBal) end_segment();
+                }
+                if (elect_one()) tc_commit(bar(kTmemDone));
+                if (warp == 11) return;
+                // free TMEM only after every softmax warp has finished reading it and every MMA is through
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar(kTmemDone), 0, kLongWait)) && lane == 0) {
+                    *abort_flag = 1;
+                    if (p.status) atomicOr(p.status, 16);
+                }
+                __syncwarp();
+                if (*abort_flag) {
+                    const uint32_t word = requested[0];
+                    const RingCopies copies = kBal ? RingCopies{word, requested[1]}
+                                                   : copies_of_units(has_draft ? 1 : 0, word == ~0u ? n_total : (int)word, NS);
+                    for (int stage = 0; stage < NS; ++stage)
+                        if (copies.waits_for(stage) && !mbar_wait_bounded(bar(kFull + stage), copies.parity(stage), kLongWait) && lane == 0 && p.status)
+                            atomicOr(p.status, 1);
+                }
+            } else {
+                constexpr uint32_t idesc_pv = umma_idesc_bf16(MT, 128, true);
+                const uint64_t dp = umma_desc_sw128(smem0 + kOffP, 16, 1024);
+                const uint64_t dv = umma_desc_sw128(smem0 + 2 * kTile, kTile, 1024);
+                const uint32_t dp_lo = (uint32_t)dp, dv_lo = (uint32_t)dv;
+                const uint64_t dp_hi = dp & 0xFFFFFFFF00000000ull, dv_hi = dv & 0xFFFFFFFF00000000ull;
+                for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
+                if constexpr (kBal) {
+                    next_segment(seg);
+                    if (end || dead) break;
+                }
+                const int n_issue = kPair ? n_total * n_wg : n_total;
+                for (int x = 0, stage = ring % NS; x < n_issue && !dead; ++x) {
+                    const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
+                    const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = kPair ? u : (u >> 1);
+                    if (!warp_wait(kPReady + g, (k + (g ? done1 : done0)) & 1)) {
+                        give_up(32);
+                        break;
                     }
-                    tc_commit(bar(kTmemDone));
-                    if (warp == 11) return;
-                    // free TMEM only after every softmax warp has finished reading it and every MMA is through
-                    if (!mbar_wait_bounded(bar(kTmemDone), 0, kLongWait)) {
-                        *abort_flag = 1;
-                        if (p.status) atomicOr(p.status, 16);
-                    }
-                    if (*abort_flag) {
-                        const uint32_t word = requested[0];
-                        const RingCopies copies = kBal ? RingCopies{word, requested[1]}
-                                                       : copies_of_units(has_draft ? 1 : 0, word == ~0u ? n_total : (int)word, NS);
-                        for (int stage = 0; stage < NS; ++stage)
-                            if (copies.waits_for(stage) && !mbar_wait_bounded(bar(kFull + stage), copies.parity(stage), kLongWait) && p.status)
-                                atomicOr(p.status, 1);
-                    }
-                } else {
-                    constexpr uint32_t idesc_pv = umma_idesc_bf16(MT, 128, true);
-                    const uint64_t dp = umma_desc_sw128(smem0 + kOffP, 16, 1024);
-                    const uint64_t dv = umma_desc_sw128(smem0 + 2 * kTile, kTile, 1024);
-                    const uint32_t dp_lo = (uint32_t)dp, dv_lo = (uint32_t)dv;
-                    const uint64_t dp_hi = dp & 0xFFFFFFFF00000000ull, dv_hi = dv & 0xFFFFFFFF00000000ull;
-                    for (int seg = 0; kBal ? !dead : seg < 1; ++seg) {
-                    if constexpr (kBal) {
-                        next_segment(seg);
-                        if (end || dead) break;
-                    }
-                    const int n_issue = kPair ? n_total * n_wg : n_total;
-                    for (int x = 0, stage = ring % NS; x < n_issue && !dead; ++x) {
-                        const int u = kPair ? (n_wg == 2 ? x >> 1 : x) : x;
-                        const int g = kPair ? (n_wg == 2 ? (x & 1) : 0) : (u & 1), k = kPair ? u : (u >> 1);
-                        if (!wait_for(kPReady + g, (k + (g ? done1 : done0)) & 1)) {
-                            dead = true;
-                            *abort_flag = 1;
-                            if (p.status) atomicOr(p.status, 32);
-                            break;
-                        }
-                        tc_fence_after_sync();
-                        const uint32_t v_lo = dv_lo + (uint32_t)((stage * kStageBytes) >> 4);
-                        const uint32_t p_lo = dp_lo + (uint32_t)((g * kPBytes) >> 4);
-                        const uint32_t d = tmem_base + 128 + g * 128;
+                    tc_fence_after_sync();
+                    const uint32_t v_lo = dv_lo + (uint32_t)((stage * kStageBytes) >> 4);
+                    const uint32_t p_lo = dp_lo + (uint32_t)((g * kPBytes) >> 4);
+                    const uint32_t d = tmem_base + 128 + g * 128;
+                    const bool last_reader = !kPair || g == n_wg - 1;   // of the stage
+                    if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {   // (the warpgroup's first unit starts O)
                             if constexpr (kPTmem)   // A = P from tensor memory: 16 keys = 8 packed columns per instruction
@@ -741,15 +763,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                                             idesc_pv, (k > 0 || kk > 0) ? 1u : 0u);
                         }
                         tc_commit(bar(kOReady + g));
-                        if (!kPair || g == n_wg - 1) {   // the last reader of the stage
-                            tc_commit(bar(kEmpty + stage));
-                            if (++stage == NS) stage = 0;
-                        }
+                        if (last_reader) tc_commit(bar(kEmpty + stage));
                     }
-                    if constexpr (kBal) end_segment();
-                    }
-                    tc_commit(bar(kTmemDone));   // (arrives behind the last PV that was issued)
+                    __syncwarp();
+                    if (last_reader && ++stage == NS) stage = 0;
                 }
+                if constexpr (kBal) end_segment();
+                }
+                if (elect_one()) tc_commit(bar(kTmemDone));   // (arrives behind the last PV that was issued)
             }
             if (warp == 9) {
                 __syncwarp();
