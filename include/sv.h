@@ -449,7 +449,8 @@ SV_API sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom *geo
                                           void *workspace, size_t workspace_bytes, int32_t *status_word, int32_t refresh_tail,
                                           const uint8_t *refresh_which, void *stream_in, void *stream_out, void *stream);
 
-/* Number of KV splits (CTAs per (sequence, KV head)) sv_verify_attn uses for this geometry. */
+/* Number of KV splits (CTAs per (sequence, KV head)) that the workspace of this geometry has room for.  sv_verify_attn uses as many, or
+ * fewer where the CTAs of a thread-block cluster merge their splits themselves (the workspace is then not written). */
 SV_API int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel);
 
 #ifdef __cplusplus

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "sv.h"
+#include "sv_ptx.cuh"
 
 namespace svk {
 
@@ -43,6 +44,7 @@ struct AttnParams {
     int n_pages;     // pages in each pool: page ids from the block table are clamped to it
     int n_claims;       // > 0: that many lists are handed out to one CTA per SM (splits = 1)
     uint32_t *claims;   // ... through these two words (list_claims.h), zero before and after the launch
+    int cluster;     // 1: the splits of a (sequence, KV head) are a cluster that merges them itself (no partials, no merge kernel)
     int early_gather;   // 1: nothing the gather reads comes from the kernel just before; it starts ahead of the dependency wait
 };
 
@@ -53,6 +55,42 @@ struct StackAttnParams : AttnParams {
     int S;                            // sequences of a layer
     uint8_t list_of[SV_MAX_LAYERS];   // block list of a layer: the ordinal of the last anchor up to it
 };
+
+// The sum over the splits of a row, four output dims: o = sum_j 2^(m_j - m) o_j / sum_j 2^(m_j - m) l_j, a batch of splits at a time.
+struct SplitSum {
+    float M = -INFINITY, l = 0.f;
+    float4 acc = {0.f, 0.f, 0.f, 0.f};
+    template <int U>
+    __device__ void add(const float2 (&ml)[U], const float4 (&o)[U])
+    {
+        float Mb = M;
+#pragma unroll
+        for (int u = 0; u < U; ++u) Mb = fmaxf(Mb, ml[u].x);
+        const float M_use = (Mb == -INFINITY) ? 0.f : Mb;
+        const float c = fast_exp2(M - M_use);   // rescale what earlier batches accumulated
+        acc.x *= c, acc.y *= c, acc.z *= c, acc.w *= c;
+        l *= c;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const float w = fast_exp2(ml[u].x - M_use);
+            acc.x += w * o[u].x, acc.y += w * o[u].y, acc.z += w * o[u].z, acc.w += w * o[u].w;
+            l += w * ml[u].y;
+        }
+        M = Mb;
+    }
+    __device__ uint2 out() const
+    {
+        const float inv = 1.f / l;
+        return make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+    }
+    __device__ float lse() const { return (M + log2f(l)) * 0.69314718055994531f; }
+};
+
+constexpr int kMaxCluster = 8;   // CTAs of a cluster that merges its splits (the portable size)
+// Whether a cluster of `splits` CTAs has room for each other's partials of `rows` query rows, and how many clusters of a size the
+// device runs at once (0: none, or no device).
+bool cluster_holds_partials(int splits, int rows);
+int clusters_at_once(int size);
 
 // tcgen05 / TMEM attention kernel (verify_attn_tc.cu): rows = G*T <= 128 packed as one M=128 tile.
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid,

@@ -85,6 +85,12 @@ __device__ __forceinline__ void st_async_cluster_v4(uint32_t addr, uint4 v, uint
                  "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(remote_bar)
                  : "memory");
 }
+__device__ __forceinline__ void st_async_cluster_v2(uint32_t addr, uint2 v, uint32_t remote_bar)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(addr), "r"(v.x),
+                 "r"(v.y), "r"(remote_bar)
+                 : "memory");
+}
 __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint32_t bar, uint32_t parity, uint32_t limit = (1u << 19))
 {
     for (uint32_t i = 0; i < limit; ++i) {

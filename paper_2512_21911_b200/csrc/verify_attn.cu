@@ -53,8 +53,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_splits_kernel(const AttnP
     const size_t sh = (size_t)s * p.Hkv + h;
     const float2 *ml = reinterpret_cast<const float2 *>(p.ws_ml) + sh * p.splits * rows + row;
     const float4 *po = reinterpret_cast<const float4 *>(p.ws_o) + (sh * p.splits * rows + row) * 32 + c4;
-    float M = -INFINITY, lsum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    SplitSum sum;
     for (int j0 = 0; j0 < p.splits; j0 += U) {
         float2 mlv[U];
         float4 ov[U];
@@ -64,29 +63,12 @@ __global__ void __launch_bounds__(kMergeThreads) merge_splits_kernel(const AttnP
             mlv[u] = in ? ml[(size_t)(j0 + u) * rows] : make_float2(-INFINITY, 0.f);
             ov[u] = in ? po[(size_t)(j0 + u) * rows * 32] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        float Mb = M;
-#pragma unroll
-        for (int u = 0; u < U; ++u) Mb = fmaxf(Mb, mlv[u].x);
-        const float M_use = (Mb == -INFINITY) ? 0.f : Mb;
-        const float c = fast_exp2(M - M_use);   // rescale what earlier batches accumulated
-        acc.x *= c, acc.y *= c, acc.z *= c, acc.w *= c;
-        lsum *= c;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const float w = fast_exp2(mlv[u].x - M_use);
-            acc.x += w * ov[u].x, acc.y += w * ov[u].y, acc.z += w * ov[u].z, acc.w += w * ov[u].w;
-            lsum += w * mlv[u].y;
-        }
-        M = Mb;
+        sum.add(mlv, ov);
     }
     const int i = row / p.G, g = row - i * p.G;
     const size_t orow = ((size_t)s * p.T + i) * p.Hq + h * p.G + g;
-    const float inv = 1.f / lsum;
-    uint2 pk;
-    pk.x = pack_bf16(acc.x * inv, acc.y * inv);
-    pk.y = pack_bf16(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2 *>(p.out + orow * 128 + c4 * 4) = pk;
-    if (p.lse && c4 == 0) p.lse[orow] = (M + log2f(lsum)) * 0.69314718055994531f;
+    *reinterpret_cast<uint2 *>(p.out + orow * 128 + c4 * 4) = sum.out();
+    if (p.lse && c4 == 0) p.lse[orow] = sum.lse();
 }
 
 // ---------------------------------------------------------------------- host side
@@ -179,6 +161,32 @@ int choose_splits(const sv_geom *g, int n_blocks, bool balance = true)
     return (n_blocks + blocks_per_cta - 1) / blocks_per_cta;
 }
 
+// CTAs of a cluster that takes such a list and merges its splits itself (verify_attn_tc.cu, kCluster), or 0: the splits of
+// choose_splits, merged by a kernel.  What it saves is the merge kernel: its launch, two boundaries and the trip of the partials through
+// L2, 2.5 us where the host's launches are the limit (2 KV heads x 16 units, selection and attention: 13.8 -> 11.25 us) and
+// 0.5 to 2 us on the device (4 sequences x 8 heads x 32 units, 32 rows: 18.1 -> 16.5).  All clusters have to be resident together: a GPC's
+// SMs hold 33 clusters of four, 22 of six, 15 of eight CTAs.
+// Where that, or the eight CTAs of a portable cluster, leaves fewer splits, each has more units: up to kMoreUnits more pay with up to
+// 64 rows (16 pairs x 100 units in 6 instead of 9: 20.0 -> 19.0; 8 more do not: 8 pairs x 128 in 8 instead of 16, 16.2 -> 17.0).
+// A 128-row tile pushes 64 KB per CTA: with two CTAs a cluster is faster (64 pairs x 32 units 28.3 -> 27.25), with four about
+// equal (28.9 and 28.8; 18.4 and 18.8), with fewer splits slower (16 pairs, 80 rows, 6 instead of 8: 17.0 -> 17.2).
+// Slices of more than kLongSlice units are left to the merge kernel: CTAs that run for long end further apart, and a cluster's SMs are
+// idle until the last of its CTAs has ended (32 pairs x 257 units, 44.2 -> 44.8 us).
+constexpr int kMoreUnits = 5, kLongSlice = 48;
+int choose_cluster(const sv_geom *g, int n_blocks, int splits)
+{
+    const int rows = g->n_q_heads / g->n_kv_heads * g->n_draft, pairs = g->n_seq * g->n_kv_heads;
+    if (splits < 2 || svh::row_tiles(g) > 1 || g->n_draft > 32 || pairs > sm_count() / 2) return 0;
+    if (rows > 64 && splits > 2) return 0;
+    const int upb = g->block_size / kUnit, split_blocks = (n_blocks + splits - 1) / splits;
+    for (int most = std::min(splits, kMaxCluster); most > 1; --most) {
+        const int blocks = (n_blocks + most - 1) / most, c = (n_blocks + blocks - 1) / blocks;
+        if ((blocks - split_blocks) * upb > kMoreUnits || blocks * upb > kLongSlice) return 0;
+        if (cluster_holds_partials(c, rows) && clusters_at_once(c) >= pairs) return c;
+    }
+    return 0;
+}
+
 }  // namespace
 
 extern "C" int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel)
@@ -227,6 +235,9 @@ static void fill_params(AttnParams &p, const sv_geom *geom, const sv_geom *rule,
     p.NBmax = geom->max_blocks, p.max_sel = max_sel, p.splits = splits;
     p.Tt = svh::tokens_per_tile(geom), p.tiles = svh::row_tiles(geom);
     p.pair = svh::pair_row_tiles(rule) ? 1 : 0;
+    const int cluster = choose_cluster(rule, max_sel, splits);
+    p.cluster = cluster > 1;
+    if (p.cluster) p.splits = cluster;
     p.early_gather = 0;
     p.n_claims = 0, p.claims = nullptr;
     const float scale = softmax_scale > 0.f ? softmax_scale : 0.08838834764831845f;   // 1/sqrt(128)
@@ -241,7 +252,7 @@ static sv_status launch_attn(Params &p, const sv_geom *rule, int n_batch, cudaSt
     p.ws_ml = p.ws_o ? p.ws_o + (size_t)n_batch * p.Hkv * p.splits * rows * 128 : nullptr;
     const dim3 grid(p.splits * svh::row_groups(rule), p.Hkv, n_batch);   // one CTA per (row tile or pair of row tiles, split)
     if (attend(grid) != cudaSuccess) return SV_ERR_CUDA;
-    if (p.splits > 1) {
+    if (p.splits > 1 && !p.cluster) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((rows * 32 + kMergeThreads - 1) / kMergeThreads, p.Hkv, n_batch);
         cfg.blockDim = dim3(kMergeThreads);

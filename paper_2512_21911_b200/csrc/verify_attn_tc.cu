@@ -33,6 +33,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "attn_common.cuh"
@@ -57,9 +58,9 @@ constexpr int kOffP = kStages * kStageBytes + kQBytes;   // (= 4 stages + 2 Q ti
 constexpr int kOffDraft = 0;                     // the draft unit is the first occupant of ring stage 0 (last split only)
 constexpr int kOffMisc = kOffP + 2 * kPBytes;
 constexpr int kSmemBytes = 1024 + kOffMisc + 1024;
-constexpr int kSmemBytesBal = kSmemBytes + 1024;   // (kBal) two sets of masks, segment descriptors
+constexpr int kSmemBytesBal = kSmemBytes + 1024;   // (kBal) two sets of masks, segment descriptors; (kCluster) the partials' (m, l)
 static_assert(kSmemBytesBal <= 232448, "shared memory budget");
-static_assert(2 * kMaxStages + 17 <= 32, "one lane of the producer warp per barrier");
+static_assert(2 * kMaxStages + 18 <= 32, "one lane of the producer warp per barrier");
 static_assert((kStages - 1) * kStageBytes + 2 * kQBytes == kOffP, "both layouts put P at the same offset");
 constexpr int kTmemCols = 512;                   // S: 2 x 64 columns, O: 2 x 128 columns; 128-row tiles also P: 2 x 32 and
                                                  // Q: 64, or (two row tiles per CTA) Q: 2 x 64
@@ -81,7 +82,8 @@ enum Bar {
     kSlot = kTaken + 1,         // (kBal) the stage of the next draft unit is free
     kClaim = kSlot + 1,         // (kBal) [2] the segment after next is known (segments take the two in turn)
     kClaimTaken = kClaim + 2,   // (kBal) [2] ... and warp 11 has noted it
-    kNumBars = kClaimTaken + 2
+    kReceived = kClaimTaken + 2,   // (kCluster) the other CTAs' partials of this CTA's rows are in shared memory
+    kNumBars = kReceived + 1
 };
 
 // (kBal) One segment: the list of a (layer, sequence, KV head) and its draft tokens.
@@ -114,7 +116,12 @@ struct ClaimWords {
 // of 8 lists of 65 units: 112.5 -> 106.9 us per step; 64 x 8 lists of 49 units: 155.7 -> 143.6).  Cutting lists so that all CTAs
 // end together costs more than it gains: the CTAs that are left have the HBM bandwidth to themselves, and partials have
 // to be written and merged (117 and 149 us).
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal>
+// kCluster (one row tile): the CTAs of a (sequence, KV head) are a thread-block cluster that merges its splits itself: no partials in
+// memory, no merge kernel.  CTA r writes the r-th share of the rows; the others push their partials of these rows into its
+// shared memory with stores that count their bytes on a barrier there, so that nothing but the data is waited for (two cluster
+// barriers around a pull, as this was first tried, cost what the merge kernel does).  Bound by latency: readout, the push, one wait.  A layer of
+// 2 KV heads x 16 units 12.0 -> 9.9 us (launches), 4 sequences x 8 heads x 32 units, 32 rows 18.1 -> 16.5, 64 pairs x 32 units 22.4 -> 21.2.
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                           const std::conditional_t<kStack, StackAttnParams, AttnParams> p)
@@ -155,6 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         return false;
     };
 
+    static_assert(!kCluster || (!kWide && !kBal), "clusters merge a single row tile of up to 32 draft tokens");
     static_assert(!kBal || (kStack && NH < 4), "lists are handed out for stacks, in tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
     // 128-row tiles are bound by the tensor pipe when every MMA fetches both operands from shared memory (S = Q K^T: eight
@@ -240,6 +248,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     const float inv_g = 1.f / (float)p.G;
     auto div_g = [&](int r) { return (int)(((float)r + 0.5f) * inv_g); };
+    // (kCluster) Rows share_begin(r) .. + share_rows(r) - 1 are written by CTA r.  Its shared memory takes a partial per other CTA
+    // (share x 512 bytes each, in the order of the ranks) in the ring stage behind its last unit, with 128-row tiles in the Q
+    // tile first (which is in tensor memory by then); a peer that is done first waits for these to be free at the cluster's barrier.
+    const int share = kCluster ? (rows + p.splits - 1) / p.splits : 1;
+    auto share_rows = [&](int r) { return max(0, min(share, rows - r * share)); };
     // The TMA producer warp initialises the barriers and runs ahead; everybody else meets it at a named
     // barrier (the producer only arrives), with the TMEM allocation done by warp 9 on the way.
     if (warp == 8) {
@@ -252,6 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == kTaken) count = na0 + (n_wg == 2 ? na1 : 0) + 2;   // the softmax warps and both issuers
             mbar_init(bar(lane), count);
             mbar_fence_init();
+            if (kCluster && lane == kReceived) mbar_arrive_expect_tx(bar(kReceived), (p.splits - 1) * share_rows(split) * (512 + 8));
         }
         if (lane == 0) *abort_flag = 0, requested[0] = kBal ? 0u : ~0u, requested[1] = 0;
         __syncwarp();
@@ -319,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp >= 8) {
         reg_dealloc<kRegsFew>();   // hand registers to the softmax warpgroups
+        if (kCluster && warp != 8) cluster_arrive();
         if (warp == 8) {
             // ---------------------------------------------------------- TMA producer
             const CUtensorMap *mk = &tm_k, *mv = &tm_v;
@@ -540,6 +555,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             if (lane == 0) mbar_arrive(bar(kTmemDone));
+            if constexpr (kCluster) {   // the stage that peers write to is free (as far as this CTA gets)
+                if (turn > 0 && !dead) warp_wait(kEmpty + stage, (turn - 1) & 1);
+                __syncwarp();
+                cluster_arrive();
+            }
         } else if (kBal && warp == 11) {
             // ---------------------------------------------------------- (kBal) segments: descriptor, Q tile, masks, draft unit
             int ring = 0, n_drafts = 0;
@@ -713,7 +733,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if constexpr (kBal) end_segment();
                 }
                 if (elect_one()) tc_commit(bar(kTmemDone));
-                if (warp == 11) return;
+                if (warp == 11) {
+                    if constexpr (kCluster) cluster_wait();
+                    return;
+                }
                 // free TMEM only after every softmax warp has finished reading it and every MMA is through
                 if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar(kTmemDone), 0, kLongWait)) && lane == 0) {
                     *abort_flag = 1;
@@ -777,6 +800,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc_fence_after_sync();
                 tmem_dealloc(tmem_base, kTmemCols);
             }
+        }
+        if constexpr (kCluster) {   // (every warp waits once for what it has arrived at)
+            __syncwarp();
+            cluster_wait();
         }
         return;
     }
@@ -886,6 +913,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!kBal && has_draft && tid == 0) mbar_arrive(bar(kFull + 0));   // the draft unit fills stage 0 in place of a TMA load
 
     const int wg = warp >> 2, quad = warp & 3;
+    if constexpr (kCluster) {
+        __syncwarp();
+        cluster_arrive();
+        if (quad >= n_active) cluster_wait();
+    }
     if (quad >= n_active) return;                                 // this warp's TMEM lanes hold padding only
     const int qd = lane & 3, lr = lane >> 2;
     const uint32_t t_lane = (uint32_t)(quad * 32) << 16;
@@ -1260,6 +1292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // a warpgroup without units never wrote its accumulator
     const bool have_mine = k > 0 && !dead, have_other = !kPair && n_total >= (wg == 0 ? 2 : 1);
     const uint32_t t_o_other = tmem_base + t_lane + 128 + (wg ^ 1) * 128;
+    if constexpr (kCluster) cluster_wait();   // every CTA's place for the partials is free
     bool stop = !kBal;
     const int out_z = kBal ? seg_item / p.Hkv : z, out_h = kBal ? seg_item - out_z * p.Hkv : h;
     for (int ch = kPair ? 0 : wg; ch < (kPair ? 2 : wg + 1); ++ch) {   // column half: 64 output dims
@@ -1308,6 +1341,40 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < NH; ++i) {
             const float M = row_m[i], lsum = row_l[i];
             const int row = lrow[i];
+            if constexpr (kCluster) {
+                // Lanes that differ in their lowest bit swap halves, for stores of 16 bytes: the even lane has columns 8 j + 2 qd .. + 3
+                // of the even j, the odd one those of the odd j.
+                const int r = min((int)(((float)row + 0.5f) / (float)share), p.splits - 1), local = row - r * share;
+                const bool mine = r == split;
+                const int src = split - (split > r);   // among the partials r receives
+                const int n_r = slice_units(r, n_sel) + (r == p.splits - 1);
+                const int in_q = NH == 4 ? kQBytes / (share * 512) : 0;
+                const uint32_t at = mine ? (uint32_t)((n_total + 1) % NS) * kStageBytes
+                                    : src < in_q ? OFFQ + (uint32_t)(src * share) * 512
+                                                 : (uint32_t)(n_r % NS) * kStageBytes + (uint32_t)((src - in_q) * share) * 512;
+                const uint32_t dst = smem0 + at + local * 512 + (ch * 64 + (qd & 1) * 8 + (qd >> 1) * 4) * 4;
+                const uint32_t to = cluster_map_shared(dst, r), to_bar = cluster_map_shared(bar(kReceived), r);
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const bool odd = qd & 1;
+                    const float g0 = __shfl_xor_sync(0xffffffffu, odd ? o[i][2 * j] : o[i][2 * j + 2], 1);
+                    const float g1 = __shfl_xor_sync(0xffffffffu, odd ? o[i][2 * j + 1] : o[i][2 * j + 3], 1);
+                    const float4 v = odd ? make_float4(g0, g1, o[i][2 * j + 2], o[i][2 * j + 3]) : make_float4(o[i][2 * j], o[i][2 * j + 1], g0, g1);
+                    if (row >= rows) continue;
+                    if (mine)
+                        *reinterpret_cast<float4 *>(smem + (dst - smem0) + j * 32) = v;
+                    else
+                        st_async_cluster_v4(to + j * 32, make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)), to_bar);
+                }
+                if (ch == 0 && qd == 0 && row < rows) {
+                    if (mine)
+                        *reinterpret_cast<float2 *>(misc + 512 + local * 8) = make_float2(M, lsum);
+                    else
+                        st_async_cluster_v2(cluster_map_shared(smem0 + kOffMisc + 1024 + (src * share + local) * 8, r),
+                                            make_uint2(__float_as_uint(M), __float_as_uint(lsum)), to_bar);
+                }
+                continue;
+            }
             if (row >= rows || (kBal && dead)) continue;
             if (kBal || p.splits == 1) {
                 const int ii = div_g(row), g = row - ii * p.G;
@@ -1326,6 +1393,41 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
     }
+    if constexpr (kCluster) {
+        named_bar_sync(1, n_sm);   // this CTA's own partial of its rows
+        const int n_rows = share_rows(split), in_q = NH == 4 ? kQBytes / (share * 512) : 0;
+        const uint8_t *stage_own = smem + ((n_total + 1) % NS) * kStageBytes, *stage_in = smem + (n_total % NS) * kStageBytes;
+        if (!__all_sync(0xffffffffu, mbar_wait_cluster_bounded(bar(kReceived), 0))) {
+            // What is missing may still come: stay until the other CTAs have left (or wait here too).
+            if (p.status && lane == 0) atomicOr(p.status, 4);
+            __syncwarp();
+            cluster_arrive();
+            cluster_wait();
+            return;
+        }
+        for (int idx = wg * wg_threads + t; idx < n_rows * 32; idx += n_sm) {
+            const int local = idx >> 5, c4 = idx & 31;
+            float2 ml[kMaxCluster];
+            float4 part[kMaxCluster];
+#pragma unroll
+            for (int j = 0; j < kMaxCluster; ++j) {
+                const int src = j - (j > split);
+                const uint8_t *o_from = j == split ? stage_own
+                                        : src < in_q ? smem + OFFQ + src * share * 512
+                                                     : stage_in + (src - in_q) * share * 512;
+                const uint8_t *ml_from = j == split ? misc + 512 : misc + 1024 + src * share * 8;
+                const bool in = j < p.splits;
+                ml[j] = in ? *reinterpret_cast<const float2 *>(ml_from + local * 8) : make_float2(-INFINITY, 0.f);
+                part[j] = in ? *reinterpret_cast<const float4 *>(o_from + local * 512 + c4 * 16) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            SplitSum sum;
+            sum.add(ml, part);
+            const int row = split * share + local, ii = div_g(row), g = row - ii * p.G;
+            const size_t orow = ((size_t)out_z * p.T + ii) * p.Hq + out_h * p.G + g;
+            *reinterpret_cast<uint2 *>(p.out + orow * 128 + c4 * 4) = sum.out();
+            if (p.lse && c4 == 0) p.lse[orow] = sum.lse();
+        }
+    }
     if (stop) break;
     ring += n_total, k_before += k;
     }
@@ -1333,11 +1435,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kBal = false, class Params>
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kBal = false, bool kCluster = false, class Params>
 static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
-    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>, kBal>;
-    constexpr int smem = kBal ? kSmemBytesBal : kSmemBytes;
+    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>, kBal, kCluster>;
+    constexpr int smem = kBal || kCluster ? kSmemBytesBal : kSmemBytes;
     static svh::OncePerDevice once;   // function attributes belong to a device
     const cudaError_t ce = once.run([] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
     if (ce != cudaSuccess) return ce;
@@ -1346,10 +1448,17 @@ static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, c
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     svh::pdl_attribute(attr);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (kCluster) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = p.splits;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, tm_k, tm_v, p);
 }
 
@@ -1364,6 +1473,12 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
                           : launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
     }
     const bool units = p.B == 128;   // 128-row tiles over blocks of 128 tokens: slices cut at 64-key units
+    if (p.cluster) {   // (one row tile of up to 32 draft tokens)
+        if (rows <= 32) return launch_tc<1, false, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        if (rows <= 64) return launch_tc<2, false, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        return units ? launch_tc<4, false, false, true, false, true>(tm_k, tm_v, p, grid, stream)
+                     : launch_tc<4, false, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+    }
     if (p.pair) {   // (a full tile has more than 64 rows)
         return units ? launch_tc<4, true, true, true>(tm_k, tm_v, p, grid, stream)
                      : launch_tc<4, true, true, false>(tm_k, tm_v, p, grid, stream);
@@ -1378,6 +1493,42 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
     if (rows <= 64) return launch_tc<2, false, false, false>(tm_k, tm_v, p, grid, stream);
     return units ? launch_tc<4, false, false, true>(tm_k, tm_v, p, grid, stream)
                  : launch_tc<4, false, false, false>(tm_k, tm_v, p, grid, stream);
+}
+
+bool cluster_holds_partials(int splits, int rows)
+{
+    const int share = (rows + splits - 1) / splits, each = kStageBytes / (share * 512);   // partials in a stage, or in a Q tile
+    return (splits - 1) * share * 8 <= 1024 && share * 8 <= 512 && splits - 1 <= (rows > 64 ? 2 * each : each);
+}
+
+int clusters_at_once(int size)
+{
+    static std::atomic<int> known[svh::kMaxDevices][kMaxCluster + 1];   // 1 + the answer
+    const int dev = svh::current_device();
+    if (size < 2 || size > kMaxCluster || dev < 0 || dev >= svh::kMaxDevices) return 0;
+    int n = known[dev][size].load(std::memory_order_acquire);
+    if (n == 0) {
+        constexpr auto kernel = verify_attn_tc_kernel<4, false, false, false, false, false, true>;   // (all forms take a whole SM a CTA)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(size, 1, 1);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = kSmemBytesBal;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = size;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int fit = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesBal) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) != cudaSuccess)
+            fit = 0;
+        (void)cudaGetLastError();   // a refusal is an answer, not an error of the call that asked
+        n = 1 + fit;
+        known[dev][size].store(n, std::memory_order_release);
+    }
+    return n - 1;
 }
 
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid, cudaStream_t stream)
