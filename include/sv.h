@@ -449,6 +449,19 @@ SV_API sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom *geo
                                           void *workspace, size_t workspace_bytes, int32_t *status_word, int32_t refresh_tail,
                                           const uint8_t *refresh_which, void *stream_in, void *stream_out, void *stream);
 
+/*
+ * The same step without chunks: the attention launch reads each list's rows from host memory when it takes the list (writing them to
+ * q / draft_k / draft_v as well) and writes its outputs to out_host and out.  For stacks whose lists are handed out to resident CTAs (more
+ * lists than SMs, at most 64 query rows a KV head, lists that are not split) and 16-byte aligned pinned memory; else nothing is
+ * launched and SV_ERR_UNSUPPORTED is returned.  Outputs are those of sv_verify_attn_layers, bit for bit.
+ */
+SV_API sv_status sv_verify_step_from_host_direct(const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors, const void *q_host,
+                                                 const void *draft_k_host, const void *draft_v_host, void *q, void *draft_k,
+                                                 void *draft_v, const int32_t *parent, float *reps, const int32_t *budget_blocks,
+                                                 int32_t n_sink, int32_t n_local, int32_t *idx, int32_t *cnt, int32_t max_sel, void *out,
+                                                 void *out_host, void *workspace, size_t workspace_bytes, int32_t *status_word,
+                                                 int32_t refresh_tail, const uint8_t *refresh_which, void *stream);
+
 /* Number of KV splits (CTAs per (sequence, KV head)) that the workspace of this geometry has room for.  sv_verify_attn uses as many, or
  * fewer where the CTAs of a thread-block cluster merge their splits themselves (the workspace is then not written). */
 SV_API int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel);

@@ -31,7 +31,7 @@ EXPORTS = ("sv_strerror", "sv_status_word_check", "sv_budget_blocks", "sv_worksp
            "sv_select_blocks_tokens", "sv_token_overlap", "sv_select_blocks_global", "sv_accept",
            "sv_block_reps_bf16", "sv_select_blocks_bf16reps", "sv_layer_table_bytes", "sv_layer_table", "sv_workspace_bytes_layers",
            "sv_block_reps_layers", "sv_select_blocks_layers", "sv_verify_attn_layers", "sv_kv_append_layers", "sv_host_step_create",
-           "sv_host_step_destroy", "sv_verify_step_from_host", "sv_workspace_bytes_host_step")
+           "sv_host_step_destroy", "sv_verify_step_from_host", "sv_verify_step_from_host_direct", "sv_workspace_bytes_host_step")
 SV_MAX_LAYERS = 256
 SV_STACK_STATE_BYTES = 256   # what a stack's launches keep at the start of their workspace
 

@@ -54,6 +54,10 @@ struct StackAttnParams : AttnParams {
     const LayerRow *layers;           // device layer table, from the launch's first layer on
     int S;                            // sequences of a layer
     uint8_t list_of[SV_MAX_LAYERS];   // block list of a layer: the ordinal of the last anchor up to it
+    // Not null: queries and draft K/V are read from these (pinned host memory), and copied to q, draft_k and draft_v on the way; the
+    // outputs go to out_host as well.
+    const __nv_bfloat16 *q_host = nullptr, *draft_k_host = nullptr, *draft_v_host = nullptr;
+    __nv_bfloat16 *out_host = nullptr;
 };
 
 // The sum over the splits of a row, four output dims: o = sum_j 2^(m_j - m) o_j / sum_j 2^(m_j - m) l_j, a batch of splits at a time.

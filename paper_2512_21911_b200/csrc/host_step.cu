@@ -43,17 +43,6 @@ __global__ void __launch_bounds__(kCopyThreads) copy_parts_kernel(const Parts p)
     }
 }
 
-// The address at which the current device can read and write this host memory, or null (memory that is not pinned).
-void *mapped(const void *host)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return nullptr;
-    }
-    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
-}
-
 }  // namespace
 
 // Events are kept: creating and destroying them costs as much as a launch each.
@@ -133,8 +122,8 @@ extern "C" sv_status sv_verify_step_from_host(sv_host_step *step, const sv_geom 
         cfg.numAttrs = 1;
         cuda(cudaLaunchKernelEx(&cfg, copy_parts_kernel, p));
     };
-    const void *q_map = mapped(q_host), *k_map = mapped(draft_k_host), *v_map = mapped(draft_v_host);
-    void *out_map = mapped(out_host);
+    const void *q_map = svh::mapped(q_host), *k_map = svh::mapped(draft_k_host), *v_map = svh::mapped(draft_v_host);
+    void *out_map = svh::mapped(out_host);
     auto words = [&](size_t layer, int c) { return (chunk_end[c] - (c ? chunk_end[c - 1] : 0)) * layer / 16; };
     const bool direct_in = q_map && k_map && v_map && words(q_layer + 2 * kv_layer, 0) < 1u << 31 && svh::aligned(q_map, 16) &&
                            svh::aligned(k_map, 16) && svh::aligned(v_map, 16);

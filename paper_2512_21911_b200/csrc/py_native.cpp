@@ -440,12 +440,14 @@ PyObject *host_step(PyObject *, PyObject *const *, Py_ssize_t n)
 // step, geom, table, kv, anchors, chunk_end (sequence of int), q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, parent, reps, budget,
 // n_sink, n_local, idx, cnt, out, out_host, workspace, status_word, refresh_tail, refresh_which (bytes or None),
 // stream_in, stream_out
-// -> status, or False when the tensors are not stacked ones
+// -> status, or False when the tensors are not stacked ones.  chunk_end None: without chunks (the streams are then not looked at), and
+// False also where that has no form
 PyObject *verify_step_from_host(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return checked(n, 27, [&]() -> PyObject * {
-        sv_host_step *h = static_cast<sv_host_step *>(PyCapsule_GetPointer(a[0], "sv_host_step"));
-        if (!h) throw ArgError{};
+        const bool direct = a[5] == Py_None;
+        sv_host_step *h = direct ? nullptr : static_cast<sv_host_step *>(PyCapsule_GetPointer(a[0], "sv_host_step"));
+        if (!h && !direct) throw ArgError{};
         const sv_geom g = geometry(a[1]);
         const sv_layers layers = stack(a[2], a[3]);
         void *dev[4], *host[4];   // q, draft K, draft V, out
@@ -460,7 +462,7 @@ PyObject *verify_step_from_host(PyObject *, PyObject *const *a, Py_ssize_t n)
             if (!host[i]) Py_RETURN_FALSE;
         }
         int32_t ends[SV_MAX_HOST_CHUNKS];
-        const Py_ssize_t chunks = PySequence_Fast_GET_SIZE(a[5]);
+        const Py_ssize_t chunks = direct ? 0 : PySequence_Fast_GET_SIZE(a[5]);
         if (chunks > SV_MAX_HOST_CHUNKS) Py_RETURN_FALSE;
         for (Py_ssize_t c = 0; c < chunks; ++c) ends[c] = int32(PySequence_Fast_GET_ITEM(a[5], c));
         const Scratch ws = scratch(a[21]);
@@ -470,18 +472,22 @@ PyObject *verify_step_from_host(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int32_t sink = int32(a[15]), local = int32(a[16]), max_sel = row_length(a[17], "idx");
         int32_t *const idx = i32(a[17], "idx"), *const cnt = i32(a[18], "cnt"), *const word = i32(a[22], "status_word");
         const bool refresh = truth(a[23]);
-        void *const in = stream(a[25]), *const back = stream(a[26]), *const s = stream(Py_None);
+        void *const s = stream(Py_None), *const in = direct ? s : stream(a[25]), *const back = direct ? s : stream(a[26]);
         const sv_status st = unlocked([&] {
+            if (direct)
+                return sv_verify_step_from_host_direct(&g, &layers, anchors, host[0], host[1], host[2], dev[0], dev[1], dev[2], parent, reps, budget,
+                                                       sink, local, idx, cnt, max_sel, dev[3], host[3], ws.p, ws.bytes, word, refresh, which, s);
             return sv_verify_step_from_host(h, &g, &layers, anchors, ends, (int32_t)chunks, host[0], host[1], host[2], dev[0], dev[1], dev[2],
                                             parent, reps, budget, sink, local, idx, cnt, max_sel, dev[3], host[3], ws.p, ws.bytes, word,
                                             refresh, which, in, back, s);
         });
+        if (direct && st == SV_ERR_UNSUPPORTED) Py_RETURN_FALSE;
         // the allocator of pinned memory must not hand these out again before the copies are through
         const auto device = c10::cuda::current_device();
         for (int i = 0; i < 4; ++i) {
             const at::Tensor &t = THPVariable_Unpack(i < 3 ? a[6 + i] : a[20]);
             void *const context = t.storage().data_ptr().get_context();
-            at::getHostAllocator(at::kCUDA)->record_event(
+            if (!direct) at::getHostAllocator(at::kCUDA)->record_event(
                 host[i], context, c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(i < 3 ? in : back), device).unwrap());
             at::getHostAllocator(at::kCUDA)->record_event(host[i], context, c10::cuda::getCurrentCUDAStream().unwrap());
         }

@@ -152,6 +152,30 @@ sv_status verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32
                              const int32_t *sel_cnt, int32_t max_sel, float softmax_scale, void *out, void *workspace,
                              size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits);
 
+// The address at which the current device can read and write this host memory, or null (memory that is not pinned).
+inline void *mapped(const void *host)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+}
+
+// Attention of a whole stack whose inputs are read from pinned host memory (device addresses of it) and whose outputs go there too
+// (kHost in verify_attn_tc.cu); q, draft_k, draft_v and out are written on the way.  SV_ERR_UNSUPPORTED, with nothing launched, where the
+// stack's lists are not handed out.
+struct HostTensors {
+    const void *q, *draft_k, *draft_v;
+    void *out;
+};
+sv_status verify_attn_from_host(const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors, const HostTensors &host, void *q,
+                                void *draft_k, void *draft_v, const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream);
+// Whether it would.
+bool lists_handed_out(const sv_geom *geom, const sv_layers *layers, int32_t max_sel);
+
 inline sv_status launch_status()
 {
     return cudaGetLastError() == cudaSuccess ? SV_OK : SV_ERR_CUDA;

@@ -429,11 +429,11 @@ extern "C" size_t sv_workspace_bytes_host_step(const sv_geom *geom, int32_t n_la
     return most ? std::max(whole, (size_t)SV_STACK_STATE_BYTES + most) : whole;
 }
 
-sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+static sv_status attn_layers_impl(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
                                   const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
                                   const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
                                   int32_t max_sel, float softmax_scale, void *out, void *workspace,
-                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits)
+                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits, const svh::HostTensors *host)
 {
     sv_status st = svh::check_layers(geom, layers, first, end);
     if (st != SV_OK) return st;
@@ -472,6 +472,11 @@ sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, 
         if (l >= first) p.list_of[l - first] = (uint8_t)(list < 0 ? 0 : list);
     }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
+    if (host) {
+        if (!handed) return SV_ERR_UNSUPPORTED;
+        p.q_host = static_cast<const __nv_bfloat16 *>(host->q), p.out_host = static_cast<__nv_bfloat16 *>(host->out);
+        p.draft_k_host = static_cast<const __nv_bfloat16 *>(host->draft_k), p.draft_v_host = static_cast<const __nv_bfloat16 *>(host->draft_v);
+    }
     if (handed) {
         p.n_claims = (end - first) * geom->n_seq * geom->n_kv_heads;
         p.claims = static_cast<uint32_t *>(workspace);
@@ -479,6 +484,30 @@ sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, 
         return launch_attn_tc_stack(p, dim3(std::min(sm_count(), p.n_claims)), cs) == cudaSuccess ? SV_OK : SV_ERR_CUDA;
     }
     return launch_attn(p, &rule, geom->n_seq * (end - first), cs, [&](dim3 grid) { return launch_attn_tc_stack(p, grid, cs); });
+}
+
+sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,
+                                  const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
+                                  const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                  int32_t max_sel, float softmax_scale, void *out, void *workspace,
+                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits)
+{
+    return attn_layers_impl(geom, layers, first, end, anchors, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel, softmax_scale, out,
+                            workspace, workspace_bytes, status_word, stream, own_splits, nullptr);
+}
+
+sv_status svh::verify_attn_from_host(const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors, const HostTensors &host, void *q,
+                                     void *draft_k, void *draft_v, const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
+                                     int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream)
+{
+    return attn_layers_impl(geom, layers, 0, layers ? layers->n_layers : 1, anchors, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel,
+                            0.f, out, workspace, workspace_bytes, status_word, stream, false, &host);
+}
+
+bool svh::lists_handed_out(const sv_geom *geom, const sv_layers *layers, int32_t max_sel)
+{
+    const sv_geom rule = stack_geom(geom, layers->n_layers);
+    return max_sel >= 1 && hand_out(&rule, max_sel);
 }
 
 extern "C" sv_status sv_verify_attn_layers(const sv_geom *geom, const sv_layers *layers, int32_t first, int32_t end,

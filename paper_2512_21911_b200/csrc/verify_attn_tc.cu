@@ -121,7 +121,9 @@ struct ClaimWords {
 // shared memory with stores that count their bytes on a barrier there, so that nothing but the data is waited for (two cluster
 // barriers around a pull, as this was first tried, cost what the merge kernel does).  Bound by latency: readout, the push, one wait.  A layer of
 // 2 KV heads x 16 units 12.0 -> 9.9 us (launches), 4 sequences x 8 heads x 32 units, 32 rows 18.1 -> 16.5, 64 pairs x 32 units 22.4 -> 21.2.
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal, bool kCluster>
+// kHost (with kBal): the step's inputs are in pinned host memory and its outputs wanted there.  A list's rows are read when a CTA takes
+// it and written when it is through, so the bus works while the lists are gathered, instead of ahead of them and behind them.
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kStack, bool kBal, bool kCluster, bool kHost>
 __global__ void __launch_bounds__(kThreads, 1)
     verify_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                           const std::conditional_t<kStack, StackAttnParams, AttnParams> p)
@@ -163,6 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
 
     static_assert(!kCluster || (!kWide && !kBal), "clusters merge a single row tile of up to 32 draft tokens");
+    static_assert(!kHost || kBal, "lists that are handed out");
     static_assert(!kBal || (kStack && NH < 4), "lists are handed out for stacks, in tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
     // 128-row tiles are bound by the tensor pipe when every MMA fetches both operands from shared memory (S = Q K^T: eight
@@ -327,6 +330,49 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T, c = idx & 15;
             cp_async_16(unit_at + which * (2 * kTile) + (c >> 3) * kTile + swz128(r, c & 7),
                         (which ? p.draft_v : p.draft_k) + (((size_t)z_d * p.T + r) * p.Hkv + h_d) * 128 + c * 8);
+        }
+    };
+    // (kHost) the same from host memory, through registers, and to the device tensors on the way: eight loads of a thread in flight
+    auto fetch_q = [&](uint8_t *to, int z_q, int h_q, int t, int n) {
+        if constexpr (kHost) {
+            const int c = t & 15, step = n >> 4;
+            const size_t at = (((size_t)z_q * p.T + i0) * p.Hq + h_q * p.G) * 128 + c * 8;
+            for (int r0 = t >> 4; r0 < rows; r0 += 8 * step) {
+                uint4 v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = r0 + i * step;
+                    if (r < rows) v[i] = __ldcv(reinterpret_cast<const uint4 *>(p.q_host + at + (r + div_g(r) * (p.Hq - p.G)) * 128));
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = r0 + i * step;
+                    if (r >= rows) continue;
+                    *reinterpret_cast<uint4 *>(to + (c >> 3) * (kQBytes / 2) + swz128((r / RPQ) * QR + (r % RPQ), c & 7)) = v[i];
+                    *reinterpret_cast<uint4 *>(const_cast<__nv_bfloat16 *>(p.q) + at + (r + div_g(r) * (p.Hq - p.G)) * 128) = v[i];
+                }
+            }
+        }
+    };
+    // the draft tokens' K and V to the device tensors, from where copy_draft, by the same threads, takes them when their unit's stage is free
+    auto fetch_draft = [&](int z_d, int h_d, int t, int n) {
+        if constexpr (kHost) {
+            for (int i0 = t; i0 < 2 * p.T * 16; i0 += 8 * n) {
+                uint4 v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int idx = i0 + i * n, which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T;
+                    const size_t at = (((size_t)z_d * p.T + r) * p.Hkv + h_d) * 128 + (idx & 15) * 8;
+                    if (idx < 2 * p.T * 16) v[i] = __ldcv(reinterpret_cast<const uint4 *>((which ? p.draft_v_host : p.draft_k_host) + at));
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int idx = i0 + i * n, which = (idx >> 4) >= p.T, r = (idx >> 4) - which * p.T;
+                    const size_t at = (((size_t)z_d * p.T + r) * p.Hkv + h_d) * 128 + (idx & 15) * 8;
+                    if (idx < 2 * p.T * 16) *reinterpret_cast<uint4 *>(const_cast<__nv_bfloat16 *>(which ? p.draft_v : p.draft_k) + at) = v[i];
+                }
+            }
+            __threadfence();
         }
     };
     const uint32_t tmem_base = warp == 8 && !kBal ? 0u : __shfl_sync(0xffffffffu, *tmem_slot, 0);
@@ -590,7 +636,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const Item it = item_at(claim);
                 const int n_total = item_blocks(it) * upb + 1;
                 if (seg > 0) {   // (the first segment's is brought by the softmax warps)
-                    copy_q(smem0 + OFFQ + (seg & 1) * 8192, it.z, it.h, lane, 32);   // (an M = 64 tile fills half of either half)
+                    if constexpr (kHost)   // (an M = 64 tile fills half of either half)
+                        fetch_q(smem + OFFQ + (seg & 1) * 8192, it.z, it.h, lane, 32);
+                    else
+                        copy_q(smem0 + OFFQ + (seg & 1) * 8192, it.z, it.h, lane, 32);
                 }
                 {   // lane i: tokens i and (kWide) 32 + i
 #pragma unroll
@@ -625,6 +674,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (seg == 0) named_bar_sync(2, 288);   // the padding rows of the Q tiles are zero
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kLoaded));
+                fetch_draft(it.z, it.h, lane, 32);
                 {   // the last unit of the segment
                     const int stage = (ring + n_total - 1) % NS;
                     if (!__all_sync(0xffffffffu, !*abort_flag && long_wait(kSlot, n_drafts++ & 1))) {
@@ -831,7 +881,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if constexpr (kBal) {
         const Item it = item_at(blockIdx.x);
-        copy_q(smem0 + OFFQ, it.z, it.h, qtid, kQThreads);   // (first segment)
+        if constexpr (kHost) {
+            // The first lists' queries are asked for one CTA after the other, 60 bytes a nanosecond, about as the bus delivers them: the
+            // CTAs then start, and end, one after the other, instead of all of them waiting for the last word.  (32 layers of 8 lists of
+            // 64 units: 131.5 us; all at once 132.4, 46 bytes a nanosecond with the draft's rows counted 138; 24 layers x 16 lists of 16
+            // units: 107, 113.5, 109.5.)
+            if (blockIdx.x > 0) __nanosleep(min(1000000u, blockIdx.x * (unsigned)rows * 256u / 60u));
+            fetch_q(smem + OFFQ, it.z, it.h, qtid, kQThreads);
+        } else {
+            copy_q(smem0 + OFFQ, it.z, it.h, qtid, kQThreads);   // (first segment)
+        }
     } else if (has_draft) {
         for (int idx = tid; idx < 2 * kUnit * 16; idx += 256) {
             const int which = idx / (kUnit * 16);   // 0: K, 1: V
@@ -1375,6 +1434,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 continue;
             }
+            if constexpr (kHost) {
+                // The four lanes of a row change words so that each stores 16 bytes: lane qd those of columns 8 (4 half + qd) .. + 7.
+                const int ii = div_g(row), g = row - ii * p.G;
+                const size_t at = (((size_t)out_z * p.T + i0 + ii) * p.Hq + out_h * p.G + g) * 128 + ch * 64 + qd * 8;
+                const float inv = 1.f / lsum;
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) w[j] = pack_bf16(o[i][8 * half + 2 * j] * inv, o[i][8 * half + 2 * j + 1] * inv);
+                    const bool odd = qd & 1, high = qd & 2;
+                    const uint32_t r0 = __shfl_xor_sync(0xffffffffu, odd ? w[0] : w[1], 1), r1 = __shfl_xor_sync(0xffffffffu, odd ? w[2] : w[3], 1);
+                    const uint2 a = odd ? make_uint2(r0, w[1]) : make_uint2(w[0], r0), b = odd ? make_uint2(r1, w[3]) : make_uint2(w[2], r1);
+                    const uint32_t x = __shfl_xor_sync(0xffffffffu, high ? a.x : b.x, 2), y = __shfl_xor_sync(0xffffffffu, high ? a.y : b.y, 2);
+                    if (row >= rows || dead) continue;
+                    const uint4 v = high ? make_uint4(x, y, b.x, b.y) : make_uint4(a.x, a.y, x, y);
+                    *reinterpret_cast<uint4 *>(p.out_host + at + half * 32) = v;
+                    *reinterpret_cast<uint4 *>(p.out + at + half * 32) = v;
+                }
+                continue;
+            }
             if (row >= rows || (kBal && dead)) continue;
             if (kBal || p.splits == 1) {
                 const int ii = div_g(row), g = row - ii * p.G;
@@ -1435,10 +1515,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kBal = false, bool kCluster = false, class Params>
+template <int NH, bool kWide, bool kPair, bool kUnitSlices, bool kBal = false, bool kCluster = false, bool kHost = false, class Params>
 static cudaError_t launch_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
-    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>, kBal, kCluster>;
+    constexpr auto kernel = verify_attn_tc_kernel<NH, kWide, kPair, kUnitSlices, std::is_same_v<Params, StackAttnParams>, kBal, kCluster, kHost>;
     constexpr int smem = kBal || kCluster ? kSmemBytesBal : kSmemBytes;
     static svh::OncePerDevice once;   // function attributes belong to a device
     const cudaError_t ce = once.run([] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); });
@@ -1467,7 +1547,11 @@ template <class Params>
 static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const Params &p, dim3 grid, cudaStream_t stream)
 {
     const int rows = p.G * p.Tt;   // rows of a full row tile
-    if constexpr (std::is_same_v<Params, StackAttnParams>) if (p.n_claims > 0) {
+    if constexpr (std::is_same_v<Params, StackAttnParams>) if (p.q_host) {
+        if (p.T > 32) return launch_tc<2, true, false, false, true, false, true>(tm_k, tm_v, p, grid, stream);
+        return rows <= 32 ? launch_tc<1, false, false, false, true, false, true>(tm_k, tm_v, p, grid, stream)
+                          : launch_tc<2, false, false, false, true, false, true>(tm_k, tm_v, p, grid, stream);
+    } else if (p.n_claims > 0) {
         if (p.T > 32) return launch_tc<2, true, false, false, true>(tm_k, tm_v, p, grid, stream);
         return rows <= 32 ? launch_tc<1, false, false, false, true>(tm_k, tm_v, p, grid, stream)
                           : launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
@@ -1508,7 +1592,7 @@ int clusters_at_once(int size)
     if (size < 2 || size > kMaxCluster || dev < 0 || dev >= svh::kMaxDevices) return 0;
     int n = known[dev][size].load(std::memory_order_acquire);
     if (n == 0) {
-        constexpr auto kernel = verify_attn_tc_kernel<4, false, false, false, false, false, true>;   // (all forms take a whole SM a CTA)
+        constexpr auto kernel = verify_attn_tc_kernel<4, false, false, false, false, false, true, false>;   // (all forms take a whole SM a CTA)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(size, 1, 1);
         cfg.blockDim = dim3(kThreads);

@@ -17,6 +17,7 @@ import torch
 from . import binding as sv
 
 
+DIRECT_BYTES = 24 << 20   # what a host-fed step may upload and still go without chunks (SparseVerifier._direct)
 # What the schedule of a host-fed step reckons with: bytes per microsecond up, down, from HBM and by one CTA alone, microseconds per
 # chunk (its launches; the copies of a further one).  Fitted to the differences between the schedules of 184 stacks on two
 # machines (the sums come out 4 % high on average): a B200 on a PCIe 5 link, of which only the proportions matter here.
@@ -99,6 +100,10 @@ class SparseVerifier:
         # are scratch of many megabytes, written before they are read: made when they are needed.
         need = [sv._native.workspace_bytes_layers(self.geom, n_layers, n) if stackable else 0 for n in (max_sel, self.geom.max_blocks)]
         keeps = [n == sv.SV_STACK_STATE_BYTES for n in need]
+        # A host-fed step of a stack whose lists go to resident CTAs needs no chunks.  90 such stacks (4 to 30 layers, 1 to 8 sequences of
+        # 1K to 42K tokens, 1 to 16 draft tokens) take 0.81 of the time of the schedule above in the geometric mean, 1.01 or more only one
+        # of them, with 33 MB to read: there the bus is all that counts, and the copy engine has a few percent more of it.
+        self._direct = keeps[0] and n_layers * rows * (n_q_heads + 2 * n_kv_heads) <= DIRECT_BYTES
         self._stack_bytes = [sv._native.workspace_bytes_host_step(self.geom, n_layers, max_sel) if stackable else 0, need[1]]
         self._stack_workspace = [torch.zeros(n, dtype=torch.uint8, device=dev) if k else None for n, k in zip(self._stack_bytes, keeps)]
 
@@ -229,9 +234,16 @@ class SparseVerifier:
         ones.  Returns with everything enqueued; the current stream ends behind the last download.  Capturable in a
         CUDA graph (the side streams fork from and join the current stream).
 
+        Where the stack's lists are handed out to resident CTAs (more lists than SMs, at most 64 query rows a KV head) and no
+        chunks are asked for, there are none: the attention launch itself reads a list's rows from pinned memory when a CTA takes the
+        list and writes its outputs there.
+
         A chunk of few lists is split over the SMs for itself, so the outputs are those of verify_step to bf16 rounding.  Large
         chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 178 us in two
-        chunks, 188 in chunks of eight layers, 241 of four, 613 of one)."""
+        chunks, 188 in chunks of eight layers, 241 of four, 613 of one; 131 without chunks)."""
+        if layers_per_chunk is None and self._direct and self._stacked() and \
+                self._from_host(None, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host, refresh_tail):
+            return
         chunks = self._chunks(layers_per_chunk)
         if self._copy_streams is None:
             self._copy_streams = (torch.cuda.Stream(device=q.device), torch.cuda.Stream(device=q.device))
@@ -285,15 +297,15 @@ class SparseVerifier:
     def _from_host(self, chunks, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host, refresh_tail) -> bool:
         """verify_step_from_host in one call of the library.  False when the tensors are not stacked ones."""
         flags = self._anchor_flags()
-        if self._host_step is None:
+        if chunks is not None and self._host_step is None:
             self._host_step = sv._native.host_step()
             if isinstance(self._host_step, int):
                 raise sv.SvError(self._host_step, "sv_host_step_create")
         st = sv._native.verify_step_from_host(
-            self._host_step, self.geom, self._table, self.kv[0], flags, [c1 for _, c1 in chunks], q_host, draft_k_host, draft_v_host, q,
+            self._host_step, self.geom, self._table, self.kv[0], flags, chunks and [c1 for _, c1 in chunks], q_host, draft_k_host, draft_v_host, q,
             draft_k, draft_v, self.parent, self.reps, self.budget, self.n_sink, self.n_local, self._lists_idx, self._lists_cnt, out,
             out_host, self._workspace_of_stack(False), self.status, refresh_tail, None if self._one_allocation else flags,
-            *self._copy_streams)
+            *(self._copy_streams if chunks else (None, None)))
         if st is False:
             return False
         sv._check(st, "sv_verify_step_from_host")
