@@ -91,6 +91,14 @@ __device__ __forceinline__ void st_async_cluster_v2(uint32_t addr, uint2 v, uint
                  "r"(v.y), "r"(remote_bar)
                  : "memory");
 }
+// bytes (a multiple of 16, both addresses on 16-byte boundaries) of this CTA's shared memory into another CTA's, reported to an mbarrier
+// there; this CTA's memory has to stay until they have arrived
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t remote_bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes),
+                 "r"(remote_bar)
+                 : "memory");
+}
 __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint32_t bar, uint32_t parity, uint32_t limit = (1u << 19))
 {
     for (uint32_t i = 0; i < limit; ++i) {

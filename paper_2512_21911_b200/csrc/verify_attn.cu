@@ -168,20 +168,21 @@ int choose_splits(const sv_geom *g, int n_blocks, bool balance = true)
 // SMs hold 33 clusters of four, 22 of six, 15 of eight CTAs.
 // Where that, or the eight CTAs of a portable cluster, leaves fewer splits, each has more units: up to kMoreUnits more pay with up to
 // 64 rows (16 pairs x 100 units in 6 instead of 9: 20.0 -> 19.0; 8 more do not: 8 pairs x 128 in 8 instead of 16, 16.2 -> 17.0).
-// A 128-row tile pushes 64 KB per CTA: with two CTAs a cluster is faster (64 pairs x 32 units 28.3 -> 27.25), with four about
-// equal (28.9 and 28.8; 18.4 and 18.8), with fewer splits slower (16 pairs, 80 rows, 6 instead of 8: 17.0 -> 17.2).
+// With 65 to 128 rows, in clusters of up to four CTAs: four more units or half as many again (64 pairs x 32 units 28.4 -> 25.2 us, 32 pairs x
+// 64 units 28.9 -> 28.2, 32 pairs x 12 units 16.3 -> 14.7; 24 pairs x 64 units in 4 instead of 6 24.7 -> 23.2; 4 pairs x 24 units in 4
+// instead of 24 13.65 -> 13.8).
 // Slices of more than kLongSlice units are left to the merge kernel: CTAs that run for long end further apart, and a cluster's SMs are
 // idle until the last of its CTAs has ended (32 pairs x 257 units, 44.2 -> 44.8 us).
-constexpr int kMoreUnits = 5, kLongSlice = 48;
+constexpr int kMoreUnits = 5, kMoreUnitsWide = 4, kLongSlice = 48;
 int choose_cluster(const sv_geom *g, int n_blocks, int splits)
 {
     const int rows = g->n_q_heads / g->n_kv_heads * g->n_draft, pairs = g->n_seq * g->n_kv_heads;
     if (splits < 2 || svh::row_tiles(g) > 1 || g->n_draft > 32 || pairs > sm_count() / 2) return 0;
-    if (rows > 64 && splits > 2) return 0;
     const int upb = g->block_size / kUnit, split_blocks = (n_blocks + splits - 1) / splits;
     for (int most = std::min(splits, kMaxCluster); most > 1; --most) {
         const int blocks = (n_blocks + most - 1) / most, c = (n_blocks + blocks - 1) / blocks;
-        if ((blocks - split_blocks) * upb > kMoreUnits || blocks * upb > kLongSlice) return 0;
+        const int more = rows > 64 ? std::max(kMoreUnitsWide, split_blocks * upb / 2) : kMoreUnits;
+        if ((blocks - split_blocks) * upb > more || blocks * upb > kLongSlice) return 0;
         if (cluster_holds_partials(c, rows) && clusters_at_once(c) >= pairs) return c;
     }
     return 0;

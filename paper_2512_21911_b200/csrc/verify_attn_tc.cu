@@ -1300,7 +1300,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if constexpr (kTurns)
         for (int x = turns_taken, u = 2 * x + wg; u < n_total; ++x, u += 2) turn_begin(x), turn_end(x, u);
-    if constexpr (NH == 4) {
+    constexpr bool kRowOut = kCluster && NH == 4;   // the read-out of 128-row tiles in clusters: a thread a row
+    if constexpr (NH == 4 && !kRowOut) {
         // back to the four-threads-per-row slots the read-out uses: slot i of this thread is row 8 i + lane / 4 of the warp
         const float m_row = m[0], l_row = l[0];
 #pragma unroll
@@ -1328,9 +1329,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (!kPair && kPTmem) {
         // no P tiles in shared memory: the exchange goes through the warpgroup's own (now idle) S columns, thread for
         // thread (this thread's slots live on TMEM lane quad * 32 + lane in either warpgroup)
-        uint32_t ml_ours[8];
+        uint32_t ml_ours[8] = {__float_as_uint(m[0]), __float_as_uint(l[0])};
 #pragma unroll
-        for (int i = 0; i < NH; ++i) ml_ours[2 * i] = __float_as_uint(m[i]), ml_ours[2 * i + 1] = __float_as_uint(l[i]);
+        for (int i = 0; i < (kRowOut ? 0 : NH); ++i) ml_ours[2 * i] = __float_as_uint(m[i]), ml_ours[2 * i + 1] = __float_as_uint(l[i]);
         tmem_st_x8(tmem_base + t_lane + wg * kUnit, ml_ours);
         tmem_st_wait();
         tc_fence_before_sync();
@@ -1354,7 +1355,54 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (kCluster) cluster_wait();   // every CTA's place for the partials is free
     bool stop = !kBal;
     const int out_z = kBal ? seg_item / p.Hkv : z, out_h = kBal ? seg_item - out_z * p.Hkv : h;
-    for (int ch = kPair ? 0 : wg; ch < (kPair ? 2 : wg + 1); ++ch) {   // column half: 64 output dims
+    if constexpr (kRowOut) {
+        // Thread = row: its 64 columns of this warpgroup's half in two steps, both accumulators, to a tile in shared memory (16-byte words,
+        // changed about by row so that neither side has bank conflicts), from where the peers get their rows by one asynchronous copy each:
+        // 6000 cycles until they have arrived, 6800 with 16-byte stores from the registers of four threads a row; the merge, by eight lanes a
+        // row, takes 1400 instead of 3000.  (Partials for the merge kernel take 3900 cycles either way and are left to the form below.)
+        const int row = quad * 32 + lane;
+        const float m1 = __uint_as_float(ml_theirs[0]), l1 = __uint_as_float(ml_theirs[1]);
+        const float M = fmaxf(m[0], m1), M_use = (M == -INFINITY) ? 0.f : M;
+        const float w0 = fast_exp2(m[0] - M_use), w1 = fast_exp2(m1 - M_use), lsum = w0 * l[0] + w1 * l1;
+        uint8_t *half_tile = smem + ((n_total + 1 + wg) % NS) * kStageBytes;   // [128][256 bytes]
+#pragma unroll 1
+        for (int cb = 0; cb < 2; ++cb) {
+            uint32_t r0[32], r1[32];
+            if (have_mine) tmem_ld_x32(t_o + wg * 64 + cb * 32, r0);
+            if (have_other) tmem_ld_x32(t_o_other + wg * 64 + cb * 32, r1);
+            tmem_ld_wait();
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    v[e] = (have_mine ? w0 * __uint_as_float(r0[4 * x + e]) : 0.f) + (have_other ? w1 * __uint_as_float(r1[4 * x + e]) : 0.f);
+                *reinterpret_cast<float4 *>(half_tile + row * 256 + (((cb * 8 + x) ^ (row & 7)) * 16)) = make_float4(v[0], v[1], v[2], v[3]);
+            }
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kTmemDone));   // this warp reads TMEM no more
+        if (wg == 0 && row < rows) {
+            const int r = min((int)(((float)row + 0.5f) / (float)share), p.splits - 1), local = row - r * share, src = split - (split > r);
+            if (r == split)
+                *reinterpret_cast<float2 *>(misc + 512 + local * 8) = make_float2(M, lsum);
+            else
+                st_async_cluster_v2(cluster_map_shared(smem0 + kOffMisc + 1024 + (src * share + local) * 8, r),
+                                    make_uint2(__float_as_uint(M), __float_as_uint(lsum)), cluster_map_shared(bar(kReceived), r));
+        }
+        fence_proxy_async();                   // (the copies read the tile)
+        named_bar_sync(12 + wg, wg_threads);   // the half tile is complete
+        const int r = t, src = split - (split > r), n_rows = r < p.splits && r != split ? share_rows(r) : 0;
+        if (n_rows > 0) {
+            const int n_r = slice_units(r, n_sel) + (r == p.splits - 1), in_q = kQBytes / (share * 512);
+            const uint32_t at = src < in_q ? OFFQ + (uint32_t)(src * share) * 512
+                                           : (uint32_t)(n_r % NS) * kStageBytes + (uint32_t)((src - in_q) * share) * 512;
+            bulk_copy_cluster(cluster_map_shared(smem0 + at + wg * share * 256, r), smem_u32(half_tile) + r * share * 256, n_rows * 256,
+                              cluster_map_shared(bar(kReceived), r));
+        }
+    }
+    for (int ch = kPair ? 0 : wg; !kRowOut && ch < (kPair ? 2 : wg + 1); ++ch) {   // column half: 64 output dims
         // this warp's rows of O, 16 output dims 64 ch + 8 j + 2 qd + e (index 2 j + e)
         float o[NH][16], row_m[NH], row_l[NH];
 #pragma unroll
@@ -1400,18 +1448,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < NH; ++i) {
             const float M = row_m[i], lsum = row_l[i];
             const int row = lrow[i];
-            if constexpr (kCluster) {
+            if constexpr (kCluster && !kRowOut) {
                 // Lanes that differ in their lowest bit swap halves, for stores of 16 bytes: the even lane has columns 8 j + 2 qd .. + 3
                 // of the even j, the odd one those of the odd j.
                 const int r = min((int)(((float)row + 0.5f) / (float)share), p.splits - 1), local = row - r * share;
                 const bool mine = r == split;
                 const int src = split - (split > r);   // among the partials r receives
                 const int n_r = slice_units(r, n_sel) + (r == p.splits - 1);
-                const int in_q = NH == 4 ? kQBytes / (share * 512) : 0;
                 const uint32_t at = mine ? (uint32_t)((n_total + 1) % NS) * kStageBytes
-                                    : src < in_q ? OFFQ + (uint32_t)(src * share) * 512
-                                                 : (uint32_t)(n_r % NS) * kStageBytes + (uint32_t)((src - in_q) * share) * 512;
+                                         : (uint32_t)(n_r % NS) * kStageBytes + (uint32_t)(src * share) * 512;
                 const uint32_t dst = smem0 + at + local * 512 + (ch * 64 + (qd & 1) * 8 + (qd >> 1) * 4) * 4;
+                const uint32_t flip = (local & 1) * 64;   // rows are 512 bytes apart: two that follow one another take different banks
                 const uint32_t to = cluster_map_shared(dst, r), to_bar = cluster_map_shared(bar(kReceived), r);
 #pragma unroll
                 for (int j = 0; j < 8; j += 2) {
@@ -1421,9 +1468,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float4 v = odd ? make_float4(g0, g1, o[i][2 * j + 2], o[i][2 * j + 3]) : make_float4(o[i][2 * j], o[i][2 * j + 1], g0, g1);
                     if (row >= rows) continue;
                     if (mine)
-                        *reinterpret_cast<float4 *>(smem + (dst - smem0) + j * 32) = v;
+                        *reinterpret_cast<float4 *>(smem + (dst - smem0) + ((j * 32) ^ flip)) = v;
                     else
-                        st_async_cluster_v4(to + j * 32, make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)), to_bar);
+                        st_async_cluster_v4(to + ((j * 32) ^ flip), make_uint4(__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)), to_bar);
                 }
                 if (ch == 0 && qd == 0 && row < rows) {
                     if (mine)
@@ -1476,37 +1523,51 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (kCluster) {
         named_bar_sync(1, n_sm);   // this CTA's own partial of its rows
         const int n_rows = share_rows(split), in_q = NH == 4 ? kQBytes / (share * 512) : 0;
-        const uint8_t *stage_own = smem + ((n_total + 1) % NS) * kStageBytes, *stage_in = smem + (n_total % NS) * kStageBytes;
-        if (!__all_sync(0xffffffffu, mbar_wait_cluster_bounded(bar(kReceived), 0))) {
-            // What is missing may still come: stay until the other CTAs have left (or wait here too).
-            if (p.status && lane == 0) atomicOr(p.status, 4);
-            __syncwarp();
-            cluster_arrive();
-            cluster_wait();
-            return;
-        }
-        for (int idx = wg * wg_threads + t; idx < n_rows * 32; idx += n_sm) {
-            const int local = idx >> 5, c4 = idx & 31;
-            float2 ml[kMaxCluster];
-            float4 part[kMaxCluster];
+        const bool received = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(bar(kReceived), 0));
+        if (!received && p.status && lane == 0) atomicOr(p.status, 4);
+        // Who copied from shared memory stays until the others have received it, who has given up until nothing more can come (warps that
+        // have left are not waited for).  Stores need neither: the arrival would wait for them, 500 cycles.
+        const bool stays = NH == 4 || !received;
+        __syncwarp();
+        if (stays) cluster_arrive();
+        // kLanes lanes write a row, each kWords 4-dim words of it, by the row's weights.
+        constexpr int kLanes = NH == 4 ? 8 : 32, kWords = 32 / kLanes, kIn = NH == 4 ? 4 : kMaxCluster;
+        const int sub = lane % kLanes;
+        for (int local = (wg * wg_threads + t) / kLanes; local < n_rows && received; local += n_sm / kLanes) {
+            const int row = split * share + local;
+            float2 ml[kIn];
+            float4 part[kWords][kIn];
 #pragma unroll
-            for (int j = 0; j < kMaxCluster; ++j) {
-                const int src = j - (j > split);
-                const uint8_t *o_from = j == split ? stage_own
-                                        : src < in_q ? smem + OFFQ + src * share * 512
-                                                     : stage_in + (src - in_q) * share * 512;
-                const uint8_t *ml_from = j == split ? misc + 512 : misc + 1024 + src * share * 8;
+            for (int j = 0; j < kIn; ++j) {
                 const bool in = j < p.splits;
-                ml[j] = in ? *reinterpret_cast<const float2 *>(ml_from + local * 8) : make_float2(-INFINITY, 0.f);
-                part[j] = in ? *reinterpret_cast<const float4 *>(o_from + local * 512 + c4 * 16) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int src = j - (j > split);
+                ml[j] = in ? *reinterpret_cast<const float2 *>((j == split ? misc + 512 : misc + 1024 + src * share * 8) + local * 8) : make_float2(-INFINITY, 0.f);
+                const uint8_t *from = smem + ((n_total % NS) * kStageBytes) + (src - in_q) * share * 512;
+                if (NH == 4 && src < in_q) from = smem + OFFQ + src * share * 512;
+                if (NH < 4 && j == split) from = smem + ((n_total + 1) % NS) * kStageBytes;
+#pragma unroll
+                for (int x = 0; x < kWords; ++x) {
+                    const int c4 = sub + x * kLanes;   // (128-row tiles: half, word of the half)
+                    const uint8_t *word = from + local * 512 + ((c4 * 16) ^ ((local & 1) * 64));
+                    if (NH == 4) {
+                        const int half = c4 >> 4, w = ((c4 & 15) ^ (row & 7)) * 16;
+                        word = j == split ? smem + ((n_total + 1 + half) % NS) * kStageBytes + row * 256 + w : from + (half * share + local) * 256 + w;
+                    }
+                    part[x][j] = in ? *reinterpret_cast<const float4 *>(word) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
             }
-            SplitSum sum;
-            sum.add(ml, part);
-            const int row = split * share + local, ii = div_g(row), g = row - ii * p.G;
+            const int ii = div_g(row), g = row - ii * p.G;
             const size_t orow = ((size_t)out_z * p.T + ii) * p.Hq + out_h * p.G + g;
-            *reinterpret_cast<uint2 *>(p.out + orow * 128 + c4 * 4) = sum.out();
-            if (p.lse && c4 == 0) p.lse[orow] = sum.lse();
+#pragma unroll
+            for (int x = 0; x < kWords; ++x) {
+                SplitSum sum;
+                sum.add(ml, part[x]);
+                *reinterpret_cast<uint2 *>(p.out + orow * 128 + (sub + x * kLanes) * 4) = sum.out();
+                if (x == 0 && p.lse && sub == 0) p.lse[orow] = sum.lse();
+            }
         }
+        __syncwarp();
+        if (stays) cluster_wait();
     }
     if (stop) break;
     ring += n_total, k_before += k;
@@ -1582,7 +1643,7 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
 bool cluster_holds_partials(int splits, int rows)
 {
     const int share = (rows + splits - 1) / splits, each = kStageBytes / (share * 512);   // partials in a stage, or in a Q tile
-    return (splits - 1) * share * 8 <= 1024 && share * 8 <= 512 && splits - 1 <= (rows > 64 ? 2 * each : each);
+    return splits <= (rows > 64 ? 4 : kMaxCluster) && (splits - 1) * share * 8 <= 1024 && share * 8 <= 512 && splits - 1 <= (rows > 64 ? 2 * each : each);
 }
 
 int clusters_at_once(int size)

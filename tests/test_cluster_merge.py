@@ -20,6 +20,10 @@ SHAPES = [  # seqs, heads, kv_heads, block, draft, tree
     (9, 32, 8, 64, 16, True),     # 64 rows, two CTAs
     (9, 64, 8, 64, 16, True),     # 128 rows, two CTAs
     (18, 28, 4, 128, 10, False),  # 70 rows, blocks of 128
+    (4, 64, 8, 64, 16, False),    # 128 rows, four CTAs
+    (4, 64, 8, 128, 16, True),    # ... cut at units
+    (8, 28, 4, 64, 11, True),     # 77 rows over four CTAs
+    (9, 40, 5, 64, 14, False),    # 112 rows over three CTAs
 ]
 
 
