@@ -170,20 +170,24 @@ int choose_splits(const sv_geom *g, int n_blocks, bool balance = true)
 // 64 rows (16 pairs x 100 units in 6 instead of 9: 20.0 -> 19.0; 8 more do not: 8 pairs x 128 in 8 instead of 16, 16.2 -> 17.0).
 // With 65 to 128 rows, in clusters of up to four CTAs: four more units or half as many again (64 pairs x 32 units 28.4 -> 25.2 us, 32 pairs x
 // 64 units 28.9 -> 28.2, 32 pairs x 12 units 16.3 -> 14.7; 24 pairs x 64 units in 4 instead of 6 24.7 -> 23.2; 4 pairs x 24 units in 4
-// instead of 24 13.65 -> 13.8).
+// instead of 24 13.65 -> 13.8).  Several row tiles are as many lists (8 x 2 tiles x 20 units 15.4 -> 14.6, 5 x 2 x 8 14.6 -> 13.5, dense 16 x 2 x
+// 32 14.7 -> 13.3).  Not for 64 rows or fewer of more than 32 draft tokens, whose last split has the longest draft unit of all: 16 pairs x 32
+// units, 40 rows 15.4 -> 16.1, 64 x 12 17.4 -> 17.9.
+// Lists of at most kUnsplitUnits stay whole: in clusters of two to four 0.5 us slower (8 pairs x 4 units, device 7.7 -> 8.4).
 // Slices of more than kLongSlice units are left to the merge kernel: CTAs that run for long end further apart, and a cluster's SMs are
 // idle until the last of its CTAs has ended (32 pairs x 257 units, 44.2 -> 44.8 us).
 constexpr int kMoreUnits = 5, kMoreUnitsWide = 4, kLongSlice = 48;
 int choose_cluster(const sv_geom *g, int n_blocks, int splits)
 {
-    const int rows = g->n_q_heads / g->n_kv_heads * g->n_draft, pairs = g->n_seq * g->n_kv_heads;
-    if (splits < 2 || svh::row_tiles(g) > 1 || g->n_draft > 32 || pairs > sm_count() / 2) return 0;
-    const int upb = g->block_size / kUnit, split_blocks = (n_blocks + splits - 1) / splits;
+    const int tiles = svh::row_tiles(g), rows = g->n_q_heads / g->n_kv_heads * svh::tokens_per_tile(g);
+    const int lists = g->n_seq * g->n_kv_heads * tiles, upb = g->block_size / kUnit;   // (a list per row tile)
+    if (splits < 2 || svh::pair_row_tiles(g) || lists > sm_count() / 2 || (rows <= 64 && g->n_draft > 32)) return 0;
+    const int split_blocks = (n_blocks + splits - 1) / splits;
     for (int most = std::min(splits, kMaxCluster); most > 1; --most) {
         const int blocks = (n_blocks + most - 1) / most, c = (n_blocks + blocks - 1) / blocks;
         const int more = rows > 64 ? std::max(kMoreUnitsWide, split_blocks * upb / 2) : kMoreUnits;
         if ((blocks - split_blocks) * upb > more || blocks * upb > kLongSlice) return 0;
-        if (cluster_holds_partials(c, rows) && clusters_at_once(c) >= pairs) return c;
+        if (cluster_holds_partials(c, rows) && clusters_at_once(c) >= lists) return c;
     }
     return 0;
 }

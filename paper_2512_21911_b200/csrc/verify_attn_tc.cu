@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         return false;
     };
 
-    static_assert(!kCluster || (!kWide && !kBal), "clusters merge a single row tile of up to 32 draft tokens");
+    static_assert(!kCluster || (!kPair && !kBal && (!kWide || NH == 4)), "a cluster merges the splits of one row tile");
     static_assert(!kHost || kBal, "lists that are handed out");
     static_assert(!kBal || (kStack && NH < 4), "lists are handed out for stacks, in tiles of up to 64 rows");
     static_assert(!kPair || (kWide && NH == 4), "row-tile pairs exist only where one tile is full (more than 64 rows)");
@@ -200,7 +200,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // those of the executing warpgroup (the query rows of draft tokens i0 .. i0 + Tq - 1).
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform, for all that hangs on it)
     const int n_groups = kPair ? (p.tiles + 1) / 2 : p.tiles;
-    const int split = kBal ? 0 : kWide ? blockIdx.x / n_groups : blockIdx.x, h = blockIdx.y, z = blockIdx.z;   // (kBal: per segment)
+    // (kCluster: a tile's splits are neighbours, for they are a cluster; kBal: per segment)
+    const int split = kBal ? 0 : !kWide ? blockIdx.x : kCluster ? blockIdx.x % p.splits : blockIdx.x / n_groups, h = blockIdx.y, z = blockIdx.z;
     // z numbers what the layer owns (q, out, draft, partials), s its sequence (tables, lengths, parents), lz its list
     int s = z, lz = z;
     const LayerRow *layer = nullptr;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         lz = p.list_of[l] * p.S + s;
         layer = p.layers + l;
     }
-    const int group = kWide && !kBal ? blockIdx.x - split * n_groups : 0;
+    const int group = !kWide || kBal ? 0 : kCluster ? blockIdx.x / p.splits : blockIdx.x - split * n_groups;
     const int tile = kPair ? 2 * group + ((warp >> 2) & 1) : group;
     const int i0 = kWide ? tile * p.Tt : 0, Tq = kWide ? max(0, min(p.Tt, p.T - i0)) : p.T;
     const int upb = p.B / kUnit;
@@ -1557,7 +1558,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
             const int ii = div_g(row), g = row - ii * p.G;
-            const size_t orow = ((size_t)out_z * p.T + ii) * p.Hq + out_h * p.G + g;
+            const size_t orow = ((size_t)out_z * p.T + i0 + ii) * p.Hq + out_h * p.G + g;
 #pragma unroll
             for (int x = 0; x < kWords; ++x) {
                 SplitSum sum;
@@ -1618,7 +1619,11 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
                           : launch_tc<2, false, false, false, true>(tm_k, tm_v, p, grid, stream);
     }
     const bool units = p.B == 128;   // 128-row tiles over blocks of 128 tokens: slices cut at 64-key units
-    if (p.cluster) {   // (one row tile of up to 32 draft tokens)
+    if (p.cluster) {
+        if (p.tiles > 1 || p.T > 32) {   // (more than 64 rows, see choose_cluster)
+            return units ? launch_tc<4, true, false, true, false, true>(tm_k, tm_v, p, grid, stream)
+                         : launch_tc<4, true, false, false, false, true>(tm_k, tm_v, p, grid, stream);
+        }
         if (rows <= 32) return launch_tc<1, false, false, false, false, true>(tm_k, tm_v, p, grid, stream);
         if (rows <= 64) return launch_tc<2, false, false, false, false, true>(tm_k, tm_v, p, grid, stream);
         return units ? launch_tc<4, false, false, true, false, true>(tm_k, tm_v, p, grid, stream)

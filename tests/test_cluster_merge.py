@@ -24,6 +24,10 @@ SHAPES = [  # seqs, heads, kv_heads, block, draft, tree
     (4, 64, 8, 128, 16, True),    # ... cut at units
     (8, 28, 4, 64, 11, True),     # 77 rows over four CTAs
     (9, 40, 5, 64, 14, False),    # 112 rows over three CTAs
+    (3, 8, 4, 64, 60, True),      # 120 rows of 60 draft tokens
+    (2, 32, 8, 64, 60, True),     # two tiles, 128 and 112 rows, clusters of four
+    (1, 28, 4, 128, 58, True),    # four tiles, the last one of 28 rows, cut at units
+    (4, 32, 8, 64, 33, False),    # two tiles, the second one of four rows, clusters of two
 ]
 
 
