@@ -99,6 +99,8 @@ int clusters_at_once(int size);
 // tcgen05 / TMEM attention kernel (verify_attn_tc.cu): rows = G*T <= 128 packed as one M=128 tile.
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid,
                            cudaStream_t stream);
+// the lists of a single layer, handed out (layers and claims null: CTA i takes lists i, i + CTAs, ...)
+cudaError_t launch_attn_tc_handed(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const StackAttnParams &p, dim3 grid, cudaStream_t stream);
 cudaError_t launch_attn_tc_stack(const StackAttnParams &p, dim3 grid, cudaStream_t stream);
 
 }  // namespace svk

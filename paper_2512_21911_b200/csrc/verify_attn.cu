@@ -294,6 +294,45 @@ static sv_status check_workspace(int splits, const void *workspace, size_t bytes
     return bytes < needed ? SV_ERR_WORKSPACE : SV_OK;
 }
 
+// Whether a stack's lists are handed out to resident CTAs (see verify_attn_tc.cu, kBal): more lists than SMs, so that CTAs
+// take several, and lists that are not cut to even out their lengths (choose_splits).  Tiles of up to 64 rows only: 128-row
+// tiles are bound by their softmax, not by the gather, and the roles' bookkeeping takes registers from it (8 layers x 4
+// sequences of 96 rows: 95 us handed out, 84 with a CTA per list; 40 layers of 112 rows: 135 and 124).  The rule looks at
+// the whole stack: a layer's result is the same whichever layers a launch covers.
+static bool hand_out(const sv_geom *rule, int max_sel)
+{
+    return svh::row_tiles(rule) == 1 && rule->n_q_heads / rule->n_kv_heads * rule->n_draft <= 64 &&
+           (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
+}
+
+// The same for a single layer, whose CTAs take its lists by turns: from 1.6 lists per SM on (336 lists x 8 units 33.0 -> 30.5 us, 480 x 12 52.1 ->
+// 47.9, 256 x 4 19.0 -> 17.5, 248 x 5 22.9 -> 21.7, 256 x 16 the same; with fewer the second lists run on a part of the SMs, and a CTA
+// of its own has the shorter loop: 192 x 30 46.0 -> 47.1).
+static bool hand_out_layer(const sv_geom *g, int max_sel)
+{
+    return 5 * (long long)g->n_seq * g->n_kv_heads >= 8 * sm_count() && hand_out(g, max_sel);
+}
+
+// Sequences of a layer whose lists go whole, a CTA a list, in a first launch, where the few lists of the others, which would run behind the
+// last full wave on a part of the SMs, do better in clusters in a second one.  A list alone takes 0.43 us a unit; in clusters of c that
+// is 1 / c of it, or what 84 lists take HBM, whichever is longer, and the launch costs about 5 us: 152 lists x 30 units 43.4 -> 37.7
+// us, 152 x 40 58.3 -> 47.2, 160 x 30 of 128 rows 52.8 -> 45.2, 168 x 24 45.7 -> 43.0, 192 x 30 46.0 -> 45.4; below the line 216 x 20 35.5
+// -> 37.3, 176 x 9 22.2 -> 23.4.  (Dense lists differ in length, and the longest of the first launch then keep the second waiting.)
+static int whole_waves(const sv_geom *g, int max_sel)
+{
+    const int sms = sm_count();
+    const long long lists = (long long)g->n_seq * g->n_kv_heads;
+    if (svh::row_tiles(g) > 1 || lists <= sms) return g->n_seq;
+    sv_geom rest = *g;
+    const int whole = (int)(lists / sms * sms / g->n_kv_heads);
+    rest.n_seq = g->n_seq - whole;
+    if (whole < 1 || rest.n_seq < 1) return g->n_seq;
+    const int c = choose_cluster(&rest, max_sel, choose_splits(&rest, max_sel));
+    if (c < 2) return g->n_seq;
+    const double saved = 1.0 - std::max(1.0 / c, rest.n_seq * rest.n_kv_heads / 84.0);
+    return max_sel * (g->block_size / kUnit) * saved * 0.43 >= 5.0 ? whole : g->n_seq;
+}
+
 // `balance`: see choose_splits (the built-in-scratch entry point gives it up when the partials would not fit)
 static sv_status verify_attn_impl(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
                                   const void *draft_v, const int32_t *parent, const int32_t *sel_idx,
@@ -316,15 +355,34 @@ static sv_status verify_attn_impl(const sv_geom *geom, const void *q, const sv_k
     const int64_t n_rows = (int64_t)kv->n_pages * geom->n_kv_heads * geom->block_size;
     if (!pool_tensor_map(kv->k_pool, n_rows, &tk) || !pool_tensor_map(kv->v_pool, n_rows, &tv)) return SV_ERR_CUDA;
 
-    AttnParams p;
-    fill_params(p, geom, geom, splits, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel, softmax_scale, out, lse, workspace,
-                status_word);
-    p.block_table = kv->block_table;
-    p.seq_lens = kv->seq_lens;
-    p.n_pages = kv->n_pages;
-    p.early_gather = early_gather ? 1 : 0;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
-    return launch_attn(p, geom, geom->n_seq, cs, [&](dim3 grid) { return launch_attn_tc(tk, tv, p, grid, cs); });
+    // sequences first .. of a launch of its own
+    const auto launch = [&](const sv_geom &g, int first, int own_splits, bool early) {
+        const auto bf16 = [&](const void *x, int heads) { return static_cast<const __nv_bfloat16 *>(x) + (size_t)first * g.n_draft * heads * 128; };
+        const size_t lists = (size_t)first * g.n_kv_heads;
+        StackAttnParams p;
+        fill_params(p, &g, &g, own_splits, bf16(q, g.n_q_heads), bf16(draft_k, g.n_kv_heads), bf16(draft_v, g.n_kv_heads),
+                    parent ? parent + (size_t)first * g.n_draft : nullptr, sel_idx ? sel_idx + lists * max_sel : nullptr,
+                    sel_cnt ? sel_cnt + lists : nullptr, max_sel, softmax_scale, const_cast<__nv_bfloat16 *>(bf16(out, g.n_q_heads)),
+                    lse ? lse + (size_t)first * g.n_draft * g.n_q_heads : nullptr, workspace, status_word);
+        p.block_table = kv->block_table + (size_t)first * g.max_blocks;
+        p.seq_lens = kv->seq_lens + first;
+        p.n_pages = kv->n_pages;
+        p.early_gather = early ? 1 : 0;
+        if (sel_idx && !early && own_splits == 1 && hand_out_layer(&g, max_sel)) {
+            p.n_claims = g.n_seq * g.n_kv_heads;
+            p.layers = nullptr, p.S = g.n_seq, p.list_of[0] = 0;
+            return launch_attn_tc_handed(tk, tv, p, dim3(std::min(sm_count(), p.n_claims)), cs) == cudaSuccess ? SV_OK : SV_ERR_CUDA;
+        }
+        AttnParams &one = p;
+        return launch_attn(one, &g, g.n_seq, cs, [&](dim3 grid) { return launch_attn_tc(tk, tv, one, grid, cs); });
+    };
+    const int whole = sel_idx && splits == 1 && !early_gather ? whole_waves(geom, max_sel) : geom->n_seq;
+    if (whole == geom->n_seq) return launch(*geom, 0, splits, early_gather);
+    sv_geom head = *geom, rest = *geom;
+    head.n_seq = whole, rest.n_seq = geom->n_seq - whole;
+    st = launch(head, 0, 1, false);
+    return st == SV_OK ? launch(rest, whole, choose_splits(&rest, max_sel, balance), true) : st;
 }
 
 extern "C" sv_status sv_verify_attn(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
@@ -371,17 +429,6 @@ extern "C" sv_status sv_layer_table(const sv_geom *geom, const sv_kv *kv, int32_
         memcpy(static_cast<char *>(table_host) + l * sizeof(LayerRow), &row, sizeof row);
     }
     return SV_OK;
-}
-
-// Whether a stack's lists are handed out to resident CTAs (see verify_attn_tc.cu, kBal): more lists than SMs, so that CTAs
-// take several, and lists that are not cut to even out their lengths (choose_splits).  Tiles of up to 64 rows only: 128-row
-// tiles are bound by their softmax, not by the gather, and the roles' bookkeeping takes registers from it (8 layers x 4
-// sequences of 96 rows: 95 us handed out, 84 with a CTA per list; 40 layers of 112 rows: 135 and 124).  The rule looks at
-// the whole stack: a layer's result is the same whichever layers a launch covers.
-static bool hand_out(const sv_geom *rule, int max_sel)
-{
-    return svh::row_tiles(rule) == 1 && rule->n_q_heads / rule->n_kv_heads * rule->n_draft <= 64 &&
-           (long long)rule->n_seq * rule->n_kv_heads > sm_count() && choose_splits(rule, max_sel) == 1;
 }
 
 // The geometry the split rules see for a stack: every (layer, sequence) is a sequence of one batch.

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // a negative count marks a list that block selection could not produce: attend over the draft tokens
                     // only, and say so
                     if (p.sel_idx && count < 0 && lane == 0 && p.status) atomicOr(p.status, kStatusNoList);
-                    if (cur.l != layer_at) {
+                    if (p.layers && cur.l != layer_at) {
                         mk = &p.layers[cur.l].k_map, mv = &p.layers[cur.l].v_map;
                         n_pages = p.layers[cur.l].n_pages;
                         layer_at = cur.l;
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                     int count_next = 0, L_next = 0, blk_next = 0, page_next = 0, step = 0;
-                    if (lane == 0) claim = (int)ClaimWords{p.claims}.add(0, 1u);
+                    if (lane == 0 && p.claims) claim = (int)ClaimWords{p.claims}.add(0, 1u);   // (else by turns: what comes before is this list)
                     auto prepare_next = [&] {
                         if (step == 0) {
                             claim = claimed_list((uint32_t)__shfl_sync(0xffffffffu, claim, 0), p.n_claims, (int)gridDim.x);
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 if (lane == 0) {
                     __threadfence();   // (this CTA's claims are made before it leaves)
-                    leave_claims(ClaimWords{p.claims}, (int)gridDim.x);
+                    if (p.claims) leave_claims(ClaimWords{p.claims}, (int)gridDim.x);
                     requested[0] = copies.stages, requested[1] = copies.odd;
                     mbar_arrive(bar(kTmemDone));
                 }
@@ -1682,6 +1682,11 @@ int clusters_at_once(int size)
 }
 
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid, cudaStream_t stream)
+{
+    return launch_any(tm_k, tm_v, p, grid, stream);
+}
+
+cudaError_t launch_attn_tc_handed(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const StackAttnParams &p, dim3 grid, cudaStream_t stream)
 {
     return launch_any(tm_k, tm_v, p, grid, stream);
 }
