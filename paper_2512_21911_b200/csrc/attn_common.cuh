@@ -43,7 +43,7 @@ struct AttnParams {
     int pair;        // 1: a CTA serves two row tiles (grid.x = splits x ceil(tiles / 2)); 0: one (grid.x = splits x tiles)
     int n_pages;     // pages in each pool: page ids from the block table are clamped to it
     int n_claims;       // > 0: that many lists are handed out to one CTA per SM (splits = 1)
-    uint32_t *claims;   // ... through these two words (list_claims.h), zero before and after the launch
+    uint32_t *claims;   // ... through these two words (list_claims.h), zero before and after the launch; null: by turns
     int cluster;     // 1: the splits of a (sequence, KV head) are a cluster that merges them itself (no partials, no merge kernel)
     int early_gather;   // 1: nothing the gather reads comes from the kernel just before; it starts ahead of the dependency wait
 };

@@ -1,7 +1,7 @@
 // sv_verify_step_from_host: a verification step whose inputs are in pinned host memory and whose outputs are wanted there.
 // The layers go in chunks: a chunk's inputs are uploaded on one side stream while the chunk before it computes, its
 // outputs leave on another while the chunk behind it computes, so only the first upload and the last download are not
-// hidden.  Bound by PCIe for those two and by the launches between them (32 layers of a 32K context, 3 MiB up, 2 MiB down, two
+// hidden.  (Stacks whose lists are handed out have a form without chunks: host_direct.cu.)  Bound by PCIe for those two and by the launches between them (32 layers of a 32K context, 3 MiB up, 2 MiB down, two
 // halves: 178 us, of which the layers' kernels 113 and the two bare transfers 51).  Everything is enqueued here, in one
 // call: the same sequence of copies, launches and events from Python took about 5 us each, and the step waited for it
 // (245 us).

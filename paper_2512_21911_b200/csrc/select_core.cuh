@@ -1,7 +1,6 @@
 // Exact top-N selection over the order-preserving keys of one (sequence, KV head), run by kThreads threads of
 // one CTA on keys that sit in its shared memory (Section 3.1: the N best-scoring blocks, the first / last few
-// always kept).  Used by the stand-alone selection kernel (select_blocks.cu) and by the attention kernel
-// that selects for itself (verify_attn_tc.cu).  Device code only.
+// always kept).  Device code only.
 //
 // Up to three keys for every sixteen threads are ranked against one another (rank_select below).  Else:
 // fast path (up to 8 keys per thread, scores not all equal): the scores are mapped linearly onto 0..65535

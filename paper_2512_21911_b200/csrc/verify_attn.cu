@@ -7,8 +7,8 @@
 // Grid (split [x row tile], KV head, sequence).  A CTA owns a contiguous slice of the ascending block list
 // of its (sequence, KV head) and the G*T query rows of that KV head (GQA group x draft tokens packed as the
 // M dimension of the tensor-core tiles).  With one split the CTA writes bf16 output directly; otherwise
-// fp32 partials (m, l, o) go to the workspace and the merge kernel below combines them.  The path is bound
-// by HBM bandwidth (512 bytes of K/V per cached token and KV head).
+// fp32 partials (m, l, o) go to the workspace and the merge kernel below combines them, or the CTAs of a list are a
+// cluster that merges its splits itself (choose_cluster).  The path is bound by HBM bandwidth (512 bytes of K/V per cached token and KV head).
 //
 // All device-side waits are bounded: a wait that gives up sets *status_word and the CTA drains without
 // hanging.  Block indices and page ids are clamped into their tables before any address is formed; a

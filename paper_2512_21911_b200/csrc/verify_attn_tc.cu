@@ -26,7 +26,8 @@
 // second), one thread of warp 10 issues every O += P V.  The
 // third warpgroup gives its registers to the other two (setmaxnreg).  Everything is chained with mbarriers; tcgen05.commit signals MMA completion.
 // At the end warpgroup 0 reads both accumulators from TMEM (warp q of either warpgroup owns lane quadrant q),
-// merges them in registers and writes the rows (or the fp32 partial of its split) out.
+// merges them in registers and writes the rows (or the fp32 partial of its split) out.  Where the CTAs of a list are a thread-block
+// cluster (kCluster), they exchange their partials through one another's shared memory and write the rows between them.
 // All waits are bounded; a wait that gives up sets *status and the CTA drains: warp 9 leaves last, and before it
 // frees the TMEM and the CTA its shared memory it waits (again with a limit) for the MMAs that have been issued and, when somebody
 // has given up, for the copies that have been requested (else all of them have been read).
@@ -109,8 +110,8 @@ struct ClaimWords {
 // row tile 2 * pair + w -- its own Q tile, S / P / O buffers -- and takes every unit instead of every other one.  The
 // host chooses it where it saves enough waves of CTAs (svh::pair_row_tiles).
 // kStack: several layers in one launch (StackAttnParams; the tensor maps are then those of the layer table).
-// kBal: one resident CTA per SM that takes whole lists from a counter until there are none left (launches of more lists
-// than SMs).  Between two lists nothing drains: the TMA ring runs on into the next list, and warp 11 has that list's Q
+// kBal: one resident CTA per SM that takes whole lists from a counter (a single layer's by turns) until there are none left (launches
+// of more lists than SMs).  Between two lists nothing drains: the TMA ring runs on into the next list, and warp 11 has that list's Q
 // tile, masks and draft K/V in shared memory by the time the warpgroups have written the last one's rows.  With one CTA
 // per list every list after an SM's first begins with an empty ring, 3 to 4 us of latencies for 45 us of HBM time (32 layers
 // of 8 lists of 65 units: 112.5 -> 106.9 us per step; 64 x 8 lists of 49 units: 155.7 -> 143.6).  Cutting lists so that all CTAs

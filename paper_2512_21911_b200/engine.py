@@ -354,8 +354,9 @@ class SparseVerifier:
 
     def kernels_per_step(self, refresh_tail: bool = False, dense: bool = False) -> int:
         """Kernel launches of one step taken layer by layer (verify_layer, the order in which a model reaches its layers):
-        tail refresh, select per anchor layer, attention (+ merge) per layer.  At most: short lists whose splits are merged inside
-        a cluster have no merge launch, which is counted here all the same."""
+        tail refresh, select per anchor layer, attention (+ merge) per layer.  Lists that are merged inside a
+        cluster have no merge launch, which is counted here all the same; the second attention launch that a batch of a few more
+        lists than SMs may take is not."""
         splits = sv.sv_verify_attn_splits(self.geom, self.geom.max_blocks if dense else self.max_sel)
         attn = self.n_layers * (2 if splits > 1 else 1)
         if dense:
