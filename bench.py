@@ -346,7 +346,7 @@ def run_gpu(args):
         ms = time_replays(g_step, args.steps, args.warmup)
         if rank == 0:
             print(json.dumps({"only_step": True, "layers": w.n_layers, "us_per_layer": ms * 1e3 / w.n_layers,
-                              "kernels_per_step": eng.kernels_per_step(refresh_tail=True)}))
+                              "kernels_per_step": eng.launches_per_step(refresh_tail=True)}))
         return
     g_reuse = capture(lambda: by_layer(eng_reuse))
     g_chain = capture(lambda: by_layer(eng_chain))
@@ -500,13 +500,13 @@ def run_gpu(args):
         "e2e": {"value": ms_e2e * 1e3 / (w.n_layers * world), "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h,
                 "note": "steps one after the other (a decoding loop cannot overlap neighbouring steps: the next queries "
-                        "depend on this step's acceptance); within a step all layers' queries are there at once and the layers of "
-                        "a chunk run together, which a transformer's layers cannot (the queries of a layer depend on the output "
+                        "depend on this step's acceptance); within a step all layers' queries are there at once and the layers "
+                        "run together, which a transformer's layers cannot (the queries of a layer depend on the output "
                         "of the one before), so this is not `value`, which goes layer by layer, plus the copies: that is "
                         "one_stream_value; every step is one call of SparseVerifier.verify_step_from_host: "
                         "Q and draft K/V of all layers from pinned host memory, the step, the outputs back to pinned host "
-                        "memory, the copies in chunks of layers, in the background so that all but the first upload "
-                        "and the last download run under the step's kernels; the KV cache is device-resident state",
+                        "memory, by the attention launch itself as it takes and leaves each list (in chunks of layers, where asked "
+                        "for: copies in the background); the KV cache is device-resident state",
                 "layers_per_chunk": e2e_chunks if e2e_chunks is not None else "the engine's schedule",
                 "one_stream_value": ms_e2e_one_stream * 1e3 / (w.n_layers * world),
                 "one_stream_note": "the step layer by layer, as in `value`, with the same bytes copied whole before and after it on "
@@ -514,8 +514,8 @@ def run_gpu(args):
                 "pipelined_value": ms_e2e_pipelined * 1e3 / (w.n_layers * world),
                 "pipelined_note": "the same copies with two buffer sets and three streams, so that the copies of steps "
                                   "i+1 / i-1 run under the kernels of step i (an upper bound no real loop reaches)"},
-        "gpu_launches": args.steps * eng.kernels_per_step(refresh_tail=True),
-        "kernels_per_step": eng.kernels_per_step(refresh_tail=True),
+        "gpu_launches": args.steps * eng.launches_per_step(refresh_tail=True),
+        "kernels_per_step": eng.launches_per_step(refresh_tail=True),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "peak_kind": f"of {peak_kind}",
                      # dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu capture of this shape, if one
@@ -527,12 +527,12 @@ def run_gpu(args):
         "kv_gathered_gbs": gathered / (us_attn * 1e-6) / 1e9,
         "pct_of_8tbs": 100.0 * gathered / (us_attn * 1e-6) / 8e12,
         "tokens_verified_per_s": S * T * world / (ms_step * 1e-3),
-        "reuse_even_anchors": {"us_per_layer": ms_reuse * 1e3 / w.n_layers, "kernels_per_step": eng_reuse.kernels_per_step(True)},
-        "reuse_previous_layer": {"us_per_layer": ms_chain * 1e3 / w.n_layers, "kernels_per_step": eng_chain.kernels_per_step(True),
+        "reuse_even_anchors": {"us_per_layer": ms_reuse * 1e3 / w.n_layers, "kernels_per_step": eng_reuse.launches_per_step(True)},
+        "reuse_previous_layer": {"us_per_layer": ms_chain * 1e3 / w.n_layers, "kernels_per_step": eng_chain.launches_per_step(True),
                                  "note": "only layer 0 retrieves; every later layer attends over the previous layer's blocks"},
         "all_layers_at_once": {"us_per_layer": ms_stack * 1e3 / w.n_layers,
                                "note": "verify_step with the inputs of all layers in hand: one launch for all selections, one "
-                                       "for all attention (what the host-fed step runs per chunk); `value` goes layer by layer"},
+                                       "for all attention (what the host-fed step runs); `value` goes layer by layer"},
         "dense_verify": {"us_per_layer": us_dense, "gbs": dense_bytes / (us_dense * 1e-6) / 1e9,
                          "frac": dense_bytes / (us_dense * 1e-6) / 1e9 / peak, "bytes_per_launch": dense_bytes},
         "block_reps_rebuild": {"us_per_layer": ms_reps * 1e3 / w.n_layers, "bytes_per_launch": reps_bytes,

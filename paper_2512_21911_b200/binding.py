@@ -27,7 +27,7 @@ SV_STATUS_WAIT_MASK, SV_STATUS_INDEX, SV_STATUS_NO_LIST = 0x0FF, 0x100, 0x200
 SV_NOALLOC_SCRATCH_BYTES = 4 * 1024 * 1024   # size of the library's built-in scratch (sv_verify_attn_noalloc)
 
 EXPORTS = ("sv_strerror", "sv_status_word_check", "sv_budget_blocks", "sv_workspace_bytes", "sv_block_reps", "sv_select_blocks",
-           "sv_verify_attn", "sv_verify_attn_reused", "sv_verify_attn_splits", "sv_verify_attn_noalloc", "sv_kv_append", "sv_anchor_jaccard", "sv_pick_anchors",
+           "sv_verify_attn", "sv_verify_attn_reused", "sv_verify_attn_splits", "sv_verify_attn_launches", "sv_verify_attn_noalloc", "sv_kv_append", "sv_anchor_jaccard", "sv_pick_anchors",
            "sv_select_blocks_tokens", "sv_token_overlap", "sv_select_blocks_global", "sv_accept",
            "sv_block_reps_bf16", "sv_select_blocks_bf16reps", "sv_layer_table_bytes", "sv_layer_table", "sv_workspace_bytes_layers",
            "sv_block_reps_layers", "sv_select_blocks_layers", "sv_verify_attn_layers", "sv_kv_append_layers", "sv_host_step_create",
@@ -71,6 +71,8 @@ def _load() -> ctypes.CDLL:
     lib.sv_workspace_bytes.argtypes = [gp, i32]
     lib.sv_verify_attn_splits.restype = i32
     lib.sv_verify_attn_splits.argtypes = [gp, i32]
+    lib.sv_verify_attn_launches.restype = i32
+    lib.sv_verify_attn_launches.argtypes = [gp, i32]
     lib.sv_block_reps.restype = ctypes.c_int
     lib.sv_block_reps.argtypes = [gp, kp, i32, i32, vp, vp]
     lib.sv_select_blocks.restype = ctypes.c_int
@@ -157,6 +159,10 @@ def sv_workspace_bytes(geom: sv_geom, max_sel: int) -> int:
 
 def sv_verify_attn_splits(geom: sv_geom, max_sel: int) -> int:
     return int(_lib.sv_verify_attn_splits(ctypes.byref(geom), max_sel))
+
+
+def sv_verify_attn_launches(geom: sv_geom, max_sel: int) -> int:
+    return int(_lib.sv_verify_attn_launches(ctypes.byref(geom), max_sel))
 
 
 def sv_block_reps(geom: sv_geom, kv: sv_kv, reps: torch.Tensor, block_begin: int = 0, block_end: int = -1,

@@ -385,6 +385,14 @@ static sv_status verify_attn_impl(const sv_geom *geom, const void *q, const sv_k
     return st == SV_OK ? launch(rest, whole, choose_splits(&rest, max_sel, balance), true) : st;
 }
 
+extern "C" int32_t sv_verify_attn_launches(const sv_geom *geom, int32_t max_sel)
+{
+    if (svh::check_geom(geom) != SV_OK || max_sel < 1) return 0;
+    const int splits = choose_splits(geom, max_sel);
+    if (splits > 1) return choose_cluster(geom, max_sel, splits) > 1 ? 1 : 2;
+    return whole_waves(geom, max_sel) < geom->n_seq ? 2 : 1;
+}
+
 extern "C" sv_status sv_verify_attn(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
                                     const void *draft_v, const int32_t *parent, const int32_t *sel_idx,
                                     const int32_t *sel_cnt, int32_t max_sel, float softmax_scale, void *out,

@@ -354,12 +354,17 @@ class SparseVerifier:
 
     def kernels_per_step(self, refresh_tail: bool = False, dense: bool = False) -> int:
         """Kernel launches of one step taken layer by layer (verify_layer, the order in which a model reaches its layers):
-        tail refresh, select per anchor layer, attention (+ merge) per layer.  Lists that are merged inside a
-        cluster have no merge launch, which is counted here all the same; the second attention launch that a batch of a few more
-        lists than SMs may take is not."""
+        tail refresh, select per anchor layer, attention (+ merge) per layer.  Lists that are merged inside a cluster
+        have no merge launch, which is counted here all the same; launches_per_step
+        leaves it out."""
         splits = sv.sv_verify_attn_splits(self.geom, self.geom.max_blocks if dense else self.max_sel)
         attn = self.n_layers * (2 if splits > 1 else 1)
         if dense:
             return attn
         refresh = 0 if not refresh_tail else (1 if self._stacked() else sum(self.anchors))
         return refresh + sum(self.anchors) + attn
+
+    def launches_per_step(self, refresh_tail: bool = False) -> int:
+        """Kernel launches of one sparse step taken layer by layer, as they are made on this device."""
+        refresh = 0 if not refresh_tail else (1 if self._stacked() else sum(self.anchors))
+        return refresh + sum(self.anchors) + self.n_layers * sv.sv_verify_attn_launches(self.geom, self.max_sel)
