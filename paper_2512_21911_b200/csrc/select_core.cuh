@@ -17,22 +17,19 @@
 
 #include <type_traits>
 
+#include "order_key.h"
+
 namespace svsel {
 
 // Histogram bin -> shared-memory slot: one pad word per 32 bins, so that a warp whose lane j reads bins
 // 8j .. 8j+7 (the scan below) touches 32 different banks with every load.
 constexpr int kHistSlots = 256 + 8;
 constexpr int kFastCap = 64;     // at most this many keys left at the boundary after the histogram levels
-constexpr uint32_t kForcedKey = 0xFFFFFFFFu;   // key of a block that is kept whatever its score (sink / local)
 
 __device__ __forceinline__ uint32_t hist_slot(uint32_t bin) { return bin + (bin >> 5); }
 
 // Order-preserving map float -> uint32 (larger score, larger key; -0 and +0 coincide) and its inverse.
-__device__ __forceinline__ uint32_t order_key(float x)
-{
-    const uint32_t u = __float_as_uint(x + 0.0f);   // -0 -> +0
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
+__device__ __forceinline__ uint32_t order_key(float x) { return key_of_bits(__float_as_uint(x + 0.0f)); }   // (+ 0: -0 -> +0)
 __device__ __forceinline__ float key_score(uint32_t k)
 {
     return __uint_as_float((k & 0x80000000u) ? (k ^ 0x80000000u) : ~k);
