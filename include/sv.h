@@ -178,7 +178,8 @@ SV_API sv_status sv_kv_append(const sv_geom *geom, void *k_pool, void *v_pool, i
  * reuse_prev == 0: score[s][h][b] = mean_g(q[s][0][h*G+g]) . reps[s][h][b] in
  *   fp32; the first n_sink and last n_local blocks are always kept (they count
  *   against the budget); then the highest scores until budget_blocks[s] blocks
- *   are kept (equal scores: smaller block index first).  A budget >= the
+ *   are kept (equal scores: smaller block index first; a NaN ranks between
+ *   the negative scores and zero).  A budget >= the
  *   number of blocks keeps all of them.  The effective budget is clamped to
  *   [forced blocks, max_sel].
  * reuse_prev != 0: out_idx / out_cnt become copies of prev_idx / prev_cnt

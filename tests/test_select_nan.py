@@ -1,5 +1,5 @@
 """Scores that are not numbers: the key of a score (csrc/order_key.h), driven on the host, is never that of a block kept without eviction; on the
-GPU a NaN query or NaN representatives leave every list at its length, with the NaN blocks ahead of the numbers, and nothing behind it written."""
+GPU a NaN query or NaN representatives leave every list at its length, with the NaN blocks between the negative scores and zero, and nothing behind it written."""
 import math
 import os
 import subprocess
@@ -21,14 +21,14 @@ int main()
     using svsel::key_of_bits;
     for (uint64_t b = 0; b < 1ull << 32; b += (b & 0x7FFFFF) < 3 || (b & 0x7FFFFF) > 0x7FFFF0 ? 1 : 61)
         if (key_of_bits((uint32_t)b) == svsel::kForcedKey) return printf("%08x has the key of a forced block\n", (unsigned)b), 1;
-    // neighbouring numbers, from -inf to +inf, in their order; a NaN with its sign clear above all of them
+    // neighbouring numbers, from -inf to +inf, in their order; every NaN between the largest negative one and zero
     for (uint32_t b = 0x807FFFFFu; b < 0xFF800000u; b += 4099)
         if (!(number(b + 1) < number(b) && key_of_bits(b + 1) < key_of_bits(b))) return printf("order at %08x\n", b), 1;
     for (uint32_t b = 0; b < 0x7F800000u; b += 4099)
         if (!(number(b) < number(b + 1) && key_of_bits(b) < key_of_bits(b + 1))) return printf("order at %08x\n", b), 1;
     if (!(key_of_bits(0xFF800000u) < key_of_bits(0x80800000u) && key_of_bits(0x80000001u) < key_of_bits(0u))) return printf("signs\n"), 1;
-    for (uint32_t nan : {0x7FFFFFFFu, 0x7FC00000u, 0x7FFFFFFEu, 0x7F800001u})
-        if (!std::isnan(number(nan)) || key_of_bits(nan) <= key_of_bits(0x7F800000u)) return printf("NaN %08x\n", nan), 1;
+    for (uint32_t nan : {0x7FFFFFFFu, 0x7FC00000u, 0x7FFFFFFEu, 0x7F800001u, 0xFFFFFFFFu, 0xFFC00000u, 0xFF800001u})
+        if (!std::isnan(number(nan)) || key_of_bits(nan) <= key_of_bits(0x80000001u) || key_of_bits(nan) >= key_of_bits(0u)) return printf("NaN %08x\n", nan), 1;
     return 0;
 }
 """
@@ -71,5 +71,5 @@ def test_lists_of_nan_scores_keep_their_length(seqs, nb):
     forced = [0, nb - 2, nb - 1]
     got = idx.cpu()
     for s, of in enumerate(scores.tolist()):
-        rest = sorted(range(1, nb - 2), key=lambda b: (0, 0.0, b) if math.isnan(of[b]) else (1, -of[b], b))
+        rest = sorted(range(1, nb - 2), key=lambda b: (-of[b], b) if not math.isnan(of[b]) else (1e-40, b))
         assert got[s, 0].tolist() == sorted(forced + rest[:keep - 3]), (s, nb)
