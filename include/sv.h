@@ -467,7 +467,8 @@ SV_API sv_status sv_verify_step_from_host_direct(const sv_geom *geom, const sv_l
  * fewer where the CTAs of a thread-block cluster merge their splits themselves (the workspace is then not written). */
 SV_API int32_t sv_verify_attn_splits(const sv_geom *geom, int32_t max_sel);
 /* Kernels that sv_verify_attn launches over lists of up to max_sel blocks: the merge of the splits and the rest of a batch of a few more lists than
- * SMs are launches of their own.  0 for an invalid geometry. */
+ * SMs are launches of their own.  (Dense calls and sv_verify_attn_reused have no such rest: one launch where sv_verify_attn_splits is 1, this
+ * number where it is more.)  0 for an invalid geometry. */
 SV_API int32_t sv_verify_attn_launches(const sv_geom *geom, int32_t max_sel);
 
 #ifdef __cplusplus

@@ -353,18 +353,24 @@ class SparseVerifier:
             self.dense_layer(l, q[l], draft_k[l], draft_v[l], out[l])
 
     def kernels_per_step(self, refresh_tail: bool = False, dense: bool = False) -> int:
-        """Kernel launches of one step taken layer by layer (verify_layer, the order in which a model reaches its layers):
-        tail refresh, select per anchor layer, attention (+ merge) per layer.  Lists that are merged inside a cluster
-        have no merge launch, which is counted here all the same; launches_per_step
-        leaves it out."""
+        """An upper bound for the kernel launches of one step taken layer by layer (verify_layer, the order in which a model reaches
+        its layers): tail refresh, select per anchor layer, attention per layer and, where lists are split, a merge kernel, which the
+        splits that a cluster merges do not have; two launches where the rest of a batch goes by itself.  A sparse step's own number
+        is launches_per_step."""
         splits = sv.sv_verify_attn_splits(self.geom, self.geom.max_blocks if dense else self.max_sel)
         attn = self.n_layers * (2 if splits > 1 else 1)
         if dense:
             return attn
+        attn = max(attn, self.n_layers * sv.sv_verify_attn_launches(self.geom, self.max_sel))
         refresh = 0 if not refresh_tail else (1 if self._stacked() else sum(self.anchors))
         return refresh + sum(self.anchors) + attn
 
     def launches_per_step(self, refresh_tail: bool = False) -> int:
-        """Kernel launches of one sparse step taken layer by layer, as they are made on this device."""
+        """Kernel launches of one sparse step taken layer by layer, each behind its own preceding layer (verify_layer with
+        behind_own_layer, as in verify_step), as they are made on this device."""
         refresh = 0 if not refresh_tail else (1 if self._stacked() else sum(self.anchors))
-        return refresh + sum(self.anchors) + self.n_layers * sv.sv_verify_attn_launches(self.geom, self.max_sel)
+        selecting = sv.sv_verify_attn_launches(self.geom, self.max_sel)
+        # (a reused list of more lists than SMs has no second launch for the rest, see sv_verify_attn_launches)
+        reusing = 1 if sv.sv_verify_attn_splits(self.geom, self.max_sel) == 1 else selecting
+        n = sum(map(bool, self.anchors))
+        return refresh + n + n * selecting + (self.n_layers - n) * reusing
