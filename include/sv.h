@@ -235,7 +235,9 @@ SV_API sv_status sv_verify_attn(const sv_geom *geom, const void *q, const sv_kv 
 /*
  * sv_verify_attn for a layer that reuses a block list selected by an earlier layer (Section 3.3, Eq. 9: a
  * non-anchor layer takes the preceding anchor's blocks, so nothing has to be retrieved before it attends).
- * Same arguments and results.  The caller vouches that nothing the gather reads -- sel_idx, sel_cnt,
+ * Same arguments; the results are equal to bf16 rounding, and bit for bit where sv_verify_attn takes the lists the same way: in a batch of
+ * more lists than SMs it may hand them out by turns, or take the last few in a launch of their own, which this call does not.  The
+ * caller vouches that nothing the gather reads -- sel_idx, sel_cnt,
  * block_table, seq_lens and the K/V pools -- is written by the kernel that immediately precedes this call in the
  * stream (q, draft_k, draft_v and parent may be).  The kernels of this library are chained by programmatic
  * dependent launch, so the call's thread blocks are resident while that kernel drains; with the promise they
