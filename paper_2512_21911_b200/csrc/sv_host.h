@@ -106,6 +106,27 @@ struct OncePerDevice {
     }
 };
 
+// What the current device answers to a question (0 or more), asked until it does: a query that fails (`ask` returns less than 0) is an answer
+// of 0 for this call and asked again by the next.
+struct AnswerPerDevice {
+    std::atomic<int> known[kMaxDevices] = {};   // 1 + the answer
+    template <class F>
+    int get(F ask)
+    {
+        const int dev = current_device();
+        if (dev < 0 || dev >= kMaxDevices) return 0;
+        const int v = known[dev].load(std::memory_order_acquire);
+        if (v > 0) return v - 1;
+        const int n = ask();
+        if (n < 0) {
+            (void)cudaGetLastError();   // (not an error of the call that asked)
+            return 0;
+        }
+        known[dev].store(1 + n, std::memory_order_release);
+        return n;
+    }
+};
+
 // SMs of the current device (148 when there is no device to ask).
 inline int sm_count()
 {

@@ -34,7 +34,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
-#include <atomic>
+#include <algorithm>
 #include <type_traits>
 
 #include "attn_common.cuh"
@@ -1654,11 +1654,9 @@ bool cluster_holds_partials(int splits, int rows)
 
 int clusters_at_once(int size)
 {
-    static std::atomic<int> known[svh::kMaxDevices][kMaxCluster + 1];   // 1 + the answer
-    const int dev = svh::current_device();
-    if (size < 2 || size > kMaxCluster || dev < 0 || dev >= svh::kMaxDevices) return 0;
-    int n = known[dev][size].load(std::memory_order_acquire);
-    if (n == 0) {
+    if (size < 2 || size > kMaxCluster) return 0;
+    static svh::AnswerPerDevice known[kMaxCluster + 1];
+    return known[size].get([size] {
         constexpr auto kernel = verify_attn_tc_kernel<4, false, false, false, false, false, true, false>;   // (all forms take a whole SM a CTA)
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(size, 1, 1);
@@ -1672,14 +1670,10 @@ int clusters_at_once(int size)
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int fit = 0;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesBal) != cudaSuccess ||
-            cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) != cudaSuccess)
-            fit = 0;
-        (void)cudaGetLastError();   // a refusal is an answer, not an error of the call that asked
-        n = 1 + fit;
-        known[dev][size].store(n, std::memory_order_release);
-    }
-    return n - 1;
+        const bool answered = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytesBal) == cudaSuccess &&
+                              cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess;
+        return answered ? std::max(fit, 0) : -1;
+    });
 }
 
 cudaError_t launch_attn_tc(const CUtensorMap &tm_k, const CUtensorMap &tm_v, const AttnParams &p, dim3 grid, cudaStream_t stream)
