@@ -48,7 +48,14 @@ extern "C" sv_status sv_verify_step_from_host_direct(const sv_geom *geom, const 
     const svh::HostTensors host = {svh::mapped(q_host), svh::mapped(draft_k_host), svh::mapped(draft_v_host), svh::mapped(out_host)};
     for (const void *p : {host.q, host.draft_k, host.draft_v, static_cast<const void *>(host.out)})
         if (!p || !svh::aligned(p, 16)) return SV_ERR_UNSUPPORTED;
-    if (!svh::aligned(q, 16) || !svh::aligned(draft_k, 16) || !svh::aligned(draft_v, 16)) return SV_ERR_ALIGN;
+    // everything that a later launch would refuse, ahead of the first one
+    const auto attend = [&](bool check_only) {
+        return svh::verify_attn_from_host(geom, layers, anchors, host, q, draft_k, draft_v, parent, idx, cnt, max_sel, out, workspace,
+                                          workspace_bytes, status_word, stream, check_only);
+    };
+    st = svh::check_select_layers(geom, anchors, q, reps, budget_blocks, n_sink, n_local, idx, cnt, max_sel);
+    if (st == SV_OK) st = attend(true);
+    if (st != SV_OK) return st;
     FirstRows rows;
     rows.from = static_cast<const uint4 *>(host.q), rows.to = static_cast<uint4 *>(q);
     rows.words = geom->n_q_heads * 16, rows.pitch = geom->n_draft * geom->n_q_heads * 16, rows.S = geom->n_seq;
@@ -75,6 +82,5 @@ extern "C" sv_status sv_verify_step_from_host_direct(const sv_geom *geom, const 
     }
     st = sv_select_blocks_layers(geom, layers, 0, layers->n_layers, anchors, q, reps, budget_blocks, n_sink, n_local, idx, cnt, max_sel, stream);
     if (st != SV_OK) return st;
-    return svh::verify_attn_from_host(geom, layers, anchors, host, q, draft_k, draft_v, parent, idx, cnt, max_sel, out, workspace, workspace_bytes,
-                                      status_word, stream);
+    return attend(false);
 }

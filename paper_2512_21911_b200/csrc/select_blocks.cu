@@ -395,13 +395,9 @@ extern "C" sv_status sv_select_blocks_layers(const sv_geom *geom, const sv_layer
                                              const int32_t *budget_blocks, int32_t n_sink, int32_t n_local, int32_t *out_idx,
                                              int32_t *out_cnt, int32_t max_sel, void *stream)
 {
-    const sv_status st = svh::check_layers(geom, layers, first, end);
+    sv_status st = svh::check_layers(geom, layers, first, end);
+    if (st == SV_OK) st = svh::check_select_layers(geom, anchors, q, reps, budget_blocks, n_sink, n_local, out_idx, out_cnt, max_sel);
     if (st != SV_OK) return st;
-    if (!anchors || !q || !reps || !budget_blocks || !out_idx || !out_cnt) return SV_ERR_NULL;
-    if (!svh::aligned(q, 16) || !svh::aligned(reps, 16)) return SV_ERR_ALIGN;
-    if (max_sel < 1 || n_sink < 0 || n_local < 0) return SV_ERR_SHAPE;
-    if (n_sink + n_local > max_sel) return SV_ERR_BUDGET;
-    if (geom->max_blocks > svh::kMaxBlocksSelect) return SV_ERR_UNSUPPORTED;
     StackSelectParams p;
     int before = 0, n = 0;   // anchors ahead of `first`, anchors of this call
     for (int l = 0; l < end; ++l) {

@@ -67,6 +67,17 @@ inline sv_status check_layers(const sv_geom *g, const sv_layers *layers, int32_t
     return SV_OK;
 }
 
+// What sv_select_blocks_layers takes besides the layers.
+inline sv_status check_select_layers(const sv_geom *g, const uint8_t *anchors, const void *q, const float *reps, const int32_t *budget_blocks,
+                                     int32_t n_sink, int32_t n_local, const int32_t *out_idx, const int32_t *out_cnt, int32_t max_sel)
+{
+    if (!anchors || !q || !reps || !budget_blocks || !out_idx || !out_cnt) return SV_ERR_NULL;
+    if (!aligned(q, 16) || !aligned(reps, 16)) return SV_ERR_ALIGN;
+    if (max_sel < 1 || n_sink < 0 || n_local < 0) return SV_ERR_SHAPE;
+    if ((int64_t)n_sink + n_local > max_sel) return SV_ERR_BUDGET;
+    return g->max_blocks > kMaxBlocksSelect ? SV_ERR_UNSUPPORTED : SV_OK;
+}
+
 // Launch attribute for programmatic dependent launch: the kernel may be scheduled while its
 // predecessor in the stream drains; every kernel of the library executes griddepcontrol.wait before it
 // reads anything the predecessor wrote.
@@ -186,15 +197,16 @@ inline void *mapped(const void *host)
 
 // Attention of a whole stack whose inputs are read from pinned host memory (device addresses of it) and whose outputs go there too
 // (kHost in verify_attn_tc.cu); q, draft_k, draft_v and out are written on the way.  SV_ERR_UNSUPPORTED, with nothing launched, where the
-// stack's lists are not handed out.
+// stack's lists are not handed out.  check_only: what the call would say to its arguments, with nothing launched.
 struct HostTensors {
     const void *q, *draft_k, *draft_v;
     void *out;
 };
 sv_status verify_attn_from_host(const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors, const HostTensors &host, void *q,
                                 void *draft_k, void *draft_v, const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
-                                int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream);
-// Whether it would.
+                                int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream,
+                                bool check_only);
+// Whether they are.
 bool lists_handed_out(const sv_geom *geom, const sv_layers *layers, int32_t max_sel);
 
 inline sv_status launch_status()

@@ -493,7 +493,8 @@ static sv_status attn_layers_impl(const sv_geom *geom, const sv_layers *layers, 
                                   const uint8_t *anchors, const void *q, const void *draft_k, const void *draft_v,
                                   const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
                                   int32_t max_sel, float softmax_scale, void *out, void *workspace,
-                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits, const svh::HostTensors *host)
+                                  size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits, const svh::HostTensors *host,
+                                  bool check_only)
 {
     sv_status st = svh::check_layers(geom, layers, first, end);
     if (st != SV_OK) return st;
@@ -516,6 +517,8 @@ static sv_status attn_layers_impl(const sv_geom *geom, const sv_layers *layers, 
     st = check_workspace(handed ? 2 : splits, workspace, workspace_bytes,
                          handed ? (size_t)SV_STACK_STATE_BYTES : workspace_bytes_for(&rule, max_sel, true));
     if (st != SV_OK) return st;
+    if (host && !handed) return SV_ERR_UNSUPPORTED;
+    if (check_only) return SV_OK;
     StackAttnParams p;
     const size_t skip = (size_t)first * geom->n_seq * geom->n_draft * 128;   // rows of the layers ahead, per head
     const auto from_first = [&](const void *x, int heads) { return static_cast<const __nv_bfloat16 *>(x) + skip * heads; };
@@ -533,7 +536,6 @@ static sv_status attn_layers_impl(const sv_geom *geom, const sv_layers *layers, 
     }
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     if (host) {
-        if (!handed) return SV_ERR_UNSUPPORTED;
         p.q_host = static_cast<const __nv_bfloat16 *>(host->q), p.out_host = static_cast<__nv_bfloat16 *>(host->out);
         p.draft_k_host = static_cast<const __nv_bfloat16 *>(host->draft_k), p.draft_v_host = static_cast<const __nv_bfloat16 *>(host->draft_v);
     }
@@ -553,15 +555,16 @@ sv_status svh::verify_attn_layers(const sv_geom *geom, const sv_layers *layers, 
                                   size_t workspace_bytes, int32_t *status_word, void *stream, bool own_splits)
 {
     return attn_layers_impl(geom, layers, first, end, anchors, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel, softmax_scale, out,
-                            workspace, workspace_bytes, status_word, stream, own_splits, nullptr);
+                            workspace, workspace_bytes, status_word, stream, own_splits, nullptr, false);
 }
 
 sv_status svh::verify_attn_from_host(const sv_geom *geom, const sv_layers *layers, const uint8_t *anchors, const HostTensors &host, void *q,
                                      void *draft_k, void *draft_v, const int32_t *parent, const int32_t *sel_idx, const int32_t *sel_cnt,
-                                     int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream)
+                                     int32_t max_sel, void *out, void *workspace, size_t workspace_bytes, int32_t *status_word, void *stream,
+                                     bool check_only)
 {
     return attn_layers_impl(geom, layers, 0, layers ? layers->n_layers : 1, anchors, q, draft_k, draft_v, parent, sel_idx, sel_cnt, max_sel,
-                            0.f, out, workspace, workspace_bytes, status_word, stream, false, &host);
+                            0.f, out, workspace, workspace_bytes, status_word, stream, false, &host, check_only);
 }
 
 bool svh::lists_handed_out(const sv_geom *geom, const sv_layers *layers, int32_t max_sel)
