@@ -304,7 +304,7 @@ static sv_status select_impl(const sv_geom *geom, const void *q, const void *rep
     if (!q || !reps || !seq_lens || !budget_blocks) return SV_ERR_NULL;
     if (!svh::aligned(q, 16) || !svh::aligned(reps, 16)) return SV_ERR_ALIGN;
     if (n_sink < 0 || n_local < 0) return SV_ERR_SHAPE;
-    if (n_sink + n_local > max_sel) return SV_ERR_BUDGET;
+    if ((int64_t)n_sink + n_local > max_sel) return SV_ERR_BUDGET;   // (their sum may not fit 32 bits)
     if (geom->max_blocks > svh::kMaxBlocksSelect) return SV_ERR_UNSUPPORTED;
 
     SelectParams p;

@@ -73,3 +73,15 @@ def test_lists_of_nan_scores_keep_their_length(seqs, nb):
     for s, of in enumerate(scores.tolist()):
         rest = sorted(range(1, nb - 2), key=lambda b: (-of[b], b) if not math.isnan(of[b]) else (1e-40, b))
         assert got[s, 0].tolist() == sorted(forced + rest[:keep - 3]), (s, nb)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_sink, n_local", [(1 << 30, 1 << 30), (2 ** 31 - 1, 1), (2 ** 31 - 1, 2 ** 31 - 1), (12, 0)])
+def test_forced_blocks_beyond_the_list_are_refused(n_sink, n_local):
+    import paper_2512_21911_b200 as sv
+    q, reps = torch.ones((1, 1, 1, 128), device="cuda").bfloat16(), torch.zeros((1, 1, 64, 128), device="cuda")
+    idx, cnt = torch.full((1, 1, 11), -7, dtype=torch.int32, device="cuda"), torch.full((1, 1), -7, dtype=torch.int32, device="cuda")
+    i32 = lambda x: torch.tensor([x], dtype=torch.int32, device="cuda")
+    with pytest.raises(sv.SvError) as e:
+        sv.sv_select_blocks(sv.make_geom(1, 1, 1, 128, 64, 64, 1), q, reps, i32(64 * 64), i32(11), n_sink, n_local, idx, cnt)
+    assert e.value.status == 4 and bool((idx == -7).all()) and int(cnt) == -7
