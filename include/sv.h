@@ -225,7 +225,9 @@ SV_API sv_status sv_select_blocks(const sv_geom *geom, const void *q, const floa
  *                   that may overlap on the GPU need distinct workspaces.
  *   status_word     dev int32 or NULL: bits are set if a kernel gave up on a bounded
  *                   wait or had to clamp an index (see "Device status word" above;
- *                   the output is then invalid)
+ *                   the output is then invalid: where a wait gave up, rows of out and
+ *                   lse, of several lists where a thread block has several, may hold
+ *                   what they held before)
  */
 SV_API sv_status sv_verify_attn(const sv_geom *geom, const void *q, const sv_kv *kv, const void *draft_k,
                          const void *draft_v, const int32_t *parent, const int32_t *sel_idx,

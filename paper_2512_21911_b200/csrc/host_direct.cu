@@ -2,8 +2,9 @@
 // launches: tail blocks, the queries that select, selection, attention.  The attention kernel reads a list's rows from host memory when a
 // CTA takes the list and writes its outputs there when it is through (kHost in verify_attn_tc.cu); there are no copies ahead of it or
 // behind it, no side streams and no chunks whose launches wait for one another.  Bound by what the K/V take from HBM, by the bus where the
-// queries are many.  32 layers of 8 lists of 64 units, 3 MiB up, 2 MiB down: 176.5 us in two chunks, 137 this way (89 of them HBM); 24 layers
-// x 16 lists of 16 units 139 -> 107; 16 layers x 32 lists x 48 units 257 -> 202.
+// queries are many.  32 layers of 8 lists of 64 units, 3 MiB up, 2 MiB down, all
+// selecting: 176 us in two chunks, 142 this way (100 with everything on the device); every second one selecting 174 and 132 to 137.  On
+// another machine 24 layers x 16 lists of 16 units 139 -> 107, 16 layers x 32 lists x 48 units 257 -> 202.
 #include <cuda_runtime.h>
 
 #include "sv.h"

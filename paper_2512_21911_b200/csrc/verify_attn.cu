@@ -10,8 +10,8 @@
 // fp32 partials (m, l, o) go to the workspace and the merge kernel below combines them, or the CTAs of a list are a
 // cluster that merges its splits itself (choose_cluster).  The path is bound by HBM bandwidth (512 bytes of K/V per cached token and KV head).
 //
-// All device-side waits are bounded: a wait that gives up sets *status_word and the CTA drains without
-// hanging.  Block indices and page ids are clamped into their tables before any address is formed; a
+// All device-side waits for data are bounded: a wait that gives up sets *status_word and the CTA drains without
+// hanging (the barriers of a cluster have no limit of their own: every warp comes to them behind bounded waits, or has left).  Block indices and page ids are clamped into their tables before any address is formed; a
 // clamp that fires also sets a bit of *status_word.
 #include <cuda.h>
 #include <cuda_bf16.h>

@@ -28,7 +28,9 @@
 // At the end warpgroup 0 reads both accumulators from TMEM (warp q of either warpgroup owns lane quadrant q),
 // merges them in registers and writes the rows (or the fp32 partial of its split) out.  Where the CTAs of a list are a thread-block
 // cluster (kCluster), they exchange their partials through one another's shared memory and write the rows between them.
-// All waits are bounded; a wait that gives up sets *status and the CTA drains: warp 9 leaves last, and before it
+// All waits on mbarriers are bounded; a wait that gives up sets *status and the CTA drains.  barrier.cluster.wait (kCluster) has no limit, and
+// needs none: before it a warp only waits on mbarriers of its own CTA, within their limits, and it arrives or leaves whether or not they
+// gave up, so that every warp of every CTA gets there.  When a CTA drains, warp 9 leaves last, and before it
 // frees the TMEM and the CTA its shared memory it waits (again with a limit) for the MMAs that have been issued and, when somebody
 // has given up, for the copies that have been requested (else all of them have been read).
 #include <cuda.h>
@@ -117,6 +119,8 @@ struct ClaimWords {
 // of 8 lists of 65 units: 112.5 -> 106.9 us per step; 64 x 8 lists of 49 units: 155.7 -> 143.6).  Cutting lists so that all CTAs
 // end together costs more than it gains: the CTAs that are left have the HBM bandwidth to themselves, and partials have
 // to be written and merged (117 and 149 us).
+// A CTA that gives up leaves the rows of the list it has, and by turns of all lists that would have been its, as the caller had them in
+// out and lse (the counter's go to other CTAs); the status word says so.
 // kCluster (one row tile): the CTAs of a (sequence, KV head) are a thread-block cluster that merges its splits itself: no partials in
 // memory, no merge kernel.  CTA r writes the r-th share of the rows; the others push their partials of these rows into its
 // shared memory with stores that count their bytes on a barrier there, so that nothing but the data is waited for (two cluster
@@ -500,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         next_stage();
                     }
                     while (step < 2) prepare_next();
-                    // a CTA that has given up claims nothing more: the lists that are left go to the others
+                    // a CTA that has given up claims nothing more: the counter's lists go to the others, by turns its own stay undone
                     if (claim < 0 || __any_sync(0xffffffffu, dead || *abort_flag)) break;
                     cur = nxt, count = uniform(count_next), n_sel = blocks_of(count), L = uniform(L_next), blk_in = blk_next, page_in = page_next;
                 }
@@ -884,10 +888,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if constexpr (kBal) {
         const Item it = item_at(blockIdx.x);
         if constexpr (kHost) {
-            // The first lists' queries are asked for one CTA after the other, 60 bytes a nanosecond, about as the bus delivers them: the
-            // CTAs then start, and end, one after the other, instead of all of them waiting for the last word.  (32 layers of 8 lists of
-            // 64 units: 131.5 us; all at once 132.4, 46 bytes a nanosecond with the draft's rows counted 138; 24 layers x 16 lists of 16
-            // units: 107, 113.5, 109.5.)
+            // The first lists' queries are asked for one CTA after the other, 60 bytes a nanosecond, about as a PCIe 5 link delivers them: the
+            // CTAs then start, and end, one after the other, instead of all of them waiting for the last word.  A hint, not a wait: the
+            // instruction sleeps for anything up to twice the time, nothing depends on it, and on a slower link it only gains less.  (Against all
+            // at once, one box: 32 layers of 8 lists of 64 units 1 % less, 24 layers x 16 lists of 16 units 6 %; at 46 bytes a nanosecond with
+            // the draft's rows counted 4 % more and 4 % less.)
             if (blockIdx.x > 0) __nanosleep(min(1000000u, blockIdx.x * (unsigned)rows * 256u / 60u));
             fetch_q(smem + OFFQ, it.z, it.h, qtid, kQThreads);
         } else {
@@ -1646,6 +1651,8 @@ static cudaError_t launch_any(const CUtensorMap &tm_k, const CUtensorMap &tm_v, 
                  : launch_tc<4, false, false, false>(tm_k, tm_v, p, grid, stream);
 }
 
+// (128-row tiles in at most four CTAs: a lane of the merge holds the partials of all of them in registers, kIn of them for each of its four
+// words.  Clusters of five and six would take batches there, and have not been measured.)
 bool cluster_holds_partials(int splits, int rows)
 {
     const int share = (rows + splits - 1) / splits, each = kStageBytes / (share * 512);   // partials in a stage, or in a Q tile

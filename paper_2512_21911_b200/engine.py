@@ -215,8 +215,8 @@ class SparseVerifier:
         grew when the previous step's accepted tokens were appended), in one launch: of all layers when the pools were
         given with set_kv_stack, else of the anchor layers.
 
-        All layers' selections are one launch and all their attention another (32 layers of a 32K context: about 115 us
-        instead of 470 layer by layer, where every layer pays the latency chain of its kernels).  A model whose layers
+        All layers' selections are one launch and all their attention another (32 layers of a 32K context: about 110 us
+        instead of 440 layer by layer, where every layer pays the latency chain of its kernels).  A model whose layers
         wait for one another calls verify_layer."""
         if refresh_tail:
             self._refresh_tail(None if self._one_allocation else self._anchor_flags())
@@ -227,20 +227,23 @@ class SparseVerifier:
 
     def verify_step_from_host(self, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host,
                               layers_per_chunk=None, refresh_tail: bool = False) -> None:
-        """verify_step with the step's inputs in pinned host memory and its outputs wanted there.  The copies go in chunks
-        of a few layers (layers_per_chunk: one size, or a list of sizes) on two side streams: a chunk's layers start as soon as its inputs have arrived, its outputs leave
-        while the next chunk computes, so only the first upload and the last download are not hidden behind kernels.
-        q/draft_k/draft_v/out are the device staging tensors (shapes as for verify_step); the *_host tensors the pinned
-        ones.  Returns with everything enqueued; the current stream ends behind the last download.  Capturable in a
-        CUDA graph (the side streams fork from and join the current stream).
+        """verify_step with the step's inputs in pinned host memory and its outputs wanted there.  q/draft_k/draft_v/out are the
+        device staging tensors (shapes as for verify_step); the *_host tensors the pinned ones.  Returns with everything enqueued; the
+        current stream ends behind the last byte that is brought back.  Capturable in a CUDA graph.
 
-        Where the stack's lists are handed out to resident CTAs (more lists than SMs, at most 64 query rows a KV head) and no
-        chunks are asked for, there are none: the attention launch itself reads a list's rows from pinned memory when a CTA takes the
-        list and writes its outputs there.
+        Where the stack's lists are handed out to resident CTAs (more lists than SMs, at most 64 query rows a KV head), the step
+        uploads no more than DIRECT_BYTES, the memory is pinned and 16-byte aligned and no chunks are asked for, there are none: the
+        attention launch itself reads a list's rows from host memory when a CTA takes the list and writes its outputs there, and the
+        outputs are those of verify_step bit for bit.
 
-        A chunk of few lists is split over the SMs for itself, so the outputs are those of verify_step to bf16 rounding.  Large
-        chunks are faster: each is a launch of its own that the next one waits for (32 layers of a 32K context: 178 us in two
-        chunks, 188 in chunks of eight layers, 241 of four, 613 of one; 131 without chunks)."""
+        Else the copies go in chunks of a few layers (layers_per_chunk: one size, or a list of sizes) on two side streams, which fork
+        from and join the current one: a chunk's layers start as soon as its inputs have arrived, its outputs leave while the next
+        chunk computes, so only the first upload and the last download are not hidden behind kernels.  A chunk of few lists is
+        split over the SMs for itself, so the outputs are those of verify_step to bf16 rounding.  Large chunks are faster: each is a
+        launch of its own that the next one waits for.
+
+        32 layers of a 32K context that all select, on one machine: 142 us without chunks, 176 in two, 184 in chunks of eight layers,
+        224 of four, 550 of one."""
         if layers_per_chunk is None and self._direct and self._stacked() and \
                 self._from_host(None, q_host, draft_k_host, draft_v_host, q, draft_k, draft_v, out, out_host, refresh_tail):
             return
